@@ -855,7 +855,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1) stream_tail_kernel(const __g
 
     if (warp == NW) {
         // ---------------- producer: stream the slab, once per chunk of hidden rows ----------------
-        if (lane == 0) {
+        if (elect_one()) {
             const int total = nchunks * nslots;
             const uint16_t* slab = p.W + (size_t)v0 * p.d;
             int st = 0, round = 0, slot = 0;

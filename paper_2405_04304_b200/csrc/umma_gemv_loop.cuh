@@ -249,7 +249,7 @@ umma_gemv_loop_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_c
         // ------------------------------ producer ------------------------------
         // One thread requests every LM-head stage of every step.  Its loop keeps running counters (no
         // divisions) and does nothing but test two barriers and issue copies; it sleeps when there is nothing to do.
-        if (lane == 0 && total > 0) {
+        if (total > 0 && elect_one()) {
             const uint32_t w_bytes = (uint32_t)g.TRN * 128u;
             int w_step = 0, w_n = 0, w_tile = 0, w_kb = 0;     // the next stage to request: step, stage of the step, tile, k-block
             int w_row = v_begin;                                // first LM-head row of that step's slab in the tensor map
@@ -333,7 +333,7 @@ umma_gemv_loop_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_c
         }
     } else if (warp == 1) {
         // ------------------------------ MMA issuer ------------------------------
-        if (lane == 0 && total > 0) {
+        if (total > 0 && elect_one()) {
             const uint32_t idesc = umma_idesc(g.TRN);
             int slot = 0, fill = 0, t_global = 0;
             for (int step0 = 0; step0 < lp.steps; ++step0) {

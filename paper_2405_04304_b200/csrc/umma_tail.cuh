@@ -81,12 +81,15 @@ struct UmmaParams {
 // ---------------------------------------------------------------------------------------------
 // PTX wrappers
 // ---------------------------------------------------------------------------------------------
-__device__ __forceinline__ void tma_load_2d(void* dst_smem, const CUtensorMap* tmap, int c0, int c1, uint64_t* bar) {
+__device__ __forceinline__ void tma_load_2d(uint32_t dst_smem, const CUtensorMap* tmap, int c0, int c1, uint32_t bar) {
     asm volatile(
         "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
-            smem_addr(dst_smem)),
-        "l"(tmap), "r"(c0), "r"(c1), "r"(smem_addr(bar))
+            dst_smem),
+        "l"(tmap), "r"(c0), "r"(c1), "r"(bar)
         : "memory");
+}
+__device__ __forceinline__ void tma_load_2d(void* dst_smem, const CUtensorMap* tmap, int c0, int c1, uint64_t* bar) {
+    tma_load_2d(smem_addr(dst_smem), tmap, c0, c1, smem_addr(bar));
 }
 // Bring one box of a tensor map into L2 (no shared-memory destination, nothing to wait for).
 __device__ __forceinline__ void tma_prefetch_l2_2d(const CUtensorMap* tmap, int c0, int c1) {
@@ -108,10 +111,10 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_commit(uint64_t* bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_addr(bar))
-                 : "memory");
+__device__ __forceinline__ void tc_commit(uint32_t bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
+__device__ __forceinline__ void tc_commit(uint64_t* bar) { tc_commit(smem_addr(bar)); }
 __device__ __forceinline__ void tc_mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
                                             uint32_t accumulate) {
     asm volatile(
@@ -277,70 +280,77 @@ umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_consta
 
     if (warp == 0) {
         // ------------------------------ producer ------------------------------
-        if (lane == 0 && live) {
-            int stage = 0, phase = 0;
+        if (live && elect_one()) {
+            // A single thread: running addresses and counters, as few instructions per stage as possible.
+            const uint32_t full0 = smem_addr(full), empty0 = smem_addr(empty), a0 = smem_addr(a_tiles), b0 = smem_addr(b_tiles);
             const uint32_t bytes = (uint32_t)(p.rep * p.a_rows + p.TRN) * 128u;   // the boxes of the two tensor maps
+            const int k_end = KB * kUmmaBK, h_row = m_tile * 128;
             // The LM head is never written by this library: its first tiles are requested before the
             // dependency wait, the hidden-state tiles of the same stages right after it.
-            int pre = 0;
-            {
-                const int v0 = nslot * gTPC * gTR;
-                if (v0 < p.V) {
-                    pre = min(p.stages, KB);
-                    for (int kb = 0; kb < pre; ++kb) {
-                        mbar_arrive_expect_tx(&full[kb], bytes);
-                        tma_load_2d(b_tiles + kb * p.b_bytes, &tmap_W, kb * kUmmaBK, v0, &full[kb]);
-                    }
-                }
+            int v0 = nslot * gTPC * gTR;
+            const int pre = v0 < p.V ? min(p.stages, KB) : 0;
+            auto load_h = [&](uint32_t dst, int k, uint32_t bar) {
+                for (int c = 0; c < p.rep; ++c) tma_load_2d(dst + c * p.rows_pad * 128, &tmap_H, k, h_row, bar);
+            };
+            for (int n = 0; n < pre; ++n) {
+                mbar_arrive_expect_tx(full0 + n * 8, bytes);
+                tma_load_2d(b0 + n * p.b_bytes, &tmap_W, n * kUmmaBK, v0, full0 + n * 8);
             }
             asm volatile("griddepcontrol.wait;" ::: "memory");
-            int n = 0;
-            for (int i = 0; i < gTPC; ++i) {
-                const int v0 = (nslot * gTPC + i) * gTR;
-                if (v0 >= p.V) break;
-                for (int kb = 0; kb < KB; ++kb, ++n) {
-                    if (n >= pre) {
-                        mbar_wait(&empty[stage], phase ^ 1, p.status);
-                        mbar_arrive_expect_tx(&full[stage], bytes);
-                        tma_load_2d(b_tiles + stage * p.b_bytes, &tmap_W, kb * kUmmaBK, v0, &full[stage]);
-                    }
-                    for (int c = 0; c < p.rep; ++c)
-                        tma_load_2d(a_tiles + stage * p.a_bytes + c * p.rows_pad * 128, &tmap_H, kb * kUmmaBK,
-                                    m_tile * 128, &full[stage]);
+            for (int n = 0; n < pre; ++n) load_h(a0 + n * p.a_bytes, n * kUmmaBK, full0 + n * 8);
+            int stage = pre == p.stages ? 0 : pre, phase = pre == p.stages ? 1 : 0;
+            int k = pre * kUmmaBK;
+            uint32_t at_a = a0 + stage * p.a_bytes, at_b = b0 + stage * p.b_bytes;
+            for (int i = 0; i < gTPC && v0 < p.V; ++i, v0 += gTR, k = 0) {
+                for (; k < k_end; k += kUmmaBK) {
+                    const uint32_t bar = full0 + stage * 8;
+                    mbar_wait(empty0 + stage * 8, phase ^ 1, p.status);
+                    mbar_arrive_expect_tx(bar, bytes);
+                    tma_load_2d(at_b, &tmap_W, k, v0, bar);
+                    load_h(at_a, k, bar);
+                    at_a += p.a_bytes;
+                    at_b += p.b_bytes;
                     if (++stage == p.stages) {
                         stage = 0;
                         phase ^= 1;
+                        at_a = a0;
+                        at_b = b0;
                     }
                 }
             }
         }
     } else if (warp == 1) {
         // ------------------------------ MMA issuer ------------------------------
-        if (lane == 0 && live) {
-            int stage = 0, phase = 0, it = 0;
+        if (live && elect_one()) {
             const uint32_t idesc = umma_idesc(gTRN);
+            const uint32_t full0 = smem_addr(full), empty0 = smem_addr(empty);
+            const uint64_t a0 = umma_smem_desc(a_tiles), b0 = umma_smem_desc(b_tiles);
+            const uint32_t a_step = (uint32_t)p.a_bytes >> 4, b_step = (uint32_t)p.b_bytes >> 4;   // descriptor units
+            uint64_t a_desc = a0, b_desc = b0;
+            int stage = 0, phase = 0;
             for (int i = 0; i < gTPC; ++i) {
                 if ((nslot * gTPC + i) * gTR >= p.V) break;
-                const int buf = it & 1;
-                mbar_wait(&tmem_empty[buf], ((it >> 1) & 1) ^ 1, p.status);
+                const int buf = i & 1;
+                mbar_wait(&tmem_empty[buf], ((i >> 1) & 1) ^ 1, p.status);
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + buf * 256;
                 for (int kb = 0; kb < KB; ++kb) {
-                    mbar_wait(&full[stage], phase, p.status);
+                    mbar_wait(full0 + stage * 8, phase, p.status);
                     tc_fence_after();
-                    const uint64_t a_desc = umma_smem_desc(a_tiles + stage * p.a_bytes);
-                    const uint64_t b_desc = umma_smem_desc(b_tiles + stage * p.b_bytes);
 #pragma unroll
                     for (int k = 0; k < kUmmaBK / 16; ++k)  // 16 k-elements = 32 bytes = 2 descriptor units
                         tc_mma_bf16(d_tmem, a_desc + 2 * k, b_desc + 2 * k, idesc, (kb | k) != 0);
-                    tc_commit(&empty[stage]);
+                    tc_commit(empty0 + stage * 8);
+                    a_desc += a_step;
+                    b_desc += b_step;
                     if (++stage == p.stages) {
                         stage = 0;
                         phase ^= 1;
+                        a_desc = a0;
+                        b_desc = b0;
                     }
                 }
                 tc_commit(&tmem_full[buf]);
-                ++it;
             }
         }
     } else if (live) {
