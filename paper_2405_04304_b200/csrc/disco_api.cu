@@ -12,6 +12,7 @@
 #include "disco.h"
 #include "stream_tail.cuh"
 #include "umma_tail.cuh"
+#include "draft_batch.cuh"
 #include "sample.cuh"
 #include "umma_gemv.cuh"
 #include "umma_gemv_loop.cuh"
@@ -70,6 +71,7 @@ struct disco_ctx {
     void* loop_rec;                // persistent draft-phase kernel: stamped 80-byte records, [4][CTA]; written by nothing else
     void* part_rec;                // draft step: 64-byte partial records, [sequence][CTA]
     void* stamped_rec;             // batched draft step: stamped 80-byte records, [sequence][CTA]; written by nothing else
+    unsigned int* row_bound;       // batched draft step: two sets of [part_rows][kDbBoundStride] words, see DraftBatchParams
     int part_slots;                // partials per row the buffers can hold
     void* encode_tiled;            // cuTensorMapEncodeTiled, resolved through the runtime
     // device staging for the *_host entry points
@@ -217,10 +219,8 @@ bool umma_possible(const disco_ctx* c, int R) {
     return c->encode_tiled != nullptr && MT <= c->sm_count;
 }
 
-// Launch the tcgen05 kernel for R hidden rows of width d against the LM head W [V, d].
-template <bool DRAFT, bool STATS = false>
-int launch_umma(disco_ctx* c, const void* W, const void* H, int d, int R, float* probs,
-                const DraftFinalParams* draft_final, const UmmaParams* fused, cudaStream_t st,
+// Launch the tcgen05 verification kernel for R hidden rows of width d against the LM head W [V, d].
+int launch_umma(disco_ctx* c, const void* W, const void* H, int d, int R, const UmmaParams* fused, cudaStream_t st,
                 const int32_t* dev_R = nullptr) {
     UmmaParams p{};
     if (fused) p = *fused;  // verification finished by the main kernel's last CTA
@@ -229,66 +229,97 @@ int launch_umma(disco_ctx* c, const void* W, const void* H, int d, int R, float*
     p.R = R;
     p.MT = (R + 127) / 128;
     p.CN = c->sm_count / p.MT;
-    // Vocabulary rows per tile: up to 256 for verification (its epilogue is a compare per logit); the
-    // draft step's epilogue is heavy (soft-max, top-10), so it gets several small tiles per CTA and
-    // the epilogue of one tile runs under the loads of the next.
-    const int tile_target = (DRAFT && !STATS) ? (R <= 128 ? 128 : 256) : 256;
-    p.TPC = std::max(1, (c->V + tile_target * p.CN - 1) / (tile_target * p.CN));
+    p.TPC = std::max(1, (c->V + 256 * p.CN - 1) / (256 * p.CN));
     p.TR = (c->V + p.CN * p.TPC - 1) / (p.CN * p.TPC);
     p.TRN = std::max(16, (p.TR + 15) / 16 * 16);
     p.dev_R = dev_R;
     if (dev_R) p.TRN = 256;   // the kernel derives the tiling from the device-side row count; the box is the largest tile
     p.a_rows = p.MT > 1 ? 128 : std::max(8, (R + 7) / 8 * 8);
-    // Draft step with few rows: copies of the rows fill the other TMEM lane quadrants, so that the
-    // epilogue (heavy there) runs on every warp scheduler.  Verification's epilogue is a compare per
-    // logit and keeps the smaller stage instead.
-    p.rep = (DRAFT && !STATS && R <= 64) ? (R <= 32 ? 4 : 2) : 1;   // (measured: no gain for the statistics-only epilogue)
-    p.rows_pad = 128 / p.rep;
-    // The A stage holds a_rows rows (rep copies, rows_pad rows apart).  The MMA still reads 128 rows from
-    // its start: what lies behind the tile (other stages of the ring, always inside it) or between the
-    // copies only feeds accumulator lanes nobody reads.
-    p.a_bytes = p.rep > 1 ? 128 * 128 : (p.a_rows * 128 + 1023) / 1024 * 1024;
+    // The A stage holds a_rows rows.  The MMA still reads 128 rows from its start: what lies behind the tile (other
+    // stages of the ring, always inside it) only feeds accumulator lanes nobody reads.
+    p.a_bytes = (p.a_rows * 128 + 1023) / 1024 * 1024;
     p.b_bytes = (p.TRN * 128 + 1023) / 1024 * 1024;
-    // (the draft step's epilogue keeps its candidate queues in the last bytes of the ring)
-    const int ring_bytes = kUmmaRingBytes - ((DRAFT && !STATS) ? kUmmaQueueBytes : 0);
-    p.stages = std::max(2, std::min(kUmmaMaxStages, ring_bytes / (p.a_bytes + p.b_bytes)));
+    p.stages = std::max(2, std::min(kUmmaMaxStages, kUmmaRingBytes / (p.a_bytes + p.b_bytes)));
     p.status = c->status;
     p.keys = c->keys;
-    p.part_rec = reinterpret_cast<float4*>(c->stamped_rec);
-    p.probs = probs;
-    if (DRAFT && ((size_t)R * p.CN > (size_t)128 * c->sm_count || R > c->part_rows)) return DISCO_ERR_WORKSPACE;
     CUtensorMap tmap_W, tmap_H;
     if (!encode_bf16_2d(c, &tmap_W, W, c->V, d, p.TRN) || !encode_bf16_2d(c, &tmap_H, H, R, d, p.a_rows))
         return DISCO_ERR_CUDA;
-    auto kern = umma_tail_kernel<DRAFT, STATS>;
     static KernelSetup setup;
-    if (!raise_smem_limit(c, setup, kern, (size_t)kUmmaSmemBytes + umma_clf_bytes(DISCO_MAX_CLF_HIDDEN), nullptr))
-        return DISCO_ERR_CUDA;
+    if (!raise_smem_limit(c, setup, umma_tail_kernel, (size_t)kUmmaSmemBytes, nullptr)) return DISCO_ERR_CUDA;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(dev_R ? c->sm_count : p.MT * p.CN));
     cfg.blockDim = dim3(kUmmaThreads);
-    cfg.dynamicSmemBytes = kUmmaSmemBytes + (draft_final ? umma_clf_bytes(draft_final->clf_H) : 0);
+    cfg.dynamicSmemBytes = kUmmaSmemBytes;
     cfg.stream = st;
-    // The draft step's second phase waits for every CTA of the grid: a cooperative launch makes the
-    // driver refuse the launch unless all of them can be resident at once.
-    cudaLaunchAttribute attr[2];
-    int na = 0;
-    if (DRAFT) {
-        attr[na].id = cudaLaunchAttributeCooperative;
-        attr[na].val.cooperative = 1;
-        ++na;
-    }
-    if (c->pdl) {
-        attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[na].val.programmaticStreamSerializationAllowed = 1;
-        ++na;
-    }
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = na;
-    const DraftFinalParams f = draft_final ? *draft_final : DraftFinalParams{};
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tmap_W, tmap_H, p, f);
+    cfg.numAttrs = c->pdl ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, umma_tail_kernel, tmap_W, tmap_H, p);
     c->launches += 1;
     return cuda_ok(e, "umma_tail_kernel launch") ? DISCO_OK : DISCO_ERR_CUDA;
+}
+
+// The batched draft step and its relatives need at most kDbMaxRecords CTAs per tile of rows and 28-bit token ids.
+bool draft_batch_possible(const disco_ctx* c, int R) {
+    const int MT = (R + 127) / 128;
+    return c->encode_tiled != nullptr && MT <= c->sm_count && c->sm_count / MT <= kDbMaxRecords && c->V < (int)kDbNoIndex;
+}
+
+// Launch the batched draft step (STATS: arg-max and statistics only) for R hidden rows of width d against W [V, d].
+template <bool STATS>
+int launch_draft_batch(disco_ctx* c, const void* W, const void* H, int d, int R, float* probs, const DraftFinalParams& f,
+                       cudaStream_t st) {
+    DraftBatchParams p{};
+    p.V = c->V;
+    p.d = d;
+    p.R = R;
+    p.MT = (R + 127) / 128;
+    p.CN = c->sm_count / p.MT;
+    // One tile of hidden rows: the LM head arrives slower than the tensor pipe works, so the tiles are small and the
+    // epilogue of one runs under the loads of the next.  More tiles of rows: the rows' tile is loaded again for every
+    // vocabulary tile, and that traffic (L2 to shared memory) is the bound, so the vocabulary tiles are the widest.
+    const int tile_target = R <= 128 ? 128 : 256;
+    p.TPC = std::max(1, (c->V + tile_target * p.CN - 1) / (tile_target * p.CN));
+    p.TR = (c->V + p.CN * p.TPC - 1) / (p.CN * p.TPC);
+    p.TRN = std::max(16, (p.TR + 15) / 16 * 16);
+    p.a_rows = p.MT > 1 ? 128 : std::max(8, (R + 7) / 8 * 8);
+    p.a_bytes = (p.a_rows * 128 + 1023) / 1024 * 1024;
+    p.b_bytes = (p.TRN * 128 + 1023) / 1024 * 1024;
+    if ((size_t)R * p.CN > (size_t)128 * c->sm_count || R > c->part_rows) return DISCO_ERR_WORKSPACE;
+    auto kern = umma_draft_batch_kernel<STATS>;
+    static KernelSetup setup;
+    size_t dyn_limit = 0;
+    if (!raise_smem_limit(c, setup, kern, 0, &dyn_limit)) return DISCO_ERR_CUDA;
+    const size_t fixed = 1024 + 512 + kDbXchBytes + (size_t)(kDbFinWarps * kDbFinWords + 128) * 4 + umma_clf_bytes(f.clf_H) + 128;
+    if (dyn_limit < fixed + 2 * (size_t)(p.a_bytes + p.b_bytes)) return DISCO_ERR_UNSUPPORTED_SHAPE;
+    p.stages = (int)std::min<size_t>(kDbMaxStages, (dyn_limit - fixed) / (p.a_bytes + p.b_bytes));
+    p.ring_bytes = p.stages * (p.a_bytes + p.b_bytes);
+    p.status = c->status;
+    p.part_rec = reinterpret_cast<float4*>(c->stamped_rec);
+    p.probs = probs;
+    p.bound = c->row_bound;
+    p.set_words = (size_t)c->part_rows * kDbBoundStride;
+    p.sync = c->ticket + 48;
+    p.rows_per_claim = (R + kDbFinWarps * p.MT * p.CN - 1) / (kDbFinWarps * p.MT * p.CN);
+    CUtensorMap tmap_W, tmap_H;
+    if (!encode_bf16_2d(c, &tmap_W, W, c->V, d, p.TRN) || !encode_bf16_2d(c, &tmap_H, H, R, d, p.a_rows))
+        return DISCO_ERR_CUDA;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(p.MT * p.CN));
+    cfg.blockDim = dim3(kDbThreads);
+    cfg.dynamicSmemBytes = fixed + p.ring_bytes;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = c->pdl ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tmap_W, tmap_H, p, f);
+    c->launches += 1;
+    return cuda_ok(e, "umma_draft_batch_kernel launch") ? DISCO_OK : DISCO_ERR_CUDA;
 }
 
 
@@ -512,6 +543,8 @@ int disco_create(disco_ctx** out, int V, int d_draft, int d_target, int max_batc
     // R rows take R * (sm_count / ceil(R / 128)) <= 128 * sm_count records
     ok = ok && cudaMalloc(&c->stamped_rec, (size_t)128 * c->sm_count * 80) == cudaSuccess;
     ok = ok && cudaMemset(c->stamped_rec, 0, (size_t)128 * c->sm_count * 80) == cudaSuccess;  // no stamp yet
+    ok = ok && cudaMalloc(&c->row_bound, (size_t)2 * c->part_rows * kDbBoundStride * 4) == cudaSuccess;
+    ok = ok && cudaMemset(c->row_bound, 0, (size_t)2 * c->part_rows * kDbBoundStride * 4) == cudaSuccess;
     ok = ok && cudaMemset(c->status, 0, 256) == cudaSuccess;
     ok = ok && cudaDeviceSynchronize() == cudaSuccess;
     if (!ok) {
@@ -527,6 +560,7 @@ int disco_destroy(disco_ctx* c) {
     cudaFree(c->keys);
     cudaFree(c->part_rec);
     cudaFree(c->stamped_rec);
+    cudaFree(c->row_bound);
     cudaFree(c->ticket);
     cudaFree(c->status);
     cudaFree(c->final_stats);
@@ -673,7 +707,7 @@ int draft_step_common(disco_ctx* c, const void* W_D, const void* h_D, int d, int
     const bool gemv_ok = c->encode_tiled != nullptr && B <= kGemvMaxRows && !stats_only &&
                          (size_t)((d + kUmmaBK - 1) / kUmmaBK) * (B <= 8 ? 8 : 16) * 128 <= 48 * 1024;
     const bool use_gemv = gemv_ok && (c->path == 3 || (c->path == 0 && B <= 4));
-    const bool use_umma = !use_gemv && umma_possible(c, B) && (c->path == 2 || c->path == 3 || (c->path == 0 && B >= 2));
+    const bool use_umma = !use_gemv && draft_batch_possible(c, B) && (c->path == 2 || c->path == 3 || (c->path == 0 && B >= 2));
     // Sampled step: the kernels that end in a last-CTA second phase draw the token there (their records are
     // at most 160 and in vocabulary order); the batched kernel leaves the draw to a follow-up kernel.
     const bool fused_draw = u_draw && probs && !use_umma && (use_gemv || c->max_grid <= 160);
@@ -706,13 +740,12 @@ int draft_step_common(disco_ctx* c, const void* W_D, const void* h_D, int d, int
         f.final_stats = c->final_stats;
         f.nll_sum = nll_sum;
         f.stats_only = stats_only;
-        f.epoch = c->ticket + 48;
         f.test_stamp_skew = c->test_stamp_skew;
         f.clear_words = clear_words;
         f.clear_n = clear_n;
         if (chain) f.chain = *chain;
-        rc = stats_only == 1 ? launch_umma<true, true>(c, W_D, h_D, d, B, probs, &f, nullptr, st)
-                        : launch_umma<true>(c, W_D, h_D, d, B, probs, &f, nullptr, st);
+        rc = stats_only == 1 ? launch_draft_batch<true>(c, W_D, h_D, d, B, probs, f, st)
+                             : launch_draft_batch<false>(c, W_D, h_D, d, B, probs, f, st);
         if (rc) return rc;
     } else {
         rc = run_stream<true>(c, p, clf->H, st);
@@ -789,9 +822,9 @@ int verify_common(disco_ctx* c, const void* W_T, const void* H_T, const int32_t*
         fp.bonus = bonus;
         fp.target_ids = target_ids;
         fp.padded = p.padded;
-        return launch_umma<false>(c, W_T, H_T, c->d_target, R, nullptr, nullptr, &fp, st, dev_R);
+        return launch_umma(c, W_T, H_T, c->d_target, R, &fp, st, dev_R);
     }
-    int rc = launch_umma<false>(c, W_T, H_T, c->d_target, R, nullptr, nullptr, nullptr, st, dev_R);
+    int rc = launch_umma(c, W_T, H_T, c->d_target, R, nullptr, st, dev_R);
     if (rc) return rc;
     VerifyFinalParams f{};
     f.keys = c->keys;

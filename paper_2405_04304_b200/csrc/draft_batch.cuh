@@ -1,0 +1,869 @@
+// Tensor-core draft step for a batch (and, with other epilogue switches, every other pass over an LM head that wants
+// soft-max statistics: the target rows of a verification with sampling, bulk feature extraction).
+//
+//   D[r, v] = sum_k H[r, k] * W[v, k]      r on the 128 TMEM lanes, v on the TMEM columns
+//
+//   * warp 0      producer: one TMA box of H (A operand, up to 128 rows x 64 k) and one of W (B operand, one
+//                 vocabulary tile x 64 k) per stage; the LM-head boxes of the first stages are requested before the
+//                 dependency wait;
+//   * warp 1      issues tcgen05.mma (M = 128, N = tile rows) into one of two or four accumulator buffers in TMEM;
+//   * warps 2-9   epilogue: every thread owns one hidden row and walks over its share of a tile's columns: soft-max
+//                 statistics in registers, and the few logits that can still be among the row's ten largest;
+//   * warps 10-11 finish rows: one warp merges the per-CTA records of a hidden row, forms the features of Eq. 2, runs
+//                 the halt classifier and the stopping rule.
+//
+// What the design is built around:
+//   * The ten largest.  A CTA sees a few hundred columns of each row, so "above this CTA's tenth largest" is no
+//     filter (a tenth of all logits pass), and an insertion network fed by it is half of the epilogue.  The rows share a
+//     bound instead: twelve words per row, each the largest logit published so far by every twelfth CTA of the grid
+//     (atomicMax).  Ten of the twelve groups have a logit at or above the third smallest word, so that is a lower bound
+//     of the row's tenth largest logit, at any time and whatever the timing; the final list is exact.  About twenty of a
+//     row's logits pass it, over all CTAs.
+//   * No waiting on CTAs that may not run.  The finishing warps wait for other CTAs' records, but only once every CTA of
+//     the grid has started (a counter); a CTA that is done before that leaves.  The CTA that starts last always finds
+//     the counter full, so every row is finished by somebody, with any number of other kernels on the device.  So the
+//     launch need not be cooperative, and its prologue and first loads run under the tail of the kernel before it (a
+//     cooperative launch was measured to cost 4 - 5 us in a stream).
+//   * Code that runs once per launch is fetched from L2 instruction by instruction.  Both the finishing code and what
+//     follows the column loop run once for nothing while the first tile is awaited.
+#pragma once
+
+#include "umma_tail.cuh"
+
+namespace disco {
+
+constexpr int kDbEpiWarps = 8;
+constexpr int kDbFinWarps = 2;
+constexpr int kDbThreads = (2 + kDbEpiWarps + kDbFinWarps) * 32;
+constexpr int kDbMaxStages = 16;
+constexpr int kDbMaxRecords = 160;     // records per row a finishing warp takes in: five per lane
+constexpr int kDbCandidates = 128;
+constexpr int kDbXchBytes = 128 * 64;  // states handed between the two warps that share a hidden row
+constexpr int kDbFinWords = 16 + kDbCandidates + 16;   // features, candidates, result; per finishing warp
+constexpr int kDbBoundSlots = 12;      // words of the shared bound per row
+constexpr int kDbBoundStride = 16;     // (rows 64 bytes apart)
+constexpr int kDbChunks = 4;           // chunks of 32 columns per warp and tile, at most
+constexpr uint32_t kDbNoIndex = 0x0fffffffu;           // record word: arg-max index in 28 bits, list length above it
+constexpr float kLog2e = 1.4426950408889634f, kLn2 = 0.6931471805599453f;
+
+struct DraftBatchParams {
+    int V, d, R;
+    int MT;      // tiles of 128 hidden rows
+    int CN;      // CTAs per tile of hidden rows (grid = MT * CN)
+    int TPC;     // vocabulary tiles per CTA
+    int TR;      // vocabulary rows per tile; the MMA and the TMA box use TRN = TR rounded up to 16
+    int TRN;
+    int a_rows;  // rows of the H box (multiple of 8, <= 128)
+    int stages, a_bytes, b_bytes, ring_bytes;
+    int* status;
+    float4* part_rec;      // [R][CN] stamped records of 80 bytes
+    float* probs;          // optional [R][V]: raw logits are written here
+    // Two sets of [set_words / kDbBoundStride] rows: ordered bits of the groups' maxima.  A launch uses the set of its
+    // stamp's parity, which starts zeroed, and zeroes the other one (whose launch is over, so nothing of it is in flight).
+    unsigned int* bound;
+    size_t set_words;
+    // [0] launches so far (the stamp of this launch is that + 1); [2], [3] rows of the last launch of each parity; from
+    // [4] on two sets of (CTAs started, rows claimed), four words apart, used by parity: a launch clears the other
+    unsigned int* sync;
+    int rows_per_claim;
+};
+
+__device__ __forceinline__ float ex2_approx(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float max3f(float a, float b, float c) { return RegTop10::max3(a, b, c); }
+
+__device__ __forceinline__ uint4 ld_relaxed_v4_u32(const unsigned int* p) {
+    uint4 v;
+    asm volatile("ld.relaxed.gpu.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "l"(p)
+                 : "memory");
+    return v;
+}
+// Two columns of the accumulator: lane r of the quadrant receives row r of each.
+__device__ __forceinline__ void tmem_ld_columns(uint32_t a, uint32_t b, float& x, float& y) {
+    uint32_t r, s;
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(a) : "memory");
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(s) : "r"(b) : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(r), "+r"(s)::"memory");
+    x = __uint_as_float(r);
+    y = __uint_as_float(s);
+}
+__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
+    asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+// A shared-memory word that another warp of the CTA is about to make non-zero (bounded).
+__device__ __forceinline__ uint32_t smem_word(const uint32_t* p, int* status) {
+    for (int i = 0; i < (1 << 22); ++i) {
+        const uint32_t v = *reinterpret_cast<const volatile uint32_t*>(p);
+        if (v) return v;
+    }
+    record_status(status, DISCO_ERR_TIMEOUT);
+    return 1u;
+}
+
+// From the twelve words of a row: the bound of its tenth largest logit (the third smallest word); TOP1: of its largest.
+template <bool TOP1>
+__device__ __forceinline__ float row_bound_of(const uint4& a, const uint4& b, const uint4& c) {
+    const unsigned int v[kDbBoundSlots] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z, c.w};
+    unsigned int k;
+    if (TOP1) {
+        k = v[0];
+#pragma unroll
+        for (int i = 1; i < kDbBoundSlots; ++i) k = max(k, v[i]);
+    } else {
+        unsigned int s0 = 0xffffffffu, s1 = 0xffffffffu, s2 = 0xffffffffu;
+#pragma unroll
+        for (int i = 0; i < kDbBoundSlots; ++i) {
+            s2 = min(s2, max(s1, v[i]));
+            s1 = min(s1, max(s0, v[i]));
+            s0 = min(s0, v[i]);
+        }
+        k = s2;
+    }
+    return k ? from_ordered_bits(k) : DISCO_NEG_INF;
+}
+static_assert(kDbBoundSlots - kTopK == 2, "the third smallest of the words bounds the tenth largest logit");
+
+// ---------------------------------------------------------------------------------------------
+// second phase: one warp finishes one hidden row
+// ---------------------------------------------------------------------------------------------
+// A record (five stamped 16-byte pieces, see kStampedPieces): m Z S | word l0 bound | l1 l2 l3 | l4 l5 l6 | l7 l8 l9.
+// word: the arg-max index if the CTA's largest logit passed the bound (kDbNoIndex otherwise), and the number of list
+// entries.  l: the CTA's logits above the bound (at most its ten largest), descending.  bound: the largest bound used.
+// The last two pieces are written only if there are more than four entries.
+//
+// What the lists leave out is at most B = the largest of the records' bounds, and at least ten logits of the row are at
+// or above B: so the row's k-th largest logit is max(B, the k-th largest list entry), for k <= 10.
+
+// Many list entries that cannot be told apart by a threshold (ties, or one CTA holding them all): ten rounds of
+// "largest entry after the last one" over the lists in memory, entries ordered by value, then position.
+static __device__ __noinline__ void db_select_slow(const float4* recs, int NP, uint32_t stamp, float* res, int lane) {
+    float last_v = __int_as_float(0x7f800000);
+    int last_pos = -1;
+    for (int k = 0; k < kTopK; ++k) {
+        float bv = DISCO_NEG_INF;
+        int bp = kNoIndex;
+        for (int c = lane; c < NP; c += 32) {
+            const float4* src = recs + (size_t)c * kStampedPieces;
+            const float4 h = load_relaxed_v4(src + 1);
+            const int cnt = min(kTopK, static_cast<int>(__float_as_uint(h.x) >> 28));
+            for (int i = 0; i < cnt; ++i) {
+                const float4 x = load_relaxed_v4(src + 2 + (i - 1) / 3);
+                // (a late piece of a list is not stamped yet only if nothing of it is wanted: the caller has seen the others)
+                if (i > 0 && __float_as_uint(x.w) != stamp) continue;
+                const int w = (i - 1) % 3;
+                const float v = i == 0 ? h.y : (w == 0 ? x.x : (w == 1 ? x.y : x.z));
+                const int pos = c * 16 + i;
+                const bool after = v < last_v || (v == last_v && pos > last_pos);
+                if (after && v > bv) {   // (positions ascend: the first of equal values stays)
+                    bv = v;
+                    bp = pos;
+                }
+            }
+        }
+        const uint32_t top = __reduce_max_sync(kFullMask, ordered_bits(bv));
+        const int pos = __reduce_min_sync(kFullMask, ordered_bits(bv) == top ? bp : kNoIndex);
+        last_v = from_ordered_bits(top);
+        last_pos = pos;
+        if (lane == 0) res[k] = last_v;
+        if (pos == kNoIndex) break;
+    }
+    __syncwarp();
+}
+
+// real = false: the same instructions on made-up records, nothing read from or written to global memory.
+__device__ __forceinline__ void db_finish_row(const DraftBatchParams& p, const DraftFinalParams& f, int b, bool real,
+                                              uint32_t stamp, float* sm, const float* clf_s, bool stats, int lane) {
+    constexpr int PER = kDbMaxRecords / 32;
+    float* cand = sm + 16;
+    float* res = cand + kDbCandidates;
+    const int NP = real ? p.CN : 0;
+    const float4* recs = p.part_rec + (size_t)b * p.CN * kStampedPieces;
+    // issued with the first poll: what the epilogue needs besides the records
+    const bool chain = f.chain.alive != nullptr;
+    float fpos = 0.f;
+    int nd = 1;
+    bool act = false;
+    if (real) {
+        act = chain_seq_live(f.chain, f.active, b);
+        fpos = chain ? static_cast<float>(f.chain.pos0[b] + f.chain.step) : (f.pos ? static_cast<float>(f.pos[b]) : 0.f);
+        nd = chain ? f.chain.step : (f.n_drafted ? f.n_drafted[b] : 1);
+    }
+    float4 q[PER][3];
+    {
+        const long long t0 = clock64();
+        for (int polls = 0;;) {
+#pragma unroll
+            for (int j = 0; j < PER; ++j) {
+                const float4* src = recs + (size_t)(j * 32 + lane) * kStampedPieces;
+                const bool has = j * 32 + lane < NP;
+#pragma unroll
+                for (int i = 0; i < 3; ++i)
+                    q[j][i] = has ? load_relaxed_v4(src + i) : make_float4(0.f, 0.f, 0.f, __uint_as_float(stamp));
+            }
+            if (!real) {   // made-up records, so that the loops below run
+                q[0][0] = make_float4(lane * 0.125f, 1.f, 0.f, q[0][0].w);
+                q[0][1] = make_float4(__uint_as_float(1u << 28 | lane), lane * 0.125f, 0.f, q[0][1].w);
+            }
+            bool good = true;
+#pragma unroll
+            for (int j = 0; j < PER; ++j)
+#pragma unroll
+                for (int i = 0; i < 3; ++i) good = good && __float_as_uint(q[j][i].w) == stamp;
+            if (__all_sync(kFullMask, good)) break;
+            if ((++polls & 63) == 0) {
+                const bool out = *reinterpret_cast<volatile int*>(p.status) == DISCO_ERR_TIMEOUT ||
+                                 clock64() - t0 > kWaitBudgetClocks;
+                if (__any_sync(kFullMask, out)) {
+                    record_status(p.status, DISCO_ERR_TIMEOUT);
+                    break;
+                }
+            }
+        }
+    }
+    // statistics, arg-max, the largest bound
+    float lm = DISCO_NEG_INF, bound = DISCO_NEG_INF;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        if (q[j][0].y > 0.f) {
+            lm = fmaxf(lm, q[j][0].x);
+            bound = fmaxf(bound, q[j][1].z);
+        }
+    }
+    const float M = from_ordered_bits(__reduce_max_sync(kFullMask, ordered_bits(lm)));
+    bound = from_ordered_bits(__reduce_max_sync(kFullMask, ordered_bits(bound)));
+    float Z = 0.f, S = 0.f;
+    uint32_t idx = kDbNoIndex;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        if (q[j][0].y > 0.f) {
+            const float dm = q[j][0].x - M;
+            const float e = ex2_approx(dm * kLog2e);
+            Z = fmaf(q[j][0].y, e, Z);
+            S = fmaf(e, fmaf(dm, q[j][0].y, q[j][0].z), S);
+            if (dm == 0.f) idx = min(idx, __float_as_uint(q[j][1].x) & kDbNoIndex);
+        }
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        Z += __shfl_xor_sync(kFullMask, Z, off);
+        S += __shfl_xor_sync(kFullMask, S, off);
+    }
+    idx = __reduce_min_sync(kFullMask, idx);
+    float sel = DISCO_NEG_INF;
+    if (!stats) {
+        // Entries above the bound move to shared memory; each lane counts its own first.  More than 32 of them (a grid that
+        // had no bound in time): only those not below theta, the tenth largest of the lanes' largest entries.
+        float theta = DISCO_NEG_INF;
+        int n = 0, mine = 0, incl = 0;
+        bool more = false;    // some list goes on past its fourth entry
+        for (int round = 0; round < 2; ++round) {
+            mine = 0;
+            more = false;
+#pragma unroll
+            for (int j = 0; j < PER; ++j) {
+                const int cnt = static_cast<int>(__float_as_uint(q[j][1].x) >> 28);
+                const float l[4] = {q[j][1].y, q[j][2].x, q[j][2].y, q[j][2].z};
+#pragma unroll
+                for (int k = 0; k < 4; ++k) mine += (k < cnt && l[k] > bound && l[k] >= theta) ? 1 : 0;
+                more = more || (cnt > 4 && l[3] > bound && l[3] >= theta);
+            }
+            incl = mine;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int o = __shfl_up_sync(kFullMask, incl, off);
+                if (lane >= off) incl += o;
+            }
+            n = __shfl_sync(kFullMask, incl, 31);
+            if (n <= 32) break;
+            float head = DISCO_NEG_INF;
+#pragma unroll
+            for (int j = 0; j < PER; ++j)
+                if (__float_as_uint(q[j][1].x) >> 28) head = fmaxf(head, q[j][1].y);
+            const int rank = rank_in_warp(head, lane, cand);
+            theta = __shfl_sync(kFullMask, head, __ffs(__ballot_sync(kFullMask, rank == kTopK - 1)) - 1);
+        }
+        int at = incl - mine;
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+            const int cnt = static_cast<int>(__float_as_uint(q[j][1].x) >> 28);
+            const float l[4] = {q[j][1].y, q[j][2].x, q[j][2].y, q[j][2].z};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                if (k < cnt && l[k] > bound && l[k] >= theta) {
+                    if (at < kDbCandidates) cand[at] = l[k];
+                    ++at;
+                }
+            }
+        }
+        if (__any_sync(kFullMask, more)) {   // (rare) the rest of the long lists
+#pragma unroll 1
+            for (int j = 0; j < PER; ++j) {
+                const int c = j * 32 + lane;
+                int cnt = 0;
+                if (c < NP) cnt = static_cast<int>(__float_as_uint(__ldcg(&recs[(size_t)c * kStampedPieces + 1].x)) >> 28);
+#pragma unroll 1
+                for (int i = 4; i < kTopK; ++i) {
+                    float v = DISCO_NEG_INF;
+                    if (i < cnt) {
+                        const float4* piece = recs + (size_t)c * kStampedPieces + 3 + (i - 4) / 3;
+                        float4 x = load_relaxed_v4(piece);
+                        const long long t0 = clock64();
+                        while (__float_as_uint(x.w) != stamp && clock64() - t0 < kWaitBudgetClocks) x = load_relaxed_v4(piece);
+                        if (__float_as_uint(x.w) != stamp) record_status(p.status, DISCO_ERR_TIMEOUT);
+                        const int w = (i - 4) % 3;
+                        v = w == 0 ? x.x : (w == 1 ? x.y : x.z);
+                    }
+                    const bool take = v > bound && v >= theta && v > DISCO_NEG_INF;
+                    const unsigned mask = __ballot_sync(kFullMask, take);
+                    const int slot = n + __popc(mask & ((1u << lane) - 1u));
+                    if (take && slot < kDbCandidates) cand[slot] = v;
+                    n += __popc(mask);
+                }
+            }
+        }
+        if (lane < kTopK) res[lane] = DISCO_NEG_INF;
+        __syncwarp();
+        if (n <= kDbCandidates) {
+            for (int i = n + lane; i < ((n + 31) & ~31); i += 32) cand[i] = DISCO_NEG_INF;
+            __syncwarp();
+            for (int i = lane; i < n; i += 32) {
+                const float x = cand[i];
+                const int r = rank_in_list(cand, n, x, i);
+                if (r < kTopK) res[r] = x;
+            }
+            __syncwarp();
+        } else {
+            db_select_slow(recs, NP, stamp, res, lane);
+        }
+        if (lane < kTopK) sel = fmaxf(res[lane], bound);
+        __syncwarp();
+    }
+    if (real && !act) return;    // masked: its records were awaited all the same, nothing is written
+    SoftmaxState st;
+    st.m = M, st.Z = Z, st.S = S;
+    const unsigned long long key = argmax_key(M, static_cast<int>(idx));
+    const DraftOutputs o{f.token, f.conf, f.halt, f.feats, f.final_stats, f.nll_sum, f.stats_only, f.chain, real};
+    const int Hc = f.clf_H;
+    warp_draft_epilogue(st, key, sel, fpos, nd, f.tau, f.sl_max, sm, clf_s, clf_s + Hc * kNFeat, clf_s + Hc * (kNFeat + 1),
+                        clf_s + Hc * (kNFeat + 2), Hc, b, o, lane);
+}
+
+// ---------------------------------------------------------------------------------------------
+// main kernel
+// ---------------------------------------------------------------------------------------------
+// STATS: arg-max and soft-max statistics only (f.stats_only == 1), no list of the ten largest.
+template <bool STATS>
+__global__ void __launch_bounds__(kDbThreads, 1)
+umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_constant__ CUtensorMap tmap_H,
+                        const DraftBatchParams p, const DraftFinalParams f) {
+    extern __shared__ uint8_t smem_dyn[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023));
+    uint8_t* a_tiles = smem;
+    uint8_t* b_tiles = smem + p.stages * p.a_bytes;
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + p.ring_bytes);
+    uint64_t* empty = full + kDbMaxStages;
+    uint64_t* tmem_full = empty + kDbMaxStages;
+    uint64_t* tmem_empty = tmem_full + 4;
+    uint32_t* tmem_base_s = reinterpret_cast<uint32_t*>(tmem_empty + 4);
+    int* s_done = reinterpret_cast<int*>(tmem_base_s + 1);    // epilogue warps that have published their records
+    uint32_t* s_stamp = tmem_base_s + 2;                      // stamp of this launch (0: not read yet, or nothing to do)
+    float4* xch = reinterpret_cast<float4*>(reinterpret_cast<uint8_t*>(full) + 512);
+    float* fin_s = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(xch) + kDbXchBytes);
+    float* row_thr_s = fin_s + kDbFinWarps * kDbFinWords;     // [128] the rows' bounds
+    float* clf_s = row_thr_s + 128;
+
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+
+    const int warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
+    const int KB = (p.d + kUmmaBK - 1) / kUmmaBK;
+    const int m_tile = blockIdx.x % p.MT;
+    const int nslot = blockIdx.x / p.MT;
+    const int v_first = nslot * p.TPC * p.TR;                 // this CTA's vocabulary rows: its tiles in sequence
+    const int tiles = v_first < p.V ? min(p.TPC, (p.V - v_first + p.TR - 1) / p.TR) : 0;
+    const bool chained = f.chain.alive != nullptr && f.chain.step > 1;
+    const int nbuf = p.TRN <= 128 ? 4 : 2, buf_cols = 512 / nbuf;   // accumulator buffers in TMEM
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < p.stages; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        for (int b = 0; b < nbuf; ++b) {
+            mbar_init(&tmem_full[b], 1);
+            mbar_init(&tmem_empty[b], kDbEpiWarps);
+        }
+        *s_done = 0;
+        *s_stamp = 0u;
+        fence_mbar_init();
+        prefetch_tensormap(&tmap_W);
+        prefetch_tensormap(&tmap_H);
+    }
+    if (warp == 1) {
+        tmem_alloc(tmem_base_s, 512);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_base_s;
+
+    if (warp == 0) {
+        // ------------------------------ producer ------------------------------
+        const int total = tiles * KB;
+        const uint32_t w_bytes = (uint32_t)p.TRN * 128u, h_bytes = (uint32_t)p.a_rows * 128u;
+        // The LM head is never written by this library: its first stages are requested before the dependency wait.
+        // (A step of a draft phase that has already ended does not: the flags are read ahead of the wait for that,
+        // they may be old and decide nothing else.)
+        int pre = min(p.stages, total);
+        if (chained && !chain_any_live(f.chain, f.B, lane)) pre = 0;
+        // Every CTA reads the same hidden rows.  Each starts at another k-block, so that they do not all ask the same few
+        // L2 slices for the same lines at the same time.
+        const int rot = nslot % KB;
+        // A single thread issues everything: running addresses and counters, as few instructions per stage as possible.
+        const uint32_t full0 = smem_addr(full), empty0 = smem_addr(empty), a0 = smem_addr(a_tiles), b0 = smem_addr(b_tiles);
+        const int k_end = KB * kUmmaBK, k_first = rot * kUmmaBK, h_row = m_tile * 128;
+        int k = k_first, v0 = v_first, left = KB;      // the next stage to request: k, vocabulary row, k-blocks left of the tile
+        auto advance = [&]() {
+            k += kUmmaBK;
+            if (k == k_end) k = 0;
+            if (--left == 0) {
+                left = KB;
+                v0 += p.TR;
+            }
+        };
+        if (elect_one()) {
+            for (int n = 0; n < pre; ++n, advance()) {
+                mbar_expect_tx(full0 + n * 8, w_bytes);
+                tma_load_2d(b0 + n * p.b_bytes, &tmap_W, k, v0, full0 + n * 8);
+            }
+        }
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        const bool live = !chained || chain_any_live(f.chain, f.B, lane);
+        if (!live) {
+            if (elect_one()) {
+                for (int n = 0; n < pre; ++n) mbar_arrive(&full[n]);
+                for (int n = 0; n < pre; ++n) mbar_wait(&full[n], 0, p.status);   // nothing may still be landing at exit
+            }
+        } else if (elect_one()) {
+            int kh = k_first;
+            for (int n = 0; n < pre; ++n) {
+                mbar_arrive_expect_tx(full0 + n * 8, h_bytes);
+                tma_load_2d(a0 + n * p.a_bytes, &tmap_H, kh, h_row, full0 + n * 8);
+                kh += kUmmaBK;
+                if (kh == k_end) kh = 0;
+            }
+            int stage = pre == p.stages ? 0 : pre, phase = pre == p.stages ? 1 : 0;
+            k = k_first, v0 = v_first, left = KB;      // (the elected thread need not be the one of before)
+            for (int n = 0; n < pre; ++n) advance();
+            uint32_t at_a = a0 + stage * p.a_bytes, at_b = b0 + stage * p.b_bytes;
+            for (int n = pre; n < total; ++n, advance()) {
+                const uint32_t bar = full0 + stage * 8;
+                mbar_wait(empty0 + stage * 8, phase ^ 1, p.status);
+                mbar_arrive_expect_tx(bar, w_bytes + h_bytes);
+                tma_load_2d(at_b, &tmap_W, k, v0, bar);
+                tma_load_2d(at_a, &tmap_H, k, h_row, bar);
+                at_a += p.a_bytes;
+                at_b += p.b_bytes;
+                if (++stage == p.stages) {
+                    stage = 0;
+                    phase ^= 1;
+                    at_a = a0;
+                    at_b = b0;
+                }
+            }
+        }
+    } else if (warp == 1) {
+        // ------------------------------ MMA issuer ------------------------------
+        bool live = true;
+        if (chained) {
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            live = chain_any_live(f.chain, f.B, lane);
+        }
+        if (live && elect_one()) {
+            const uint32_t idesc = umma_idesc(p.TRN);
+            const uint32_t full0 = smem_addr(full), empty0 = smem_addr(empty);
+            // Up to eight rows: the A operand is the one 8-row box read 16 times over (zero stride between the 8-row groups
+            // of the descriptor).  More: the MMA reads 128 rows from the start of the stage; what lies behind the box
+            // (further stages, inside the ring) only feeds accumulator lanes nobody reads.
+            const uint64_t a0 = umma_smem_desc(a_tiles) & (p.a_rows == 8 ? ~(0x3fffull << 32) : ~0ull);
+            const uint64_t b0 = umma_smem_desc(b_tiles);
+            const uint32_t a_step = (uint32_t)p.a_bytes >> 4, b_step = (uint32_t)p.b_bytes >> 4;   // descriptor units
+            uint64_t a_desc = a0, b_desc = b0;
+            int stage = 0, phase = 0;
+            for (int t = 0; t < tiles; ++t) {
+                const int buf = t % nbuf;
+                mbar_wait(&tmem_empty[buf], ((t / nbuf) & 1) ^ 1, p.status);
+                tc_fence_after();
+                const uint32_t d_tmem = tmem_base + buf * buf_cols;
+                for (int kb = 0; kb < KB; ++kb) {
+                    mbar_wait(full0 + stage * 8, phase, p.status);
+                    tc_fence_after();
+#pragma unroll
+                    for (int k = 0; k < kUmmaBK / 16; ++k)  // 16 k-elements = 32 bytes = 2 descriptor units
+                        tc_mma_bf16(d_tmem, a_desc + 2 * k, b_desc + 2 * k, idesc, (kb | k) != 0);
+                    tc_commit(empty0 + stage * 8);
+                    a_desc += a_step;
+                    b_desc += b_step;
+                    if (++stage == p.stages) {
+                        stage = 0;
+                        phase ^= 1;
+                        a_desc = a0;
+                        b_desc = b0;
+                    }
+                }
+                tc_commit(&tmem_full[buf]);
+            }
+        }
+    } else if (warp < 2 + kDbEpiWarps) {
+        // ------------------------------ epilogue ------------------------------
+        const int ew = warp - 2;
+        const int quad = warp & 3;              // TMEM lane quadrant this warp may read
+        const int share = ew >> 2;              // the two warps of a quadrant split the columns of a tile
+        const int tile_row = quad * 32 + lane;  // row within this tile of hidden rows
+        const int row = m_tile * 128 + tile_row;
+        const bool warp_has_rows = m_tile * 128 + quad * 32 < p.R;
+        const bool valid = row < p.R;
+        // A single narrow tile is not worth a bound.  With four accumulator buffers the candidates of a tile are looked for
+        // one tile later, when the bound that everybody's tiles give has long arrived; otherwise the first tile waits for it.
+        const bool use_bound = p.TPC > 1 || p.TR > 32;
+        const bool defer = nbuf == 4 && tiles > 1;
+        const uint32_t t_quad = tmem_base + (static_cast<uint32_t>(quad * 32) << 16);
+        volatile float* thr_s = row_thr_s + tile_row;
+        // Twice: a rehearsal without columns before the dependency wait (what follows the column loop is on the critical
+        // path, and its instructions would come from L2 one after the other), then for good.
+        for (int phase = 0; phase < 2; ++phase) {
+            bool keep_logits = false;
+            unsigned int *slots = nullptr, *my_slot = nullptr;
+            float m = DISCO_NEG_INF, Z = 0.f, S2 = 0.f;      // S2 = sum e^(z - m) (z - m) / ln 2
+            float best_v = DISCO_NEG_INF;
+            int best_i = 0;
+            RegTop10 top;
+            top.init();
+            float thr = DISCO_NEG_INF;     // logits at or below it are not among the row's ten largest (or equal its bound)
+            float bound_used = DISCO_NEG_INF;
+            if (phase == 0) {
+                m = best_v = top.t[0] = static_cast<float>(lane);
+                Z = 1.f;
+            } else {
+                asm volatile("griddepcontrol.wait;" ::: "memory");  // scratch and outputs belong to the predecessor until now
+                if (chained && !chain_any_live(f.chain, f.B, lane)) break;
+                const uint32_t stamp = *reinterpret_cast<volatile unsigned int*>(p.sync) + 1u;
+                const uint32_t par = stamp & 1u;
+                const int old_rows = *reinterpret_cast<volatile unsigned int*>(p.sync + 2 + (par ^ 1u));
+                if (blockIdx.x == 0)
+                    for (int i = ew * 32 + lane; i < f.clear_n; i += kDbEpiWarps * 32) f.clear_words[i] = 0u;
+                // the optional probs output receives the raw logits of this row, unless the sequence is masked
+                keep_logits = p.probs && valid && (!f.active || f.active[row]);
+                slots = p.bound + par * p.set_words + (size_t)(valid ? row : 0) * kDbBoundStride;
+                my_slot = slots + nslot % kDbBoundSlots;
+                uint4* old = reinterpret_cast<uint4*>(p.bound + (par ^ 1u) * p.set_words);
+                for (int i = blockIdx.x * (kDbEpiWarps * 32) + ew * 32 + lane; i < old_rows * (kDbBoundStride / 4);
+                     i += gridDim.x * (kDbEpiWarps * 32))
+                    old[i] = make_uint4(0, 0, 0, 0);
+                __syncwarp();
+                if (ew == 0 && lane == 0) {
+                    // This CTA has started, now that it has read the stamp (nobody moves it before all CTAs have started).
+                    *reinterpret_cast<volatile uint32_t*>(s_stamp) = stamp;
+                    atomicAdd(p.sync + 4 + 4 * par, 1u);
+                }
+            }
+            const int phase_tiles = phase == 0 ? 0 : tiles;
+
+            // Tile by tile: statistics and the chunks' maxima, the tile's maximum to the shared bound, then the candidates.
+            float cm[kDbChunks], cm_prev[kDbChunks];
+#pragma unroll
+            for (int i = 0; i < kDbChunks; ++i) cm[i] = cm_prev[i] = DISCO_NEG_INF;
+            for (int t = 0; t < phase_tiles; ++t) {
+                mbar_wait(&tmem_full[t % nbuf], (t / nbuf) & 1, p.status);
+                tc_fence_after();
+                const int ncols = min(p.TR, p.V - (v_first + t * p.TR));  // further columns belong to the next tile or lie past V
+                const int half = (((ncols + 31) >> 5) + 1) >> 1;
+                const int c_lo = share == 0 ? 0 : half, c_hi = share == 0 ? half : (ncols + 31) >> 5;
+                const uint32_t t_buf = t_quad + (t % nbuf) * buf_cols;
+                const bool look = use_bound && valid && share == 0;   // one thread per row looks the bound up
+                uint4 sa = make_uint4(0, 0, 0, 0), sb = sa, sc = sa;  // (on its way during the statistics)
+                if (look && t > 0) {
+                    sa = ld_relaxed_v4_u32(slots);
+                    sb = ld_relaxed_v4_u32(slots + 4);
+                    sc = ld_relaxed_v4_u32(slots + 8);
+                }
+                if (warp_has_rows) {
+                    float tile_max = DISCO_NEG_INF;
+#pragma unroll
+                    for (int i = 0; i < kDbChunks; ++i) cm_prev[i] = cm[i];
+#pragma unroll 1
+                    for (int c = c_lo; c < c_hi; ++c) {
+                        float z[32];
+                        tmem_ld32(t_buf + c * 32, z);
+                        const int n = ncols - c * 32;           // columns of the chunk that count
+                        if (n < 32) {
+#pragma unroll
+                            for (int j = 0; j < 32; ++j)
+                                if (j >= n) z[j] = DISCO_NEG_INF;
+                        }
+                        float g[4];
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const float x = max3f(z[8 * q], z[8 * q + 1], z[8 * q + 2]), y = max3f(z[8 * q + 3], z[8 * q + 4], z[8 * q + 5]);
+                            g[q] = max3f(x, y, fmaxf(z[8 * q + 6], z[8 * q + 7]));
+                        }
+                        const float cmax = fmaxf(max3f(g[0], g[1], g[2]), g[3]);
+                        tile_max = fmaxf(tile_max, cmax);
+#pragma unroll
+                        for (int i = kDbChunks - 1; i > 0; --i) cm[i] = cm[i - 1];   // cm[0]: the tile's last chunk
+                        cm[0] = cmax;
+                        // the reference maximum moves first, then the chunk is added
+                        const float mn = fmaxf(m, cmax);
+                        const float dm = fmaxf((m - mn) * kLog2e, -1000.f);
+                        const float em = ex2_approx(dm);
+                        m = mn;
+                        if (n < 32) {   // masked columns: finite, far below the maximum (e = 0, and 0 * -inf is avoided)
+#pragma unroll
+                            for (int j = 0; j < 32; ++j)
+                                if (j >= n) z[j] = mn - 1000.f;
+                        }
+                        const float nm = -mn * kLog2e;
+                        float Za = 0.f, Sa = 0.f, Zb = 0.f, Sb = 0.f;
+#pragma unroll
+                        for (int j = 0; j < 32; j += 2) {
+                            const float ta = fmaf(z[j], kLog2e, nm), tb = fmaf(z[j + 1], kLog2e, nm);
+                            const float ea = ex2_approx(ta), eb = ex2_approx(tb);
+                            Za += ea;
+                            Sa = fmaf(ea, ta, Sa);
+                            Zb += eb;
+                            Sb = fmaf(eb, tb, Sb);
+                        }
+                        S2 = fmaf(em, fmaf(dm, Z, S2), Sa + Sb);   // (Z = S2 = 0 before the first chunk)
+                        Z = fmaf(Z, em, Za + Zb);
+                        if (keep_logits) {
+                            const int v = v_first + t * p.TR + c * 32;
+                            float* dst = p.probs + (size_t)row * p.V + v;
+                            if ((((uintptr_t)p.probs & 15) | ((p.V | v) & 3)) == 0 && n >= 32) {  // 16-byte stores
+#pragma unroll
+                                for (int j = 0; j < 32; j += 4)
+                                    *reinterpret_cast<float4*>(dst + j) = make_float4(z[j], z[j + 1], z[j + 2], z[j + 3]);
+                            } else {
+#pragma unroll
+                                for (int j = 0; j < 32; ++j)
+                                    if (j < n) dst[j] = z[j];
+                            }
+                        }
+                    }
+                    if (use_bound) {
+                        if (valid && c_lo < c_hi && (t == 0 || t + 1 < tiles) && tile_max > bound_used)
+                            atomicMax(my_slot, ordered_bits(tile_max + 0.f));
+                        if (t > 0 || !defer) {
+                            if (t == 0 && share == 0) {
+                                // (not waited for longer than the round trips of this CTA's own word and a slow neighbour's:
+                                // the bound only saves work)
+                                for (int k = 0; k < 4; ++k) {
+                                    if (look) {
+                                        sa = ld_relaxed_v4_u32(slots);
+                                        sb = ld_relaxed_v4_u32(slots + 4);
+                                        sc = ld_relaxed_v4_u32(slots + 8);
+                                    }
+                                    if (__all_sync(kFullMask, !valid || row_bound_of<STATS>(sa, sb, sc) > DISCO_NEG_INF)) break;
+                                }
+                            }
+                            if (look) *thr_s = row_bound_of<STATS>(sa, sb, sc);
+                            named_barrier_sync(4 + quad, 64);   // the two warps of the quadrant (a later bound would do too)
+                            if (valid) bound_used = fmaxf(bound_used, *thr_s);
+                        }
+                    }
+                }
+                for (int tc = defer && t > 0 ? t - 1 : t; tc <= t; ++tc) {
+                    if (defer && tc == t && t + 1 < tiles) break;       // later, with a better bound
+                    const int nc = min(p.TR, p.V - (v_first + tc * p.TR));
+                    const int mid = (((nc + 31) >> 5) + 1) >> 1;
+                    const int lo = share == 0 ? 0 : mid, hi = share == 0 ? mid : (nc + 31) >> 5;
+                    thr = fmaxf(thr, bound_used);
+                    // Chunks that hold a logit that can still be among some row's ten largest (STATS: its largest).  A logit
+                    // equal to the bound counts for the arg-max only: the finishing warp fills the list up with the bound.
+                    unsigned flagged = 0u;
+#pragma unroll
+                    for (int i = 0; i < kDbChunks; ++i) {
+                        const float x = tc == t ? cm[i] : cm_prev[i];
+                        const bool want = valid && x >= thr && (x > best_v || (!STATS && x > thr));
+                        if (warp_has_rows && hi - lo > i && __any_sync(kFullMask, want)) flagged |= 1u << i;
+                    }
+                    while (flagged) {   // (bit i: the i-th last chunk; the first columns come first)
+                        const int i = 31 - __clz(flagged);
+                        flagged &= ~(1u << i);
+                        const int c = hi - 1 - i;
+                        const uint32_t t_chunk = t_quad + (tc % nbuf) * buf_cols + c * 32;
+                        float z[32];
+                        tmem_ld32(t_chunk, z);
+                        const int n = nc - c * 32;
+                        float cut = thr;
+                        if (STATS) {   // only the chunk's largest can be the row's
+#pragma unroll
+                            for (int j = 0; j < 32; ++j) cut = fmaxf(cut, j < n ? z[j] : DISCO_NEG_INF);
+                        }
+                        unsigned bits = 0u;
+#pragma unroll
+                        for (int j = 0; j < 32; ++j)
+                            if (z[j] >= cut) bits |= 1u << j;
+                        if (n < 32) bits &= (1u << n) - 1u;
+                        if (!valid) bits = 0u;
+                        const int v = v_first + tc * p.TR + c * 32;
+                        for (unsigned left = __reduce_or_sync(kFullMask, bits); left != 0u;) {
+                            // two columns at a time (the second may be the first again: it is then left out)
+                            const int j = __ffs(left) - 1;
+                            left &= left - 1u;
+                            const int k = left ? __ffs(left) - 1 : j;
+                            left &= left - 1u;
+                            float x, y;
+                            tmem_ld_columns(t_chunk + j, t_chunk + k, x, y);
+                            x = (bits >> j) & 1u ? x : DISCO_NEG_INF;
+                            y = ((bits >> k) & 1u) && k != j ? y : DISCO_NEG_INF;
+                            if (x > best_v) {
+                                best_v = x;
+                                best_i = v + j;
+                            }
+                            if (y > best_v) {
+                                best_v = y;
+                                best_i = v + k;
+                            }
+                            if (!STATS) {
+                                top.push2(x > thr ? x : DISCO_NEG_INF, y > thr ? y : DISCO_NEG_INF);
+                                thr = fmaxf(thr, top.t[kTopK - 1]);
+                            }
+                        }
+                    }
+                    // this tile's accumulator columns are free again
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&tmem_empty[tc % nbuf]);
+                }
+            }
+
+            // one record per hidden row and CTA: the warp with share 1 hands its rows' state to the one with share 0
+            float4* xrow = xch + tile_row * 4;
+            if (share != 0) {
+                xrow[0] = make_float4(m, Z, S2, __int_as_float(best_i));
+                xrow[1] = make_float4(best_v, bound_used, top.t[0], top.t[1]);
+                xrow[2] = make_float4(top.t[2], top.t[3], top.t[4], top.t[5]);
+                xrow[3] = make_float4(top.t[6], top.t[7], top.t[8], top.t[9]);
+            }
+            named_barrier_sync(2, kDbEpiWarps * 32);
+            if (share == 0 && warp_has_rows) {
+                const float4 a = xrow[0], b4 = xrow[1], c4 = xrow[2], d4 = xrow[3];
+                // (a share without columns has Z = 0 and m = -inf; a CTA without columns leaves a record with Z = 0)
+                const float M = fmaxf(m, a.x);
+                const float d1 = Z > 0.f ? (m - M) * kLog2e : 0.f, d2 = a.y > 0.f ? (a.x - M) * kLog2e : 0.f;
+                const float e1 = ex2_approx(d1), e2 = ex2_approx(d2);
+                S2 = e1 * fmaf(d1, Z, S2) + e2 * fmaf(d2, a.y, a.z);
+                Z = Z * e1 + a.y * e2;
+                m = M;
+                const int i2 = __float_as_int(a.w);
+                if (b4.x > best_v || (b4.x == best_v && i2 < best_i)) {
+                    best_v = b4.x;
+                    best_i = i2;
+                }
+                bound_used = fmaxf(bound_used, b4.y);
+                uint32_t cnt = 0;
+                if (!STATS) {
+                    const float theirs[kTopK] = {b4.z, b4.w, c4.x, c4.y, c4.z, c4.w, d4.x, d4.y, d4.z, d4.w};
+                    top.merge(theirs);
+#pragma unroll
+                    for (int k = 0; k < kTopK; ++k) {
+                        cnt += top.t[k] > DISCO_NEG_INF ? 1u : 0u;
+                        top.t[k] += 0.f;   // -0 and +0 are the same logit
+                    }
+                }
+                if (valid && phase == 1) {
+                    const uint32_t word = (cnt << 28) | (best_v == m && Z > 0.f ? (uint32_t)best_i : kDbNoIndex);
+                    float4* rec = p.part_rec + ((size_t)row * p.CN + nslot) * kStampedPieces;
+                    const float sf = __uint_as_float(smem_word(s_stamp, p.status));   // (written microseconds ago)
+                    store_relaxed_v4(rec, m + 0.f, Z, S2 * kLn2, sf);
+                    store_relaxed_v4(rec + 1, __uint_as_float(word), top.t[0], bound_used, sf);
+                    store_relaxed_v4(rec + 2, top.t[1], top.t[2], top.t[3], sf);
+                    if (cnt > 4) {
+                        store_relaxed_v4(rec + 3, top.t[4], top.t[5], top.t[6], sf);
+                        store_relaxed_v4(rec + 4, top.t[7], top.t[8], top.t[9], sf);
+                    }
+                }
+            }
+            __syncwarp();
+            if (lane == 0 && phase == 1) {
+                __threadfence_block();
+                atomicAdd(s_done, 1);
+            }
+        }
+    } else {
+        // ------------------------------ finishing warps ------------------------------
+        const int fw = warp - 2 - kDbEpiWarps;
+        float* sm = fin_s + fw * kDbFinWords;
+        if (f.clf_H > 0) {   // classifier parameters -> shared
+            const int Hc = f.clf_H, n1 = Hc * kNFeat;
+            for (int i = fw * 32 + lane; i < n1 + 2 * Hc + 1; i += kDbFinWarps * 32) {
+                const float* src = i < n1 ? f.clf_W1 + i
+                                          : (i < n1 + Hc ? f.clf_b1 + (i - n1)
+                                                         : (i < n1 + 2 * Hc ? f.clf_w2 + (i - n1 - Hc) : f.clf_b2));
+                cp_async4(clf_s + i, src);
+            }
+            cp_async_commit();
+        }
+        uint32_t stamp = 1u;
+        unsigned int* set = nullptr;
+        int b = 0, b_end = 0;
+        for (bool real = false;; real = true) {
+            db_finish_row(p, f, b, real, stamp + (real ? f.test_stamp_skew : 0u), sm, clf_s, STATS, lane);
+            if (real) {
+                ++b;
+            } else {
+                cp_async_wait_all();
+                named_barrier_sync(3, kDbFinWarps * 32);
+                asm volatile("griddepcontrol.wait;" ::: "memory");
+                if (chained && !chain_any_live(f.chain, f.B, lane)) break;
+                stamp = smem_word(s_stamp, p.status);
+                __syncwarp();
+                set = p.sync + 4 + 4 * (stamp & 1u);
+                // Have all CTAs of the grid started?  Until then none of their records may be waited for.
+                int all = 0;
+                if (lane == 0) {
+                    for (;;) {
+                        const bool done = *reinterpret_cast<volatile int*>(s_done) == kDbEpiWarps;
+                        __threadfence_block();
+                        all = ld_relaxed_u32(set) == gridDim.x;
+                        if (all || done) break;
+                        __nanosleep(300);   // (148 CTAs polling one word without a pause held everybody up by 5 us)
+                    }
+                }
+                if (!__shfl_sync(kFullMask, all, 0)) break;
+            }
+            if (b >= b_end) {   // the next rows nobody has taken
+                int first = 0;
+                if (lane == 0) first = (int)atomicAdd(set + 1, 1u);
+                first = __shfl_sync(kFullMask, first, 0);
+                if (first == 0 && lane == 0) {
+                    // All CTAs have started: the stamp can move on, and the counters of the next launch (this one's may
+                    // still be looked at) start at zero.
+                    unsigned int* other = p.sync + 4 + 4 * ((stamp + 1u) & 1u);
+                    other[0] = 0u;
+                    other[1] = 0u;
+                    p.sync[2 + (stamp & 1u)] = (unsigned int)p.R;
+                    p.sync[0] = stamp == 0xffffffffu ? 1u : stamp;   // never zero, and the two sets keep alternating
+                }
+                b = first * p.rows_per_claim;
+                b_end = min(f.B, b + p.rows_per_claim);
+                if (b >= f.B) break;
+            }
+        }
+    }
+
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc(tmem_base, 512);
+    }
+}
+
+}  // namespace disco

@@ -525,17 +525,25 @@ __device__ __forceinline__ void warp_store_record(float* rec, const LaneRecord& 
 // ---------------------------------------------------------------------------------------------
 
 // Halt classifier of Eq. 2 by one warp: C = sigmoid(w2 . relu(W1 x + b1) + b2).  x (lane < 12) is the
-// feature held by that lane; feat_s is 16 words of shared scratch owned by the warp.
+// feature held by that lane; feat_s is 16 words of shared scratch owned by the warp.  feat_s and W1 are shared memory,
+// 16-byte aligned.
 __device__ __forceinline__ float warp_halt_classifier(float x, float* feat_s, const float* W1, const float* b1,
                                                       const float* w2, const float* b2p, int Hc, int lane) {
     if (lane < kNFeat) feat_s[lane] = x;
     __syncwarp();
     const float b2 = b2p[0];
     float acc = 0.f;
+    // (a row of W1 is 48 bytes: three vector loads per unit, the eight lanes of a quarter-warp on all 32 banks)
+    static_assert(kNFeat == 12, "three float4 per row of W1");
+    const float4 f0 = *reinterpret_cast<const float4*>(feat_s), f1 = *reinterpret_cast<const float4*>(feat_s + 4),
+                 f2 = *reinterpret_cast<const float4*>(feat_s + 8);
     for (int j = lane; j < Hc; j += 32) {
+        const float4* w = reinterpret_cast<const float4*>(W1 + j * kNFeat);
+        const float4 q0 = w[0], q1 = w[1], q2 = w[2];
         float a = b1[j];
-#pragma unroll
-        for (int i = 0; i < kNFeat; ++i) a = fmaf(W1[j * kNFeat + i], feat_s[i], a);
+        a = fmaf(q0.x, f0.x, a), a = fmaf(q0.y, f0.y, a), a = fmaf(q0.z, f0.z, a), a = fmaf(q0.w, f0.w, a);
+        a = fmaf(q1.x, f1.x, a), a = fmaf(q1.y, f1.y, a), a = fmaf(q1.z, f1.z, a), a = fmaf(q1.w, f1.w, a);
+        a = fmaf(q2.x, f2.x, a), a = fmaf(q2.y, f2.y, a), a = fmaf(q2.z, f2.z, a), a = fmaf(q2.w, f2.w, a);
         acc = fmaf(w2[j], fmaxf(a, 0.f), acc);
     }
 #pragma unroll
@@ -556,13 +564,14 @@ struct DraftOutputs {
     int stats_only;  // 1: arg-max and soft-max statistics only (rows of a verification with sampling);
                      // 2: token and features, no classifier (bulk feature extraction)
     ChainLink chain; // draft phase chained on the device: the look-ahead bookkeeping goes with the halt flag
+    bool write = true;   // false: compute, write nothing (a warp that only wants the code in its instruction cache)
 };
 __device__ __forceinline__ bool warp_draft_epilogue(const SoftmaxState& st, unsigned long long key, float sel, float fpos,
                                                     int n_drafted, float tau, int sl_max, float* feat_s, const float* W1,
                                                     const float* b1, const float* w2, const float* b2, int Hc, int b,
                                                     const DraftOutputs& o, int lane) {
     if (o.stats_only == 1) {
-        if (lane == 0) {
+        if (lane == 0 && o.write) {
             if (o.token) o.token[b] = key_index(key);
             o.final_stats[2 * b] = st.m;
             o.final_stats[2 * b + 1] = st.Z;
@@ -573,7 +582,7 @@ __device__ __forceinline__ bool warp_draft_epilogue(const SoftmaxState& st, unsi
         // Perplexity rule: the greedy token attains the largest logit, so -ln y(token) = ln Z.  The caller
         // keeps the running sum over the tokens drafted in this iteration; halt when the perplexity of
         // that run exceeds the bound (here passed in tau) or the cap is reached.
-        if (lane == 0) {
+        if (lane == 0 && o.write) {
             const float nll = o.nll_sum[b] + logf(st.Z);
             const float ppl = expf(nll / static_cast<float>(n_drafted));
             o.nll_sum[b] = nll;
@@ -590,17 +599,17 @@ __device__ __forceinline__ bool warp_draft_epilogue(const SoftmaxState& st, unsi
     const float ent = __logf(st.Z) - st.S * inv_Z;
     const float x = lane < kTopK ? prob : (lane == kTopK ? ent : (lane == kTopK + 1 ? fpos : 0.f));
     if (o.stats_only == 2) {
-        if (lane == 0) {
+        if (lane == 0 && o.write) {
             if (o.token) o.token[b] = key_index(key);
             o.final_stats[2 * b] = st.m;
             o.final_stats[2 * b + 1] = st.Z;
         }
-        if (o.feats && lane < kNFeat) o.feats[(size_t)b * kNFeat + lane] = x;
+        if (o.feats && o.write && lane < kNFeat) o.feats[(size_t)b * kNFeat + lane] = x;
         return false;
     }
     const float C = warp_halt_classifier(x, feat_s, W1, b1, w2, b2, Hc, lane);
     bool goes_on = false;
-    if (lane == 0) {
+    if (lane == 0 && o.write) {
         const bool halt = (C < tau) || (n_drafted >= sl_max);
         o.token[b] = key_index(key);
         o.conf[b] = C;
@@ -609,7 +618,7 @@ __device__ __forceinline__ bool warp_draft_epilogue(const SoftmaxState& st, unsi
         o.final_stats[2 * b] = st.m;
         o.final_stats[2 * b + 1] = st.Z;
     }
-    if (o.feats && lane < kNFeat) o.feats[(size_t)b * kNFeat + lane] = x;
+    if (o.feats && o.write && lane < kNFeat) o.feats[(size_t)b * kNFeat + lane] = x;
     return goes_on;   // lane 0: the sequence drafts another token after this one
 }
 

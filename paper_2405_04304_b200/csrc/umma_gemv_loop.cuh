@@ -48,11 +48,6 @@ struct GemvLoopParams {
     float4* records;       // [sequence][CTA] stamped records of 80 bytes; written by this kernel only, starts zeroed
 };
 
-__device__ __forceinline__ unsigned int ld_relaxed_u32(const unsigned int* p) {
-    unsigned int v;
-    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
 __device__ __forceinline__ void st_relaxed_u32(unsigned int* p, unsigned int v) {
     asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
