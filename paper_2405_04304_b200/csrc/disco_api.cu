@@ -284,6 +284,7 @@ int launch_draft_batch(disco_ctx* c, const void* W, const void* H, int d, int R,
     const int tile_target = R <= 128 ? 128 : 256;
     p.TPC = std::max(1, (c->V + tile_target * p.CN - 1) / (tile_target * p.CN));
     p.TR = (c->V + p.CN * p.TPC - 1) / (p.CN * p.TPC);
+    if (probs) p.TR = (p.TR + 3) & ~3;   // rows of logits are stored 16 bytes at a time
     p.TRN = std::max(16, (p.TR + 15) / 16 * 16);
     p.a_rows = p.MT > 1 ? 128 : std::max(8, (R + 7) / 8 * 8);
     p.a_bytes = (p.a_rows * 128 + 1023) / 1024 * 1024;
@@ -293,7 +294,10 @@ int launch_draft_batch(disco_ctx* c, const void* W, const void* H, int d, int R,
     static KernelSetup setup;
     size_t dyn_limit = 0;
     if (!raise_smem_limit(c, setup, kern, 0, &dyn_limit)) return DISCO_ERR_CUDA;
-    const size_t fixed = 1024 + 512 + kDbXchBytes + (size_t)(kDbFinWarps * kDbFinWords + 128) * 4 + umma_clf_bytes(f.clf_H) + 128;
+    p.all_finish = R > kDbFinWarps * p.MT * p.CN;
+    const int fin_warps = kDbFinWarps + (p.all_finish ? kDbEpiWarps : 0);
+    const size_t fixed = 1024 + 512 + kDbXchBytes + (size_t)(fin_warps * kDbFinWords + 128) * 4 +
+                         (probs ? kDbEpiWarps * 32 * kDbTurnStride * 4 : 0) + umma_clf_bytes(f.clf_H) + 128;
     if (dyn_limit < fixed + 2 * (size_t)(p.a_bytes + p.b_bytes)) return DISCO_ERR_UNSUPPORTED_SHAPE;
     p.stages = (int)std::min<size_t>(kDbMaxStages, (dyn_limit - fixed) / (p.a_bytes + p.b_bytes));
     p.ring_bytes = p.stages * (p.a_bytes + p.b_bytes);
@@ -303,7 +307,6 @@ int launch_draft_batch(disco_ctx* c, const void* W, const void* H, int d, int R,
     p.bound = c->row_bound;
     p.set_words = (size_t)c->part_rows * kDbBoundStride;
     p.sync = c->ticket + 48;
-    p.rows_per_claim = (R + kDbFinWarps * p.MT * p.CN - 1) / (kDbFinWarps * p.MT * p.CN);
     CUtensorMap tmap_W, tmap_H;
     if (!encode_bf16_2d(c, &tmap_W, W, c->V, d, p.TRN) || !encode_bf16_2d(c, &tmap_H, H, R, d, p.a_rows))
         return DISCO_ERR_CUDA;

@@ -42,6 +42,7 @@ constexpr int kDbXchBytes = 128 * 64;  // states handed between the two warps th
 constexpr int kDbFinWords = 16 + kDbCandidates + 16;   // features, candidates, result; per finishing warp
 constexpr int kDbBoundSlots = 12;      // words of the shared bound per row
 constexpr int kDbBoundStride = 16;     // (rows 64 bytes apart)
+constexpr int kDbTurnStride = 36;      // floats per row of the area that turns a chunk of logits round (no bank conflicts)
 constexpr int kDbChunks = 4;           // chunks of 32 columns per warp and tile, at most
 constexpr uint32_t kDbNoIndex = 0x0fffffffu;           // record word: arg-max index in 28 bits, list length above it
 constexpr float kLog2e = 1.4426950408889634f, kLn2 = 0.6931471805599453f;
@@ -65,7 +66,7 @@ struct DraftBatchParams {
     // [0] launches so far (the stamp of this launch is that + 1); [2], [3] rows of the last launch of each parity; from
     // [4] on two sets of (CTAs started, rows claimed), four words apart, used by parity: a launch clears the other
     unsigned int* sync;
-    int rows_per_claim;
+    int all_finish;        // more rows than finishing warps in the grid: the epilogue warps help
 };
 
 __device__ __forceinline__ float ex2_approx(float x) {
@@ -256,49 +257,39 @@ __device__ __forceinline__ void db_finish_row(const DraftBatchParams& p, const D
     idx = __reduce_min_sync(kFullMask, idx);
     float sel = DISCO_NEG_INF;
     if (!stats) {
-        // Entries above the bound move to shared memory; each lane counts its own first.  More than 32 of them (a grid that
+        // Entries above the bound move to shared memory (about twenty, over all records).  More than 64 of them (a grid that
         // had no bound in time): only those not below theta, the tenth largest of the lanes' largest entries.
         float theta = DISCO_NEG_INF;
-        int n = 0, mine = 0, incl = 0;
+        int n = 0;
         bool more = false;    // some list goes on past its fourth entry
+        const unsigned lt = (1u << lane) - 1u;
         for (int round = 0; round < 2; ++round) {
-            mine = 0;
+            n = 0;
             more = false;
 #pragma unroll
             for (int j = 0; j < PER; ++j) {
                 const int cnt = static_cast<int>(__float_as_uint(q[j][1].x) >> 28);
                 const float l[4] = {q[j][1].y, q[j][2].x, q[j][2].y, q[j][2].z};
 #pragma unroll
-                for (int k = 0; k < 4; ++k) mine += (k < cnt && l[k] > bound && l[k] >= theta) ? 1 : 0;
-                more = more || (cnt > 4 && l[3] > bound && l[3] >= theta);
+                for (int k = 0; k < 4; ++k) {
+                    const bool take = k < cnt && l[k] > bound && l[k] >= theta;
+                    const unsigned mask = __ballot_sync(kFullMask, take);
+                    if (mask == 0u) break;
+                    const int at = n + __popc(mask & lt);
+                    if (take && at < kDbCandidates) cand[at] = l[k];
+                    n += __popc(mask);
+                    if (k == 3) more = more || (take && cnt > 4);
+                }
             }
-            incl = mine;
-#pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const int o = __shfl_up_sync(kFullMask, incl, off);
-                if (lane >= off) incl += o;
-            }
-            n = __shfl_sync(kFullMask, incl, 31);
-            if (n <= 32) break;
+            if (n <= 64) break;
             float head = DISCO_NEG_INF;
 #pragma unroll
             for (int j = 0; j < PER; ++j)
                 if (__float_as_uint(q[j][1].x) >> 28) head = fmaxf(head, q[j][1].y);
+            __syncwarp();
             const int rank = rank_in_warp(head, lane, cand);
             theta = __shfl_sync(kFullMask, head, __ffs(__ballot_sync(kFullMask, rank == kTopK - 1)) - 1);
-        }
-        int at = incl - mine;
-#pragma unroll
-        for (int j = 0; j < PER; ++j) {
-            const int cnt = static_cast<int>(__float_as_uint(q[j][1].x) >> 28);
-            const float l[4] = {q[j][1].y, q[j][2].x, q[j][2].y, q[j][2].z};
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                if (k < cnt && l[k] > bound && l[k] >= theta) {
-                    if (at < kDbCandidates) cand[at] = l[k];
-                    ++at;
-                }
-            }
+            if (round == 1) n = kDbCandidates + 1;   // (the candidates were overwritten)
         }
         if (__any_sync(kFullMask, more)) {   // (rare) the rest of the long lists
 #pragma unroll 1
@@ -371,11 +362,13 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
     uint64_t* tmem_empty = tmem_full + 4;
     uint32_t* tmem_base_s = reinterpret_cast<uint32_t*>(tmem_empty + 4);
     int* s_done = reinterpret_cast<int*>(tmem_base_s + 1);    // epilogue warps that have published their records
+    uint32_t* s_clf = tmem_base_s + 3;                        // set once the classifier is in shared memory
     uint32_t* s_stamp = tmem_base_s + 2;                      // stamp of this launch (0: not read yet, or nothing to do)
     float4* xch = reinterpret_cast<float4*>(reinterpret_cast<uint8_t*>(full) + 512);
     float* fin_s = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(xch) + kDbXchBytes);
-    float* row_thr_s = fin_s + kDbFinWarps * kDbFinWords;     // [128] the rows' bounds
-    float* clf_s = row_thr_s + 128;
+    float* row_thr_s = fin_s + (p.all_finish ? kDbFinWarps + kDbEpiWarps : kDbFinWarps) * kDbFinWords;     // [128] the rows' bounds
+    float* turn_s = row_thr_s + 128;                          // with probs: 32 rows of one chunk per epilogue warp
+    float* clf_s = turn_s + (p.probs ? kDbEpiWarps * 32 * kDbTurnStride : 0);
 
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
@@ -400,6 +393,7 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
         }
         *s_done = 0;
         *s_stamp = 0u;
+        *s_clf = 0u;
         fence_mbar_init();
         prefetch_tensormap(&tmap_W);
         prefetch_tensormap(&tmap_H);
@@ -520,7 +514,8 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
                 tc_commit(&tmem_full[buf]);
             }
         }
-    } else if (warp < 2 + kDbEpiWarps) {
+    }
+    if (warp >= 2 && warp < 2 + kDbEpiWarps) {
         // ------------------------------ epilogue ------------------------------
         const int ew = warp - 2;
         const int quad = warp & 3;              // TMEM lane quadrant this warp may read
@@ -535,10 +530,11 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
         const bool defer = nbuf == 4 && tiles > 1;
         const uint32_t t_quad = tmem_base + (static_cast<uint32_t>(quad * 32) << 16);
         volatile float* thr_s = row_thr_s + tile_row;
+        float* turn = turn_s + ew * 32 * kDbTurnStride;
         // Twice: a rehearsal without columns before the dependency wait (what follows the column loop is on the critical
         // path, and its instructions would come from L2 one after the other), then for good.
         for (int phase = 0; phase < 2; ++phase) {
-            bool keep_logits = false;
+            unsigned keep_mask = 0u;       // rows of this warp whose raw logits go to probs (none of a masked sequence's)
             unsigned int *slots = nullptr, *my_slot = nullptr;
             float m = DISCO_NEG_INF, Z = 0.f, S2 = 0.f;      // S2 = sum e^(z - m) (z - m) / ln 2
             float best_v = DISCO_NEG_INF;
@@ -558,8 +554,7 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
                 const int old_rows = *reinterpret_cast<volatile unsigned int*>(p.sync + 2 + (par ^ 1u));
                 if (blockIdx.x == 0)
                     for (int i = ew * 32 + lane; i < f.clear_n; i += kDbEpiWarps * 32) f.clear_words[i] = 0u;
-                // the optional probs output receives the raw logits of this row, unless the sequence is masked
-                keep_logits = p.probs && valid && (!f.active || f.active[row]);
+                keep_mask = __ballot_sync(kFullMask, p.probs && valid && (!f.active || f.active[row]));
                 slots = p.bound + par * p.set_words + (size_t)(valid ? row : 0) * kDbBoundStride;
                 my_slot = slots + nslot % kDbBoundSlots;
                 uint4* old = reinterpret_cast<uint4*>(p.bound + (par ^ 1u) * p.set_words);
@@ -641,18 +636,31 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
                         }
                         S2 = fmaf(em, fmaf(dm, Z, S2), Sa + Sb);   // (Z = S2 = 0 before the first chunk)
                         Z = fmaf(Z, em, Za + Zb);
-                        if (keep_logits) {
+                        if (keep_mask) {
+                            // A thread holds one row: the chunk goes through shared memory so that every store instruction
+                            // writes whole lines (four rows of 128 bytes; 32 bytes at a time per row halved the rate of
+                            // the whole pass: 278 against 68 us for 1000 rows of the 32000 x 768 head).
                             const int v = v_first + t * p.TR + c * 32;
-                            float* dst = p.probs + (size_t)row * p.V + v;
-                            if ((((uintptr_t)p.probs & 15) | ((p.V | v) & 3)) == 0 && n >= 32) {  // 16-byte stores
+                            float4* mine = reinterpret_cast<float4*>(turn + lane * kDbTurnStride);
 #pragma unroll
-                                for (int j = 0; j < 32; j += 4)
-                                    *reinterpret_cast<float4*>(dst + j) = make_float4(z[j], z[j + 1], z[j + 2], z[j + 3]);
+                            for (int j = 0; j < 8; ++j) mine[j] = make_float4(z[4 * j], z[4 * j + 1], z[4 * j + 2], z[4 * j + 3]);
+                            __syncwarp();
+                            float* dst = p.probs + (size_t)(m_tile * 128 + quad * 32) * p.V + v;
+                            if (((p.V | v) & 3) == 0 && n >= 32 && (reinterpret_cast<uintptr_t>(p.probs) & 15) == 0) {
+#pragma unroll
+                                for (int j = 0; j < 8; ++j) {
+                                    const int r = 4 * j + (lane >> 3), col = (lane & 7) * 4;
+                                    const float4 x = *reinterpret_cast<const float4*>(turn + r * kDbTurnStride + col);
+                                    if ((keep_mask >> r) & 1u) *reinterpret_cast<float4*>(dst + (size_t)r * p.V + col) = x;
+                                }
                             } else {
-#pragma unroll
-                                for (int j = 0; j < 32; ++j)
-                                    if (j < n) dst[j] = z[j];
+#pragma unroll 4
+                                for (int r = 0; r < 32; ++r) {
+                                    const float x = turn[r * kDbTurnStride + lane];
+                                    if (((keep_mask >> r) & 1u) && lane < n) dst[(size_t)r * p.V + lane] = x;
+                                }
                             }
+                            __syncwarp();
                         }
                     }
                     if (use_bound) {
@@ -796,11 +804,15 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
                 atomicAdd(s_done, 1);
             }
         }
-    } else {
-        // ------------------------------ finishing warps ------------------------------
-        const int fw = warp - 2 - kDbEpiWarps;
+    }
+    // ------------------------------ finishing rows ------------------------------
+    // The finishing warps, from the start of the launch; with more rows than those of the whole grid, the epilogue warps as
+    // well once their records are out.
+    const bool epi = warp < 2 + kDbEpiWarps;
+    if (warp >= 2 && (!epi || p.all_finish)) {
+        const int fw = epi ? kDbFinWarps + warp - 2 : warp - 2 - kDbEpiWarps;
         float* sm = fin_s + fw * kDbFinWords;
-        if (f.clf_H > 0) {   // classifier parameters -> shared
+        if (!epi && f.clf_H > 0) {   // classifier parameters -> shared
             const int Hc = f.clf_H, n1 = Hc * kNFeat;
             for (int i = fw * 32 + lane; i < n1 + 2 * Hc + 1; i += kDbFinWarps * 32) {
                 const float* src = i < n1 ? f.clf_W1 + i
@@ -812,16 +824,23 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
         }
         uint32_t stamp = 1u;
         unsigned int* set = nullptr;
-        int b = 0, b_end = 0;
+        int b = 0;
+        bool run = !epi;
         for (bool real = false;; real = true) {
-            db_finish_row(p, f, b, real, stamp + (real ? f.test_stamp_skew : 0u), sm, clf_s, STATS, lane);
-            if (real) {
-                ++b;
-            } else {
-                cp_async_wait_all();
-                named_barrier_sync(3, kDbFinWarps * 32);
-                asm volatile("griddepcontrol.wait;" ::: "memory");
+            if (run) db_finish_row(p, f, b, real, stamp + (real ? f.test_stamp_skew : 0u), sm, clf_s, STATS, lane);
+            run = true;
+            if (!real) {
+                if (!epi) {
+                    cp_async_wait_all();
+                    named_barrier_sync(3, kDbFinWarps * 32);
+                    if (fw == 0 && lane == 0) {
+                        __threadfence_block();
+                        *reinterpret_cast<volatile uint32_t*>(s_clf) = 1u;
+                    }
+                    asm volatile("griddepcontrol.wait;" ::: "memory");
+                }
                 if (chained && !chain_any_live(f.chain, f.B, lane)) break;
+                if (epi) smem_word(s_clf, p.status);
                 stamp = smem_word(s_stamp, p.status);
                 __syncwarp();
                 set = p.sync + 4 + 4 * (stamp & 1u);
@@ -838,23 +857,20 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
                 }
                 if (!__shfl_sync(kFullMask, all, 0)) break;
             }
-            if (b >= b_end) {   // the next rows nobody has taken
-                int first = 0;
-                if (lane == 0) first = (int)atomicAdd(set + 1, 1u);
-                first = __shfl_sync(kFullMask, first, 0);
-                if (first == 0 && lane == 0) {
-                    // All CTAs have started: the stamp can move on, and the counters of the next launch (this one's may
-                    // still be looked at) start at zero.
-                    unsigned int* other = p.sync + 4 + 4 * ((stamp + 1u) & 1u);
-                    other[0] = 0u;
-                    other[1] = 0u;
-                    p.sync[2 + (stamp & 1u)] = (unsigned int)p.R;
-                    p.sync[0] = stamp == 0xffffffffu ? 1u : stamp;   // never zero, and the two sets keep alternating
-                }
-                b = first * p.rows_per_claim;
-                b_end = min(f.B, b + p.rows_per_claim);
-                if (b >= f.B) break;
+            // the next row nobody has taken
+            int first = 0;
+            if (lane == 0) first = (int)atomicAdd(set + 1, 1u);
+            b = __shfl_sync(kFullMask, first, 0);
+            if (b == 0 && lane == 0) {
+                // All CTAs have started: the stamp can move on, and the counters of the next launch (this one's may
+                // still be looked at) start at zero.
+                unsigned int* other = p.sync + 4 + 4 * ((stamp + 1u) & 1u);
+                other[0] = 0u;
+                other[1] = 0u;
+                p.sync[2 + (stamp & 1u)] = (unsigned int)p.R;
+                p.sync[0] = stamp == 0xffffffffu ? 1u : stamp;   // never zero, and the two sets keep alternating
             }
+            if (b >= f.B) break;
         }
     }
 
