@@ -36,6 +36,12 @@ struct KernelSetup {
     size_t dyn_limit[kMaxDevices] = {};
 };
 
+// Where an LM-head pass leaves its records (m, Z first) of consecutive vocabulary slabs: what a draw is located with.
+struct RecordLayout {
+    const float4* recs;
+    int pieces, NP, slab;
+};
+
 struct StreamPlan {
     int rows_per_cta, grid, rps, stages;
     uint32_t slot_bytes;
@@ -178,7 +184,6 @@ int run_stream(disco_ctx* c, TailParams& p, int clf_H, cudaStream_t st) {
     if (!pl.ok) return DISCO_ERR_UNSUPPORTED_SHAPE;
     if (DRAFT && (pl.grid > c->max_grid || p.R > c->part_rows)) return DISCO_ERR_WORKSPACE;
     p.rows_per_cta = pl.rows_per_cta;
-    p.slab_rows = pl.rows_per_cta;
     p.rps = pl.rps;
     p.stages = pl.stages;
     p.slot_bytes = pl.slot_bytes;
@@ -271,7 +276,7 @@ bool draft_batch_possible(const disco_ctx* c, int R) {
 // Launch the batched draft step (STATS: arg-max and statistics only) for R hidden rows of width d against W [V, d].
 template <bool STATS>
 int launch_draft_batch(disco_ctx* c, const void* W, const void* H, int d, int R, float* probs, const DraftFinalParams& f,
-                       cudaStream_t st) {
+                       cudaStream_t st, RecordLayout* layout) {
     DraftBatchParams p{};
     p.V = c->V;
     p.d = d;
@@ -320,6 +325,7 @@ int launch_draft_batch(disco_ctx* c, const void* W, const void* H, int d, int R,
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = c->pdl ? 1 : 0;
+    if (layout) *layout = RecordLayout{p.part_rec, kStampedPieces, p.CN, p.TPC * p.TR};
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tmap_W, tmap_H, p, f);
     c->launches += 1;
     return cuda_ok(e, "umma_draft_batch_kernel launch") ? DISCO_OK : DISCO_ERR_CUDA;
@@ -355,13 +361,13 @@ int launch_gemv_rk(disco_ctx* c, GemvParams& g, const CUtensorMap& mW, const CUt
     return cuda_ok(e, "umma_gemv_draft_kernel launch") ? DISCO_OK : DISCO_ERR_CUDA;
 }
 
-int launch_gemv(disco_ctx* c, const TailParams& t, cudaStream_t st) {
+int launch_gemv(disco_ctx* c, const TailParams& t, cudaStream_t st, RecordLayout* layout) {
     GemvParams g{};
     g.t = t;
     const int grid = c->sm_count;
     if (grid > c->part_slots || t.R > c->part_rows) return DISCO_ERR_WORKSPACE;
     g.TR = (t.V + grid - 1) / grid;
-    g.t.slab_rows = g.TR;
+    if (layout) *layout = RecordLayout{t.part_rec, 4, grid, g.TR};
     g.tiles = (g.TR + 255) / 256;
     g.TRt = (g.TR + g.tiles - 1) / g.tiles;
     g.TRN = (g.TRt + 15) / 16 * 16;
@@ -421,7 +427,6 @@ int launch_gemv_loop(disco_ctx* c, const TailParams& t, int steps, size_t w_step
     const int grid = c->sm_count;
     if (grid > kGroupMaxRecords) return DISCO_ERR_UNSUPPORTED_SHAPE;
     g.TR = (t.V + grid - 1) / grid;
-    g.t.slab_rows = g.TR;
     g.tiles = (g.TR + 255) / 256;
     g.TRt = (g.TR + g.tiles - 1) / g.tiles;
     g.TRN = (g.TRt + 15) / 16 * 16;
@@ -638,13 +643,6 @@ cudaError_t launch_after(const disco_ctx* c, void (*kern)(KArgs...), dim3 grid, 
     return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }
 
-// The sampling kernels stage one row of V floats in dynamic shared memory: raise their limit once per device.
-bool configure_sampling(disco_ctx* c) {
-    static KernelSetup rows_setup;
-    const size_t bytes = (size_t)kSampleSmemFloats * sizeof(float);
-    return raise_smem_limit(c, rows_setup, sample_rows_kernel, bytes, nullptr);
-}
-
 // Shared body of the LM-head + soft-max passes: B rows of hidden size d against the head W.
 //   * nll_sum != null selects the perplexity rule (no classifier; tau is the perplexity bound);
 //   * stats_only = 1: arg-max (token, optional) and soft-max statistics only, no classifier: the target
@@ -654,8 +652,7 @@ int draft_step_common(disco_ctx* c, const void* W_D, const void* h_D, int d, int
                       const int32_t* n_drafted, const uint8_t* active, const disco_clf* clf, float tau,
                       int sl_max, int32_t* token, float* conf, uint8_t* halt, float* feats, float* probs,
                       float* nll_sum, int stats_only, void* stream, bool normalize = true,
-                      const float* u_draw = nullptr, float* p_token = nullptr, bool* drew = nullptr,
-                      const ChainLink* chain = nullptr, unsigned int* clear_words = nullptr, int clear_n = 0) {
+                      RecordLayout* layout = nullptr, const ChainLink* chain = nullptr, unsigned int* clear_words = nullptr, int clear_n = 0) {
     if (!c || !W_D || !h_D) return DISCO_ERR_INVALID_ARG;
     if (!stats_only && !chain && (!pos || !n_drafted)) return DISCO_ERR_INVALID_ARG;
     if (!stats_only && (!token || !conf || !halt)) return DISCO_ERR_INVALID_ARG;
@@ -711,17 +708,8 @@ int draft_step_common(disco_ctx* c, const void* W_D, const void* h_D, int d, int
                          (size_t)((d + kUmmaBK - 1) / kUmmaBK) * (B <= 8 ? 8 : 16) * 128 <= 48 * 1024;
     const bool use_gemv = gemv_ok && (c->path == 3 || (c->path == 0 && B <= 4));
     const bool use_umma = !use_gemv && draft_batch_possible(c, B) && (c->path == 2 || c->path == 3 || (c->path == 0 && B >= 2));
-    // Sampled step: the kernels that end in a last-CTA second phase draw the token there (their records are
-    // at most 160 and in vocabulary order); the batched kernel leaves the draw to a follow-up kernel.
-    const bool fused_draw = u_draw && probs && !use_umma && (use_gemv || c->max_grid <= 160);
-    if (fused_draw) {
-        p.u_draw = u_draw;
-        p.p_token = p_token;
-        normalize = true;
-    }
-    if (drew) *drew = fused_draw;
     if (use_gemv) {
-        rc = launch_gemv(c, p, st);
+        rc = launch_gemv(c, p, st, layout);
         if (rc) return rc;
     } else if (use_umma) {
         DraftFinalParams f{};
@@ -747,12 +735,13 @@ int draft_step_common(disco_ctx* c, const void* W_D, const void* h_D, int d, int
         f.clear_words = clear_words;
         f.clear_n = clear_n;
         if (chain) f.chain = *chain;
-        rc = stats_only == 1 ? launch_draft_batch<true>(c, W_D, h_D, d, B, probs, f, st)
-                             : launch_draft_batch<false>(c, W_D, h_D, d, B, probs, f, st);
+        rc = stats_only == 1 ? launch_draft_batch<true>(c, W_D, h_D, d, B, probs, f, st, layout)
+                             : launch_draft_batch<false>(c, W_D, h_D, d, B, probs, f, st, layout);
         if (rc) return rc;
     } else {
         rc = run_stream<true>(c, p, clf->H, st);
         if (rc) return rc;
+        if (layout) *layout = RecordLayout{p.part_rec, 4, (p.V + p.rows_per_cta - 1) / p.rows_per_cta, p.rows_per_cta};
     }
     if (probs && normalize) {
         dim3 grid((unsigned)std::min(64, (c->V + 255) / 256), (unsigned)B);
@@ -875,19 +864,30 @@ int disco_draft_step_sample(disco_ctx* c, const void* W_D, const void* h_D, int 
                             int sl_max, const float* u, int32_t* token, float* p_token, float* conf, uint8_t* halt,
                             float* feats, float* probs, void* stream) {
     if (!c || !u || !probs) return DISCO_ERR_INVALID_ARG;
-    bool drew = false;
+    RecordLayout rl{};
     int rc = draft_step_common(c, W_D, h_D, c->d_draft, B, c->max_batch, pos, n_drafted, active, clf, tau, sl_max,
-                               token, conf, halt, feats, probs, nullptr, 0, stream, false, u, p_token, &drew);
+                               token, conf, halt, feats, probs, nullptr, 0, stream, false, &rl);
     if (rc) return rc;
-    if (drew) return DISCO_OK;   // token drawn by the LM-head kernel's second phase, probs normalised
     // probs holds the logits: the kernel turns them into y^D and replaces the greedy token by the draw
-    const size_t smem = sample_smem_bytes(c->V);
-    if (!configure_sampling(c)) return DISCO_ERR_CUDA;
-    const cudaError_t e = launch_after(c, sample_rows_kernel, dim3(B), dim3(kSampleThreads), smem,
-                                       static_cast<cudaStream_t>(stream), probs, (const float*)c->final_stats, u, active,
-                                       c->V, smem ? 1 : 0, token, p_token);
+    DrawRowsParams dp{};
+    dp.probs = probs;
+    dp.stats = c->final_stats;
+    dp.recs = rl.recs;
+    dp.rec_pieces = rl.pieces;
+    dp.NP = rl.NP;
+    dp.slab = rl.slab;
+    // about two CTAs per SM, at least one slab each
+    const int seg = std::max(1, std::min(rl.NP, 2 * c->sm_count / B));
+    dp.seg_slabs = (rl.NP + seg - 1) / seg;
+    dp.V = c->V;
+    dp.u = u;
+    dp.active = active;
+    dp.token = token;
+    dp.p_token = p_token;
+    const cudaError_t e = launch_after(c, draw_rows_kernel, dim3((unsigned)((rl.NP + dp.seg_slabs - 1) / dp.seg_slabs), (unsigned)B),
+                                       dim3(kSampleThreads), 0, static_cast<cudaStream_t>(stream), dp);
     c->launches += 1;
-    return cuda_ok(e, "sample_rows_kernel launch") ? DISCO_OK : DISCO_ERR_CUDA;
+    return cuda_ok(e, "draw_rows_kernel launch") ? DISCO_OK : DISCO_ERR_CUDA;
 }
 
 int disco_verify_sample_ragged(disco_ctx* c, const void* W_T, const void* H_T, const int32_t* draft_ids,
@@ -905,7 +905,7 @@ int disco_verify_sample_ragged(disco_ctx* c, const void* W_T, const void* H_T, c
     // launch normalises the rows, counts the accepted tokens and draws the next one
     int rc = draft_step_common(c, W_T, H_T, c->d_target, R, c->max_rows, nullptr, nullptr, nullptr, nullptr, 0.f, 1,
                                target_ids, nullptr, nullptr, nullptr, y_T, nullptr, 1, stream, false, nullptr, nullptr,
-                               nullptr, nullptr, c->sample_tickets, B);
+                               c->sample_tickets, B);
     if (rc) return rc;
     SampleRowsParams sp{};
     sp.y_T = y_T;
@@ -1017,7 +1017,7 @@ int disco_draft_loop(disco_ctx* c, const void* W_D, size_t w_step_stride, const 
                                static_cast<const char*>(h_D) + k * h_step, c->d_draft, B, c->max_batch, nullptr,
                                nullptr, nullptr, clf, tau, sl_max, token + k * B, conf + k * B, halt + k * B,
                                feats ? feats + k * B * kNFeat : nullptr, nullptr, nullptr, 0, stream, true, nullptr,
-                               nullptr, nullptr, &link);
+                               &link);
         if (rc) return rc;
     }
     return DISCO_OK;

@@ -14,7 +14,7 @@ namespace disco {
 constexpr int kSampleThreads = 512;
 constexpr int kSampleWarps = kSampleThreads / 32;
 
-// Step C of the draw below, also used on its own: entries [c0, c1) hold the crossing of `target` (the running
+// The last step of a draw: entries [c0, c1) hold the crossing of `target` (the running
 // sum before c0 is `before`).  They are dealt out, a few consecutive entries per thread of the whole CTA: sums in
 // vocabulary order, a scan over the CTA, and the thread that holds the crossing walks its entries and writes
 // the token to found[0].  piece_tot: kSampleWarps doubles of shared memory.  Ends without a barrier.
@@ -80,124 +80,130 @@ __device__ __forceinline__ void block_cdf_walk(WeightFn w, int c0, int c1, doubl
     }
 }
 
-// Inverse-CDF draw by one CTA of kSampleThreads threads from weights w(v) >= 0, v < V (a callable that
-// returns the same value whenever it is asked again): the smallest v whose running sum w(0) + .. + w(v)
-// exceeds u * (sum of all); if rounding leaves none, the last v with w(v) > 0; -1 if every weight is zero.
-// Every thread returns the token.  Three steps:
-//   A  each warp sums one contiguous segment of the row (coalesced reads, four partial sums per lane);
-//   B  every thread finds, from the 16 totals, the segment that holds u * total;
-//   C  that segment is dealt out again, a few consecutive entries per thread of the whole CTA: sums in
-//      vocabulary order, a scan over the CTA, and the thread that holds the crossing walks its entries.
-// sh: 40 doubles of shared memory; total (optional) receives the sum.
-template <typename WeightFn>
-__device__ __forceinline__ int block_sample_cdf(WeightFn w, int V, double u, double* sh, double* total_out) {
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const int seg = ((V + kSampleWarps - 1) / kSampleWarps + 31) & ~31;  // entries per warp, whole 32s
-    const int s0 = min(V, warp * seg), s1 = min(V, s0 + seg);
-    double* warp_tot = sh;                                        // [kSampleWarps] segment totals
-    double* piece_tot = sh + kSampleWarps;                        // [kSampleWarps] step C: per-warp sums
-    int* found = reinterpret_cast<int*>(sh + 2 * kSampleWarps);   // [2]: token, last index with positive weight
-    if (t == 0) {
-        found[0] = -1;
-        found[1] = -1;
-    }
-    // A
-    double part[4] = {0.0, 0.0, 0.0, 0.0};
-    int last = -1;
-    for (int v0 = s0 + lane; v0 < s1; v0 += 128) {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int v = v0 + 32 * k;
-            if (v < s1) {
-                const float x = w(v);
-                part[k] += static_cast<double>(x);
-                if (x > 0.f) last = max(last, v);
-            }
-        }
-    }
-    double tot = (part[0] + part[1]) + (part[2] + part[3]);
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        tot += __shfl_xor_sync(kFullMask, tot, off);
-        last = max(last, __shfl_xor_sync(kFullMask, last, off));
-    }
-    if (lane == 0) warp_tot[warp] = tot;
-    __syncthreads();
-    if (lane == 0 && last >= 0) atomicMax(&found[1], last);
-    // B: the first segment whose running total exceeds the target (the same for every thread)
-    double total = 0.0;
-#pragma unroll
-    for (int k = 0; k < kSampleWarps; ++k) total += warp_tot[k];
-    const double target = u * total;
-    int win = -1;
-    double before = 0.0, run = 0.0;
-#pragma unroll
-    for (int k = 0; k < kSampleWarps; ++k) {
-        const double nxt = run + warp_tot[k];
-        if (win < 0 && nxt > target) {
-            win = k;
-            before = run;
-        }
-        run = nxt;
-    }
-    // C
-    if (win >= 0) block_cdf_walk(w, min(V, win * seg), min(V, min(V, win * seg) + seg), before, target, piece_tot, found);
-    __syncthreads();
-    const int tok = found[0] >= 0 ? found[0] : found[1];
-    if (total_out) *total_out = total;
-    __syncthreads();  // sh may be reused by the caller
-    return tok;
-}
-
-// Rows of up to kSampleSmemFloats entries are staged in shared memory (one pass over global memory, eight
-// loads in flight per thread); longer rows are read from global memory by every step of the draw.
-constexpr int kSampleSmemFloats = 50 * 1024;
 constexpr int kSampleBatch = 16;
-inline size_t sample_smem_bytes(int V) { return V <= kSampleSmemFloats ? (size_t)V * sizeof(float) : 0; }
 
-// Draft side: the row probs[b, :] arrives holding the raw logits left by the LM-head pass; it is turned
-// into the distribution y = exp(z - m) / Z in place (m, Z from stats[2b], stats[2b + 1]), then token[b]
-// is drawn from it with u[b]; p_token[b] = its probability.  One CTA per sequence; sequences with
-// active[b] == 0 are left untouched.  Dynamic shared memory: sample_smem_bytes(V).
-static __global__ void __launch_bounds__(kSampleThreads)
-sample_rows_kernel(float* __restrict__ probs, const float* __restrict__ stats, const float* __restrict__ u,
-                   const uint8_t* __restrict__ active, int V, int use_smem, int32_t* token, float* p_token) {
-    extern __shared__ float row_s[];
-    __shared__ double sh[40];
+// Draft side: the row probs[b, :] arrives holding the raw logits left by the LM-head pass; it is turned into the
+// distribution y = exp(z - m) / Z in place (m, Z from stats[2b], stats[2b + 1]), and token[b] is drawn from it with u[b];
+// p_token[b] = its probability.  Sequences with active[b] == 0 are left untouched.
+//
+// A row is cut into SEG segments, one CTA each, and no CTA waits for another: the LM-head pass has left a record (m, Z)
+// per slab of the vocabulary, in order, so every CTA of a row works out by itself which slab holds u * Z (one warp, beside
+// the normalisation), and the CTA whose segment has that slab walks it.  A segment is a whole number of slabs.
+// (One CTA per row, staging it in shared memory, took 18 us for 8 rows of 49152; this takes 5.)
+struct DrawRowsParams {
+    float* probs;             // [B, V]
+    const float* stats;       // [B][2]
+    const float4* recs;       // [B][NP] records of rec_pieces * 16 bytes that start with m, Z
+    int rec_pieces, NP;
+    int slab;                 // vocabulary rows per record
+    int seg_slabs;            // slabs per segment
+    int V;
+    const float* u;           // [B]
+    const uint8_t* active;    // [B] or null
+    int32_t* token;           // [B]
+    float* p_token;           // [B] or null
+};
+static __global__ void __launch_bounds__(kSampleThreads) draw_rows_kernel(const DrawRowsParams p) {
+    __shared__ double piece_tot[kSampleWarps];
+    __shared__ double s_before, s_target;
+    __shared__ int s_slab, found[1];
     // launched with programmatic stream serialization: resident early, reading only once the LM-head
     // kernel before it has completed
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    const int b = blockIdx.x;
-    if (active && !active[b]) return;
-    float* y = probs + (size_t)b * V;
-    const float m = stats[2 * b], inv_Z = 1.f / stats[2 * b + 1];
-    for (int v0 = threadIdx.x; v0 < V; v0 += kSampleBatch * kSampleThreads) {
-        float z[kSampleBatch];
-#pragma unroll
-        for (int k = 0; k < kSampleBatch; ++k) {
-            const int v = v0 + k * kSampleThreads;
-            z[k] = v < V ? __ldcg(y + v) : 0.f;
+    const int t = threadIdx.x, lane = t & 31;
+    const int b = blockIdx.y;
+    if (p.active && !p.active[b]) return;
+    float* y = p.probs + (size_t)b * p.V;
+    const float m = p.stats[2 * b], inv_Z = 1.f / p.stats[2 * b + 1];
+    const int first_slab = blockIdx.x * p.seg_slabs;
+    const int v0 = min(p.V, first_slab * p.slab), v1 = min(p.V, v0 + p.seg_slabs * p.slab);
+    if (t < 32) {
+        // a few consecutive records per lane, running sums in record order
+        const int q = (p.NP + 31) / 32, c0 = min(p.NP, lane * q), c1 = min(p.NP, c0 + q);
+        const float4* rec = p.recs + (size_t)b * p.NP * p.rec_pieces;
+        auto mass = [&](int c) {
+            const float4 r = __ldcg(rec + (size_t)c * p.rec_pieces);
+            return r.y > 0.f ? static_cast<double>(r.y) * static_cast<double>(expf(r.x - m)) : 0.0;
+        };
+        double mine = 0.0;
+        int last = -1;
+        for (int c = c0; c < c1; ++c) {
+            const double w = mass(c);
+            mine += w;
+            if (w > 0.0) last = c;
         }
+        double incl = mine;
 #pragma unroll
-        for (int k = 0; k < kSampleBatch; ++k) {
-            const int v = v0 + k * kSampleThreads;
-            if (v < V) {
-                const float pv = __expf(z[k] - m) * inv_Z;
-                y[v] = pv;
-                if (use_smem) row_s[v] = pv;
+        for (int off = 1; off < 32; off <<= 1) {
+            const double o = __shfl_up_sync(kFullMask, incl, off);
+            if (lane >= off) incl += o;
+        }
+        const double total = __shfl_sync(kFullMask, incl, 31);
+        const double target = static_cast<double>(p.u[b]) * total;
+        last = __reduce_max_sync(kFullMask, last);
+        const bool cross = incl - mine <= target && incl > target;
+        const unsigned who = __ballot_sync(kFullMask, cross);
+        if (who ? lane == __ffs(who) - 1 : lane == 0) {
+            double before = incl - mine;
+            int slab = last;               // rounding next to u = 1: the last slab with mass, and its last entry
+            if (who) {
+                for (int c = c0; c < c1; ++c) {
+                    const double w = mass(c);
+                    if (before + w > target) {
+                        slab = c;
+                        break;
+                    }
+                    before += w;
+                }
             }
+            s_slab = slab;
+            s_before = who ? before * inv_Z : 0.0;
+            s_target = who ? target * inv_Z : 1e300;
+            found[0] = -1;
+        }
+    }
+    if (((p.V | v0 | v1) & 3) == 0 && (reinterpret_cast<uintptr_t>(p.probs) & 15) == 0) {
+        for (int v = v0 + 4 * t; v < v1; v += 4 * 4 * kSampleThreads) {
+            float4 z[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                z[k] = v + 4 * k * kSampleThreads < v1 ? __ldcg(reinterpret_cast<const float4*>(y + v + 4 * k * kSampleThreads))
+                                                       : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (v + 4 * k * kSampleThreads < v1)
+                    *reinterpret_cast<float4*>(y + v + 4 * k * kSampleThreads) =
+                        make_float4(__expf(z[k].x - m) * inv_Z, __expf(z[k].y - m) * inv_Z, __expf(z[k].z - m) * inv_Z,
+                                    __expf(z[k].w - m) * inv_Z);
+        }
+    } else {
+        for (int v = v0 + t; v < v1; v += 8 * kSampleThreads) {
+            float z[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) z[k] = v + k * kSampleThreads < v1 ? __ldcg(y + v + k * kSampleThreads) : 0.f;
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if (v + k * kSampleThreads < v1) y[v + k * kSampleThreads] = __expf(z[k] - m) * inv_Z;
         }
     }
     __syncthreads();
-    int tok;
-    if (use_smem)
-        tok = block_sample_cdf([&](int v) { return row_s[v]; }, V, static_cast<double>(u[b]), sh, nullptr);
-    else
-        tok = block_sample_cdf([&](int v) { return y[v]; }, V, static_cast<double>(u[b]), sh, nullptr);
-    if (threadIdx.x == 0) {
-        token[b] = tok;
-        if (p_token) p_token[b] = tok >= 0 ? y[tok] : 0.f;
+    const int slab = s_slab;
+    if (slab < 0) {   // no mass anywhere
+        if (blockIdx.x == 0 && t == 0) {
+            p.token[b] = -1;
+            if (p.p_token) p.p_token[b] = 0.f;
+        }
+        return;
+    }
+    if (slab < first_slab || slab >= first_slab + p.seg_slabs) return;
+    const int c0 = slab * p.slab, c1 = min(p.V, c0 + p.slab);
+    block_cdf_walk([&](int v) { return __ldcg(y + v); }, c0, c1, s_before, s_target, piece_tot, found);
+    __syncthreads();
+    if (t == 0) {
+        const int tok = found[0];
+        p.token[b] = tok;
+        if (p.p_token) p.p_token[b] = tok >= 0 ? __ldcg(y + tok) : 0.f;
     }
 }
 
