@@ -109,9 +109,18 @@ def _ptr(t, dtype=None, cuda=True):
     return t.data_ptr()
 
 
+# The address of the current stream without a torch.cuda.Stream object around it (0.1 us instead of 3 us per call, which
+# is a fifth of the smallest calls); torch.cuda.current_stream() where this torch does not offer it.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_get_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream(stream) -> int:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return s.cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is not None and _get_device is not None:
+        return _raw_stream(_get_device())
+    return torch.cuda.current_stream().cuda_stream
 
 
 class Classifier:

@@ -14,7 +14,6 @@
 #include "umma_tail.cuh"
 #include "draft_batch.cuh"
 #include "sample.cuh"
-#include "umma_gemv.cuh"
 #include "umma_gemv_loop.cuh"
 
 using namespace disco;
@@ -67,7 +66,8 @@ struct disco_ctx {
     unsigned long long* keys;
     unsigned int* ticket;
     int* status;
-    float* final_stats;
+    float* final_stats;            // [part_rows][2] (m, Z) of the rows of a pass
+    float* final_stats2;           // the same for the second pass of a feature extraction
     uint8_t* chain_alive;          // [max_batch] draft phase on the device: which sequences still draft
     double* sample_seg_tot;        // verification with sampling: [max_batch][kSampleMaxSegments][2] sums of weights
     int32_t* sample_seg_last;      //   the same shape: last index with positive weight
@@ -332,57 +332,6 @@ int launch_draft_batch(disco_ctx* c, const void* W, const void* H, int d, int R,
 }
 
 
-// Launch the tensor-core GEMV-shaped draft step (1..16 sequences).
-template <int RK>
-int launch_gemv_rk(disco_ctx* c, GemvParams& g, const CUtensorMap& mW, const CUtensorMap& mH, cudaStream_t st) {
-    auto kern = umma_gemv_draft_kernel<RK>;
-    static KernelSetup setup;
-    size_t dyn_limit = 0;
-    if (!raise_smem_limit(c, setup, kern, 0, &dyn_limit)) return DISCO_ERR_CUDA;
-    // the ring takes what the fixed part leaves; it must hold at least two stages and the 16 KB that the
-    // MMA reads behind the last box of hidden rows
-    const size_t fixed = gemv_fixed_smem_bytes(RK, g.t.clf_H, g.t.d, g.h_rows);
-    if (dyn_limit < fixed + 2 * (size_t)g.b_bytes) return DISCO_ERR_UNSUPPORTED_SHAPE;
-    g.stages = (int)std::min<size_t>(kGemvMaxStages, (dyn_limit - fixed) / g.b_bytes);
-    if ((size_t)g.stages * g.b_bytes < 16384) return DISCO_ERR_UNSUPPORTED_SHAPE;
-    const size_t smem = gemv_smem_bytes(RK, g.t.clf_H, g.t.d, g.h_rows, g.stages, g.b_bytes);
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)c->sm_count);
-    cfg.blockDim = dim3(kGemvThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = c->pdl ? 1 : 0;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, mW, mH, g);
-    c->launches += 1;
-    return cuda_ok(e, "umma_gemv_draft_kernel launch") ? DISCO_OK : DISCO_ERR_CUDA;
-}
-
-int launch_gemv(disco_ctx* c, const TailParams& t, cudaStream_t st, RecordLayout* layout) {
-    GemvParams g{};
-    g.t = t;
-    const int grid = c->sm_count;
-    if (grid > c->part_slots || t.R > c->part_rows) return DISCO_ERR_WORKSPACE;
-    g.TR = (t.V + grid - 1) / grid;
-    if (layout) *layout = RecordLayout{t.part_rec, 4, grid, g.TR};
-    g.tiles = (g.TR + 255) / 256;
-    g.TRt = (g.TR + g.tiles - 1) / g.tiles;
-    g.TRN = (g.TRt + 15) / 16 * 16;
-    g.b_bytes = (g.TRN * 128 + 1023) / 1024 * 1024;
-    g.h_rows = t.R <= 8 ? 8 : 16;
-    CUtensorMap mW, mH;
-    if (!encode_bf16_2d(c, &mW, t.W, t.V, t.d, g.TRN) || !encode_bf16_2d(c, &mH, t.H, t.R, t.d, g.h_rows))
-        return DISCO_ERR_CUDA;
-    if (t.R == 1) return launch_gemv_rk<1>(c, g, mW, mH, st);
-    if (t.R == 2) return launch_gemv_rk<2>(c, g, mW, mH, st);
-    if (t.R <= 4) return launch_gemv_rk<4>(c, g, mW, mH, st);
-    if (t.R <= 8) return launch_gemv_rk<8>(c, g, mW, mH, st);
-    return launch_gemv_rk<16>(c, g, mW, mH, st);
-}
-
 // The draft phase as one persistent kernel (1..4 sequences): see umma_gemv_loop.cuh.
 template <int RK>
 int launch_gemv_loop_rk(disco_ctx* c, GemvLoopParams& lp, const CUtensorMap& mW, const CUtensorMap& mH, cudaStream_t st) {
@@ -528,6 +477,7 @@ int disco_create(disco_ctx** out, int V, int d_draft, int d_target, int max_batc
     ok = ok && cudaMalloc(&c->ticket, 1024) == cudaSuccess;
     ok = ok && cudaMalloc(&c->status, 256) == cudaSuccess;
     ok = ok && cudaMalloc(&c->final_stats, (size_t)c->part_rows * 2 * sizeof(float)) == cudaSuccess;
+    ok = ok && cudaMalloc(&c->final_stats2, (size_t)c->part_rows * 2 * sizeof(float)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->chain_alive, (size_t)max_batch + 64) == cudaSuccess;
     ok = ok && cudaMalloc(&c->sample_seg_tot, (size_t)max_batch * kSampleMaxSegments * 2 * sizeof(double)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->sample_seg_last, (size_t)max_batch * kSampleMaxSegments * 2 * sizeof(int32_t)) == cudaSuccess;
@@ -572,6 +522,7 @@ int disco_destroy(disco_ctx* c) {
     cudaFree(c->ticket);
     cudaFree(c->status);
     cudaFree(c->final_stats);
+    cudaFree(c->final_stats2);
     cudaFree(c->chain_alive);
     cudaFree(c->sample_seg_tot);
     cudaFree(c->sample_seg_last);
@@ -652,7 +603,8 @@ int draft_step_common(disco_ctx* c, const void* W_D, const void* h_D, int d, int
                       const int32_t* n_drafted, const uint8_t* active, const disco_clf* clf, float tau,
                       int sl_max, int32_t* token, float* conf, uint8_t* halt, float* feats, float* probs,
                       float* nll_sum, int stats_only, void* stream, bool normalize = true,
-                      RecordLayout* layout = nullptr, const ChainLink* chain = nullptr, unsigned int* clear_words = nullptr, int clear_n = 0) {
+                      RecordLayout* layout = nullptr, const ChainLink* chain = nullptr, unsigned int* clear_words = nullptr, int clear_n = 0,
+                      float* stats = nullptr) {
     if (!c || !W_D || !h_D) return DISCO_ERR_INVALID_ARG;
     if (!stats_only && !chain && (!pos || !n_drafted)) return DISCO_ERR_INVALID_ARG;
     if (!stats_only && (!token || !conf || !halt)) return DISCO_ERR_INVALID_ARG;
@@ -679,6 +631,7 @@ int draft_step_common(disco_ctx* c, const void* W_D, const void* h_D, int d, int
     p.R = B;
     p.B = B;
     fill_scratch(c, p);
+    if (stats) p.final_stats = stats;
     p.stats_only = stats_only;
     p.pos = pos;
     p.n_drafted = n_drafted;
@@ -699,19 +652,10 @@ int draft_step_common(disco_ctx* c, const void* W_D, const void* h_D, int d, int
     p.feats = feats;
     p.probs = probs;
     p.nll_sum = nll_sum;
-    // Measured on B200 (Vicuna head, us per step for 1 / 2 / 3 / 4 / 6 / 8 sequences): the tensor-core kernel
-    // that folds the logits a block at a time 14.8 / 17.0 / 19.4 / 21.3 / 24.8 / 26.8, the one with a thread
-    // per hidden row 22.9 / 23.3 / 23.4 / 23.0 / 23.3 / 23.5: the first up to 4 sequences, the second beyond.
-    // The CUDA-core streaming kernel is within 5 % for one sequence and serves as the path without tensor maps.
-    // (its hidden rows stay in shared memory: up to 48 KB of them, so that the ring keeps at least 8 stages)
-    const bool gemv_ok = c->encode_tiled != nullptr && B <= kGemvMaxRows && !stats_only &&
-                         (size_t)((d + kUmmaBK - 1) / kUmmaBK) * (B <= 8 ? 8 : 16) * 128 <= 48 * 1024;
-    const bool use_gemv = gemv_ok && (c->path == 3 || (c->path == 0 && B <= 4));
-    const bool use_umma = !use_gemv && draft_batch_possible(c, B) && (c->path == 2 || c->path == 3 || (c->path == 0 && B >= 2));
-    if (use_gemv) {
-        rc = launch_gemv(c, p, st, layout);
-        if (rc) return rc;
-    } else if (use_umma) {
+    // The tensor-core kernel serves every batch (measured on the Vicuna head, us per step in a stream for 1 / 4 / 7 / 64
+    // sequences: 13.4 / 14.6 / 15.9 / 19.9); the CUDA-core streaming kernel is the path without tensor maps.
+    const bool use_umma = draft_batch_possible(c, B) && c->path != 1;
+    if (use_umma) {
         DraftFinalParams f{};
         f.B = B;
         f.pos = pos;
@@ -728,7 +672,7 @@ int draft_step_common(disco_ctx* c, const void* W_D, const void* h_D, int d, int
         f.conf = conf;
         f.halt = halt;
         f.feats = feats;
-        f.final_stats = c->final_stats;
+        f.final_stats = p.final_stats;
         f.nll_sum = nll_sum;
         f.stats_only = stats_only;
         f.test_stamp_skew = c->test_stamp_skew;
@@ -943,16 +887,19 @@ int disco_extract_features(disco_ctx* c, const void* W_D, const void* H_D, const
     // everything both passes will check, before the first of them is enqueued
     if (!W_D || !H_D || !W_T || !H_T) return DISCO_ERR_INVALID_ARG;
     if (!aligned16(W_D) || !aligned16(H_D) || !aligned16(W_T) || !aligned16(H_T)) return DISCO_ERR_INVALID_ARG;
-    // the same LM-head pass as a draft step, once per model, without the classifier
+    // the same LM-head pass as a draft step, once per model, without the classifier; y_D and y_T receive the logits
     int rc = draft_step_common(c, W_D, H_D, c->d_draft, N, c->max_rows, pos, nullptr, nullptr, nullptr, 0.f, 1, token_D,
-                               nullptr, nullptr, feats_D, y_D, nullptr, 2, stream);
+                               nullptr, nullptr, feats_D, y_D, nullptr, 2, stream, false);
     if (rc) return rc;
     rc = draft_step_common(c, W_T, H_T, c->d_target, N, c->max_rows, pos, nullptr, nullptr, nullptr, 0.f, 1, token_T,
-                           nullptr, nullptr, feats_T, y_T, nullptr, 2, stream);
+                           nullptr, nullptr, feats_T, y_T, nullptr, 2, stream, false, nullptr, nullptr, nullptr, 0,
+                           c->final_stats2);
     if (rc) return rc;
-    tv_label_kernel<<<N, 256, 0, static_cast<cudaStream_t>(stream)>>>(y_D, y_T, token_D, token_T, c->V, tv, label);
+    const cudaError_t e = launch_after(c, tv_label_kernel, dim3((unsigned)N), dim3(kFeatThreads), 0, static_cast<cudaStream_t>(stream),
+                                       y_D, y_T, (const float*)c->final_stats, (const float*)c->final_stats2,
+                                       (const int32_t*)token_D, (const int32_t*)token_T, c->V, tv, label);
     c->launches += 1;
-    return cuda_ok(cudaGetLastError(), "tv_label_kernel launch") ? DISCO_OK : DISCO_ERR_CUDA;
+    return cuda_ok(e, "tv_label_kernel launch") ? DISCO_OK : DISCO_ERR_CUDA;
 }
 
 int disco_verify_ragged(disco_ctx* c, const void* W_T, const void* H_T, const int32_t* draft_ids,

@@ -2,8 +2,9 @@
 // sl_max draft steps (Sec. 3: after every draft token the classifier decides whether the next one is
 // drafted) without leaving the GPU and without a launch per step.
 //
-// Each step is the tensor-core GEMV of umma_gemv.cuh (hidden rows on the TMEM lanes, the CTA's whole slab
-// of the vocabulary on the columns); what the loop adds:
+// Each step is a tensor-core GEMV: hidden rows on the TMEM lanes, the CTA's slab of the vocabulary on the columns (one
+// MMA wide up to 256 rows: an MMA costs the same for few rows as for 128, so the vocabulary is the wide operand).
+// What the loop adds:
 //   * one CTA per SM stays resident for all steps (cooperative launch: the steps hand over through global
 //     memory, so every CTA must be running);
 //   * the producer never stops: as soon as the MMAs of step i have released a ring stage it is refilled
@@ -26,9 +27,25 @@
 // of a batch in flight before the first use), not for few instructions.
 #pragma once
 
-#include "umma_gemv.cuh"
+#include "umma_tail.cuh"
 
 namespace disco {
+
+constexpr int kGemvEpiWarps = 8;
+constexpr int kGemvThreads = (2 + kGemvEpiWarps) * 32;
+constexpr int kGemvMaxStages = 16;
+constexpr int kGemvRowStride = 256 + 4;   // floats per hidden row in the logit staging area (padded: no bank conflicts)
+
+struct GemvParams {
+    TailParams t;     // V, d, R and everything the fused epilogue needs (scratch, classifier, outputs)
+    int TR;           // vocabulary rows per CTA (slab)
+    int tiles;        // ceil(TR / 256)
+    int TRt;          // vocabulary rows per tile
+    int TRN;          // rows of the LM-head box = N of the MMA (TRt rounded up to 16, <= 256)
+    int b_bytes;      // bytes of one ring stage (TRN * 128, a multiple of 1024)
+    int h_rows;       // rows of the hidden-state box (8)
+    int stages;       // ring depth (2 .. kGemvMaxStages)
+};
 
 constexpr int kLoopMaxSteps = 64;
 constexpr unsigned kLoopContinue = 1u, kLoopStop = 2u;
