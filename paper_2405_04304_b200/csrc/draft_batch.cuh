@@ -708,11 +708,15 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
                         float z[32];
                         tmem_ld32(t_chunk, z);
                         const int n = nc - c * 32;
-                        float cut = thr;
-                        if (STATS) {   // only the chunk's largest can be the row's
+                        if (n < 32) {
 #pragma unroll
-                            for (int j = 0; j < 32; ++j) cut = fmaxf(cut, j < n ? z[j] : DISCO_NEG_INF);
+                            for (int j = 0; j < 32; ++j)
+                                if (j >= n) z[j] = DISCO_NEG_INF;
                         }
+                        float cmax = fmaxf(z[0], z[1]);
+#pragma unroll
+                        for (int j = 2; j < 32; j += 2) cmax = max3f(cmax, z[j], z[j + 1]);
+                        const float cut = STATS ? fmaxf(thr, cmax) : thr;   // (STATS: only the chunk's largest can be the row's)
                         unsigned bits = 0u;
 #pragma unroll
                         for (int j = 0; j < 32; ++j)
@@ -720,6 +724,18 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
                         if (n < 32) bits &= (1u << n) - 1u;
                         if (!valid) bits = 0u;
                         const int v = v_first + tc * p.TR + c * 32;
+                        // Nearly always a row has at most one: its chunk maximum.
+                        if (!__any_sync(kFullMask, (bits & (bits - 1u)) != 0u)) {
+                            if (bits != 0u && cmax > best_v) {
+                                best_v = cmax;
+                                best_i = v + __ffs(bits) - 1;
+                            }
+                            if (!STATS) {
+                                top.push(bits != 0u && cmax > thr ? cmax : DISCO_NEG_INF);
+                                thr = fmaxf(thr, top.t[kTopK - 1]);
+                            }
+                            continue;
+                        }
                         for (unsigned left = __reduce_or_sync(kFullMask, bits); left != 0u;) {
                             // two columns at a time (the second may be the first again: it is then left out)
                             const int j = __ffs(left) - 1;
@@ -759,7 +775,7 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
                 xrow[2] = make_float4(top.t[2], top.t[3], top.t[4], top.t[5]);
                 xrow[3] = make_float4(top.t[6], top.t[7], top.t[8], top.t[9]);
             }
-            named_barrier_sync(2, kDbEpiWarps * 32);
+            named_barrier_sync(4 + quad, 64);
             if (share == 0 && warp_has_rows) {
                 const float4 a = xrow[0], b4 = xrow[1], c4 = xrow[2], d4 = xrow[3];
                 // (a share without columns has Z = 0 and m = -inf; a CTA without columns leaves a record with Z = 0)
