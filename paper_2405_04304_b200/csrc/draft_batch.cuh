@@ -872,6 +872,10 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
                     }
                 }
                 if (!__shfl_sync(kFullMask, all, 0)) break;
+                // The records of the other CTAs will not be there before this CTA's own: polling them earlier only loads L2.
+                if (lane == 0 && !epi)
+                    for (int i = 0; i < (1 << 20) && *reinterpret_cast<volatile int*>(s_done) != kDbEpiWarps; ++i) __nanosleep(100);
+                __syncwarp();
             }
             // the next row nobody has taken
             int first = 0;
