@@ -197,25 +197,30 @@ __device__ __forceinline__ void db_finish_row(const DraftBatchParams& p, const D
     float4 q[PER][3];
     {
         const long long t0 = clock64();
+#pragma unroll
+        for (int j = 0; j < PER; ++j)
+#pragma unroll
+            for (int i = 0; i < 3; ++i) q[j][i] = make_float4(0.f, 0.f, 0.f, __uint_as_float(stamp));
+        if (!real) {   // made-up records, so that the loops below run
+            q[0][0] = make_float4(lane * 0.125f, 1.f, 0.f, q[0][0].w);
+            q[0][1] = make_float4(__uint_as_float(1u << 28 | lane), lane * 0.125f, 0.f, q[0][1].w);
+        }
+        unsigned pend = 0u;   // the lane's records that are still awaited: only those are read again
+#pragma unroll
+        for (int j = 0; j < PER; ++j) pend |= j * 32 + lane < NP ? 1u << j : 0u;
         for (int polls = 0;;) {
 #pragma unroll
             for (int j = 0; j < PER; ++j) {
                 const float4* src = recs + (size_t)(j * 32 + lane) * kStampedPieces;
-                const bool has = j * 32 + lane < NP;
+                if ((pend >> j) & 1u)
 #pragma unroll
-                for (int i = 0; i < 3; ++i)
-                    q[j][i] = has ? load_relaxed_v4(src + i) : make_float4(0.f, 0.f, 0.f, __uint_as_float(stamp));
+                    for (int i = 0; i < 3; ++i) q[j][i] = load_relaxed_v4(src + i);
             }
-            if (!real) {   // made-up records, so that the loops below run
-                q[0][0] = make_float4(lane * 0.125f, 1.f, 0.f, q[0][0].w);
-                q[0][1] = make_float4(__uint_as_float(1u << 28 | lane), lane * 0.125f, 0.f, q[0][1].w);
-            }
-            bool good = true;
 #pragma unroll
             for (int j = 0; j < PER; ++j)
-#pragma unroll
-                for (int i = 0; i < 3; ++i) good = good && __float_as_uint(q[j][i].w) == stamp;
-            if (__all_sync(kFullMask, good)) break;
+                if (__float_as_uint(q[j][0].w) == stamp && __float_as_uint(q[j][1].w) == stamp && __float_as_uint(q[j][2].w) == stamp)
+                    pend &= ~(1u << j);
+            if (__all_sync(kFullMask, pend == 0u)) break;
             if ((++polls & 63) == 0) {
                 const bool out = *reinterpret_cast<volatile int*>(p.status) == DISCO_ERR_TIMEOUT ||
                                  clock64() - t0 > kWaitBudgetClocks;
