@@ -340,7 +340,7 @@ int launch_gemv_loop_rk(disco_ctx* c, GemvLoopParams& lp, const CUtensorMap& mW,
     size_t dyn_limit = 0;
     if (!raise_smem_limit(c, setup, kern, 0, &dyn_limit)) return DISCO_ERR_CUDA;
     GemvParams& g = lp.g;
-    const size_t fixed = gemv_loop_fixed_smem_bytes(RK, g.t.clf_H, g.t.d, g.h_rows);
+    const size_t fixed = gemv_loop_fixed_smem_bytes(RK, g.t.clf_H, g.t.d, g.h_rows, g.TRN);
     if (dyn_limit < fixed + 2 * (size_t)g.b_bytes) return DISCO_ERR_UNSUPPORTED_SHAPE;
     g.stages = (int)std::min<size_t>(kGemvMaxStages, (dyn_limit - fixed) / g.b_bytes);
     cudaLaunchConfig_t cfg{};
@@ -364,6 +364,7 @@ int launch_gemv_loop_rk(disco_ctx* c, GemvLoopParams& lp, const CUtensorMap& mW,
 bool gemv_loop_possible(const disco_ctx* c, int B, int sl_max, size_t w_step_stride) {
     if (!c->encode_tiled || B > 4 || sl_max > kLoopMaxSteps) return false;
     if (c->path != 0 && c->path != 3) return false;
+    if ((c->V + c->sm_count - 1) / c->sm_count > 256 * kGemvMaxTiles) return false;   // the fold's lists
     if (w_step_stride != 0 && w_step_stride != (size_t)c->V * c->d_draft * 2) return false;   // one tensor map over all copies
     if ((long long)c->V * sl_max > 0x7fffffffll) return false;
     return (size_t)((c->d_draft + kUmmaBK - 1) / kUmmaBK) * 8 * 128 <= 48 * 1024;

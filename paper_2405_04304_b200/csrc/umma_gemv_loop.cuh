@@ -2,22 +2,22 @@
 // sl_max draft steps (Sec. 3: after every draft token the classifier decides whether the next one is
 // drafted) without leaving the GPU and without a launch per step.
 //
-// Each step is a tensor-core GEMV: hidden rows on the TMEM lanes, the CTA's slab of the vocabulary on the columns (one
-// MMA wide up to 256 rows: an MMA costs the same for few rows as for 128, so the vocabulary is the wide operand).
-// What the loop adds:
+// Each step is a tensor-core GEMV with the vocabulary on the TMEM lanes: the A operand is 128 rows of the LM head, the B
+// operand the hidden rows (N = 16), D[v, r].  An MMA of that shape takes 39 cycles against 112 of one with the hidden rows
+// on the lanes and 224 vocabulary rows on the columns, and its accumulator has one vocabulary row per thread, which is
+// what the fold wants.  What the loop adds:
 //   * one CTA per SM stays resident for all steps (cooperative launch: the steps hand over through global
 //     memory, so every CTA must be running);
 //   * the producer never stops: as soon as the MMAs of step i have released a ring stage it is refilled
 //     with the LM head's tiles for step i + 1, while the CTA folds, publishes its record, and the step is
 //     decided.  Only the hidden rows of step i + 1 are requested after step i has been decided -- in a
 //     decoder they would not exist before;
-//   * the A operand is the one 8-row box of hidden rows read 16 times over (zero stride between the 8-row
-//     groups of the descriptor): every TMEM lane quadrant holds a copy of each row, so all eight epilogue
-//     warps fetch logits, and the MMAs read nothing outside the box (with a non-zero stride they read ring
-//     stages that the TMA unit is refilling, which halved their rate);
-//   * the step's logits of a CTA (at most 256 per hidden row and tile) are folded by the whole CTA, one
-//     logit per thread (cta_fold_tile), into one record per sequence, which is published in stamped
-//     16-byte pieces: no fence and no counter between the writer and its reader;
+//   * the B operand is the one 8-row box of hidden rows read twice over (zero stride between the 8-row groups of the
+//     descriptor), so nothing outside it is read;
+//   * every warp folds its 32 logits of a hidden row (statistics, arg-max, a descending list of ten); one barrier later a
+//     group of warps per sequence ranks the lists' entries that can be among the CTA's ten largest while another of its
+//     warps adds up the statistics, and the CTA's record is published in stamped 16-byte pieces: no fence and no counter
+//     between the writer and its reader;
 //   * CTA 0 finishes the sequences with all eight epilogue warps (group_merge_partials polls the records
 //     of the step until all carry its stamp), records which sequences go on, and publishes the decision
 //     "continue / stop" in a stamped word that every CTA polls (bounded);
@@ -34,14 +34,14 @@ namespace disco {
 constexpr int kGemvEpiWarps = 8;
 constexpr int kGemvThreads = (2 + kGemvEpiWarps) * 32;
 constexpr int kGemvMaxStages = 16;
-constexpr int kGemvRowStride = 256 + 4;   // floats per hidden row in the logit staging area (padded: no bank conflicts)
+constexpr int kGemvMaxTiles = 4;          // tiles of up to 256 vocabulary rows per CTA
 
 struct GemvParams {
     TailParams t;     // V, d, R and everything the fused epilogue needs (scratch, classifier, outputs)
     int TR;           // vocabulary rows per CTA (slab)
     int tiles;        // ceil(TR / 256)
     int TRt;          // vocabulary rows per tile
-    int TRN;          // rows of the LM-head box = N of the MMA (TRt rounded up to 16, <= 256)
+    int TRN;          // rows of the LM-head box (TRt rounded up to 16, <= 256)
     int b_bytes;      // bytes of one ring stage (TRN * 128, a multiple of 1024)
     int h_rows;       // rows of the hidden-state box (8)
     int stages;       // ring depth (2 .. kGemvMaxStages)
@@ -49,12 +49,12 @@ struct GemvParams {
 
 constexpr int kLoopMaxSteps = 64;
 constexpr unsigned kLoopContinue = 1u, kLoopStop = 2u;
-// shared memory of the CTA-wide fold (two copies, used alternately): per-warp reduction slots, the candidates
-// of the final ranking (at most the ten largest of each of the eight warps and the row's running ten), and
-// the warps' values
-constexpr int kFoldCandidates = kGemvEpiWarps * kTopK + kTopK;            // 90
-constexpr int kFoldCandidatesPad = 96;                                    // whole batches of 32, the padding is -inf
-constexpr int kFoldScratchWords = 64 + kFoldCandidatesPad + kGemvEpiWarps * 32;
+// shared memory of the fold, per sequence: the warps' lists, entry k of warp w at [k * NW + w] (NW warps over all tiles;
+// padded with -inf to whole batches of 32), and the warps' statistics
+constexpr int kFoldMaxWarps = kGemvEpiWarps * kGemvMaxTiles;
+constexpr int kFoldListWords = kTopK * kFoldMaxWarps;
+constexpr int kFoldWords = kFoldListWords + 4 * kFoldMaxWarps;
+static_assert(kFoldListWords % 32 == 0, "whole batches");
 
 struct GemvLoopParams {
     GemvParams g;          // geometry of one step; g.t: shapes, scratch, classifier, outputs of step 1, chain bookkeeping
@@ -91,57 +91,47 @@ __device__ __forceinline__ bool mbar_wait_idle(uint64_t* bar, uint32_t parity, i
     }
 }
 
-// Running result of one hidden row over the tiles of a step, in shared memory (16 words):
-// m, Z, S, -, the ten largest logits, the arg-max key.
+// Result of one hidden row of a step, in shared memory (16 words): m, Z, S, -, the ten largest logits, the arg-max key.
 struct RowState {
     float m, Z, S, pad;
     float top[kTopK];
     uint32_t key_lo, key_hi;
 };
 
-// Fold the ncols <= 256 logits of one hidden row and tile (z[c], vocabulary index v0 + c) into the row's
-// running state, by the eight epilogue warps, one logit per thread:
-//   * maximum and arg-max key by warp reductions, then across the warps through shared memory;
-//   * e^(z - M) and its first moment by one exponential per thread and shuffle sums;
-//   * the ten largest by selection: every warp ranks its 32 logits against each other; the largest of the
-//     warps' 10th-largest values (and the row's running 10th) bounds the new 10th from below, so only the
-//     warps' top-ten values and the running values at or above it are candidates (a dozen or so, at most
-//     90), and the candidates are ranked against each other.
-// Two barriers.  sm: kFoldScratchWords words, not the copy the previous call used.  tid: 0 .. 255.
-__device__ __forceinline__ void cta_fold_tile(const float* z, int ncols, int v0, RowState* rs, float* sm, int tid) {
-    constexpr int BAR_THREADS = kGemvEpiWarps * 32;
-    const int lane = tid & 31, w = tid >> 5;
-    uint32_t* wred = reinterpret_cast<uint32_t*>(sm);      // [3][8] m bits, key lo, bits of the warp's 10th largest
-    float* wsum = sm + 24;                                  // [2][8]
-    int* ncand = reinterpret_cast<int*>(sm + 40);           // [1]
-    float* cand = sm + 64;                                  // [kFoldCandidatesPad]
-    float* wvals = cand + kFoldCandidatesPad;               // [8][32] the warps' values
-    const bool valid = tid < ncols;
-    const float val = valid ? z[tid] : DISCO_NEG_INF;
+// RK consecutive accumulator columns: one logit per thread and hidden row
+template <int RK>
+__device__ __forceinline__ void tmem_ld_rows(uint32_t taddr, float (&z)[RK]) {
+    uint32_t r[RK];
+    if constexpr (RK == 1)
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r[0]) : "r"(taddr) : "memory");
+    else if constexpr (RK == 2)
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(taddr) : "memory");
+    else
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                     : "r"(taddr)
+                     : "memory");
+    if constexpr (RK == 1)
+        asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(r[0])::"memory");
+    else if constexpr (RK == 2)
+        asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(r[0]), "+r"(r[1])::"memory");
+    else
+        asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3])::"memory");
+#pragma unroll
+    for (int i = 0; i < RK; ++i) z[i] = __uint_as_float(r[i]);
+}
+
+// A warp's 32 logits of one hidden row (lane's vocabulary index v; lanes without one hold -inf), as warp w of NW: its
+// list and its statistics (m, Z, S, arg-max key low word) go to `fold`.  warp_vals: 32 words owned by the warp.
+__device__ __forceinline__ void warp_fold_row(float val, bool valid, int v, float* fold, int w, int NW, float* warp_vals,
+                                              int lane) {
     const uint32_t bits = ordered_bits(val);
     const uint32_t mb = __reduce_max_sync(kFullMask, bits);
-    // arg-max key of the warp: largest value, lowest index
-    const uint32_t klo_mine = valid && bits == mb ? 0xffffffffu - static_cast<uint32_t>(v0 + tid) : 0u;
-    const uint32_t klo = __reduce_max_sync(kFullMask, klo_mine);
-    const int rank = rank_in_warp(val, lane, wvals + w * 32);
-    if (rank == kTopK - 1) wred[16 + w] = bits;             // the warp's 10th largest (-inf with fewer than ten logits)
-    if (lane == 0) {
-        wred[w] = mb;
-        wred[8 + w] = klo;      // 0: the warp holds no logit
-    }
-    if (tid == 0) *ncand = 0;
-    if (tid < kFoldCandidatesPad) cand[tid] = DISCO_NEG_INF;
-    named_barrier_sync(1, BAR_THREADS);
-    uint32_t Mb = 0u, Klo = 0u, Tb = ordered_bits(rs->top[kTopK - 1]);
-#pragma unroll
-    for (int k = 0; k < kGemvEpiWarps; ++k) {
-        Mb = max(Mb, wred[k]);
-        Tb = max(Tb, wred[16 + k]);
-    }
-#pragma unroll
-    for (int k = 0; k < kGemvEpiWarps; ++k) Klo = max(Klo, wred[k] == Mb ? wred[8 + k] : 0u);
-    const float M = from_ordered_bits(Mb);
-    const float theta = from_ordered_bits(Tb);
+    // arg-max of the warp: largest value, lowest index (0: the warp holds no logit)
+    const uint32_t klo = __reduce_max_sync(kFullMask, valid && bits == mb ? 0xffffffffu - static_cast<uint32_t>(v) : 0u);
+    const int rank = rank_in_warp(val, lane, warp_vals);
+    if (rank < kTopK) fold[rank * NW + w] = val;
+    const float M = from_ordered_bits(mb);
     float e = 0.f, et = 0.f;
     if (valid) {
         const float t = val - M;
@@ -153,43 +143,49 @@ __device__ __forceinline__ void cta_fold_tile(const float* z, int ncols, int v0,
         e += __shfl_xor_sync(kFullMask, e, off);
         et += __shfl_xor_sync(kFullMask, et, off);
     }
-    if (lane == 0) {
-        wsum[w] = e;
-        wsum[8 + w] = et;
+    if (lane == 0) *reinterpret_cast<float4*>(fold + kFoldListWords + 4 * w) = make_float4(M, e, et, __uint_as_float(klo));
+}
+
+// The warps' results of one hidden row -> the CTA's, by a group of GT threads (whole warps; gt: index in it).  A barrier
+// lies before (the warps' results are complete, rs->top is -inf) and after it.
+template <int GT>
+__device__ __forceinline__ void group_fold_row(const float* fold, int NW, RowState* rs, int gt) {
+    const int lane = gt & 31, n = kTopK * NW;
+    // ten logits are at or above the largest of the warps' tenth largest
+    const float theta = from_ordered_bits(
+        __reduce_max_sync(kFullMask, ordered_bits(lane < NW ? fold[(kTopK - 1) * NW + lane] : DISCO_NEG_INF)));
+    // (entries that can qualify come first: the warps' largest, then their second largest, ..)
+    for (int i = gt; i < n; i += GT) {
+        const float x = fold[i];
+        if (x >= theta && x > DISCO_NEG_INF) {
+            const int r = rank_in_list(fold, n, x, i);
+            if (r < kTopK) rs->top[r] = x;
+        }
     }
-    warp_append(valid && rank < kTopK && val >= theta, val, cand, ncand, kFoldCandidatesPad, lane);
-    if (w == 0) {
-        const float run = lane < kTopK ? rs->top[lane] : DISCO_NEG_INF;
-        warp_append(run >= theta && run > DISCO_NEG_INF, run, cand, ncand, kFoldCandidatesPad, lane);
-    }
-    named_barrier_sync(1, BAR_THREADS);
-    const int n = min(*ncand, kFoldCandidatesPad);   // at most 90 by construction
-    if (tid < n) {
-        const float x = cand[tid];
-        const int r = rank_in_list(cand, n, x, tid);
-        if (r < kTopK) rs->top[r] = x;               // entries beyond n were -inf before and stay so
-    }
-    if (tid == 0 && ncols > 0) {
-        float Zt = 0.f, St = 0.f;
+    if (gt >= GT - 32) {
+        const float4 q = lane < NW ? *reinterpret_cast<const float4*>(fold + kFoldListWords + 4 * lane)
+                                   : make_float4(DISCO_NEG_INF, 0.f, 0.f, 0.f);
+        const uint32_t mine = ordered_bits(q.y > 0.f ? q.x : DISCO_NEG_INF);
+        const uint32_t Mb = __reduce_max_sync(kFullMask, mine);
+        const uint32_t klo = __reduce_max_sync(kFullMask, q.y > 0.f && mine == Mb ? __float_as_uint(q.w) : 0u);
+        const float M = from_ordered_bits(Mb);
+        float Z = 0.f, S = 0.f;
+        if (q.y > 0.f) {
+            const float dm = q.x - M;
+            const float e = __expf(dm);
+            Z = q.y * e;
+            S = e * fmaf(dm, q.y, q.z);
+        }
 #pragma unroll
-        for (int k = 0; k < kGemvEpiWarps; ++k) {
-            Zt += wsum[k];
-            St += wsum[8 + k];
+        for (int off = 16; off > 0; off >>= 1) {
+            Z += __shfl_xor_sync(kFullMask, Z, off);
+            S += __shfl_xor_sync(kFullMask, S, off);
         }
-        SoftmaxState st;
-        st.m = rs->m, st.Z = rs->Z, st.S = rs->S;
-        st.merge(M, Zt, St);
-        rs->m = st.m, rs->Z = st.Z, rs->S = st.S;
-        // a later tile holds higher indices: it takes the arg-max only with a strictly larger value
-        const unsigned long long k_tile = (static_cast<unsigned long long>(Mb) << 32) | Klo;
-        const unsigned long long k_run = (static_cast<unsigned long long>(rs->key_hi) << 32) | rs->key_lo;
-        if (k_tile > k_run) {
-            rs->key_hi = Mb;
-            rs->key_lo = Klo;
+        if (lane == 0) {
+            rs->m = M, rs->Z = Z, rs->S = S;
+            rs->key_hi = klo ? Mb : 0u, rs->key_lo = klo;
         }
     }
-    // The caller puts a barrier between this call and any reader of the row state that is not one of the
-    // threads that wrote it; the scratch copy is reused only by the call after the next.
 }
 
 // RK: compile-time bound on the sequences (1, 2 or 4); 8 / RK epilogue warps finish each sequence.
@@ -214,10 +210,10 @@ umma_gemv_loop_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_c
     uint64_t* go_bar = h_full + 1;
     uint32_t* tmem_base_s = reinterpret_cast<uint32_t*>(go_bar + 1);
     uint32_t* s_code = tmem_base_s + 2;                       // [kLoopMaxSteps] decision of each step, as this CTA saw it
-    float* lg_s = reinterpret_cast<float*>(after + 1024);     // [RK][kGemvRowStride] logits of one tile
-    RowState* row_s = reinterpret_cast<RowState*>(lg_s + RK * kGemvRowStride);   // [RK]
-    float* fold_s = reinterpret_cast<float*>(row_s + RK);     // 2 x kFoldScratchWords, used alternately
-    float* group_s = fold_s + 2 * kFoldScratchWords;          // RK x kGroupScratchWords
+    RowState* row_s = reinterpret_cast<RowState*>(after + 1024);                 // [RK]
+    float* fold_s = reinterpret_cast<float*>(row_s + RK);     // [RK][kFoldWords]
+    float* vals_s = fold_s + RK * kFoldWords;                 // [8][32] the warps' logits
+    float* group_s = vals_s + kGemvEpiWarps * 32;             // RK x kGroupScratchWords
     float* clf_s = group_s + RK * kGroupScratchWords;
     __shared__ int s_alive;
     __shared__ int s_pos0[4], s_forced[4], s_live[4];         // the finishing CTA's copy of the per-sequence inputs
@@ -346,7 +342,15 @@ umma_gemv_loop_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_c
     } else if (warp == 1) {
         // ------------------------------ MMA issuer ------------------------------
         if (total > 0 && elect_one()) {
-            const uint32_t idesc = umma_idesc(g.TRN);
+            const uint32_t idesc = umma_idesc(16);
+            const uint32_t full0 = smem_addr(full), empty0 = smem_addr(empty);
+            const uint64_t w0 = umma_smem_desc(w_tiles);
+            const uint64_t h0 = umma_smem_desc(h_tiles) & ~(0x3fffull << 32);   // zero stride between the 8-row groups
+            const uint32_t w_step = (uint32_t)g.b_bytes >> 4, h_step = (uint32_t)h_stride >> 4;   // descriptor units
+            // the rows past 128 of a tile: the last 128 of its box (a multiple of eight rows in)
+            const bool two = g.TRN > 128;
+            const uint32_t second = two ? (uint32_t)(g.TRN - 128) * 8u : 0u;
+            uint64_t w_desc = w0;
             int slot = 0, fill = 0, t_global = 0;
             for (int step0 = 0; step0 < lp.steps; ++step0) {
                 if (step0 > 0) {
@@ -359,22 +363,26 @@ umma_gemv_loop_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_c
                     const int buf = t_global & 1;
                     mbar_wait(&tmem_empty[buf], ((t_global >> 1) & 1) ^ 1, p.status);
                     tc_fence_after();
-                    const uint32_t d_tmem = tmem_base + buf * 256;
+                    const uint32_t d_tmem = tmem_base + buf * 32;
+                    uint64_t h_desc = h0;
                     for (int kb = 0; kb < KB; ++kb) {
-                        mbar_wait(&full[slot], fill & 1, p.status);
+                        mbar_wait(full0 + slot * 8, fill & 1, p.status);
                         tc_fence_after();
-                        // The A operand is the one 8-row box of hidden rows, read 16 times over (zero stride between
-                        // the 8-row groups): hidden row r lands on the TMEM lanes r, r + 8, .., r + 120, so every lane
-                        // quadrant holds a copy and all epilogue warps can fetch logits; nothing outside the box is read.
-                        const uint64_t a_desc = umma_smem_desc(h_tiles + kb * h_stride) & ~(0x3fffull << 32);
-                        const uint64_t b_desc = umma_smem_desc(w_tiles + slot * g.b_bytes);
 #pragma unroll
                         for (int k = 0; k < kUmmaBK / 16; ++k)
-                            tc_mma_bf16(d_tmem, a_desc + 2 * k, b_desc + 2 * k, idesc, (kb | k) != 0);
-                        tc_commit(&empty[slot]);
+                            tc_mma_bf16(d_tmem, w_desc + 2 * k, h_desc + 2 * k, idesc, (kb | k) != 0);
+                        if (two) {
+#pragma unroll
+                            for (int k = 0; k < kUmmaBK / 16; ++k)
+                                tc_mma_bf16(d_tmem + 16, w_desc + second + 2 * k, h_desc + 2 * k, idesc, (kb | k) != 0);
+                        }
+                        tc_commit(empty0 + slot * 8);
+                        w_desc += w_step;
+                        h_desc += h_step;
                         if (++slot == g.stages) {
                             slot = 0;
                             ++fill;
+                            w_desc = w0;
                         }
                     }
                     tc_commit(&tmem_full[buf]);
@@ -408,52 +416,39 @@ umma_gemv_loop_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_c
             s_live[tid] = 1;
         }
         cp_async_wait_all();
-        int t_global = 0, fold_calls = 0;
+        // (the padding of the lists is never written again)
+        for (int i = tid; i < RK * kFoldWords; i += BAR_THREADS) fold_s[i] = DISCO_NEG_INF;
+        named_barrier_sync(1, BAR_THREADS);
+        int t_global = 0;
+        // this thread's vocabulary row within a tile: 128 per half of the tile's box
+        const bool second_half = ew >= 4;
+        const int tile_row = quad * 32 + lane + (second_half ? g.TRN - 128 : 0);
+        const bool row_ok = second_half ? g.TRN > 128 && tile_row >= 128 : true;
+        const int NW = tiles * kGemvEpiWarps;
         int h_ahead_step = -1;     // (thread 0) step whose hidden rows were requested and not yet used
 
         for (int step0 = 0; step0 < lp.steps; ++step0) {
             // stamp of this step's records: unique among everything a reader can still find in the buffer
             const uint32_t rec_stamp = (launch_stamp << 6) | (uint32_t)(step0 & 63) | 0x80000000u;
-            if (tid < RK) {
-                RowState* rs = row_s + tid;
-                rs->m = DISCO_NEG_INF, rs->Z = 0.f, rs->S = 0.f, rs->pad = 0.f;
-#pragma unroll
-                for (int k = 0; k < kTopK; ++k) rs->top[k] = DISCO_NEG_INF;
-                rs->key_lo = 0u, rs->key_hi = 0u;
-            }
+            if (tid < RK * kTopK) row_s[tid / kTopK].top[tid % kTopK] = DISCO_NEG_INF;
             for (int tile = 0; tile < tiles; ++tile, ++t_global) {
                 const int buf = t_global & 1;
                 const int v0 = v_begin + tile * g.TRt;
                 const int ncols = min(g.TRt, v_end - v0);
-                const int nblocks = (ncols + 31) >> 5;
-                {
-                    // every warp fetches its share of the tile's columns from its own lane quadrant (lane r < 8 of a
-                    // quadrant holds hidden row r) and stages them in shared memory, row by row
-                    mbar_wait(&tmem_full[buf], (t_global >> 1) & 1, p.status);
-                    tc_fence_after();
-                    const uint32_t t_quad = tmem_base + buf * 256 + (static_cast<uint32_t>(quad * 32) << 16);
-                    for (int c = ew; c < nblocks; c += kGemvEpiWarps) {
-                        float z[32];
-                        tmem_ld32(t_quad + c * 32, z);
-                        if (lane < B) {
-                            float4* dst = reinterpret_cast<float4*>(lg_s + lane * kGemvRowStride + c * 32);
+                mbar_wait(&tmem_full[buf], (t_global >> 1) & 1, p.status);
+                tc_fence_after();
+                float z[RK];
+                tmem_ld_rows<RK>(tmem_base + buf * 32 + (second_half ? 16 : 0) + (static_cast<uint32_t>(quad * 32) << 16), z);
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&tmem_empty[buf]);
+                const bool valid = row_ok && tile_row < ncols;
 #pragma unroll
-                            for (int j = 0; j < 32; j += 4)
-                                dst[j >> 2] = make_float4(__fadd_rn(z[j], 0.f), __fadd_rn(z[j + 1], 0.f),
-                                                          __fadd_rn(z[j + 2], 0.f), __fadd_rn(z[j + 3], 0.f));
-                        }
-                    }
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&tmem_empty[buf]);
-                }
-                named_barrier_sync(1, BAR_THREADS);
-                for (int r = 0; r < B; ++r, ++fold_calls)
-                    cta_fold_tile(lg_s + r * kGemvRowStride, ncols, v0, row_s + r,
-                                  fold_s + (fold_calls & 1) * kFoldScratchWords, tid);
-                named_barrier_sync(1, BAR_THREADS);   // the staging area is overwritten by the next tile
+                for (int r = 0; r < RK; ++r)
+                    if (r < B)
+                        warp_fold_row(valid ? __fadd_rn(z[r], 0.f) : DISCO_NEG_INF, valid, v0 + tile_row, fold_s + r * kFoldWords,
+                                      tile * kGemvEpiWarps + ew, NW, vals_s + ew * 32, lane);
             }
-            if (tiles == 0) named_barrier_sync(1, BAR_THREADS);   // the cleared row states are visible
             // The MMAs of this step are done with the hidden rows: those of the next step are requested now, ahead
             // of the decision (if the phase stops here they are awaited before the CTA leaves).
             h_ahead_step = -1;
@@ -461,9 +456,16 @@ umma_gemv_loop_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_c
                 loop_issue_hidden(h_tiles, h_stride, KB, &tmap_H, (step0 + 1) * B, h_full);
                 h_ahead_step = step0 + 1;
             }
+            named_barrier_sync(1, BAR_THREADS);   // the warps' results are complete
+            const int gb = ew / GW;               // the sequence this warp's group works for
+            const int gt = (ew % GW) * 32 + lane;
+            if (gb < B) {
+                group_fold_row<GW * 32>(fold_s + gb * kFoldWords, NW, row_s + gb, gt);
+                named_barrier_sync(2 + gb, GW * 32);
+            }
             // ---- the CTA's record of this step for each sequence, in stamped pieces ----
-            if (tid < B * kStampedPieces) {
-                const int r = tid / kStampedPieces, piece = tid - r * kStampedPieces;
+            if (gb < B && gt < kStampedPieces) {
+                const int r = gb, piece = gt;
                 const RowState* rs = row_s + r;
                 float4* dst = lp.records + ((size_t)r * grid + blockIdx.x) * kStampedPieces + piece;
                 const float sf = __uint_as_float(rec_stamp);
@@ -477,8 +479,7 @@ umma_gemv_loop_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_c
             if (blockIdx.x == 0) {
                 if (tid == 0) s_alive = 0;
                 named_barrier_sync(1, BAR_THREADS);
-                const int b = ew / GW;              // the sequence this warp helps to finish
-                const int gt = (ew % GW) * 32 + lane;
+                const int b = gb;
                 if (b < B) {
                     const bool takes_part = s_live[b] != 0;
                     if (takes_part) {               // uniform over the group
@@ -552,13 +553,13 @@ umma_gemv_loop_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_c
     }
 }
 
-inline size_t gemv_loop_fixed_smem_bytes(int RK, int clf_H, int d, int h_rows) {
+inline size_t gemv_loop_fixed_smem_bytes(int RK, int clf_H, int d, int h_rows, int TRN) {
     size_t b = 1024;                                             // alignment
     b += (size_t)((d + kUmmaBK - 1) / kUmmaBK) * h_rows * 128;   // hidden rows
     b += 1024;                                                   // barriers, TMEM address, decisions
-    b += (size_t)RK * kGemvRowStride * 4;                        // logits of one tile
-    b += (size_t)RK * sizeof(RowState);                          // running results of the rows
-    b += (size_t)2 * kFoldScratchWords * 4;                      // CTA-wide fold, two copies
+    b += TRN < 128 ? 16384 : 0;                                  // an MMA reads 128 rows from the start of a stage
+    b += (size_t)RK * sizeof(RowState);                          // results of the rows
+    b += (size_t)(RK * kFoldWords + kGemvEpiWarps * 32) * 4;     // fold
     b += (size_t)RK * kGroupScratchWords * 4;                    // finishing groups
     b += ((size_t)clf_H * (kNFeat + 2) + 4) * 4;                 // classifier parameters
     return b + 128;
