@@ -32,7 +32,7 @@
 namespace disco {
 
 constexpr int kGemvEpiWarps = 8;
-constexpr int kGemvThreads = (2 + kGemvEpiWarps) * 32;
+constexpr int kGemvThreads = (3 + kGemvEpiWarps) * 32;   // producer, two MMA issuers, epilogue
 constexpr int kGemvMaxStages = 16;
 constexpr int kGemvMaxTiles = 4;          // tiles of up to 256 vocabulary rows per CTA
 
@@ -228,14 +228,15 @@ umma_gemv_loop_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_c
     const int v_end = min(p.V, v_begin + g.TR);
     const int tiles = v_begin < p.V ? (v_end - v_begin + g.TRt - 1) / g.TRt : 0;
     const int total = tiles * KB;          // LM-head stages of one step
+    const bool two = g.TRN > 128;          // a tile has rows beyond the 128 of one MMA
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < g.stages; ++s) {
             mbar_init(&full[s], 1);
-            mbar_init(&empty[s], 1);
+            mbar_init(&empty[s], two ? 2 : 1);
         }
         for (int b = 0; b < 2; ++b) {
-            mbar_init(&tmem_full[b], 1);
+            mbar_init(&tmem_full[b], two ? 2 : 1);
             mbar_init(&tmem_empty[b], kGemvEpiWarps);
         }
         mbar_init(h_full, 1);
@@ -294,10 +295,11 @@ umma_gemv_loop_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_c
             bool stopped = false;
             const long long t0 = clock64();
             int polls = 0;
+            int p_step = 0, p_n = 0;          // the next stage to bring into L2: step, stage of the step
             for (;;) {
                 bool progress = false;
                 // the decision of step `live` (its hidden rows were requested by the thread that read the decision)
-                if (live < lp.steps && mbar_try_wait(go_bar, (live - 1) & 1)) {
+                if (live < lp.steps && mbar_test(go_bar, (live - 1) & 1)) {
                     if (s_code[live - 1] != kLoopContinue) {
                         stopped = true;
                         break;
@@ -307,12 +309,26 @@ umma_gemv_loop_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_c
                 }
                 // the next LM-head stage: of a step known to take place, or of the one after it (requested ahead)
                 if (w_step < lp.steps && w_step <= live) {
-                    if (w_fill == 0 || mbar_try_wait(&empty[w_slot], (w_fill - 1) & 1)) {
+                    if (w_fill == 0 || mbar_test(&empty[w_slot], (w_fill - 1) & 1)) {
                         issue_w();
                         progress = true;
                     }
                 } else if (w_step >= lp.steps && live >= lp.steps) {
                     break;                    // everything requested, every step known to take place
+                }
+                // The ring holds a good half of the next step's slab.  Once that has landed, HBM would idle until the step has
+                // been decided: the other half is brought into L2 meanwhile, a box at a time (ten steps, 32000 x 768 head: 124 -> 115 us;
+                // 49152 x 768: 185 -> 154).
+                if (!progress && w_step == live && w_n > 0) {
+                    if (p_step != w_step) p_step = w_step, p_n = w_n;
+                    if (p_n < w_n) p_n = w_n;
+                    const int last = w_slot == 0 ? g.stages - 1 : w_slot - 1;
+                    if (p_n < total && mbar_test(&full[last], (w_slot == 0 ? w_fill - 1 : w_fill) & 1)) {
+                        const int tile = p_n / KB, kb = p_n - tile * KB;
+                        tma_prefetch_l2_2d(&tmap_W, kb * kUmmaBK, w_row + tile * g.TRt);
+                        ++p_n;
+                        progress = true;
+                    }
                 }
                 if (!progress) __nanosleep(32);   // leave the issue slots to the warps that compute
                 if (!progress && (++polls & 1023) == 0) {
@@ -339,18 +355,20 @@ umma_gemv_loop_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_c
                 }
             }
         }
-    } else if (warp == 1) {
-        // ------------------------------ MMA issuer ------------------------------
-        if (total > 0 && elect_one()) {
+    } else if (warp == 1 || warp == 2 + kGemvEpiWarps) {
+        // ------------------------------ MMA issuers ------------------------------
+        // MMAs this small are bound by their issue (39 cycles each, and a wait per stage), so the two halves of a tile have a
+        // warp each: the first 128 rows of the box, and its last 128 (a multiple of eight rows in).
+        const bool first = warp == 1;
+        if (total > 0 && (first || two) && elect_one()) {
             const uint32_t idesc = umma_idesc(16);
             const uint32_t full0 = smem_addr(full), empty0 = smem_addr(empty);
             const uint64_t w0 = umma_smem_desc(w_tiles);
             const uint64_t h0 = umma_smem_desc(h_tiles) & ~(0x3fffull << 32);   // zero stride between the 8-row groups
             const uint32_t w_step = (uint32_t)g.b_bytes >> 4, h_step = (uint32_t)h_stride >> 4;   // descriptor units
-            // the rows past 128 of a tile: the last 128 of its box (a multiple of eight rows in)
-            const bool two = g.TRN > 128;
-            const uint32_t second = two ? (uint32_t)(g.TRN - 128) * 8u : 0u;
-            uint64_t w_desc = w0;
+            const uint64_t w_base = w0 + (first ? 0u : (uint32_t)(g.TRN - 128) * 8u);
+            uint64_t w_desc = w_base;
+            int h_ahead = -1;          // step whose hidden rows were requested and not yet used
             int slot = 0, fill = 0, t_global = 0;
             for (int step0 = 0; step0 < lp.steps; ++step0) {
                 if (step0 > 0) {
@@ -358,12 +376,13 @@ umma_gemv_loop_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_c
                     if (s_code[step0 - 1] != kLoopContinue) break;
                 }
                 if (!mbar_wait(h_full, step0 & 1, p.status)) break;
+                h_ahead = -1;
                 tc_fence_after();
                 for (int tile = 0; tile < tiles; ++tile, ++t_global) {
                     const int buf = t_global & 1;
                     mbar_wait(&tmem_empty[buf], ((t_global >> 1) & 1) ^ 1, p.status);
                     tc_fence_after();
-                    const uint32_t d_tmem = tmem_base + buf * 32;
+                    const uint32_t d_tmem = tmem_base + buf * 32 + (first ? 0 : 16);
                     uint64_t h_desc = h0;
                     for (int kb = 0; kb < KB; ++kb) {
                         mbar_wait(full0 + slot * 8, fill & 1, p.status);
@@ -371,23 +390,26 @@ umma_gemv_loop_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_c
 #pragma unroll
                         for (int k = 0; k < kUmmaBK / 16; ++k)
                             tc_mma_bf16(d_tmem, w_desc + 2 * k, h_desc + 2 * k, idesc, (kb | k) != 0);
-                        if (two) {
-#pragma unroll
-                            for (int k = 0; k < kUmmaBK / 16; ++k)
-                                tc_mma_bf16(d_tmem + 16, w_desc + second + 2 * k, h_desc + 2 * k, idesc, (kb | k) != 0);
-                        }
                         tc_commit(empty0 + slot * 8);
                         w_desc += w_step;
                         h_desc += h_step;
                         if (++slot == g.stages) {
                             slot = 0;
                             ++fill;
-                            w_desc = w0;
+                            w_desc = w_base;
                         }
                     }
                     tc_commit(&tmem_full[buf]);
                 }
+                // Once the MMAs of this step are done with the hidden rows, those of the next step are requested, ahead of the
+                // decision (if the phase stops here they are awaited before the CTA leaves).
+                if (first && step0 + 1 < lp.steps) {
+                    mbar_wait(&tmem_full[(t_global - 1) & 1], ((t_global - 1) >> 1) & 1, p.status);
+                    loop_issue_hidden(h_tiles, h_stride, KB, &tmap_H, (step0 + 1) * B, h_full);
+                    h_ahead = step0 + 1;
+                }
             }
+            if (h_ahead >= 0) mbar_wait(h_full, h_ahead & 1, p.status);
         }
     } else {
         // ------------------------------ epilogue ------------------------------
@@ -425,7 +447,6 @@ umma_gemv_loop_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_c
         const int tile_row = quad * 32 + lane + (second_half ? g.TRN - 128 : 0);
         const bool row_ok = second_half ? g.TRN > 128 && tile_row >= 128 : true;
         const int NW = tiles * kGemvEpiWarps;
-        int h_ahead_step = -1;     // (thread 0) step whose hidden rows were requested and not yet used
 
         for (int step0 = 0; step0 < lp.steps; ++step0) {
             // stamp of this step's records: unique among everything a reader can still find in the buffer
@@ -448,13 +469,6 @@ umma_gemv_loop_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_c
                     if (r < B)
                         warp_fold_row(valid ? __fadd_rn(z[r], 0.f) : DISCO_NEG_INF, valid, v0 + tile_row, fold_s + r * kFoldWords,
                                       tile * kGemvEpiWarps + ew, NW, vals_s + ew * 32, lane);
-            }
-            // The MMAs of this step are done with the hidden rows: those of the next step are requested now, ahead
-            // of the decision (if the phase stops here they are awaited before the CTA leaves).
-            h_ahead_step = -1;
-            if (tid == 0 && step0 + 1 < lp.steps && total > 0) {
-                loop_issue_hidden(h_tiles, h_stride, KB, &tmap_H, (step0 + 1) * B, h_full);
-                h_ahead_step = step0 + 1;
             }
             named_barrier_sync(1, BAR_THREADS);   // the warps' results are complete
             const int gb = ew / GW;               // the sequence this warp's group works for
@@ -541,8 +555,6 @@ umma_gemv_loop_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_c
             named_barrier_sync(1, BAR_THREADS);
             if (s_code[step0] != kLoopContinue) break;
         }
-        // rows requested for a step that does not take place: their copy must land before the CTA leaves
-        if (h_ahead_step >= 0) mbar_wait(h_full, h_ahead_step & 1, p.status);
     }
 
     tc_fence_before();
