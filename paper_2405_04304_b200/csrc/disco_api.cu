@@ -777,9 +777,9 @@ int verify_common(disco_ctx* c, const void* W_T, const void* H_T, const int32_t*
     f.ticket = c->ticket + 16;
     f.padded = p.padded;
     f.dev_R = dev_R;
-    verify_finalize_kernel<<<(B + 3) / 4, 128, 0, st>>>(f);
+    const cudaError_t e = launch_after(c, verify_finalize_kernel, dim3((unsigned)((B + 3) / 4)), dim3(128), 0, st, f);
     c->launches += 1;
-    return cuda_ok(cudaGetLastError(), "verify_finalize_kernel launch") ? DISCO_OK : DISCO_ERR_CUDA;
+    return cuda_ok(e, "verify_finalize_kernel launch") ? DISCO_OK : DISCO_ERR_CUDA;
 }
 
 }  // namespace

@@ -188,9 +188,7 @@ __device__ __forceinline__ void db_finish_row(const DraftBatchParams& p, const D
     const bool chain = f.chain.alive != nullptr;
     float fpos = 0.f;
     int nd = 1;
-    bool act = false;
     if (real) {
-        act = chain_seq_live(f.chain, f.active, b);
         fpos = chain ? static_cast<float>(f.chain.pos0[b] + f.chain.step) : (f.pos ? static_cast<float>(f.pos[b]) : 0.f);
         nd = chain ? f.chain.step : (f.n_drafted ? f.n_drafted[b] : 1);
     }
@@ -339,7 +337,6 @@ __device__ __forceinline__ void db_finish_row(const DraftBatchParams& p, const D
         if (lane < kTopK) sel = fmaxf(res[lane], bound);
         __syncwarp();
     }
-    if (real && !act) return;    // masked: its records were awaited all the same, nothing is written
     SoftmaxState st;
     st.m = M, st.Z = Z, st.S = S;
     const unsigned long long key = argmax_key(M, static_cast<int>(idx));
@@ -528,7 +525,7 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
         const int tile_row = quad * 32 + lane;  // row within this tile of hidden rows
         const int row = m_tile * 128 + tile_row;
         const bool warp_has_rows = m_tile * 128 + quad * 32 < p.R;
-        const bool valid = row < p.R;
+        bool valid = row < p.R;                 // and (once that can be read) its sequence still drafts
         // A single narrow tile is not worth a bound.  With four accumulator buffers the candidates of a tile are looked for
         // one tile later, when the bound that everybody's tiles give has long arrived; otherwise the first tile waits for it.
         const bool use_bound = p.TPC > 1 || p.TR > 32;
@@ -559,7 +556,10 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
                 const int old_rows = *reinterpret_cast<volatile unsigned int*>(p.sync + 2 + (par ^ 1u));
                 if (blockIdx.x == 0)
                     for (int i = ew * 32 + lane; i < f.clear_n; i += kDbEpiWarps * 32) f.clear_words[i] = 0u;
-                keep_mask = __ballot_sync(kFullMask, p.probs && valid && (!f.active || f.active[row]));
+                // Rows of sequences that are masked or have stopped drafting: nobody wants their candidates, and no record of
+                // them is written.
+                valid = valid && chain_seq_live(f.chain, f.active, row);
+                keep_mask = __ballot_sync(kFullMask, p.probs && valid);
                 slots = p.bound + par * p.set_words + (size_t)(valid ? row : 0) * kDbBoundStride;
                 my_slot = slots + nslot % kDbBoundSlots;
                 uint4* old = reinterpret_cast<uint4*>(p.bound + (par ^ 1u) * p.set_words);
@@ -848,7 +848,7 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
         int b = 0;
         bool run = !epi;
         for (bool real = false;; real = true) {
-            if (run) db_finish_row(p, f, b, real, stamp + (real ? f.test_stamp_skew : 0u), sm, clf_s, STATS, lane);
+            if (run && !(real && !chain_seq_live(f.chain, f.active, b))) db_finish_row(p, f, b, real, stamp + (real ? f.test_stamp_skew : 0u), sm, clf_s, STATS, lane);
             run = true;
             if (!real) {
                 if (!epi) {

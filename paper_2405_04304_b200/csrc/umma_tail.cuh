@@ -409,6 +409,9 @@ struct VerifyFinalParams {
 
 __global__ void __launch_bounds__(128) verify_finalize_kernel(const VerifyFinalParams p) {
     __shared__ int s_last;
+    // launched with programmatic stream serialization: resident early, reading only once its predecessor has completed
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int b = blockIdx.x * (blockDim.x >> 5) + warp;
     const int R = p.dev_R ? min(max(__ldcg(p.dev_R), 1), p.R) : p.R;
