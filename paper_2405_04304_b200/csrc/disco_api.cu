@@ -219,10 +219,6 @@ bool encode_bf16_2d(const disco_ctx* c, CUtensorMap* map, const void* base, int 
     return r == CUDA_SUCCESS;
 }
 
-bool umma_possible(const disco_ctx* c, int R) {
-    const int MT = (R + 127) / 128;
-    return c->encode_tiled != nullptr && MT <= c->sm_count;
-}
 
 // Launch the tcgen05 verification kernel for R hidden rows of width d against the LM head W [V, d].
 int launch_umma(disco_ctx* c, const void* W, const void* H, int d, int R, const UmmaParams* fused, cudaStream_t st,
@@ -232,28 +228,25 @@ int launch_umma(disco_ctx* c, const void* W, const void* H, int d, int R, const 
     p.V = c->V;
     p.d = d;
     p.R = R;
-    p.MT = (R + 127) / 128;
-    p.CN = c->sm_count / p.MT;
-    p.TPC = std::max(1, (c->V + 256 * p.CN - 1) / (256 * p.CN));
-    p.TR = (c->V + p.CN * p.TPC - 1) / (p.CN * p.TPC);
-    p.TRN = std::max(16, (p.TR + 15) / 16 * 16);
+    p.t = VerifyTiling::make(R, c->V, d, c->sm_count);
     p.dev_R = dev_R;
-    if (dev_R) p.TRN = 256;   // the kernel derives the tiling from the device-side row count; the box is the largest tile
-    p.a_rows = p.MT > 1 ? 128 : std::max(8, (R + 7) / 8 * 8);
-    // The A stage holds a_rows rows.  The MMA still reads 128 rows from its start: what lies behind the tile (other
+    p.box_rows = dev_R ? 256 : p.t.TRN;   // (the kernel derives the tiling from the device-side row count)
+    p.pairs = dev_R || p.t.GS == 2;
+    p.a_rows = p.t.MT > 1 ? 128 : std::max(8, (R + 7) / 8 * 8);
+    // The A tile holds a_rows rows.  The MMA still reads 128 rows from its start: what lies behind the tile (other
     // stages of the ring, always inside it) only feeds accumulator lanes nobody reads.
     p.a_bytes = (p.a_rows * 128 + 1023) / 1024 * 1024;
-    p.b_bytes = (p.TRN * 128 + 1023) / 1024 * 1024;
-    p.stages = std::max(2, std::min(kUmmaMaxStages, kUmmaRingBytes / (p.a_bytes + p.b_bytes)));
+    p.b_bytes = (p.box_rows * 128 + 1023) / 1024 * 1024;
+    p.stages = std::max(2, std::min(kUmmaMaxStages, kUmmaRingBytes / (p.a_bytes * (1 + p.pairs) + p.b_bytes)));
     p.status = c->status;
     p.keys = c->keys;
     CUtensorMap tmap_W, tmap_H;
-    if (!encode_bf16_2d(c, &tmap_W, W, c->V, d, p.TRN) || !encode_bf16_2d(c, &tmap_H, H, R, d, p.a_rows))
+    if (!encode_bf16_2d(c, &tmap_W, W, c->V, d, p.box_rows) || !encode_bf16_2d(c, &tmap_H, H, R, d, p.a_rows))
         return DISCO_ERR_CUDA;
     static KernelSetup setup;
     if (!raise_smem_limit(c, setup, umma_tail_kernel, (size_t)kUmmaSmemBytes, nullptr)) return DISCO_ERR_CUDA;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)(dev_R ? c->sm_count : p.MT * p.CN));
+    cfg.gridDim = dim3((unsigned)(dev_R ? c->sm_count : p.t.groups * p.t.CN));
     cfg.blockDim = dim3(kUmmaThreads);
     cfg.dynamicSmemBytes = kUmmaSmemBytes;
     cfg.stream = st;
@@ -724,7 +717,7 @@ int verify_common(disco_ctx* c, const void* W_T, const void* H_T, const int32_t*
     p.bonus = bonus;
     p.target_ids = target_ids;
     if (pad) p.padded = *pad;
-    const bool use_umma = umma_possible(c, R) && (c->path == 2 || (c->path == 0 && R >= 2));
+    const bool use_umma = c->encode_tiled != nullptr && (c->path == 2 || (c->path == 0 && R >= 2));
     if (!use_umma) return run_stream<false>(c, p, 0, st);
     // Fixed-shape rows beyond one tile of 128: the projection is no longer free of charge for the rows that do not
     // count, so they are packed first and the tensor-core kernel tiles for the row count it finds on the device.

@@ -13,10 +13,8 @@
 //              and the logits never leave the chip.  Two warps share each TMEM lane quadrant and
 //              split the columns.
 //
-// A CTA keeps one tile of hidden rows (m_tile) and walks over a contiguous range of vocabulary
-// tiles; CTAs that share a vocabulary tile run side by side, so the LM head crosses HBM once and is
-// shared through L2.  Results leave the CTA as one atomicMax per row; the last CTA (few sequences) or a small
-// separate kernel finishes the job.
+// A CTA keeps one or two tiles of hidden rows and walks over a contiguous range of vocabulary tiles (VerifyTiling).  CTAs that share a vocabulary tile run side by side, so the LM head crosses HBM once and is shared through L2.
+// Results leave the CTA as one atomicMax per row; the last CTA (few sequences) or a small separate kernel finishes the job.
 #pragma once
 
 #include <cuda.h>
@@ -36,16 +34,39 @@ constexpr int kUmmaSmemBytes = kUmmaRingBytes + 1024 /*align*/ + 512 /*barriers*
 // shared memory of a staged classifier (draft steps)
 inline int umma_clf_bytes(int clf_H) { return (clf_H * (kNFeat + 2) + 4) * 4; }
 
+// How R hidden rows and V vocabulary rows are cut: MT tiles of 128 hidden rows, GS of them (1 or 2) to a CTA; CN CTAs per
+// such group share the vocabulary, TPC tiles of TR rows each (MMA width TRN).  The groups of a vocabulary tile run side by
+// side: with the whole of H against one vocabulary tile after the other in each CTA, the LM head came from HBM once per
+// group (1000 rows, 32000 x 5120 head: 284 us instead of 235).
+struct VerifyTiling {
+    int MT, GS, groups, CN, TPC, TR, TRN;
+    __host__ __device__ static VerifyTiling make(int R, int V, int d, int grid) {
+        VerifyTiling t;
+        t.MT = (R + 127) / 128;
+        // Two tiles of hidden rows per CTA halve the LM head's traffic from L2 (425 rows, 32000 x 5120 head: 133 -> 120 us;
+        // 130 rows, 32000 x 2048: 35 -> 31), but they use both accumulators, so the epilogue does not overlap the next
+        // tile's MMAs (1000 rows, 32000 x 768: 39 -> 43), and an odd last tile has its CTAs to itself (300 rows: 105 -> 116).
+        // So: two tiles that share every vocabulary tile always; more where the contraction is long and the CTAs' largest
+        // share of work grows by at most a twentieth.
+        const int cn_pairs = grid / ((t.MT + 1) / 2), cn_single = grid / t.MT;
+        t.GS = t.MT == 2 || (t.MT > 2 && d >= 2048 && cn_pairs * 21 >= cn_single * 40) ? 2 : 1;
+        t.groups = (t.MT + t.GS - 1) / t.GS;
+        t.CN = grid / t.groups;
+        t.TPC = (V + 256 * t.CN - 1) / (256 * t.CN);
+        t.TR = (V + t.CN * t.TPC - 1) / (t.CN * t.TPC);
+        t.TRN = (t.TR + 15) / 16 * 16;
+        return t;
+    }
+};
+
 struct UmmaParams {
     int V, d, R;
-    int MT;      // tiles of 128 hidden rows
-    int CN;      // CTAs per m_tile (grid = MT * CN)
-    int TPC;     // vocabulary tiles per CTA
-    int TR;      // vocabulary rows per tile; the MMA and the TMA box use TRN = TR rounded up to 16
-    int TRN;
-    int a_rows;  // rows of the H box (multiple of 8, <= 128)
-    int stages;  // ring depth (<= kUmmaMaxStages); stage s holds an A tile of a_bytes and a B tile of b_bytes
+    VerifyTiling t;
+    int box_rows;  // rows of the LM-head box
+    int a_rows;    // rows of the H box (multiple of 8, <= 128)
+    int stages;    // ring depth (<= kUmmaMaxStages); stage s holds one or two A tiles of a_bytes and a B tile of b_bytes
     int a_bytes, b_bytes;  // multiples of 1024
+    int pairs;     // 1: stages have room for two A tiles
     int* status;
     unsigned long long* keys;  // [R]
     // verification finished inside this kernel by the last CTA (few sequences only)
@@ -58,9 +79,8 @@ struct UmmaParams {
     int32_t* bonus;
     int32_t* target_ids;
     VerifyPadded padded;   // sl != null: fixed-shape rows, per-sequence look-ahead read from the device
-    // Verification whose row count is device memory (rows packed by the kernel before this one): R, MT, CN, TPC, TR
-    // above are then upper bounds / unused, the kernel derives the tiling from *dev_R; TRN stays the box height of
-    // the LM-head tensor map (256) and the MMAs take the tile height rounded up to 16.
+    // Verification whose row count is device memory (rows packed by the kernel before this one): R is then an upper bound,
+    // the kernel derives the tiling from *dev_R, and the LM-head box is 256 rows high.
     const int32_t* dev_R;
 };
 
@@ -187,7 +207,7 @@ umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_consta
     extern __shared__ uint8_t smem_dyn[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023));
     uint8_t* a_tiles = smem;
-    uint8_t* b_tiles = smem + p.stages * p.a_bytes;
+    uint8_t* b_tiles = smem + p.stages * p.a_bytes * (1 + p.pairs);
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + kUmmaRingBytes);
     uint64_t* empty = full + kUmmaMaxStages;
     uint64_t* tmem_full = empty + kUmmaMaxStages;
@@ -202,20 +222,19 @@ umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_consta
     const int lane = threadIdx.x & 31;
     const int KB = (p.d + kUmmaBK - 1) / kUmmaBK;
     // tiling: from the host, or (row count in device memory) derived here by the same rule
-    int gR = p.R, gMT = p.MT, gCN = p.CN, gTPC = p.TPC, gTR = p.TR, gTRN = p.TRN;
-    bool idle = false;
+    int R = p.R;
+    VerifyTiling tl = p.t;
     if (p.dev_R) {
         asm volatile("griddepcontrol.wait;" ::: "memory");   // the count is the predecessor's output
-        gR = min(max(__ldcg(p.dev_R), 1), p.R);
-        gMT = (gR + 127) / 128;
-        gCN = (int)gridDim.x / gMT;
-        gTPC = max(1, (p.V + 256 * gCN - 1) / (256 * gCN));
-        gTR = (p.V + gCN * gTPC - 1) / (gCN * gTPC);
-        gTRN = max(16, (gTR + 15) / 16 * 16);
-        idle = (int)blockIdx.x >= gMT * gCN;
+        R = min(max(__ldcg(p.dev_R), 1), p.R);
+        tl = VerifyTiling::make(R, p.V, p.d, (int)gridDim.x);
     }
-    const int m_tile = blockIdx.x % gMT;
-    const int nslot = blockIdx.x / gMT;
+    // this CTA: `size` tiles of hidden rows from m_tile on, vocabulary rows v_begin .. v_end - 1 in tiles of TR
+    const int m_tile = (int)blockIdx.x % tl.groups * tl.GS;
+    const int size = min(tl.GS, tl.MT - m_tile);
+    const int slot = (int)blockIdx.x / tl.groups;
+    const int v_begin = slot * tl.TPC * tl.TR;
+    const int v_end = min(p.V, v_begin + tl.TPC * tl.TR);
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < p.stages; ++s) {
@@ -239,36 +258,42 @@ umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_consta
     tc_fence_after();
     const uint32_t tmem_base = *tmem_base_s;
 
-    const bool live = !idle;   // a CTA beyond the tiling derived from the device-side row count has nothing to do
+    const bool live = slot < tl.CN;   // (CTAs beyond the tiling have nothing to do)
 
     if (warp == 0) {
         // ------------------------------ producer ------------------------------
         if (live && elect_one()) {
             // A single thread: running addresses and counters, as few instructions per stage as possible.
             const uint32_t full0 = smem_addr(full), empty0 = smem_addr(empty), a0 = smem_addr(a_tiles), b0 = smem_addr(b_tiles);
-            const uint32_t bytes = (uint32_t)(p.a_rows + p.TRN) * 128u;   // the boxes of the two tensor maps
-            const int k_end = KB * kUmmaBK, h_row = m_tile * 128;
+            const uint32_t a_box = (uint32_t)p.a_rows * 128u, w_box = (uint32_t)p.box_rows * 128u;   // bytes of the two boxes
+            const uint32_t a_step = (uint32_t)p.a_bytes * (1 + p.pairs);
+            const int k_end = KB * kUmmaBK;
             // The LM head is never written by this library: its first tiles are requested before the
             // dependency wait, the hidden-state tiles of the same stages right after it.
-            int v0 = nslot * gTPC * gTR;
-            const int pre = v0 < p.V ? min(p.stages, KB) : 0;
+            const int h_row = m_tile * 128;
+            int v0 = v_begin;
+            const int pre = v0 < v_end ? min(p.stages, KB) : 0;
             for (int n = 0; n < pre; ++n) {
-                mbar_arrive_expect_tx(full0 + n * 8, bytes);
+                mbar_arrive_expect_tx(full0 + n * 8, w_box + size * a_box);
                 tma_load_2d(b0 + n * p.b_bytes, &tmap_W, n * kUmmaBK, v0, full0 + n * 8);
             }
             asm volatile("griddepcontrol.wait;" ::: "memory");
-            for (int n = 0; n < pre; ++n) tma_load_2d(a0 + n * p.a_bytes, &tmap_H, n * kUmmaBK, h_row, full0 + n * 8);
+            for (int n = 0; n < pre; ++n) {
+                tma_load_2d(a0 + n * a_step, &tmap_H, n * kUmmaBK, h_row, full0 + n * 8);
+                if (size == 2) tma_load_2d(a0 + n * a_step + p.a_bytes, &tmap_H, n * kUmmaBK, h_row + 128, full0 + n * 8);
+            }
             int stage = pre == p.stages ? 0 : pre, phase = pre == p.stages ? 1 : 0;
             int k = pre * kUmmaBK;
-            uint32_t at_a = a0 + stage * p.a_bytes, at_b = b0 + stage * p.b_bytes;
-            for (int i = 0; i < gTPC && v0 < p.V; ++i, v0 += gTR, k = 0) {
+            uint32_t at_a = a0 + stage * a_step, at_b = b0 + stage * p.b_bytes;
+            for (; v0 < v_end; v0 += tl.TR, k = 0) {
                 for (; k < k_end; k += kUmmaBK) {
                     const uint32_t bar = full0 + stage * 8;
                     mbar_wait(empty0 + stage * 8, phase ^ 1, p.status);
-                    mbar_arrive_expect_tx(bar, bytes);
+                    mbar_arrive_expect_tx(bar, w_box + size * a_box);
                     tma_load_2d(at_b, &tmap_W, k, v0, bar);
                     tma_load_2d(at_a, &tmap_H, k, h_row, bar);
-                    at_a += p.a_bytes;
+                    if (size == 2) tma_load_2d(at_a + p.a_bytes, &tmap_H, k, h_row + 128, bar);
+                    at_a += a_step;
                     at_b += p.b_bytes;
                     if (++stage == p.stages) {
                         stage = 0;
@@ -282,24 +307,31 @@ umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_consta
     } else if (warp == 1) {
         // ------------------------------ MMA issuer ------------------------------
         if (live && elect_one()) {
-            const uint32_t idesc = umma_idesc(gTRN);
+            const uint32_t idesc = umma_idesc(tl.TRN);
             const uint32_t full0 = smem_addr(full), empty0 = smem_addr(empty);
             const uint64_t a0 = umma_smem_desc(a_tiles), b0 = umma_smem_desc(b_tiles);
-            const uint32_t a_step = (uint32_t)p.a_bytes >> 4, b_step = (uint32_t)p.b_bytes >> 4;   // descriptor units
+            const uint32_t a_half = (uint32_t)p.a_bytes >> 4, a_step = a_half * (1 + p.pairs), b_step = (uint32_t)p.b_bytes >> 4;   // descriptor units
             uint64_t a_desc = a0, b_desc = b0;
             int stage = 0, phase = 0;
-            for (int i = 0; i < gTPC; ++i) {
-                if ((nslot * gTPC + i) * gTR >= p.V) break;
-                const int buf = i & 1;
-                mbar_wait(&tmem_empty[buf], ((i >> 1) & 1) ^ 1, p.status);
+            // Two tiles of hidden rows use an accumulator each, one alternates between the two.
+            int it = 0;
+            for (int v0 = v_begin; v0 < v_end; v0 += tl.TR, ++it) {
+                const int first = size == 2 ? 0 : it & 1;
+                const uint32_t parity = (size == 2 ? it : it >> 1) & 1;
+                for (int j = 0; j < size; ++j) mbar_wait(&tmem_empty[first + j], parity ^ 1u, p.status);
                 tc_fence_after();
-                const uint32_t d_tmem = tmem_base + buf * 256;
+                const uint32_t d_tmem = tmem_base + first * 256;
                 for (int kb = 0; kb < KB; ++kb) {
                     mbar_wait(full0 + stage * 8, phase, p.status);
                     tc_fence_after();
 #pragma unroll
                     for (int k = 0; k < kUmmaBK / 16; ++k)  // 16 k-elements = 32 bytes = 2 descriptor units
                         tc_mma_bf16(d_tmem, a_desc + 2 * k, b_desc + 2 * k, idesc, (kb | k) != 0);
+                    if (size == 2) {
+#pragma unroll
+                        for (int k = 0; k < kUmmaBK / 16; ++k)
+                            tc_mma_bf16(d_tmem + 256, a_desc + a_half + 2 * k, b_desc + 2 * k, idesc, (kb | k) != 0);
+                    }
                     tc_commit(empty0 + stage * 8);
                     a_desc += a_step;
                     b_desc += b_step;
@@ -310,7 +342,7 @@ umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_consta
                         b_desc = b0;
                     }
                 }
-                tc_commit(&tmem_full[buf]);
+                for (int j = 0; j < size; ++j) tc_commit(&tmem_full[first + j]);
             }
         }
     } else if (live) {
@@ -319,57 +351,68 @@ umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_consta
         const int ew = warp - 2;            // 0 .. kUmmaEpiWarps-1
         const int quad = warp & 3;          // TMEM lane quadrant this warp may read
         const int share = ew >> 2;          // two warps per quadrant split the columns of a tile
-        const int row = m_tile * 128 + quad * 32 + lane;
-        const bool warp_has_rows = m_tile * 128 + quad * 32 < gR;
-        const bool valid = row < gR;
-        float best_v = DISCO_NEG_INF;
-        int best_i = kNoIndex;
-
+        float best_v[2] = {DISCO_NEG_INF, DISCO_NEG_INF};
+        int best_i[2] = {kNoIndex, kNoIndex};
         int it = 0;
-        for (int i = 0; i < gTPC; ++i) {
-            const int v0 = (nslot * gTPC + i) * gTR;
-            if (v0 >= p.V) break;
-            const int buf = it & 1;
-            mbar_wait(&tmem_full[buf], (it >> 1) & 1, p.status);
-            tc_fence_after();
-            const int ncols = min(gTR, p.V - v0);  // further columns belong to the next tile or lie past V
-            if (warp_has_rows) {
-                const int nchunks = (ncols + 31) >> 5;
-                const int c_lo = (nchunks * share + 1) / 2;
-                const int c_hi = (nchunks * (share + 1) + 1) / 2;
-                for (int c = c_lo; c < c_hi; ++c) {
-                    float z[32];
-                    tmem_ld32(tmem_base + buf * 256 + c * 32 + (static_cast<uint32_t>(quad * 32) << 16), z);
-                    const int cbase = c * 32;
+        for (int v0 = v_begin; v0 < v_end; v0 += tl.TR, ++it) {
+            const int ncols = min(tl.TR, v_end - v0);  // further columns belong to the next tile or lie past V
+            const int nchunks = (ncols + 31) >> 5;
+            const int c_lo = (nchunks * share + 1) / 2, c_hi = (nchunks * (share + 1) + 1) / 2;
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) {
-                        const float zz = __fadd_rn(z[j], 0.f);
-                        if (cbase + j < ncols && zz > best_v) {
-                            best_v = zz;
-                            best_i = v0 + cbase + j;
+            for (int j = 0; j < 2; ++j) {
+                if (j >= size) break;
+                const int b = size == 2 ? j : it & 1;
+                mbar_wait(&tmem_full[b], (size == 2 ? it : it >> 1) & 1, p.status);
+                tc_fence_after();
+                if ((m_tile + j) * 128 + quad * 32 < R) {
+                    for (int c = c_lo; c < c_hi; ++c) {
+                        float z[32];
+                        tmem_ld32(tmem_base + b * 256 + c * 32 + (static_cast<uint32_t>(quad * 32) << 16), z);
+                        const int n = ncols - c * 32;
+                        if (n < 32) {
+#pragma unroll
+                            for (int i = 0; i < 32; ++i)
+                                if (i >= n) z[i] = DISCO_NEG_INF;
+                        }
+                        float cmax = fmaxf(z[0], z[1]);
+#pragma unroll
+                        for (int i = 2; i < 32; i += 2) cmax = RegTop10::max3(cmax, z[i], z[i + 1]);
+                        // (a chunk seldom holds a new largest logit: its index is looked for only then)
+                        if (__any_sync(kFullMask, cmax > best_v[j])) {
+                            int at = 0;
+#pragma unroll
+                            for (int i = 31; i >= 0; --i)
+                                if (z[i] == cmax) at = i;
+                            if (cmax > best_v[j]) {
+                                best_v[j] = cmax;
+                                best_i[j] = v0 + c * 32 + at;
+                            }
                         }
                     }
                 }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&tmem_empty[b]);
             }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&tmem_empty[buf]);
-            ++it;
         }
-
         // one result per hidden row and CTA
-        if (valid && best_i != kNoIndex) atomicMax(p.keys + row, argmax_key(best_v, best_i));
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const int row = (m_tile + j) * 128 + quad * 32 + lane;
+            if (j < size && row < R && best_i[j] != kNoIndex)
+                atomicMax(p.keys + row, argmax_key(__fadd_rn(best_v[j], 0.f), best_i[j]));
+        }
         if (p.fuse_final) {
             // ticket: the last CTA to get here matches the prefixes and clears the keys
             __shared__ int s_last;
             __threadfence();
             named_barrier_sync(2, kUmmaEpiWarps * 32);
-            if (ew == 0 && lane == 0) s_last = atomicAdd(p.ticket, 1u) == (unsigned)(gMT * gCN) - 1u;   // idle CTAs take none
+            if (ew == 0 && lane == 0) s_last = atomicAdd(p.ticket, 1u) == (unsigned)(tl.groups * tl.CN) - 1u;   // CTAs beyond the tiling take none
             named_barrier_sync(2, kUmmaEpiWarps * 32);
             if (s_last) {
                 __threadfence();
                 for (int b = ew; b < p.B; b += kUmmaEpiWarps)
-                    verify_one_sequence(p.keys, p.draft_ids, p.row_off, p.B, p.SL, gR, b, p.n_accept, p.bonus,
+                    verify_one_sequence(p.keys, p.draft_ids, p.row_off, p.B, p.SL, R, b, p.n_accept, p.bonus,
                                         p.target_ids, p.status, lane, p.padded);
                 if (ew == 0) warp_write_row_offsets(p.padded, p.B, p.SL, lane);
                 named_barrier_sync(2, kUmmaEpiWarps * 32);
