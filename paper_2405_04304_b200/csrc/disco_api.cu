@@ -60,6 +60,8 @@ struct disco_ctx {
     long long launches;
     cudaStream_t last_stream;  // stream of the most recent enqueue (disco_last_device_status waits for it only)
     unsigned int test_stamp_skew;  // disco_test_hooks
+    void* device_mem;  // every device buffer below
+    void* host_mem;    // the pinned staging below
     // scratch for cross-block reductions
     int part_rows;  // rows the partial buffers can hold
     int max_grid;
@@ -432,8 +434,10 @@ int disco_create(disco_ctx** out, int V, int d_draft, int d_target, int max_batc
     disco_ctx* c = new (std::nothrow) disco_ctx();
     if (!c) return DISCO_ERR_CUDA;
     std::memset(c, 0, sizeof(*c));
-    cudaDeviceProp prop;
-    if (cudaGetDevice(&c->device) != cudaSuccess || cudaGetDeviceProperties(&prop, c->device) != cudaSuccess) {
+    int sms = 0, optin = 0;   // (two attributes: the whole cudaDeviceProp takes milliseconds)
+    if (cudaGetDevice(&c->device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device) != cudaSuccess) {
         delete c;
         return DISCO_ERR_CUDA;
     }
@@ -447,8 +451,8 @@ int disco_create(disco_ctx** out, int V, int d_draft, int d_target, int max_batc
         const char* e = std::getenv("DISCO_PDL");
         c->pdl = !(e && e[0] == '0');
     }
-    c->sm_count = prop.multiProcessorCount;
-    c->smem_optin = prop.sharedMemPerBlockOptin;
+    c->sm_count = sms;
+    c->smem_optin = (size_t)optin;
 
     const int rpc = std::max(1, std::min((V + c->sm_count - 1) / c->sm_count, 2048));
     c->max_grid = (V + rpc - 1) / rpc;
@@ -465,39 +469,60 @@ int disco_create(disco_ctx** out, int V, int d_draft, int d_target, int max_batc
     // the largest layout is disco_iteration_host's: 6 arrays of max_batch words and 2 of max_rows
     const size_t n_int = (size_t)8 * max_batch + (size_t)3 * max_rows + 64;
     const size_t hid = std::max((size_t)max_batch * d_draft, (size_t)max_rows * d_target) * 2;
-    bool ok = true;
-    ok = ok && cudaMalloc(&c->keys, (size_t)max_rows * sizeof(unsigned long long)) == cudaSuccess;
-    ok = ok && cudaMalloc(&c->part_rec, slots * 64) == cudaSuccess;
-    ok = ok && cudaMalloc(&c->ticket, 1024) == cudaSuccess;
-    ok = ok && cudaMalloc(&c->status, 256) == cudaSuccess;
-    ok = ok && cudaMalloc(&c->final_stats, (size_t)c->part_rows * 2 * sizeof(float)) == cudaSuccess;
-    ok = ok && cudaMalloc(&c->final_stats2, (size_t)c->part_rows * 2 * sizeof(float)) == cudaSuccess;
-    ok = ok && cudaMalloc(&c->chain_alive, (size_t)max_batch + 64) == cudaSuccess;
-    ok = ok && cudaMalloc(&c->sample_seg_tot, (size_t)max_batch * kSampleMaxSegments * 2 * sizeof(double)) == cudaSuccess;
-    ok = ok && cudaMalloc(&c->sample_seg_last, (size_t)max_batch * kSampleMaxSegments * 2 * sizeof(int32_t)) == cudaSuccess;
-    ok = ok && cudaMalloc(&c->sample_tickets, (size_t)max_batch * sizeof(unsigned int)) == cudaSuccess;
-    ok = ok && cudaMalloc(&c->pack_rows, (size_t)max_rows * d_target * 2) == cudaSuccess;
-    ok = ok && cudaMalloc(&c->pack_off, ((size_t)max_batch + 2) * sizeof(int32_t)) == cudaSuccess;
-    ok = ok && cudaMalloc(&c->loop_rec, (size_t)4 * c->sm_count * 80) == cudaSuccess;
-    ok = ok && cudaMemset(c->loop_rec, 0, (size_t)4 * c->sm_count * 80) == cudaSuccess;   // no stamp yet
-    ok = ok && cudaMalloc(&c->stage_hidden, hid) == cudaSuccess;
-    ok = ok && cudaMalloc(&c->stage_hidden_draft, (size_t)max_rows * d_draft * 2) == cudaSuccess;
+    // One device allocation and one pinned one, cut into pieces of 256 bytes; what must start at zero comes first.
+    // (A call to the allocator costs tens of microseconds to milliseconds, and there are about twenty pieces.)
+    size_t dev_bytes = 0, host_bytes = 0, zero_bytes = 0;
+    struct Piece {
+        void** p;
+        size_t at;
+    };
+    Piece pieces[32];
+    int n_pieces = 0;
+    auto device = [&](auto** p, size_t bytes) {
+        pieces[n_pieces++] = Piece{reinterpret_cast<void**>(p), dev_bytes};
+        dev_bytes += (bytes + 255) & ~(size_t)255;
+    };
+    device(&c->keys, (size_t)max_rows * sizeof(unsigned long long));
+    device(&c->ticket, 1024);
+    device(&c->status, 256);
+    device(&c->loop_rec, (size_t)4 * c->sm_count * 80);            // no stamp yet
+    // R rows take R * (sm_count / ceil(R / 128)) <= 128 * sm_count records
+    device(&c->stamped_rec, (size_t)128 * c->sm_count * 80);       // no stamp yet
+    device(&c->row_bound, (size_t)2 * c->part_rows * kDbBoundStride * 4);
+    zero_bytes = dev_bytes;
+    device(&c->part_rec, slots * 64);
+    device(&c->final_stats, (size_t)c->part_rows * 2 * sizeof(float));
+    device(&c->final_stats2, (size_t)c->part_rows * 2 * sizeof(float));
+    device(&c->chain_alive, (size_t)max_batch + 64);
+    device(&c->sample_seg_tot, (size_t)max_batch * kSampleMaxSegments * 2 * sizeof(double));
+    device(&c->sample_seg_last, (size_t)max_batch * kSampleMaxSegments * 2 * sizeof(int32_t));
+    device(&c->sample_tickets, (size_t)max_batch * sizeof(unsigned int));
+    device(&c->pack_rows, (size_t)max_rows * d_target * 2);
+    device(&c->pack_off, ((size_t)max_batch + 2) * sizeof(int32_t));
+    device(&c->stage_hidden, hid);
+    device(&c->stage_hidden_draft, (size_t)max_rows * d_draft * 2);
+    auto pinned = [&](size_t bytes) {
+        const size_t at = host_bytes;
+        host_bytes += (bytes + 255) & ~(size_t)255;
+        return at;
+    };
+    const size_t at_int = pinned(n_int * sizeof(int32_t));
+    const size_t at_float = pinned(((size_t)max_batch * (1 + kNFeat) + max_rows) * sizeof(float));
+    const size_t at_byte = pinned((size_t)max_batch * 2 + max_rows + 64);
+    void* host_d = nullptr;
+    bool ok = cudaMalloc(&c->device_mem, dev_bytes) == cudaSuccess;
+    ok = ok && cudaHostAlloc(&c->host_mem, host_bytes, cudaHostAllocMapped) == cudaSuccess;
+    ok = ok && cudaHostGetDevicePointer(&host_d, c->host_mem, 0) == cudaSuccess;
     ok = ok && cudaStreamCreateWithFlags(&c->copy_stream, cudaStreamNonBlocking) == cudaSuccess;
     ok = ok && cudaEventCreateWithFlags(&c->copy_done, cudaEventDisableTiming) == cudaSuccess;
-    ok = ok && cudaHostAlloc(&c->stage_int_h, n_int * sizeof(int32_t), cudaHostAllocMapped) == cudaSuccess;
-    ok = ok && cudaHostAlloc(&c->stage_float_h, ((size_t)max_batch * (1 + kNFeat) + max_rows) * sizeof(float), cudaHostAllocMapped) == cudaSuccess;
-    ok = ok && cudaHostAlloc(&c->stage_byte_h, (size_t)max_batch * 2 + max_rows + 64, cudaHostAllocMapped) == cudaSuccess;
-    ok = ok && cudaHostGetDevicePointer(&c->stage_int_d, c->stage_int_h, 0) == cudaSuccess;
-    ok = ok && cudaHostGetDevicePointer(&c->stage_float_d, c->stage_float_h, 0) == cudaSuccess;
-    ok = ok && cudaHostGetDevicePointer(&c->stage_byte_d, c->stage_byte_h, 0) == cudaSuccess;
-    ok = ok && cudaMemset(c->keys, 0, (size_t)max_rows * sizeof(unsigned long long)) == cudaSuccess;
-    ok = ok && cudaMemset(c->ticket, 0, 1024) == cudaSuccess;
-    // R rows take R * (sm_count / ceil(R / 128)) <= 128 * sm_count records
-    ok = ok && cudaMalloc(&c->stamped_rec, (size_t)128 * c->sm_count * 80) == cudaSuccess;
-    ok = ok && cudaMemset(c->stamped_rec, 0, (size_t)128 * c->sm_count * 80) == cudaSuccess;  // no stamp yet
-    ok = ok && cudaMalloc(&c->row_bound, (size_t)2 * c->part_rows * kDbBoundStride * 4) == cudaSuccess;
-    ok = ok && cudaMemset(c->row_bound, 0, (size_t)2 * c->part_rows * kDbBoundStride * 4) == cudaSuccess;
-    ok = ok && cudaMemset(c->status, 0, 256) == cudaSuccess;
+    ok = ok && cudaMemset(c->device_mem, 0, zero_bytes) == cudaSuccess;
+    if (ok) {
+        for (int i = 0; i < n_pieces; ++i) *pieces[i].p = static_cast<char*>(c->device_mem) + pieces[i].at;
+        char *h = static_cast<char*>(c->host_mem), *d = static_cast<char*>(host_d);
+        c->stage_int_h = reinterpret_cast<int32_t*>(h + at_int), c->stage_int_d = reinterpret_cast<int32_t*>(d + at_int);
+        c->stage_float_h = reinterpret_cast<float*>(h + at_float), c->stage_float_d = reinterpret_cast<float*>(d + at_float);
+        c->stage_byte_h = reinterpret_cast<uint8_t*>(h + at_byte), c->stage_byte_d = reinterpret_cast<uint8_t*>(d + at_byte);
+    }
     ok = ok && cudaDeviceSynchronize() == cudaSuccess;
     if (!ok) {
         disco_destroy(c);
@@ -509,28 +534,10 @@ int disco_create(disco_ctx** out, int V, int d_draft, int d_target, int max_batc
 
 int disco_destroy(disco_ctx* c) {
     if (!c) return DISCO_ERR_INVALID_ARG;
-    cudaFree(c->keys);
-    cudaFree(c->part_rec);
-    cudaFree(c->stamped_rec);
-    cudaFree(c->row_bound);
-    cudaFree(c->ticket);
-    cudaFree(c->status);
-    cudaFree(c->final_stats);
-    cudaFree(c->final_stats2);
-    cudaFree(c->chain_alive);
-    cudaFree(c->sample_seg_tot);
-    cudaFree(c->sample_seg_last);
-    cudaFree(c->sample_tickets);
-    cudaFree(c->loop_rec);
-    cudaFree(c->pack_rows);
-    cudaFree(c->pack_off);
-    cudaFree(c->stage_hidden);
-    cudaFree(c->stage_hidden_draft);
+    cudaFree(c->device_mem);
     if (c->copy_stream) cudaStreamDestroy(c->copy_stream);
     if (c->copy_done) cudaEventDestroy(c->copy_done);
-    cudaFreeHost(c->stage_int_h);
-    cudaFreeHost(c->stage_float_h);
-    cudaFreeHost(c->stage_byte_h);
+    cudaFreeHost(c->host_mem);
     delete c;
     return DISCO_OK;
 }
