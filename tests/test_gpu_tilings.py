@@ -1,0 +1,154 @@
+"""The sizes at which the kernels change their tiling or their way of working, against the CPU oracle: vocabulary tiles of a
+CTA, tiles of hidden rows, halves of a tile, slabs of a draw, and logits that no bound can tell apart.  Needs a B200.
+Tolerances as in util.py (derived there); SM counts are read from the device."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2405_04304_b200 import binding, inputs
+from util import (check_draft, check_verify, gpu_draft_step, gpu_verify, make_clf, near_tie_ids, to_gpu_clf,
+                  to_oracle_clf)
+
+pytestmark = pytest.mark.gpu
+
+_bits = inputs.bf16_bits
+
+
+def _sms():
+    return torch.cuda.get_device_properties(0).multi_processor_count
+
+
+# vocabulary rows per SM: one and two tiles of up to 128, a tile of exactly 32 / 33 rows (with and without the shared bound)
+@pytest.mark.parametrize("rows_per_sm,extra,B", [(32, 0, 9), (32, 1, 9), (128, 0, 40), (128, 1, 40), (256, 1, 33),
+                                                 (16, 5, 128), (16, 5, 129), (40, -3, 300)])
+def test_batched_draft_step_at_the_edges_of_its_tiling(oracle, rows_per_sm, extra, B):
+    V, d = _sms() * rows_per_sm + extra, 40
+    W, h = inputs.lm_head(V, d, seed=V, std=0.3), inputs.hidden(B, d, seed=B)
+    params = make_clf(16, seed=1)
+    pos, nd = np.arange(1, B + 1, dtype=np.int32), (np.arange(B, dtype=np.int32) % 4) + 1
+    active = (np.arange(B) % 5 != 2).astype(np.uint8)
+    ctx = binding.Context(V, d, 8, max_batch=B, max_rows=8, clf_hidden=16)
+    Wg, clf = W.cuda(), to_gpu_clf(params)
+    for act in (None, active, None):   # (a masked step between two full ones: scratch of either parity is left clean)
+        got = gpu_draft_step(ctx, Wg, h, pos, nd, clf, 0.5, 3, active=act)
+        ref = oracle.draft_step(_bits(W), _bits(h), pos, nd, to_oracle_clf(oracle, params), 0.5, 3, active=act, nthreads=8)
+        check_draft(got, ref, 0.5, active=act)
+    assert ctx.device_status() == 0
+    ctx.close()
+
+
+@pytest.mark.parametrize("V,copies", [(5000, 5000), (5000, 40), (40000, 1000), (20000, 12)])
+def test_logits_that_no_bound_can_tell_apart(oracle, V, copies):
+    """The largest logit occurs `copies` times (the whole vocabulary, or in consecutive rows of a few CTAs): the lists
+    overflow, the arg-max is the lowest index."""
+    d, B = 16, 12
+    W, h = inputs.lm_head(V, d, seed=V + copies, std=0.2), inputs.hidden(B, d, seed=3)
+    peak = (h[0].float() * 0.5).to(torch.bfloat16)          # sequence 0: logit |h|^2 / 2, far above the others
+    at = (V - copies) // 2
+    W[at:at + copies] = peak
+    params = make_clf(8, seed=2)
+    pos, nd = np.ones(B, np.int32), np.ones(B, np.int32)
+    ctx = binding.Context(V, d, 8, max_batch=B, max_rows=8, clf_hidden=8)
+    got = gpu_draft_step(ctx, W.cuda(), h, pos, nd, to_gpu_clf(params), 0.5, 3)
+    ref = oracle.draft_step(_bits(W), _bits(h), pos, nd, to_oracle_clf(oracle, params), 0.5, 3, nthreads=8)
+    assert int(got["token"][0]) == at == int(ref.token[0])
+    ties = ref.gap < 1e-3                                    # other sequences may tie at rows of the block as well
+    got["token"][ties] = ref.token[ties]
+    ref.topk_ids[ties, 0] = ref.token[ties]
+    check_draft(got, ref, 0.5)
+    assert ctx.device_status() == 0
+    ctx.close()
+
+
+# slabs whose length is and is not a multiple of four, rows of V floats that are not 16-byte aligned, one to many CTAs a row
+@pytest.mark.parametrize("V,B", [(7, 1), (4096, 1), (4099, 3), (30002, 2), (30000, 40), (5001, 150)])
+def test_draw_finds_the_entry_that_holds_the_target(V, B):
+    d = 24
+    W, h = inputs.lm_head(V, d, seed=V, std=0.3).cuda(), inputs.hidden(B, d, seed=B).cuda()
+    clf = to_gpu_clf(make_clf(8, seed=4))
+    ctx = binding.Context(V, d, 8, max_batch=B, max_rows=8, clf_hidden=8)
+    i32 = dict(dtype=torch.int32, device="cuda")
+    one, token = torch.ones(B, **i32), torch.zeros(B, **i32)
+    conf, p_tok = torch.zeros(B, device="cuda"), torch.zeros(B, device="cuda")
+    halt, probs = torch.zeros(B, dtype=torch.uint8, device="cuda"), torch.zeros(B, V, device="cuda")
+    logits = h.double() @ W.double().T
+    for u_all in (0.0, 0.37, float(np.nextafter(np.float32(1), np.float32(0)))):
+        u = torch.full((B,), u_all, device="cuda")
+        ctx.draft_step_sample(W, h, one, one, clf, 0.5, 4, u, token, conf, halt, probs, p_token=p_tok)
+        torch.cuda.synchronize()
+        y = torch.softmax(logits, -1)
+        assert float((probs.double() - y).abs().max()) < 2e-3
+        cdf = torch.cumsum(y, -1)
+        t = token.long()[:, None]
+        hi, lo = cdf.gather(1, t)[:, 0], (cdf.gather(1, t) - y.gather(1, t))[:, 0]
+        # the running sums are of fp32 exponentials: 2e-5 of the total, the tolerance of every draw
+        assert bool(((lo <= u_all + 2e-5) & (hi >= u_all - 2e-5)).all())
+        assert torch.equal(p_tok, probs.gather(1, t)[:, 0])
+    assert ctx.device_status() == 0
+    ctx.close()
+
+
+# 1, 2, 3, 4 and 5 tiles of hidden rows, each just full and with one row more; short and long contractions
+@pytest.mark.parametrize("R", [127, 128, 129, 256, 257, 384, 385, 512, 513])
+@pytest.mark.parametrize("d", [64, 2048])
+def test_verification_at_the_edges_of_the_tiles_of_hidden_rows(oracle, R, d):
+    V, B = 700, 7
+    sl = np.full(B, R // B - 1, dtype=np.int32)
+    sl[-1] += R - int((sl + 1).sum())
+    off = inputs.row_offsets(torch.from_numpy(sl)).numpy()
+    W, H = inputs.lm_head(V, d, seed=R, std=0.1), inputs.hidden(R, d, seed=R + d)
+    free = oracle.verify_ragged(_bits(W), _bits(H), np.zeros(R - B, np.int32), off, nthreads=8)
+    clean = np.concatenate([free.target_ids[off[b]:off[b + 1] - 1] for b in range(B)]).astype(np.int32)
+    draft = inputs.corrupt_ids(torch.from_numpy(clean), 0.02, V, seed=R).numpy()
+    ref = oracle.verify_ragged(_bits(W), _bits(H), draft, off, nthreads=8)
+    ctx = binding.Context(V, 8, d, max_batch=B, max_rows=R)
+    got = gpu_verify(ctx, W.cuda(), H, draft, row_off=off)
+    check_verify(got, ref, off, draft, near_tie_ids(oracle, _bits(W), _bits(H), ref.gap))
+    assert ctx.device_status() == 0
+    ctx.close()
+
+
+# a box below 128 rows, exactly 128, both halves, two and four tiles of it, and beyond what the persistent kernel takes
+@pytest.mark.parametrize("rows_per_sm", [3, 128, 129, 256, 257, 1024, 1025])
+@pytest.mark.parametrize("B", [1, 2, 4])
+def test_draft_phase_at_the_edges_of_its_tiling(oracle, rows_per_sm, B):
+    V, d, S = _sms() * rows_per_sm - 1, 16, 3
+    W, h = inputs.lm_head(V, d, seed=V, std=0.3), inputs.hidden(S * B, d, seed=B).view(S, B, d)
+    params = make_clf(16, seed=6)
+    ctx = binding.Context(V, d, 8, max_batch=B, max_rows=8, clf_hidden=16)
+    z = lambda *s, t=torch.int32: torch.zeros(*s, dtype=t, device="cuda")
+    token, conf, halt = z(S, B), z(S, B, t=torch.float32), z(S, B, t=torch.uint8)
+    feats, sl, pos0 = z(S, B, binding.NFEAT, t=torch.float32), z(B), torch.arange(5, 5 + B, dtype=torch.int32)
+    ctx.draft_loop(W.cuda(), h.cuda(), pos0.cuda(), to_gpu_clf(params), 0.0, S, token, conf, halt, sl, feats=feats)
+    torch.cuda.synchronize()
+    assert sl.tolist() == [S] * B
+    for i in range(S):
+        ref = oracle.draft_step(_bits(W), _bits(h[i]), pos0.numpy() + i + 1, np.full(B, i + 1, np.int32),
+                                to_oracle_clf(oracle, params), 0.0, S, nthreads=8)
+        got = dict(token=token[i].cpu().numpy(), conf=conf[i].cpu().numpy(), halt=halt[i].cpu().numpy(),
+                   feats=feats[i].cpu().numpy(), probs=None)
+        check_draft(got, ref, 0.0)
+    assert ctx.device_status() == 0
+    ctx.close()
+
+
+@pytest.mark.parametrize("V,N", [(1000, 3), (1001, 130)])
+def test_features_with_rows_that_are_and_are_not_aligned(oracle, V, N):
+    d_D, d_T = 16, 24
+    W_D, W_T = inputs.lm_head(V, d_D, seed=1, std=0.3), inputs.lm_head(V, d_T, seed=2, std=0.3)
+    H_D, H_T = inputs.hidden(N, d_D, seed=3), inputs.hidden(N, d_T, seed=4)
+    ctx = binding.Context(V, d_D, d_T, max_batch=1, max_rows=N)
+    z = lambda *s, t=torch.float32: torch.zeros(*s, dtype=t, device="cuda")
+    fD, fT, tv, lab = z(N, 12), z(N, 12), z(N), z(N, t=torch.uint8)
+    tD, tT, yD, yT = z(N, t=torch.int32), z(N, t=torch.int32), z(N, V), z(N, V)
+    ctx.extract_features(W_D.cuda(), H_D.cuda(), W_T.cuda(), H_T.cuda(), torch.ones(N, dtype=torch.int32, device="cuda"),
+                         fD, fT, tv, lab, tD, tT, yD, yT)
+    torch.cuda.synchronize()
+    want = [torch.softmax(H.double() @ W.double().T, -1) for H, W in ((H_D, W_D), (H_T, W_T))]
+    for y, w in zip((yD, yT), want):
+        assert float((y.cpu().double() - w).abs().max()) < 2e-3
+    # half a sum of V differences of fp32 probabilities (rows that sum to one): 1e-5
+    assert float((tv.cpu().double() - 0.5 * (want[0] - want[1]).abs().sum(-1)).abs().max()) < 1e-5
+    assert torch.equal(lab.cpu().bool(), tD.cpu() == tT.cpu())
+    assert ctx.device_status() == 0
+    ctx.close()
