@@ -364,6 +364,8 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
     uint64_t* tmem_empty = tmem_full + 4;
     uint32_t* tmem_base_s = reinterpret_cast<uint32_t*>(tmem_empty + 4);
     int* s_done = reinterpret_cast<int*>(tmem_base_s + 1);    // epilogue warps that have published their records
+    uint32_t* s_live = tmem_base_s + 5;                       // 1: the step takes place, 2: it does not
+    uint32_t* s_look = tmem_base_s + 4;                       // whether the step seems to take place
     uint32_t* s_clf = tmem_base_s + 3;                        // set once the classifier is in shared memory
     uint32_t* s_stamp = tmem_base_s + 2;                      // stamp of this launch (0: not read yet, or nothing to do)
     float4* xch = reinterpret_cast<float4*>(reinterpret_cast<uint8_t*>(full) + 512);
@@ -396,6 +398,7 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
         *s_done = 0;
         *s_stamp = 0u;
         *s_clf = 0u;
+        *s_live = 0u;
         fence_mbar_init();
         prefetch_tensormap(&tmap_W);
         prefetch_tensormap(&tmap_H);
@@ -404,20 +407,27 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
         tmem_alloc(tmem_base_s, 512);
         tmem_relinquish();
     }
+    // A step of a draft phase that has ended already needs neither loads nor rehearsals.  The flags are looked at ahead of
+    // the dependency wait for that, once for the whole CTA: they may be old and decide nothing else.
+    if (warp == 2) {
+        const bool any = !chained || chain_any_live(f.chain, f.B, lane);
+        if (lane == 0) *s_look = any ? 1u : 0u;
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_base_s;
+    const bool looks_live = *s_look != 0u;
+    // Does the step take place?  Read once per CTA, by the MMA issuer right after the dependency wait (a finishing warp of
+    // this launch may clear flags once this CTA's records are out), and told to the others here.
+    auto step_live = [&]() { return !chained || smem_word(s_live, p.status) == 1u; };
 
     if (warp == 0) {
         // ------------------------------ producer ------------------------------
         const int total = tiles * KB;
         const uint32_t w_bytes = (uint32_t)p.TRN * 128u, h_bytes = (uint32_t)p.a_rows * 128u;
         // The LM head is never written by this library: its first stages are requested before the dependency wait.
-        // (A step of a draft phase that has already ended does not: the flags are read ahead of the wait for that,
-        // they may be old and decide nothing else.)
-        int pre = min(p.stages, total);
-        if (chained && !chain_any_live(f.chain, f.B, lane)) pre = 0;
+        const int pre = looks_live ? min(p.stages, total) : 0;
         // Every CTA reads the same hidden rows.  Each starts at another k-block, so that they do not all ask the same few
         // L2 slices for the same lines at the same time.
         const int rot = nslot % KB;
@@ -440,7 +450,7 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
             }
         }
         asm volatile("griddepcontrol.wait;" ::: "memory");
-        const bool live = !chained || chain_any_live(f.chain, f.B, lane);
+        const bool live = step_live();
         if (!live) {
             if (elect_one()) {
                 for (int n = 0; n < pre; ++n) mbar_arrive(&full[n]);
@@ -480,6 +490,7 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
         if (chained) {
             asm volatile("griddepcontrol.wait;" ::: "memory");
             live = chain_any_live(f.chain, f.B, lane);
+            if (lane == 0) *reinterpret_cast<volatile uint32_t*>(s_live) = live ? 1u : 2u;
         }
         if (live && elect_one()) {
             const uint32_t idesc = umma_idesc(p.TRN);
@@ -535,7 +546,8 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
         float* turn = turn_s + ew * 32 * kDbTurnStride;
         // Twice: a rehearsal without columns before the dependency wait (what follows the column loop is on the critical
         // path, and its instructions would come from L2 one after the other), then for good.
-        for (int phase = 0; phase < 2; ++phase) {
+        for (int phase = looks_live ? 0 : 1; phase < 2; ++phase) {
+            bool few_kept = false;
             unsigned keep_mask = 0u;       // rows of this warp whose raw logits go to probs (none of a masked sequence's)
             unsigned int *slots = nullptr, *my_slot = nullptr;
             float m = DISCO_NEG_INF, Z = 0.f, S2 = 0.f;      // S2 = sum e^(z - m) (z - m) / ln 2
@@ -550,7 +562,7 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
                 Z = 1.f;
             } else {
                 asm volatile("griddepcontrol.wait;" ::: "memory");  // scratch and outputs belong to the predecessor until now
-                if (chained && !chain_any_live(f.chain, f.B, lane)) break;
+                if (!step_live()) break;
                 const uint32_t stamp = *reinterpret_cast<volatile unsigned int*>(p.sync) + 1u;
                 const uint32_t par = stamp & 1u;
                 const int old_rows = *reinterpret_cast<volatile unsigned int*>(p.sync + 2 + (par ^ 1u));
@@ -560,6 +572,7 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
                 // them is written.
                 valid = valid && chain_seq_live(f.chain, f.active, row);
                 keep_mask = __ballot_sync(kFullMask, p.probs && valid);
+                few_kept = keep_mask != 0u && __popc(keep_mask) <= 4;
                 slots = p.bound + par * p.set_words + (size_t)(valid ? row : 0) * kDbBoundStride;
                 my_slot = slots + nslot % kDbBoundSlots;
                 uint4* old = reinterpret_cast<uint4*>(p.bound + (par ^ 1u) * p.set_words);
@@ -641,7 +654,21 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
                         }
                         S2 = fmaf(em, fmaf(dm, Z, S2), Sa + Sb);   // (Z = S2 = 0 before the first chunk)
                         Z = fmaf(Z, em, Za + Zb);
-                        if (keep_mask) {
+                        if (few_kept) {   // a handful of rows: each by the thread that holds it
+                            const int v = v_first + t * p.TR + c * 32;
+                            float* dst = p.probs + (size_t)row * p.V + v;
+                            if ((keep_mask >> lane) & 1u) {
+                                if (((p.V | v) & 3) == 0 && n >= 32 && (reinterpret_cast<uintptr_t>(p.probs) & 15) == 0) {
+#pragma unroll
+                                    for (int j = 0; j < 32; j += 4)
+                                        *reinterpret_cast<float4*>(dst + j) = make_float4(z[j], z[j + 1], z[j + 2], z[j + 3]);
+                                } else {
+#pragma unroll
+                                    for (int j = 0; j < 32; ++j)
+                                        if (j < n) dst[j] = z[j];
+                                }
+                            }
+                        } else if (keep_mask) {
                             // A thread holds one row: the chunk goes through shared memory so that every store instruction
                             // writes whole lines (four rows of 128 bytes; 32 bytes at a time per row halved the rate of
                             // the whole pass: 278 against 68 us for 1000 rows of the 32000 x 768 head).
@@ -846,7 +873,7 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
         uint32_t stamp = 1u;
         unsigned int* set = nullptr;
         int b = 0;
-        bool run = !epi;
+        bool run = !epi && looks_live;
         for (bool real = false;; real = true) {
             if (run && !(real && !chain_seq_live(f.chain, f.active, b))) db_finish_row(p, f, b, real, stamp + (real ? f.test_stamp_skew : 0u), sm, clf_s, STATS, lane);
             run = true;
@@ -860,7 +887,7 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
                     }
                     asm volatile("griddepcontrol.wait;" ::: "memory");
                 }
-                if (chained && !chain_any_live(f.chain, f.B, lane)) break;
+                if (!step_live()) break;
                 if (epi) smem_word(s_clf, p.status);
                 stamp = smem_word(s_stamp, p.status);
                 __syncwarp();

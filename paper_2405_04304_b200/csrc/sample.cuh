@@ -120,13 +120,28 @@ static __global__ void __launch_bounds__(kSampleThreads) draw_rows_kernel(const 
         // a few consecutive records per lane, running sums in record order
         const int q = (p.NP + 31) / 32, c0 = min(p.NP, lane * q), c1 = min(p.NP, c0 + q);
         const float4* rec = p.recs + (size_t)b * p.NP * p.rec_pieces;
-        auto mass = [&](int c) {
-            const float4 r = __ldcg(rec + (size_t)c * p.rec_pieces);
+        // (the first few are fetched side by side: a loop of dependent loads is a round trip each)
+        constexpr int kAhead = 5;
+        float2 mz[kAhead];
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i) {
+            mz[i] = make_float2(0.f, 0.f);
+            if (c0 + i < c1) mz[i] = __ldcg(reinterpret_cast<const float2*>(rec + (size_t)(c0 + i) * p.rec_pieces));
+        }
+        auto mass_of = [&](const float2& r) {
             return r.y > 0.f ? static_cast<double>(r.y) * static_cast<double>(expf(r.x - m)) : 0.0;
         };
+        double w_first[kAhead];
         double mine = 0.0;
         int last = -1;
-        for (int c = c0; c < c1; ++c) {
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i) {
+            w_first[i] = mass_of(mz[i]);
+            mine += w_first[i];
+            if (w_first[i] > 0.0) last = c0 + i;
+        }
+        auto mass = [&](int c) { return mass_of(__ldcg(reinterpret_cast<const float2*>(rec + (size_t)c * p.rec_pieces))); };
+        for (int c = c0 + kAhead; c < c1; ++c) {
             const double w = mass(c);
             mine += w;
             if (w > 0.0) last = c;
@@ -146,14 +161,20 @@ static __global__ void __launch_bounds__(kSampleThreads) draw_rows_kernel(const 
             double before = incl - mine;
             int slab = last;               // rounding next to u = 1: the last slab with mass, and its last entry
             if (who) {
-                for (int c = c0; c < c1; ++c) {
-                    const double w = mass(c);
-                    if (before + w > target) {
-                        slab = c;
-                        break;
+                slab = -1;
+#pragma unroll
+                for (int i = 0; i < kAhead; ++i) {
+                    if (slab < 0 && c0 + i < c1) {
+                        if (before + w_first[i] > target) slab = c0 + i;
+                        else before += w_first[i];
                     }
-                    before += w;
                 }
+                for (int c = c0 + kAhead; c < c1 && slab < 0; ++c) {
+                    const double w = mass(c);
+                    if (before + w > target) slab = c;
+                    else before += w;
+                }
+                if (slab < 0) slab = last;   // (the sums above were added in another order)
             }
             s_slab = slab;
             s_before = who ? before * inv_Z : 0.0;
