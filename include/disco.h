@@ -101,7 +101,7 @@ int disco_set_kernel_path(disco_ctx* ctx, int which);
  *   wait_budget_clocks  SM clock ticks after which a wait gives up and records DISCO_ERR_TIMEOUT in the device
  *                       status word (0 restores the default of about 0.05 s); applies to every context of the
  *                       process
- *   withhold_records    non-zero: the batched draft step (the tensor-core kernel for five sequences and more)
+ *   withhold_records    non-zero: the draft step (the tensor-core kernel)
  *                       makes its finishing warps look for per-CTA records that no CTA publishes, so that
  *                       their wait runs out.  The kernel still returns by itself; its outputs are then
  *                       meaningless and the context must be destroyed (see DISCO_ERR_TIMEOUT).
