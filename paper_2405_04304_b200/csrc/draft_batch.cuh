@@ -547,7 +547,7 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
         // Twice: a rehearsal without columns before the dependency wait (what follows the column loop is on the critical
         // path, and its instructions would come from L2 one after the other), then for good.
         for (int phase = looks_live ? 0 : 1; phase < 2; ++phase) {
-            bool few_kept = false;
+            bool many_kept = false;        // enough of them to store four rows per instruction
             unsigned keep_mask = 0u;       // rows of this warp whose raw logits go to probs (none of a masked sequence's)
             unsigned int *slots = nullptr, *my_slot = nullptr;
             float m = DISCO_NEG_INF, Z = 0.f, S2 = 0.f;      // S2 = sum e^(z - m) (z - m) / ln 2
@@ -572,7 +572,7 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
                 // them is written.
                 valid = valid && chain_seq_live(f.chain, f.active, row);
                 keep_mask = __ballot_sync(kFullMask, p.probs && valid);
-                few_kept = keep_mask != 0u && __popc(keep_mask) <= 4;
+                many_kept = __popc(keep_mask) > 8 && (reinterpret_cast<uintptr_t>(p.probs) & 15) == 0;
                 slots = p.bound + par * p.set_words + (size_t)(valid ? row : 0) * kDbBoundStride;
                 my_slot = slots + nslot % kDbBoundSlots;
                 uint4* old = reinterpret_cast<uint4*>(p.bound + (par ^ 1u) * p.set_words);
@@ -654,21 +654,7 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
                         }
                         S2 = fmaf(em, fmaf(dm, Z, S2), Sa + Sb);   // (Z = S2 = 0 before the first chunk)
                         Z = fmaf(Z, em, Za + Zb);
-                        if (few_kept) {   // a handful of rows: each by the thread that holds it
-                            const int v = v_first + t * p.TR + c * 32;
-                            float* dst = p.probs + (size_t)row * p.V + v;
-                            if ((keep_mask >> lane) & 1u) {
-                                if (((p.V | v) & 3) == 0 && n >= 32 && (reinterpret_cast<uintptr_t>(p.probs) & 15) == 0) {
-#pragma unroll
-                                    for (int j = 0; j < 32; j += 4)
-                                        *reinterpret_cast<float4*>(dst + j) = make_float4(z[j], z[j + 1], z[j + 2], z[j + 3]);
-                                } else {
-#pragma unroll
-                                    for (int j = 0; j < 32; ++j)
-                                        if (j < n) dst[j] = z[j];
-                                }
-                            }
-                        } else if (keep_mask) {
+                        if (keep_mask) {
                             // A thread holds one row: the chunk goes through shared memory so that every store instruction
                             // writes whole lines (four rows of 128 bytes; 32 bytes at a time per row halved the rate of
                             // the whole pass: 278 against 68 us for 1000 rows of the 32000 x 768 head).
@@ -678,7 +664,7 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
                             for (int j = 0; j < 8; ++j) mine[j] = make_float4(z[4 * j], z[4 * j + 1], z[4 * j + 2], z[4 * j + 3]);
                             __syncwarp();
                             float* dst = p.probs + (size_t)(m_tile * 128 + quad * 32) * p.V + v;
-                            if (((p.V | v) & 3) == 0 && n >= 32 && (reinterpret_cast<uintptr_t>(p.probs) & 15) == 0) {
+                            if (many_kept && ((p.V | v) & 3) == 0 && n >= 32) {
 #pragma unroll
                                 for (int j = 0; j < 8; ++j) {
                                     const int r = 4 * j + (lane >> 3), col = (lane & 7) * 4;
@@ -686,10 +672,9 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
                                     if ((keep_mask >> r) & 1u) *reinterpret_cast<float4*>(dst + (size_t)r * p.V + col) = x;
                                 }
                             } else {
-#pragma unroll 4
-                                for (int r = 0; r < 32; ++r) {
-                                    const float x = turn[r * kDbTurnStride + lane];
-                                    if (((keep_mask >> r) & 1u) && lane < n) dst[(size_t)r * p.V + lane] = x;
+                                for (unsigned left = keep_mask; left != 0u; left &= left - 1u) {   // row by row, those there are
+                                    const int r = __ffs(left) - 1;
+                                    if (lane < n) dst[(size_t)r * p.V + lane] = turn[r * kDbTurnStride + lane];
                                 }
                             }
                             __syncwarp();
