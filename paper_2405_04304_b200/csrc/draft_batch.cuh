@@ -106,6 +106,10 @@ __device__ __forceinline__ uint32_t smem_word(const uint32_t* p, int* status) {
     return 1u;
 }
 
+// The same out of line, where it is seldom reached: inlined four times its loop costs the launches that never take it the
+// placement of their code (one row of the 32000 x 768 head 15.1 against 14.4 us, 7 rows of 40011 x 768 18.4 against 17.9).
+static __device__ __noinline__ uint32_t cold_smem_word(const uint32_t* p, int* status) { return smem_word(p, status); }
+
 // From the twelve words of a row: the bound of its tenth largest logit (the third smallest word); TOP1: of its largest.
 template <bool TOP1>
 __device__ __forceinline__ float row_bound_of(const uint4& a, const uint4& b, const uint4& c) {
@@ -383,7 +387,7 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
     const int nslot = blockIdx.x / p.MT;
     const int v_first = nslot * p.TPC * p.TR;                 // this CTA's vocabulary rows: its tiles in sequence
     const int tiles = v_first < p.V ? min(p.TPC, (p.V - v_first + p.TR - 1) / p.TR) : 0;
-    const bool chained = f.chain.alive != nullptr && f.chain.step > 1;
+    const bool chained = !STATS && f.chain.alive != nullptr && f.chain.step > 1;
     const int nbuf = p.TRN <= 128 ? 4 : 2, buf_cols = 512 / nbuf;   // accumulator buffers in TMEM
 
     if (threadIdx.x == 0) {
@@ -420,7 +424,7 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
     const bool looks_live = *s_look != 0u;
     // Does the step take place?  Read once per CTA, by the MMA issuer right after the dependency wait (a finishing warp of
     // this launch may clear flags once this CTA's records are out), and told to the others here.
-    auto step_live = [&]() { return !chained || smem_word(s_live, p.status) == 1u; };
+    auto step_live = [&]() { return !chained || cold_smem_word(s_live, p.status) == 1u; };
 
     if (warp == 0) {
         // ------------------------------ producer ------------------------------
