@@ -234,7 +234,8 @@ int launch_umma(disco_ctx* c, const void* W, const void* H, int d, int R, const 
     p.dev_R = dev_R;
     p.box_rows = dev_R ? 256 : p.t.TRN;   // (the kernel derives the tiling from the device-side row count)
     p.pairs = dev_R || p.t.GS == 2;
-    p.a_rows = p.t.MT > 1 ? 128 : std::max(8, (R + 7) / 8 * 8);
+    const bool lanes = !dev_R && R <= kUmmaLaneRows;   // vocabulary on the TMEM lanes: see umma_tail.cuh
+    p.a_rows = lanes ? (R + 15) / 16 * 16 : p.t.MT > 1 ? 128 : (R + 7) / 8 * 8;
     // The A tile holds a_rows rows.  The MMA still reads 128 rows from its start: what lies behind the tile (other
     // stages of the ring, always inside it) only feeds accumulator lanes nobody reads.
     p.a_bytes = (p.a_rows * 128 + 1023) / 1024 * 1024;
@@ -245,19 +246,21 @@ int launch_umma(disco_ctx* c, const void* W, const void* H, int d, int R, const 
     CUtensorMap tmap_W, tmap_H;
     if (!encode_bf16_2d(c, &tmap_W, W, c->V, d, p.box_rows) || !encode_bf16_2d(c, &tmap_H, H, R, d, p.a_rows))
         return DISCO_ERR_CUDA;
-    static KernelSetup setup;
-    if (!raise_smem_limit(c, setup, umma_tail_kernel, (size_t)kUmmaSmemBytes, nullptr)) return DISCO_ERR_CUDA;
+    static KernelSetup setup[2];
+    auto kern = lanes ? umma_tail_kernel<true> : umma_tail_kernel<false>;
+    const int smem_bytes = lanes ? kUmmaLaneSmemBytes : kUmmaSmemBytes;
+    if (!raise_smem_limit(c, setup[lanes], kern, (size_t)smem_bytes, nullptr)) return DISCO_ERR_CUDA;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(dev_R ? c->sm_count : p.t.groups * p.t.CN));
     cfg.blockDim = dim3(kUmmaThreads);
-    cfg.dynamicSmemBytes = kUmmaSmemBytes;
+    cfg.dynamicSmemBytes = (size_t)smem_bytes;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = c->pdl ? 1 : 0;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, umma_tail_kernel, tmap_W, tmap_H, p);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tmap_W, tmap_H, p);
     c->launches += 1;
     return cuda_ok(e, "umma_tail_kernel launch") ? DISCO_OK : DISCO_ERR_CUDA;
 }

@@ -13,6 +13,11 @@
 //              and the logits never leave the chip.  Two warps share each TMEM lane quadrant and
 //              split the columns.
 //
+// Up to 32 hidden rows (one or a few sequences) the operands change places: vocabulary rows on the TMEM lanes, hidden rows on
+// 16 or 32 columns.  HBM bounds both forms, but 11 rows on 128 lanes are eight times the multiplications that are needed, and
+// a launch that streams HBM for more than some milliseconds runs at the power limit: 11 rows,
+// 32000 x 5120 head, one launch after the other: 60.9 us at 1.29 GHz with the hidden rows on the lanes, 54.9 us at 1.78 GHz
+// with the vocabulary there (54.2 us either way in a short burst; 51.1 us at the measured copy bandwidth).
 // A CTA keeps one or two tiles of hidden rows and walks over a contiguous range of vocabulary tiles (VerifyTiling).  CTAs that share a vocabulary tile run side by side, so the LM head crosses HBM once and is shared through L2.
 // Results leave the CTA as one atomicMax per row; the last CTA (few sequences) or a small separate kernel finishes the job.
 #pragma once
@@ -31,6 +36,9 @@ constexpr int kUmmaRingBytes = 192 * 1024;  // shared memory for the operand sta
 constexpr int kUmmaEpiWarps = 8;
 constexpr int kUmmaThreads = (2 + kUmmaEpiWarps) * 32;
 constexpr int kUmmaSmemBytes = kUmmaRingBytes + 1024 /*align*/ + 512 /*barriers*/;
+constexpr int kUmmaLaneRows = 32;         // hidden rows up to which the vocabulary goes on the TMEM lanes
+// ... where an MMA reads whole blocks of 128 vocabulary rows, up to 16 KB past the last stage
+constexpr int kUmmaLaneSmemBytes = kUmmaSmemBytes + 16 * 1024;
 // shared memory of a staged classifier (draft steps)
 inline int umma_clf_bytes(int clf_H) { return (clf_H * (kNFeat + 2) + 4) * 4; }
 
@@ -201,6 +209,9 @@ struct DraftFinalParams {
 // ---------------------------------------------------------------------------------------------
 // main kernel
 // ---------------------------------------------------------------------------------------------
+// VL: vocabulary rows on the TMEM lanes (A operand, two blocks of 128 per tile), at most kUmmaLaneRows hidden rows, which all
+// CTAs read as one B operand of 16 or 32 rows.
+template <bool VL>
 __global__ void __launch_bounds__(kUmmaThreads, 1)
 umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_constant__ CUtensorMap tmap_H,
                  const UmmaParams p) {
@@ -307,7 +318,8 @@ umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_consta
     } else if (warp == 1) {
         // ------------------------------ MMA issuer ------------------------------
         if (live && elect_one()) {
-            const uint32_t idesc = umma_idesc(tl.TRN);
+            const uint32_t idesc = umma_idesc(VL ? p.a_rows : tl.TRN);
+            const bool upper = tl.TRN > 128;   // (VL)
             const uint32_t full0 = smem_addr(full), empty0 = smem_addr(empty);
             const uint64_t a0 = umma_smem_desc(a_tiles), b0 = umma_smem_desc(b_tiles);
             const uint32_t a_half = (uint32_t)p.a_bytes >> 4, a_step = a_half * (1 + p.pairs), b_step = (uint32_t)p.b_bytes >> 4;   // descriptor units
@@ -320,14 +332,25 @@ umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_consta
                 const uint32_t parity = (size == 2 ? it : it >> 1) & 1;
                 for (int j = 0; j < size; ++j) mbar_wait(&tmem_empty[first + j], parity ^ 1u, p.status);
                 tc_fence_after();
-                const uint32_t d_tmem = tmem_base + first * 256;
+                const uint32_t d_tmem = tmem_base + first * (VL ? 2 * kUmmaLaneRows : 256);
                 for (int kb = 0; kb < KB; ++kb) {
                     mbar_wait(full0 + stage * 8, phase, p.status);
                     tc_fence_after();
+                    if constexpr (VL) {
 #pragma unroll
-                    for (int k = 0; k < kUmmaBK / 16; ++k)  // 16 k-elements = 32 bytes = 2 descriptor units
-                        tc_mma_bf16(d_tmem, a_desc + 2 * k, b_desc + 2 * k, idesc, (kb | k) != 0);
-                    if (size == 2) {
+                        for (int k = 0; k < kUmmaBK / 16; ++k)
+                            tc_mma_bf16(d_tmem, b_desc + 2 * k, a_desc + 2 * k, idesc, (kb | k) != 0);
+                        if (upper) {
+#pragma unroll
+                            for (int k = 0; k < kUmmaBK / 16; ++k)   // 128 rows further on
+                                tc_mma_bf16(d_tmem + kUmmaLaneRows, b_desc + (128 * 128 >> 4) + 2 * k, a_desc + 2 * k, idesc, (kb | k) != 0);
+                        }
+                    } else {
+#pragma unroll
+                        for (int k = 0; k < kUmmaBK / 16; ++k)  // 16 k-elements = 32 bytes = 2 descriptor units
+                            tc_mma_bf16(d_tmem, a_desc + 2 * k, b_desc + 2 * k, idesc, (kb | k) != 0);
+                    }
+                    if (!VL && size == 2) {
 #pragma unroll
                         for (int k = 0; k < kUmmaBK / 16; ++k)
                             tc_mma_bf16(d_tmem + 256, a_desc + a_half + 2 * k, b_desc + 2 * k, idesc, (kb | k) != 0);
@@ -351,56 +374,103 @@ umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_consta
         const int ew = warp - 2;            // 0 .. kUmmaEpiWarps-1
         const int quad = warp & 3;          // TMEM lane quadrant this warp may read
         const int share = ew >> 2;          // two warps per quadrant split the columns of a tile
-        float best_v[2] = {DISCO_NEG_INF, DISCO_NEG_INF};
-        int best_i[2] = {kNoIndex, kNoIndex};
-        int it = 0;
-        for (int v0 = v_begin; v0 < v_end; v0 += tl.TR, ++it) {
-            const int ncols = min(tl.TR, v_end - v0);  // further columns belong to the next tile or lie past V
-            const int nchunks = (ncols + 31) >> 5;
-            const int c_lo = (nchunks * share + 1) / 2, c_hi = (nchunks * (share + 1) + 1) / 2;
+        if constexpr (VL) {
+            // a thread holds one vocabulary row of the tile, a column is a hidden row
+            float best_v[kUmmaLaneRows];
+            int best_i[kUmmaLaneRows];
 #pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                if (j >= size) break;
-                const int b = size == 2 ? j : it & 1;
-                mbar_wait(&tmem_full[b], (size == 2 ? it : it >> 1) & 1, p.status);
+            for (int r = 0; r < kUmmaLaneRows; ++r) best_v[r] = DISCO_NEG_INF, best_i[r] = kNoIndex;
+            const int tile_row = share * 128 + quad * 32 + lane;
+            int it = 0;
+            for (int v0 = v_begin; v0 < v_end; v0 += tl.TR, ++it) {
+                const int b = it & 1;
+                const int ncols = min(tl.TR, v_end - v0);
+                mbar_wait(&tmem_full[b], (it >> 1) & 1, p.status);
                 tc_fence_after();
-                if ((m_tile + j) * 128 + quad * 32 < R) {
-                    for (int c = c_lo; c < c_hi; ++c) {
-                        float z[32];
-                        tmem_ld32(tmem_base + b * 256 + c * 32 + (static_cast<uint32_t>(quad * 32) << 16), z);
-                        const int n = ncols - c * 32;
-                        if (n < 32) {
+                if (share * 128 + quad * 32 < ncols) {
+                    float z[32];
+                    tmem_ld32(tmem_base + (2 * b + share) * kUmmaLaneRows + (static_cast<uint32_t>(quad * 32) << 16), z);
+                    if (tile_row < ncols) {
 #pragma unroll
-                            for (int i = 0; i < 32; ++i)
-                                if (i >= n) z[i] = DISCO_NEG_INF;
-                        }
-                        float cmax = fmaxf(z[0], z[1]);
-#pragma unroll
-                        for (int i = 2; i < 32; i += 2) cmax = RegTop10::max3(cmax, z[i], z[i + 1]);
-                        // (a chunk seldom holds a new largest logit: its index is looked for only then)
-                        if (__any_sync(kFullMask, cmax > best_v[j])) {
-                            int at = 0;
-#pragma unroll
-                            for (int i = 31; i >= 0; --i)
-                                if (z[i] == cmax) at = i;
-                            if (cmax > best_v[j]) {
-                                best_v[j] = cmax;
-                                best_i[j] = v0 + c * 32 + at;
-                            }
-                        }
+                        for (int r = 0; r < kUmmaLaneRows; ++r)
+                            if (z[r] > best_v[r]) best_v[r] = z[r], best_i[r] = v0 + tile_row;
                     }
                 }
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&tmem_empty[b]);
             }
-        }
-        // one result per hidden row and CTA
+            // one result per hidden row and CTA: the keys of a row side by side in the ring (every load has landed and every MMA
+            // is done), a warp per row.  (32 folds in registers one after the other are 13 KB of code that comes from L2 in an
+            // iteration: 2 us.)
+            unsigned long long* keys_s = reinterpret_cast<unsigned long long*>(smem);
+            constexpr int kEpiThreads = kUmmaEpiWarps * 32;
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const int row = (m_tile + j) * 128 + quad * 32 + lane;
-            if (j < size && row < R && best_i[j] != kNoIndex)
-                atomicMax(p.keys + row, argmax_key(__fadd_rn(best_v[j], 0.f), best_i[j]));
+            for (int r = 0; r < kUmmaLaneRows; ++r)
+                if (r < R) keys_s[r * kEpiThreads + ew * 32 + lane] = best_i[r] != kNoIndex ? argmax_key(__fadd_rn(best_v[r], 0.f), best_i[r]) : 0ull;
+            named_barrier_sync(2, kEpiThreads);
+#pragma unroll 1
+            for (int r = ew; r < R; r += kUmmaEpiWarps) {
+                unsigned long long key = 0ull;
+#pragma unroll
+                for (int i = 0; i < kUmmaEpiWarps; ++i) key = max(key, keys_s[r * kEpiThreads + i * 32 + lane]);
+                const uint32_t hi = static_cast<uint32_t>(key >> 32);
+                const uint32_t top = __reduce_max_sync(kFullMask, hi);
+                const uint32_t low = __reduce_max_sync(kFullMask, hi == top ? static_cast<uint32_t>(key) : 0u);
+                if (lane == 0 && top) atomicMax(p.keys + r, static_cast<unsigned long long>(top) << 32 | low);
+            }
+        } else {
+            float best_v[2] = {DISCO_NEG_INF, DISCO_NEG_INF};
+            int best_i[2] = {kNoIndex, kNoIndex};
+            int it = 0;
+            for (int v0 = v_begin; v0 < v_end; v0 += tl.TR, ++it) {
+                const int ncols = min(tl.TR, v_end - v0);  // further columns belong to the next tile or lie past V
+                const int nchunks = (ncols + 31) >> 5;
+                const int c_lo = (nchunks * share + 1) / 2, c_hi = (nchunks * (share + 1) + 1) / 2;
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    if (j >= size) break;
+                    const int b = size == 2 ? j : it & 1;
+                    mbar_wait(&tmem_full[b], (size == 2 ? it : it >> 1) & 1, p.status);
+                    tc_fence_after();
+                    if ((m_tile + j) * 128 + quad * 32 < R) {
+                        for (int c = c_lo; c < c_hi; ++c) {
+                            float z[32];
+                            tmem_ld32(tmem_base + b * 256 + c * 32 + (static_cast<uint32_t>(quad * 32) << 16), z);
+                            const int n = ncols - c * 32;
+                            if (n < 32) {
+#pragma unroll
+                                for (int i = 0; i < 32; ++i)
+                                    if (i >= n) z[i] = DISCO_NEG_INF;
+                            }
+                            float cmax = fmaxf(z[0], z[1]);
+#pragma unroll
+                            for (int i = 2; i < 32; i += 2) cmax = RegTop10::max3(cmax, z[i], z[i + 1]);
+                            // (a chunk seldom holds a new largest logit: its index is looked for only then)
+                            if (__any_sync(kFullMask, cmax > best_v[j])) {
+                                int at = 0;
+#pragma unroll
+                                for (int i = 31; i >= 0; --i)
+                                    if (z[i] == cmax) at = i;
+                                if (cmax > best_v[j]) {
+                                    best_v[j] = cmax;
+                                    best_i[j] = v0 + c * 32 + at;
+                                }
+                            }
+                        }
+                    }
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&tmem_empty[b]);
+                }
+            }
+            // one result per hidden row and CTA
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int row = (m_tile + j) * 128 + quad * 32 + lane;
+                if (j < size && row < R && best_i[j] != kNoIndex)
+                    atomicMax(p.keys + row, argmax_key(__fadd_rn(best_v[j], 0.f), best_i[j]));
+            }
         }
         if (p.fuse_final) {
             // ticket: the last CTA to get here matches the prefixes and clears the keys

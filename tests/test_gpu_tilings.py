@@ -88,11 +88,7 @@ def test_draw_finds_the_entry_that_holds_the_target(V, B):
     ctx.close()
 
 
-# 1, 2, 3, 4 and 5 tiles of hidden rows, each just full and with one row more; short and long contractions
-@pytest.mark.parametrize("R", [127, 128, 129, 256, 257, 384, 385, 512, 513])
-@pytest.mark.parametrize("d", [64, 2048])
-def test_verification_at_the_edges_of_the_tiles_of_hidden_rows(oracle, R, d):
-    V, B = 700, 7
+def _verification_agrees(oracle, V, B, R, d):
     sl = np.full(B, R // B - 1, dtype=np.int32)
     sl[-1] += R - int((sl + 1).sum())
     off = inputs.row_offsets(torch.from_numpy(sl)).numpy()
@@ -106,6 +102,20 @@ def test_verification_at_the_edges_of_the_tiles_of_hidden_rows(oracle, R, d):
     check_verify(got, ref, off, draft, near_tie_ids(oracle, _bits(W), _bits(H), ref.gap))
     assert ctx.device_status() == 0
     ctx.close()
+
+
+# 1, 2, 3, 4 and 5 tiles of hidden rows, each just full and with one row more; short and long contractions
+@pytest.mark.parametrize("R", [127, 128, 129, 256, 257, 384, 385, 512, 513])
+@pytest.mark.parametrize("d", [64, 2048])
+def test_verification_at_the_edges_of_the_tiles_of_hidden_rows(oracle, R, d):
+    _verification_agrees(oracle, 700, 7, R, d)
+
+
+# vocabulary rows on the lanes: a block of 128 not full, full, two of them, several tiles; 16 rows per column group and one more
+@pytest.mark.parametrize("rows_per_sm", [2, 128, 129, 256, 257, 600])
+@pytest.mark.parametrize("R", [2, 16, 17, 32, 33])
+def test_verification_of_few_rows_at_the_edges_of_its_tiling(oracle, rows_per_sm, R):
+    _verification_agrees(oracle, _sms() * rows_per_sm - 1, 1, R, 24)
 
 
 # a box below 128 rows, exactly 128, both halves, two and four tiles of it, and beyond what the persistent kernel takes
