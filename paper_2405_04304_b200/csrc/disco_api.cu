@@ -233,9 +233,15 @@ int launch_umma(disco_ctx* c, const void* W, const void* H, int d, int R, const 
     p.t = VerifyTiling::make(R, c->V, d, c->sm_count);
     p.dev_R = dev_R;
     p.box_rows = dev_R ? 256 : p.t.TRN;   // (the kernel derives the tiling from the device-side row count)
-    p.pairs = dev_R || p.t.GS == 2;
-    const bool lanes = !dev_R && R <= kUmmaLaneRows;   // vocabulary on the TMEM lanes: see umma_tail.cuh
+    // Vocabulary on the TMEM lanes (umma_tail.cuh): few rows, and the first rows beyond one tile of 128, where the other form
+    // multiplies by 256.  In between and beyond it has no fewer multiplications and the dearer epilogue.  (Launches one after
+    // the other at the power limit, 32000 x 5120, 34 / 64 / 96 / 130 / 160 / 192 rows: 61.4 -> 56.2, 61.6 -> 58.2, 63.1 -> 62.5,
+    // 79.7 -> 68.9, 81.2 -> 72.6, 82.8 -> 81.1 us; 49152 x 6144, 64 / 96 / 160 / 192 rows: 113 -> 109, 115 -> 121, 158 -> 153,
+    // 160 -> 171 us.)
+    const bool wide = !dev_R && ((R > kUmmaLaneRows && R <= 64) || (R > 128 && R <= 160));
+    const bool lanes = wide || (!dev_R && R <= kUmmaLaneRows);
     p.a_rows = lanes ? (R + 15) / 16 * 16 : p.t.MT > 1 ? 128 : (R + 7) / 8 * 8;
+    p.pairs = !lanes && (dev_R || p.t.GS == 2);
     // The A tile holds a_rows rows.  The MMA still reads 128 rows from its start: what lies behind the tile (other
     // stages of the ring, always inside it) only feeds accumulator lanes nobody reads.
     p.a_bytes = (p.a_rows * 128 + 1023) / 1024 * 1024;
@@ -246,10 +252,10 @@ int launch_umma(disco_ctx* c, const void* W, const void* H, int d, int R, const 
     CUtensorMap tmap_W, tmap_H;
     if (!encode_bf16_2d(c, &tmap_W, W, c->V, d, p.box_rows) || !encode_bf16_2d(c, &tmap_H, H, R, d, p.a_rows))
         return DISCO_ERR_CUDA;
-    static KernelSetup setup[2];
-    auto kern = lanes ? umma_tail_kernel<true> : umma_tail_kernel<false>;
+    static KernelSetup setup[3];
+    auto kern = wide ? umma_tail_kernel<true, true> : lanes ? umma_tail_kernel<true, false> : umma_tail_kernel<false, false>;
     const int smem_bytes = lanes ? kUmmaLaneSmemBytes : kUmmaSmemBytes;
-    if (!raise_smem_limit(c, setup[lanes], kern, (size_t)smem_bytes, nullptr)) return DISCO_ERR_CUDA;
+    if (!raise_smem_limit(c, setup[lanes + wide], kern, (size_t)smem_bytes, nullptr)) return DISCO_ERR_CUDA;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(dev_R ? c->sm_count : p.t.groups * p.t.CN));
     cfg.blockDim = dim3(kUmmaThreads);

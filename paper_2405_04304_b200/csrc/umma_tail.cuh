@@ -13,12 +13,14 @@
 //              and the logits never leave the chip.  Two warps share each TMEM lane quadrant and
 //              split the columns.
 //
-// Up to 32 hidden rows (one or a few sequences) the operands change places: vocabulary rows on the TMEM lanes, hidden rows on
-// 16 or 32 columns.  HBM bounds both forms, but 11 rows on 128 lanes are eight times the multiplications that are needed, and
-// a launch that streams HBM for more than some milliseconds runs at the power limit: 11 rows,
-// 32000 x 5120 head, one launch after the other: 60.9 us at 1.29 GHz with the hidden rows on the lanes, 54.9 us at 1.78 GHz
-// with the vocabulary there (54.2 us either way in a short burst; 51.1 us at the measured copy bandwidth).
-// A CTA keeps one or two tiles of hidden rows and walks over a contiguous range of vocabulary tiles (VerifyTiling).  CTAs that share a vocabulary tile run side by side, so the LM head crosses HBM once and is shared through L2.
+// With few hidden rows (and some counts just beyond a tile) the operands change places: vocabulary rows on the TMEM lanes,
+// hidden rows on the columns, as many as there are in steps of 16.  HBM bounds both forms, but 11 rows on 128 lanes are eight
+// times the multiplications that are needed, and a launch that streams HBM for more than some milliseconds runs at the power
+// limit: 11 rows, 32000 x 5120 head, one launch after the other: 60.9 us at 1.29 GHz with the hidden rows on the lanes,
+// 54.9 us at 1.78 GHz with the vocabulary there (54.2 us either way in a short burst; 51.1 us at the measured copy bandwidth).
+//
+// A CTA keeps one or two tiles of hidden rows and walks over a contiguous range of vocabulary tiles (VerifyTiling).  CTAs
+// that share a vocabulary tile run side by side, so the LM head crosses HBM once and is shared through L2.
 // Results leave the CTA as one atomicMax per row; the last CTA (few sequences) or a small separate kernel finishes the job.
 #pragma once
 
@@ -36,7 +38,8 @@ constexpr int kUmmaRingBytes = 192 * 1024;  // shared memory for the operand sta
 constexpr int kUmmaEpiWarps = 8;
 constexpr int kUmmaThreads = (2 + kUmmaEpiWarps) * 32;
 constexpr int kUmmaSmemBytes = kUmmaRingBytes + 1024 /*align*/ + 512 /*barriers*/;
-constexpr int kUmmaLaneRows = 32;         // hidden rows up to which the vocabulary goes on the TMEM lanes
+constexpr int kUmmaLaneRows = 32;         // hidden rows whose arg-max a thread can hold, with a vocabulary row per lane
+constexpr int kUmmaWideRows = 256;        // hidden rows on the columns at most
 // ... where an MMA reads whole blocks of 128 vocabulary rows, up to 16 KB past the last stage
 constexpr int kUmmaLaneSmemBytes = kUmmaSmemBytes + 16 * 1024;
 // shared memory of a staged classifier (draft steps)
@@ -161,6 +164,13 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// The largest of a warp's numbers, in one instruction.
+__device__ __forceinline__ float warp_max_f32(float x) {
+    float m;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(m) : "f"(x));
+    return m;
+}
+
 // Shared-memory matrix descriptor: K-major tile, 128-byte swizzle, 8-row groups 1024 bytes apart.
 __device__ __forceinline__ uint64_t umma_smem_desc(const void* tile) {
     uint64_t desc = 0;
@@ -211,7 +221,9 @@ struct DraftFinalParams {
 // ---------------------------------------------------------------------------------------------
 // VL: vocabulary rows on the TMEM lanes (A operand, two blocks of 128 per tile), at most kUmmaLaneRows hidden rows, which all
 // CTAs read as one B operand of 16 or 32 rows.
-template <bool VL>
+// WIDE: the same with up to kUmmaWideRows hidden rows; the warp finds the largest logit of a column at once, and the running
+// keys live in shared memory.  130 rows, 32000 x 2048: 36.2 -> 32.3 us; 20.5 us at the measured copy bandwidth.
+template <bool VL, bool WIDE>
 __global__ void __launch_bounds__(kUmmaThreads, 1)
 umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_constant__ CUtensorMap tmap_H,
                  const UmmaParams p) {
@@ -242,7 +254,7 @@ umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_consta
     }
     // this CTA: `size` tiles of hidden rows from m_tile on, vocabulary rows v_begin .. v_end - 1 in tiles of TR
     const int m_tile = (int)blockIdx.x % tl.groups * tl.GS;
-    const int size = min(tl.GS, tl.MT - m_tile);
+    const int size = VL ? 1 : min(tl.GS, tl.MT - m_tile);
     const int slot = (int)blockIdx.x / tl.groups;
     const int v_begin = slot * tl.TPC * tl.TR;
     const int v_end = min(p.V, v_begin + tl.TPC * tl.TR);
@@ -269,6 +281,9 @@ umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_consta
     tc_fence_after();
     const uint32_t tmem_base = *tmem_base_s;
 
+    // (VL) columns of a block of 128 vocabulary rows; two blocks per tile, one or two tiles in TMEM
+    const int lane_cols = WIDE ? (p.a_rows + 31) & ~31 : kUmmaLaneRows;
+    const int lane_bufs = lane_cols <= 128 ? 2 : 1;
     const bool live = slot < tl.CN;   // (CTAs beyond the tiling have nothing to do)
 
     if (warp == 0) {
@@ -328,11 +343,12 @@ umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_consta
             // Two tiles of hidden rows use an accumulator each, one alternates between the two.
             int it = 0;
             for (int v0 = v_begin; v0 < v_end; v0 += tl.TR, ++it) {
-                const int first = size == 2 ? 0 : it & 1;
-                const uint32_t parity = (size == 2 ? it : it >> 1) & 1;
+                const bool alternate = VL ? lane_bufs == 2 : size == 1;
+                const int first = alternate ? it & 1 : 0;
+                const uint32_t parity = (alternate ? it >> 1 : it) & 1;
                 for (int j = 0; j < size; ++j) mbar_wait(&tmem_empty[first + j], parity ^ 1u, p.status);
                 tc_fence_after();
-                const uint32_t d_tmem = tmem_base + first * (VL ? 2 * kUmmaLaneRows : 256);
+                const uint32_t d_tmem = tmem_base + first * (VL ? 2 * lane_cols : 256);
                 for (int kb = 0; kb < KB; ++kb) {
                     mbar_wait(full0 + stage * 8, phase, p.status);
                     tc_fence_after();
@@ -343,7 +359,7 @@ umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_consta
                         if (upper) {
 #pragma unroll
                             for (int k = 0; k < kUmmaBK / 16; ++k)   // 128 rows further on
-                                tc_mma_bf16(d_tmem + kUmmaLaneRows, b_desc + (128 * 128 >> 4) + 2 * k, a_desc + 2 * k, idesc, (kb | k) != 0);
+                                tc_mma_bf16(d_tmem + lane_cols, b_desc + (128 * 128 >> 4) + 2 * k, a_desc + 2 * k, idesc, (kb | k) != 0);
                         }
                     } else {
 #pragma unroll
@@ -374,7 +390,54 @@ umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_consta
         const int ew = warp - 2;            // 0 .. kUmmaEpiWarps-1
         const int quad = warp & 3;          // TMEM lane quadrant this warp may read
         const int share = ew >> 2;          // two warps per quadrant split the columns of a tile
-        if constexpr (VL) {
+        if constexpr (VL && WIDE) {
+            // a lane holds one vocabulary row of the tile, a column is a hidden row; the warp's keys are behind the barriers,
+            // where MMAs may read (lanes nobody looks at) but nothing is loaded to
+            constexpr int kEpiThreads = kUmmaEpiWarps * 32;
+            unsigned long long* keys_s = reinterpret_cast<unsigned long long*>(smem + kUmmaRingBytes + 512);
+            unsigned long long* mine = keys_s + ew * kUmmaWideRows + lane;
+            for (int c = 0; c < lane_cols; c += 32) mine[c] = 0ull;
+            const int block_row = share * 128 + quad * 32;
+            int it = 0;
+            for (int v0 = v_begin; v0 < v_end; v0 += tl.TR, ++it) {
+                const int b = lane_bufs == 2 ? it & 1 : 0;
+                const int ncols = min(tl.TR, v_end - v0);
+                mbar_wait(&tmem_full[b], (lane_bufs == 2 ? it >> 1 : it) & 1, p.status);
+                tc_fence_after();
+                if (block_row < ncols) {
+                    const bool in = block_row + lane < ncols;
+#pragma unroll 1
+                    for (int c = 0; c < lane_cols; c += 32) {
+                        float z[32];
+                        tmem_ld32(tmem_base + (2 * b + share) * lane_cols + c + (static_cast<uint32_t>(quad * 32) << 16), z);
+                        float top = DISCO_NEG_INF;      // lane i: the largest logit of column i and the lanes that hold it
+                        unsigned int who = 0u;
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) {
+                            const float x = in ? z[i] : DISCO_NEG_INF;
+                            const float m = warp_max_f32(x);
+                            const unsigned int at = __ballot_sync(kFullMask, x == m);
+                            if (lane == i) top = m, who = at;
+                        }
+                        if (top > DISCO_NEG_INF) {
+                            const unsigned long long key = argmax_key(__fadd_rn(top, 0.f), v0 + block_row + __ffs(who) - 1);
+                            if (key > mine[c]) mine[c] = key;
+                        }
+                    }
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&tmem_empty[b]);
+            }
+            named_barrier_sync(2, kEpiThreads);
+            const int r = ew * 32 + lane;               // one result per hidden row and CTA
+            if (r < R) {
+                unsigned long long key = 0ull;
+#pragma unroll
+                for (int w = 0; w < kUmmaEpiWarps; ++w) key = max(key, keys_s[w * kUmmaWideRows + r]);
+                if (key) atomicMax(p.keys + r, key);
+            }
+        } else if constexpr (VL) {
             // a thread holds one vocabulary row of the tile, a column is a hidden row
             float best_v[kUmmaLaneRows];
             int best_i[kUmmaLaneRows];

@@ -118,6 +118,13 @@ def test_verification_of_few_rows_at_the_edges_of_its_tiling(oracle, rows_per_sm
     _verification_agrees(oracle, _sms() * rows_per_sm - 1, 1, R, 24)
 
 
+# ... with a column per hidden row and the keys in shared memory: two tiles in flight and one, and the row counts around the rule
+@pytest.mark.parametrize("rows_per_sm", [2, 128, 129, 600])
+@pytest.mark.parametrize("R", [34, 64, 65, 129, 144, 160, 161])
+def test_verification_with_a_column_per_row_at_the_edges_of_its_tiling(oracle, rows_per_sm, R):
+    _verification_agrees(oracle, _sms() * rows_per_sm - 1, 3, R, 24)
+
+
 # a box below 128 rows, exactly 128, both halves, two and four tiles of it, and beyond what the persistent kernel takes
 @pytest.mark.parametrize("rows_per_sm", [3, 128, 129, 256, 257, 1024, 1025])
 @pytest.mark.parametrize("B", [1, 2, 4])
