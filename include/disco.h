@@ -93,7 +93,8 @@ int disco_last_device_status(disco_ctx* ctx, int* out);
 int disco_launch_count(disco_ctx* ctx, long long* out);
 
 /* Kernel selection (tuning and tests): which = 0 automatic (default), 1 force the CUDA-core
- * streaming kernels, 2 force the tcgen05 kernels, one launch per draft step, 3 as 2 but with the persistent
+ * streaming kernels, 2 force the tcgen05 kernels, one launch per draft step (a verification's
+ * choice between them then takes no account of the head's size), 3 as 2 but with the persistent
  * draft-phase kernel where it applies. */
 int disco_set_kernel_path(disco_ctx* ctx, int which);
 

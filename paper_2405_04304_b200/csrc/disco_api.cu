@@ -237,9 +237,13 @@ int launch_umma(disco_ctx* c, const void* W, const void* H, int d, int R, const 
     // multiplies by 256.  In between and beyond it has no fewer multiplications and the dearer epilogue.  (Launches one after
     // the other at the power limit, 32000 x 5120, 34 / 64 / 96 / 130 / 160 / 192 rows: 61.4 -> 56.2, 61.6 -> 58.2, 63.1 -> 62.5,
     // 79.7 -> 68.9, 81.2 -> 72.6, 82.8 -> 81.1 us; 49152 x 6144, 64 / 96 / 160 / 192 rows: 113 -> 109, 115 -> 121, 158 -> 153,
-    // 160 -> 171 us.)
-    const bool wide = !dev_R && ((R > kUmmaLaneRows && R <= 64) || (R > 128 && R <= 160));
-    const bool lanes = wide || (!dev_R && R <= kUmmaLaneRows);
+    // 160 -> 171 us.)  A head that takes less than some 10 us does not reach the power limit, and its epilogue is a larger part
+    // (6 rows, 8000 x 512: 7.1 us, 7.7 with the vocabulary on the lanes).  Forced path 2 takes no account of the size.
+    const size_t head_bytes = (size_t)c->V * d * 2;
+    const bool few = R <= 64 && (head_bytes >= (size_t)64 << 20 || c->path == 2);
+    const bool beyond = R > 128 && R <= 160 && (head_bytes >= (size_t)45 << 20 || c->path == 2);
+    const bool lanes = !dev_R && (few || beyond);
+    const bool wide = lanes && R > kUmmaLaneRows;
     p.a_rows = lanes ? (R + 15) / 16 * 16 : p.t.MT > 1 ? 128 : (R + 7) / 8 * 8;
     p.pairs = !lanes && (dev_R || p.t.GS == 2);
     // The A tile holds a_rows rows.  The MMA still reads 128 rows from its start: what lies behind the tile (other

@@ -88,7 +88,7 @@ def test_draw_finds_the_entry_that_holds_the_target(V, B):
     ctx.close()
 
 
-def _verification_agrees(oracle, V, B, R, d):
+def _verification_agrees(oracle, V, B, R, d, path=0):
     sl = np.full(B, R // B - 1, dtype=np.int32)
     sl[-1] += R - int((sl + 1).sum())
     off = inputs.row_offsets(torch.from_numpy(sl)).numpy()
@@ -98,6 +98,8 @@ def _verification_agrees(oracle, V, B, R, d):
     draft = inputs.corrupt_ids(torch.from_numpy(clean), 0.02, V, seed=R).numpy()
     ref = oracle.verify_ragged(_bits(W), _bits(H), draft, off, nthreads=8)
     ctx = binding.Context(V, 8, d, max_batch=B, max_rows=R)
+    if path:
+        ctx.set_kernel_path(path)
     got = gpu_verify(ctx, W.cuda(), H, draft, row_off=off)
     check_verify(got, ref, off, draft, near_tie_ids(oracle, _bits(W), _bits(H), ref.gap))
     assert ctx.device_status() == 0
@@ -115,14 +117,14 @@ def test_verification_at_the_edges_of_the_tiles_of_hidden_rows(oracle, R, d):
 @pytest.mark.parametrize("rows_per_sm", [2, 128, 129, 256, 257, 600])
 @pytest.mark.parametrize("R", [2, 16, 17, 32, 33])
 def test_verification_of_few_rows_at_the_edges_of_its_tiling(oracle, rows_per_sm, R):
-    _verification_agrees(oracle, _sms() * rows_per_sm - 1, 1, R, 24)
+    _verification_agrees(oracle, _sms() * rows_per_sm - 1, 1, R, 24, path=2)
 
 
 # ... with a column per hidden row and the keys in shared memory: two tiles in flight and one, and the row counts around the rule
 @pytest.mark.parametrize("rows_per_sm", [2, 128, 129, 600])
 @pytest.mark.parametrize("R", [34, 64, 65, 129, 144, 160, 161])
 def test_verification_with_a_column_per_row_at_the_edges_of_its_tiling(oracle, rows_per_sm, R):
-    _verification_agrees(oracle, _sms() * rows_per_sm - 1, 3, R, 24)
+    _verification_agrees(oracle, _sms() * rows_per_sm - 1, 3, R, 24, path=2)
 
 
 # a box below 128 rows, exactly 128, both halves, two and four tiles of it, and beyond what the persistent kernel takes
