@@ -567,8 +567,18 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
             } else {
                 asm volatile("griddepcontrol.wait;" ::: "memory");  // scratch and outputs belong to the predecessor until now
                 if (!step_live()) break;
-                const uint32_t stamp = *reinterpret_cast<volatile unsigned int*>(p.sync) + 1u;
+                // The stamp may be moved on as soon as every CTA counts as started, and this CTA does when its first epilogue
+                // warp says so: that warp alone reads the word, and the others take the stamp from it.  (A warp with a read
+                // of its own could see the moved word and work on the next launch's set of bounds.)
+                uint32_t stamp;
+                if (ew == 0) {
+                    stamp = *reinterpret_cast<volatile unsigned int*>(p.sync) + 1u;
+                    if (lane == 0) *reinterpret_cast<volatile uint32_t*>(s_stamp) = stamp;
+                } else {
+                    stamp = cold_smem_word(s_stamp, p.status);
+                }
                 const uint32_t par = stamp & 1u;
+                // (that word is the other parity's: only a launch after this one writes it)
                 const int old_rows = *reinterpret_cast<volatile unsigned int*>(p.sync + 2 + (par ^ 1u));
                 if (blockIdx.x == 0)
                     for (int i = ew * 32 + lane; i < f.clear_n; i += kDbEpiWarps * 32) f.clear_words[i] = 0u;
@@ -584,11 +594,8 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
                      i += gridDim.x * (kDbEpiWarps * 32))
                     old[i] = make_uint4(0, 0, 0, 0);
                 __syncwarp();
-                if (ew == 0 && lane == 0) {
-                    // This CTA has started, now that it has read the stamp (nobody moves it before all CTAs have started).
-                    *reinterpret_cast<volatile uint32_t*>(s_stamp) = stamp;
-                    atomicAdd(p.sync + 4 + 4 * par, 1u);
-                }
+                // This CTA has started, now that its one read of the stamp is done (the word to count in depends on it).
+                if (ew == 0 && lane == 0) atomicAdd(p.sync + 4 + 4 * par, 1u);
             }
             const int phase_tiles = phase == 0 ? 0 : tiles;
 

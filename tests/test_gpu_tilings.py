@@ -60,6 +60,36 @@ def test_logits_that_no_bound_can_tell_apart(oracle, V, copies):
     ctx.close()
 
 
+# (32000 and 4000 rows leave CTAs without a vocabulary row on 148 SMs: they are done while the others have just started)
+@pytest.mark.parametrize("V", [32000, 4000])
+def test_steps_in_a_row_do_not_see_each_others_bounds(V):
+    """Back-to-back steps whose logits shrink and grow by a factor of 32 and whose row counts change: a bound left over from
+    the step before would drop all of a small step's candidates."""
+    d, counts, steps = 16, (40, 8, 1, 130), 160
+    W = inputs.lm_head(V, d, seed=V, std=0.3).cuda()
+    h = inputs.hidden(steps * 130, d, seed=11).view(steps, 130, d)
+    h[::2] *= 4.0
+    h[1::2] *= 0.125
+    h, clf = h.cuda(), to_gpu_clf(make_clf(8, seed=3))
+    ctx = binding.Context(V, d, 8, max_batch=130, max_rows=8, clf_hidden=8)
+    z = lambda *s, t=torch.float32: torch.zeros(*s, dtype=t, device="cuda")
+    one, token, feats = torch.ones(130, dtype=torch.int32, device="cuda"), z(steps, 130, t=torch.int32), z(steps, 130, 12)
+    conf, halt = z(130), z(130, t=torch.uint8)
+    rows = [counts[i // 2 % 4] for i in range(steps)]
+    for i, B in enumerate(rows):
+        ctx.draft_step(W, h[i, :B], one[:B], one[:B], clf, 0.5, 4, token[i], conf, halt, feats=feats[i])
+    assert ctx.device_status() == 0
+    for i, B in enumerate(rows):
+        logits = h[i, :B].double() @ W.double().T
+        top = logits.topk(10, -1).values
+        want = (top - torch.logsumexp(logits, -1, keepdim=True)).exp()
+        # a logit is a sum of 16 products of up to 60 in all, in fp32: 16 * 60 * 2^-24 = 6e-5 at most, e^z moves by as much
+        assert float(((feats[i, :B, :10].double() - want) / want).abs().max()) < 2e-4, f"step {i}"
+        picked = logits.gather(1, token[i, :B].long()[:, None])[:, 0]
+        assert float((top[:, 0] - picked).max()) < 2e-4, f"step {i}"
+    ctx.close()
+
+
 # slabs whose length is and is not a multiple of four, rows of V floats that are not 16-byte aligned, one to many CTAs a row
 @pytest.mark.parametrize("V,B", [(7, 1), (4096, 1), (4099, 3), (30002, 2), (30000, 40), (5001, 150)])
 def test_draw_finds_the_entry_that_holds_the_target(V, B):
