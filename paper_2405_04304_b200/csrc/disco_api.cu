@@ -737,7 +737,8 @@ int verify_common(disco_ctx* c, const void* W_T, const void* H_T, const int32_t*
     p.bonus = bonus;
     p.target_ids = target_ids;
     if (pad) p.padded = *pad;
-    const bool use_umma = c->encode_tiled != nullptr && (c->path == 2 || (c->path == 0 && R >= 2));
+    const bool use_umma = c->encode_tiled != nullptr && VerifyTiling::possible(R, c->sm_count) &&
+                          (c->path == 2 || (c->path == 0 && R >= 2));
     if (!use_umma) return run_stream<false>(c, p, 0, st);
     // Fixed-shape rows beyond one tile of 128: the projection is no longer free of charge for the rows that do not
     // count, so they are packed first and the tensor-core kernel tiles for the row count it finds on the device.

@@ -51,6 +51,8 @@ inline int umma_clf_bytes(int clf_H) { return (clf_H * (kNFeat + 2) + 4) * 4; }
 // group (1000 rows, 32000 x 5120 head: 284 us instead of 235).
 struct VerifyTiling {
     int MT, GS, groups, CN, TPC, TR, TRN;
+    // Every group of tiles needs a CTA: at most two tiles of hidden rows per CTA (37888 rows on 148 SMs).
+    __host__ __device__ static bool possible(int R, int grid) { return ((R + 127) / 128 + 1) / 2 <= grid; }
     __host__ __device__ static VerifyTiling make(int R, int V, int d, int grid) {
         VerifyTiling t;
         t.MT = (R + 127) / 128;
@@ -58,9 +60,9 @@ struct VerifyTiling {
         // 130 rows, 32000 x 2048: 35 -> 31), but they use both accumulators, so the epilogue does not overlap the next
         // tile's MMAs (1000 rows, 32000 x 768: 39 -> 43), and an odd last tile has its CTAs to itself (300 rows: 105 -> 116).
         // So: two tiles that share every vocabulary tile always; more where the contraction is long and the CTAs' largest
-        // share of work grows by at most a twentieth.
+        // share of work grows by at most a twentieth, or where there are more tiles of hidden rows than CTAs.
         const int cn_pairs = grid / ((t.MT + 1) / 2), cn_single = grid / t.MT;
-        t.GS = t.MT == 2 || (t.MT > 2 && d >= 2048 && cn_pairs * 21 >= cn_single * 40) ? 2 : 1;
+        t.GS = t.MT == 2 || t.MT > grid || (t.MT > 2 && d >= 2048 && cn_pairs * 21 >= cn_single * 40) ? 2 : 1;
         t.groups = (t.MT + t.GS - 1) / t.GS;
         t.CN = grid / t.groups;
         t.TPC = (V + 256 * t.CN - 1) / (256 * t.CN);

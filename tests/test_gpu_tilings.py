@@ -143,6 +143,47 @@ def test_verification_at_the_edges_of_the_tiles_of_hidden_rows(oracle, R, d):
     _verification_agrees(oracle, 700, 7, R, d)
 
 
+# as many tiles of hidden rows as SMs, one more (two tiles to a CTA), as many as that takes, and one more (CUDA cores)
+@pytest.mark.parametrize("tiles_per_sm,extra", [(1, 0), (1, 1), (2, 0), (2, 1)])
+@pytest.mark.parametrize("fixed_shape", [False, True])
+def test_verification_of_more_rows_than_the_sms_have_tiles_for(tiles_per_sm, extra, fixed_shape):
+    R, V, d, SL = 128 * _sms() * tiles_per_sm + extra, 300, 8, 3
+    R = R if not fixed_shape else (R + SL) // (SL + 1) * (SL + 1)
+    B = R // (SL + 1)
+    W, H = inputs.lm_head(V, d, seed=1, std=0.3).cuda(), inputs.hidden(R, d, seed=2).cuda()
+    logits = H.double() @ W.double().T
+    free = logits.argmax(-1).to(torch.int32)
+    z = lambda *s: torch.zeros(*s, dtype=torch.int32, device="cuda")
+    ctx = binding.Context(V, 8, d, max_batch=B, max_rows=R)
+    n_acc, nxt = z(B), z(B)
+    if fixed_shape:
+        sl = (torch.arange(B, device="cuda") % (SL + 1)).to(torch.int32)
+        tids, off = torch.full((B, SL + 1), -1, dtype=torch.int32, device="cuda"), z(B + 1)
+        ctx.verify_sl(W, H, free.view(B, SL + 1)[:, :SL].contiguous(), SL, 1, sl, B, SL, n_acc, nxt, target_ids=tids, row_off=off)
+        counts = torch.arange(SL + 1, device="cuda")[None] <= sl[:, None]
+        assert torch.equal(off[1:], torch.cumsum(sl + 1, 0).to(torch.int32))
+    else:   # the last sequence takes the rows that are left over
+        off = torch.arange(B + 1, dtype=torch.int32, device="cuda") * (SL + 1)
+        off[-1] = R
+        rows = torch.ones(R, dtype=torch.bool, device="cuda")
+        rows[(off[1:] - 1).long()] = False
+        tids = z(R)
+        ctx.verify_ragged(W, H, free[rows], off, B, R, n_acc, nxt, tids)
+        sl = off[1:] - off[:-1] - 1
+        counts = torch.ones(R, dtype=torch.bool, device="cuda")
+    assert ctx.device_status() == 0
+    got = tids.reshape(-1)[counts.reshape(-1)].long()
+    seen = logits[counts.reshape(-1)]
+    # a logit is a sum of 8 products of up to 10 in all, in fp32: 8 * 10 * 2^-24 = 5e-6 at most
+    assert float((seen.max(-1).values - seen.gather(1, got[:, None])[:, 0]).max()) < 1e-5
+    gap = logits.topk(2, -1).values
+    if float((gap[:, 0] - gap[:, 1]).min()) > 1e-5:
+        assert torch.equal(n_acc, sl)
+    else:   # (a row that ties may end its sequence's prefix)
+        assert float((n_acc == sl).float().mean()) > 0.99
+    ctx.close()
+
+
 # vocabulary rows on the lanes: a block of 128 not full, full, two of them, several tiles; 16 rows per column group and one more
 @pytest.mark.parametrize("rows_per_sm", [2, 128, 129, 256, 257, 600])
 @pytest.mark.parametrize("R", [2, 16, 17, 32, 33])
