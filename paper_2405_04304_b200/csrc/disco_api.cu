@@ -75,7 +75,7 @@ struct disco_ctx {
     int32_t* sample_seg_last;      //   the same shape: last index with positive weight
     unsigned int* sample_tickets;  //   [max_batch]
     void* pack_rows;               // fixed-shape verification with many rows: the rows that count, packed
-    int32_t* pack_off;             // [max_batch + 1] their offsets; the last entry is the row count
+    int32_t* pack_off;             // [max(max_batch, max_rows) + 1] their offsets; the last entry is the row count
     void* loop_rec;                // persistent draft-phase kernel: stamped 80-byte records, [4][CTA]; written by nothing else
     void* part_rec;                // draft step: 64-byte partial records, [sequence][CTA]
     void* stamped_rec;             // batched draft step: stamped 80-byte records, [sequence][CTA]; written by nothing else
@@ -511,7 +511,8 @@ int disco_create(disco_ctx** out, int V, int d_draft, int d_target, int max_batc
     device(&c->sample_seg_last, (size_t)max_batch * kSampleMaxSegments * 2 * sizeof(int32_t));
     device(&c->sample_tickets, (size_t)max_batch * sizeof(unsigned int));
     device(&c->pack_rows, (size_t)max_rows * d_target * 2);
-    device(&c->pack_off, ((size_t)max_batch + 2) * sizeof(int32_t));
+    // (a fixed-shape verification is bounded by its rows alone, and every sequence has at least one)
+    device(&c->pack_off, ((size_t)std::max(max_batch, max_rows) + 1) * sizeof(int32_t));
     device(&c->stage_hidden, hid);
     device(&c->stage_hidden_draft, (size_t)max_rows * d_draft * 2);
     auto pinned = [&](size_t bytes) {

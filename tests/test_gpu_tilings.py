@@ -184,6 +184,33 @@ def test_verification_of_more_rows_than_the_sms_have_tiles_for(tiles_per_sm, ext
     ctx.close()
 
 
+@pytest.mark.parametrize("B,SL", [(700, 0), (350, 1)])
+def test_fixed_shape_verification_is_bounded_by_its_rows_alone(B, SL):
+    """More sequences than the context's max_batch, which bounds the draft steps only; more than one tile of rows, so that the
+    rows that count are packed and B + 1 offsets are kept in scratch."""
+    V, d, R = 500, 16, B * (SL + 1)
+    W, H = inputs.lm_head(V, d, seed=3, std=0.3).cuda(), inputs.hidden(R, d, seed=4).cuda()
+    z = lambda *s: torch.zeros(*s, dtype=torch.int32, device="cuda")
+    ctx = binding.Context(V, 8, d, max_batch=1, max_rows=R)
+    n_acc, nxt, off, tids = z(B), z(B), z(B + 1), torch.full((B, SL + 1), -1, dtype=torch.int32, device="cuda")
+    sl = (torch.arange(B, device="cuda") % (SL + 1)).to(torch.int32)
+    ids = torch.full((B, max(SL, 1)), -1, dtype=torch.int32, device="cuda")   # no draft token is the target's
+    for _ in range(2):
+        ctx.verify_sl(W, H, ids if SL else None, SL, 1, sl, B, SL, n_acc, nxt, target_ids=tids, row_off=off)
+    assert ctx.device_status() == 0
+    assert torch.equal(off[1:], torch.cumsum(sl + 1, 0).to(torch.int32)) and not bool(n_acc.any())
+    logits = (H.double() @ W.double().T).view(B, SL + 1, V)
+    best = logits.max(-1).values
+    # a logit is a sum of 16 products of up to 20 in all, in fp32: 16 * 20 * 2^-24 = 2e-5 at most
+    for j in range(SL + 1):
+        on = sl >= j
+        got = tids[on, j].long()
+        assert float((best[on, j] - logits[on, j].gather(1, got[:, None])[:, 0]).max()) < 2e-5
+        assert bool((tids[~on, j] == -1).all())
+    assert torch.equal(nxt, tids[:, 0])
+    ctx.close()
+
+
 # vocabulary rows on the lanes: a block of 128 not full, full, two of them, several tiles; 16 rows per column group and one more
 @pytest.mark.parametrize("rows_per_sm", [2, 128, 129, 256, 257, 600])
 @pytest.mark.parametrize("R", [2, 16, 17, 32, 33])
