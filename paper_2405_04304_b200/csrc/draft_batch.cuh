@@ -45,7 +45,7 @@ constexpr int kDbBoundStride = 16;     // (rows 64 bytes apart)
 constexpr int kDbTurnStride = 36;      // floats per row of the area that turns a chunk of logits round (no bank conflicts)
 constexpr int kDbChunks = 4;           // chunks of 32 columns per warp and tile, at most
 constexpr uint32_t kDbNoIndex = 0x0fffffffu;           // record word: arg-max index in 28 bits, list length above it
-constexpr float kLog2e = 1.4426950408889634f, kLn2 = 0.6931471805599453f;
+constexpr float kLog2e = 1.4426950408889634f;
 
 struct DraftBatchParams {
     int V, d, R;
@@ -73,6 +73,29 @@ __device__ __forceinline__ float ex2_approx(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
+}
+// Two fp32 numbers in one register pair: an instruction for both.
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+    f32x2 d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
+    return d;
+}
+__device__ __forceinline__ void unpack2(f32x2 d, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(d)); }
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
 }
 __device__ __forceinline__ float max3f(float a, float b, float c) { return RegTop10::max3(a, b, c); }
 
@@ -554,7 +577,7 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
             bool many_kept = false;        // enough of them to store four rows per instruction
             unsigned keep_mask = 0u;       // rows of this warp whose raw logits go to probs (none of a masked sequence's)
             unsigned int *slots = nullptr, *my_slot = nullptr;
-            float m = DISCO_NEG_INF, Z = 0.f, S2 = 0.f;      // S2 = sum e^(z - m) (z - m) / ln 2
+            float m = DISCO_NEG_INF, Z = 0.f, S = 0.f;       // S = sum e^(z - m) (z - m)
             float best_v = DISCO_NEG_INF;
             int best_i = 0;
             RegTop10 top;
@@ -644,26 +667,32 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
                         cm[0] = cmax;
                         // the reference maximum moves first, then the chunk is added
                         const float mn = fmaxf(m, cmax);
-                        const float dm = fmaxf((m - mn) * kLog2e, -1000.f);
-                        const float em = ex2_approx(dm);
+                        const float dm = fmaxf(m - mn, -1000.f);
+                        const float em = ex2_approx(dm * kLog2e);
                         m = mn;
-                        if (n < 32) {   // masked columns: finite, far below the maximum (e = 0, and 0 * -inf is avoided)
+                        if (n < 32) {   // masked columns: finite, far below any logit (e = 0, and 0 * -inf is avoided)
 #pragma unroll
                             for (int j = 0; j < 32; ++j)
-                                if (j >= n) z[j] = mn - 1000.f;
+                                if (j >= n) z[j] = -2e38f;
                         }
-                        const float nm = -mn * kLog2e;
-                        float Za = 0.f, Sa = 0.f, Zb = 0.f, Sb = 0.f;
+                        // The difference to the maximum comes first: it is exact where it matters, whatever the size of the
+                        // logits.  (z * log2e - m * log2e in one instruction keeps the rounding of m * log2e: up to 5e-6 of
+                        // every probability at logits of 100, 2e-5 at 400.)  Two columns per instruction, so it costs no more.
+                        const f32x2 neg_m = pack2(-mn, -mn), log2e = pack2(kLog2e, kLog2e);
+                        f32x2 Zc = 0ull, Sc = 0ull;
 #pragma unroll
                         for (int j = 0; j < 32; j += 2) {
-                            const float ta = fmaf(z[j], kLog2e, nm), tb = fmaf(z[j + 1], kLog2e, nm);
-                            const float ea = ex2_approx(ta), eb = ex2_approx(tb);
-                            Za += ea;
-                            Sa = fmaf(ea, ta, Sa);
-                            Zb += eb;
-                            Sb = fmaf(eb, tb, Sb);
+                            const f32x2 t = add2(pack2(z[j], z[j + 1]), neg_m);
+                            float xa, xb;
+                            unpack2(mul2(t, log2e), xa, xb);
+                            const f32x2 e = pack2(ex2_approx(xa), ex2_approx(xb));
+                            Zc = add2(Zc, e);
+                            Sc = fma2(e, t, Sc);
                         }
-                        S2 = fmaf(em, fmaf(dm, Z, S2), Sa + Sb);   // (Z = S2 = 0 before the first chunk)
+                        float Za, Zb, Sa, Sb;
+                        unpack2(Zc, Za, Zb);
+                        unpack2(Sc, Sa, Sb);
+                        S = fmaf(em, fmaf(dm, Z, S), Sa + Sb);   // (Z = S = 0 before the first chunk)
                         Z = fmaf(Z, em, Za + Zb);
                         if (keep_mask) {
                             // A thread holds one row: the chunk goes through shared memory so that every store instruction
@@ -798,7 +827,7 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
             // one record per hidden row and CTA: the warp with share 1 hands its rows' state to the one with share 0
             float4* xrow = xch + tile_row * 4;
             if (share != 0) {
-                xrow[0] = make_float4(m, Z, S2, __int_as_float(best_i));
+                xrow[0] = make_float4(m, Z, S, __int_as_float(best_i));
                 xrow[1] = make_float4(best_v, bound_used, top.t[0], top.t[1]);
                 xrow[2] = make_float4(top.t[2], top.t[3], top.t[4], top.t[5]);
                 xrow[3] = make_float4(top.t[6], top.t[7], top.t[8], top.t[9]);
@@ -808,9 +837,9 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
                 const float4 a = xrow[0], b4 = xrow[1], c4 = xrow[2], d4 = xrow[3];
                 // (a share without columns has Z = 0 and m = -inf; a CTA without columns leaves a record with Z = 0)
                 const float M = fmaxf(m, a.x);
-                const float d1 = Z > 0.f ? (m - M) * kLog2e : 0.f, d2 = a.y > 0.f ? (a.x - M) * kLog2e : 0.f;
-                const float e1 = ex2_approx(d1), e2 = ex2_approx(d2);
-                S2 = e1 * fmaf(d1, Z, S2) + e2 * fmaf(d2, a.y, a.z);
+                const float d1 = Z > 0.f ? m - M : 0.f, d2 = a.y > 0.f ? a.x - M : 0.f;
+                const float e1 = ex2_approx(d1 * kLog2e), e2 = ex2_approx(d2 * kLog2e);
+                S = e1 * fmaf(d1, Z, S) + e2 * fmaf(d2, a.y, a.z);
                 Z = Z * e1 + a.y * e2;
                 m = M;
                 const int i2 = __float_as_int(a.w);
@@ -833,7 +862,7 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
                     const uint32_t word = (cnt << 28) | (best_v == m && Z > 0.f ? (uint32_t)best_i : kDbNoIndex);
                     float4* rec = p.part_rec + ((size_t)row * p.CN + nslot) * kStampedPieces;
                     const float sf = __uint_as_float(smem_word(s_stamp, p.status));   // (written microseconds ago)
-                    store_relaxed_v4(rec, m + 0.f, Z, S2 * kLn2, sf);
+                    store_relaxed_v4(rec, m + 0.f, Z, S, sf);
                     store_relaxed_v4(rec + 1, __uint_as_float(word), top.t[0], bound_used, sf);
                     store_relaxed_v4(rec + 2, top.t[1], top.t[2], top.t[3], sf);
                     if (cnt > 4) {

@@ -90,6 +90,36 @@ def test_steps_in_a_row_do_not_see_each_others_bounds(V):
     ctx.close()
 
 
+@pytest.mark.parametrize("V,B", [(32000, 1), (5001, 40), (20011, 200)])
+@pytest.mark.parametrize("path", [0, 1])
+def test_soft_max_does_not_depend_on_what_all_logits_have_in_common(V, B, path):
+    """Row b's logits are w_v + its offset, exactly (w_v a multiple of 1/32 below 4): the distribution is that of the w_v."""
+    d = 8
+    g = torch.Generator().manual_seed(V)
+    w = torch.randint(-127, 128, (V,), generator=g).double() / 32
+    W, h = torch.zeros(V, d), torch.zeros(B, d)
+    W[:, 0], W[:, 1], h[:, 1] = 1.0, w.float(), 1.0
+    h[:, 0] = torch.tensor([400.0, 0.0, 96.0, -2048.0, 131072.0, -131072.0])[torch.arange(B) % 6]
+    W, h = W.to(torch.bfloat16).cuda(), h.to(torch.bfloat16).cuda()
+    y = torch.softmax(w, -1)
+    top, ent = y.topk(10).values, -(y * y.log()).sum()
+    z = lambda *s, t=torch.float32: torch.zeros(*s, dtype=t, device="cuda")
+    one, token, nxt, conf, halt = z(B, t=torch.int32) + 1, z(B, t=torch.int32), z(B, t=torch.int32), z(B), z(B, t=torch.uint8)
+    feats, y_T = z(B, 12), z(B, V)
+    ctx = binding.Context(V, d, d, max_batch=B, max_rows=B, clf_hidden=8)
+    ctx.set_kernel_path(path)
+    ctx.draft_step(W, h, one, one, to_gpu_clf(make_clf(8, seed=5)), 0.5, 4, token, conf, halt, feats=feats)
+    ctx.verify_sample_ragged(W, h, None, None, None, B, B, None, z(B), z(B, t=torch.int32), nxt, y_T)
+    assert ctx.device_status() == 0
+    # an exponential is good to 2 ulp of its own and 2^-24 * |z - m| of its argument, |z - m| < 8: 8e-7 in all, once above
+    # and once below the fraction bar; the entropy is some 10, a difference of ln Z and S / Z of that accuracy
+    assert float(((feats[:, :10].cpu().double() - top) / top).abs().max()) < 2e-6
+    assert float((feats[:, 10].cpu().double() - ent).abs().max()) < 1e-5
+    assert float(((y_T.cpu().double() - y) / y).abs().max()) < 2e-6
+    assert token.tolist() == [int(w.argmax())] * B
+    ctx.close()
+
+
 # slabs whose length is and is not a multiple of four, rows of V floats that are not 16-byte aligned, one to many CTAs a row
 @pytest.mark.parametrize("V,B", [(7, 1), (4096, 1), (4099, 3), (30002, 2), (30000, 40), (5001, 150)])
 def test_draw_finds_the_entry_that_holds_the_target(V, B):
