@@ -120,7 +120,8 @@ int disco_test_hooks(disco_ctx* ctx, long long wait_budget_clocks, int withhold_
  *   clf        host struct         classifier parameters (device arrays)
  *   tau        threshold; halt iff C < tau (C == tau continues) or n_drafted >= sl_max
  * Outputs
- *   token      int32 [B]           greedy draft token: lowest index attaining the largest logit
+ *   token      int32 [B]           greedy draft token: lowest index attaining the largest logit (-1 if
+ *                                  the logits are not numbers, as those of a hidden state that is not)
  *   conf       float [B]           C
  *   halt       uint8 [B]           1 = stop drafting and hand over to the target
  *   feats      float [B, DISCO_NFEAT] or NULL   the feature vector (top-10 probabilities

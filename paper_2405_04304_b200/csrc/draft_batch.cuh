@@ -366,7 +366,7 @@ __device__ __forceinline__ void db_finish_row(const DraftBatchParams& p, const D
     }
     SoftmaxState st;
     st.m = M, st.Z = Z, st.S = S;
-    const unsigned long long key = argmax_key(M, static_cast<int>(idx));
+    const unsigned long long key = idx != kDbNoIndex ? argmax_key(M, static_cast<int>(idx)) : 0ull;   // (0: token -1)
     const DraftOutputs o{f.token, f.conf, f.halt, f.feats, f.final_stats, f.nll_sum, f.stats_only, f.chain, real};
     const int Hc = f.clf_H;
     warp_draft_epilogue(st, key, sel, fpos, nd, f.tau, f.sl_max, sm, clf_s, clf_s + Hc * kNFeat, clf_s + Hc * (kNFeat + 1),
@@ -721,7 +721,8 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
                         }
                     }
                     if (use_bound) {
-                        if (valid && c_lo < c_hi && (t == 0 || t + 1 < tiles) && tile_max > bound_used)
+                        // (an infinite logit bounds nothing: its CTA's statistics are no numbers, and its record is left out)
+                        if (valid && c_lo < c_hi && (t == 0 || t + 1 < tiles) && tile_max > bound_used && tile_max < -DISCO_NEG_INF)
                             atomicMax(my_slot, ordered_bits(tile_max + 0.f));
                         if (t > 0 || !defer) {
                             if (t == 0 && share == 0) {
@@ -858,6 +859,8 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
                         top.t[k] += 0.f;   // -0 and +0 are the same logit
                     }
                 }
+                // Statistics that are no numbers (logits that are infinite or no numbers themselves): the record is as good as empty.
+                if (!(Z > 0.f)) cnt = 0u;
                 if (valid && phase == 1) {
                     const uint32_t word = (cnt << 28) | (best_v == m && Z > 0.f ? (uint32_t)best_i : kDbNoIndex);
                     float4* rec = p.part_rec + ((size_t)row * p.CN + nslot) * kStampedPieces;

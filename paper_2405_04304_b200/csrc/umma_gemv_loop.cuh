@@ -169,8 +169,10 @@ __device__ __forceinline__ void group_fold_row(const float* fold, int NW, RowSta
         const uint32_t Mb = __reduce_max_sync(kFullMask, mine);
         const uint32_t klo = __reduce_max_sync(kFullMask, q.y > 0.f && mine == Mb ? __float_as_uint(q.w) : 0u);
         const float M = from_ordered_bits(Mb);
+        // (A warp whose sum is no number may have an infinite logit in its list: the CTA's sum is then no number either, and
+        // the reader leaves its record out.)
         float Z = 0.f, S = 0.f;
-        if (q.y > 0.f) {
+        if (q.y != 0.f) {
             const float dm = q.x - M;
             const float e = __expf(dm);
             Z = q.y * e;
