@@ -830,9 +830,6 @@ int disco_draft_step_sample(disco_ctx* c, const void* W_D, const void* h_D, int 
     if (rc) return rc;
     // probs holds the logits: the kernel turns them into y^D and replaces the greedy token by the draw
     DrawRowsParams dp{};
-    dp.probs = probs;
-    dp.stats = c->final_stats;
-    dp.recs = rl.recs;
     dp.rec_pieces = rl.pieces;
     dp.NP = rl.NP;
     dp.slab = rl.slab;
@@ -840,14 +837,21 @@ int disco_draft_step_sample(disco_ctx* c, const void* W_D, const void* h_D, int 
     const int seg = std::max(1, std::min(rl.NP, 2 * c->sm_count / B));
     dp.seg_slabs = (rl.NP + seg - 1) / seg;
     dp.V = c->V;
-    dp.u = u;
-    dp.active = active;
-    dp.token = token;
-    dp.p_token = p_token;
-    const cudaError_t e = launch_after(c, draw_rows_kernel, dim3((unsigned)((rl.NP + dp.seg_slabs - 1) / dp.seg_slabs), (unsigned)B),
-                                       dim3(kSampleThreads), 0, static_cast<cudaStream_t>(stream), dp);
-    c->launches += 1;
-    return cuda_ok(e, "draw_rows_kernel launch") ? DISCO_OK : DISCO_ERR_CUDA;
+    constexpr int kMaxRows = 65535;   // a grid's second dimension
+    for (size_t b0 = 0; b0 < (size_t)B; b0 += kMaxRows) {
+        dp.probs = probs + b0 * c->V;
+        dp.stats = c->final_stats + 2 * b0;
+        dp.recs = rl.recs + b0 * rl.NP * rl.pieces;
+        dp.u = u + b0;
+        dp.active = active ? active + b0 : nullptr;
+        dp.token = token + b0;
+        dp.p_token = p_token ? p_token + b0 : nullptr;
+        const dim3 grid((unsigned)((rl.NP + dp.seg_slabs - 1) / dp.seg_slabs), (unsigned)std::min<size_t>(kMaxRows, B - b0));
+        const cudaError_t e = launch_after(c, draw_rows_kernel, grid, dim3(kSampleThreads), 0, static_cast<cudaStream_t>(stream), dp);
+        c->launches += 1;
+        if (!cuda_ok(e, "draw_rows_kernel launch")) return DISCO_ERR_CUDA;
+    }
+    return DISCO_OK;
 }
 
 int disco_verify_sample_ragged(disco_ctx* c, const void* W_T, const void* H_T, const int32_t* draft_ids,

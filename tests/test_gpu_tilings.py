@@ -163,8 +163,9 @@ def test_logits_that_are_not_numbers(V, B, path):
     ctx.close()
 
 
-# slabs whose length is and is not a multiple of four, rows of V floats that are not 16-byte aligned, one to many CTAs a row
-@pytest.mark.parametrize("V,B", [(7, 1), (4096, 1), (4099, 3), (30002, 2), (30000, 40), (5001, 150)])
+# slabs whose length is and is not a multiple of four, rows of V floats that are not 16-byte aligned, one to many CTAs a row, more
+# rows than a grid's second dimension has room for
+@pytest.mark.parametrize("V,B", [(7, 1), (4096, 1), (4099, 3), (30002, 2), (30000, 40), (5001, 150), (7, 65600)])
 def test_draw_finds_the_entry_that_holds_the_target(V, B):
     d = 24
     W, h = inputs.lm_head(V, d, seed=V, std=0.3).cuda(), inputs.hidden(B, d, seed=B).cuda()
