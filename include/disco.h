@@ -94,8 +94,8 @@ int disco_launch_count(disco_ctx* ctx, long long* out);
 
 /* Kernel selection (tuning and tests): which = 0 automatic (default), 1 force the CUDA-core
  * streaming kernels, 2 force the tcgen05 kernels, one launch per draft step (a verification's
- * choice between them then takes no account of the head's size), 3 as 2 but with the persistent
- * draft-phase kernel where it applies. */
+ * choice between them then takes no account of the head's size), 3 the draft steps as 2 but with the
+ * persistent draft-phase kernel where it applies, greedy verifications as 1. */
 int disco_set_kernel_path(disco_ctx* ctx, int which);
 
 /* For the test-suite: how the bounded device-side waits behave when what they wait for never comes.
@@ -261,8 +261,8 @@ int disco_verify_ragged(disco_ctx* ctx, const void* W_T, const void* H_T, const 
  * disco_draft_step on the hidden states h_D[i-1] with pos = pos0 + i and n_drafted = i, for the sequences
  * that have not stopped yet, and the halt flag it produces is consumed on the device: no host round trip
  * between the steps.  A step that finds no sequence drafting any more returns at once.  (In this isolated
- * tail the hidden state of every step is an input; a decoder would produce h_D[i] from token i-1.  Step i
- * reads h_D[i-1] only after step i-1 has finished.)
+ * tail the hidden state of every step is an input, complete before the call like any other: a decoder would
+ * produce h_D[i] from token i-1, but the kernels may read it while step i-1 is still being decided.)
  *   W_D            bf16 [V, d_draft]            draft LM head
  *   w_step_stride  bytes between the LM heads used by consecutive steps; 0 = the same head for every step
  *                  (the normal case).  Non-zero lets a benchmark rotate through copies of the head so that

@@ -238,7 +238,14 @@ int launch_umma(disco_ctx* c, const void* W, const void* H, int d, int R, const 
     // the other at the power limit, 32000 x 5120, 34 / 64 / 96 / 130 / 160 / 192 rows: 61.4 -> 56.2, 61.6 -> 58.2, 63.1 -> 62.5,
     // 79.7 -> 68.9, 81.2 -> 72.6, 82.8 -> 81.1 us; 49152 x 6144, 64 / 96 / 160 / 192 rows: 113 -> 109, 115 -> 121, 158 -> 153,
     // 160 -> 171 us.)  A head that takes less than some 10 us does not reach the power limit, and its epilogue is a larger part
-    // (6 rows, 8000 x 512: 7.1 us, 7.7 with the vocabulary on the lanes).  Forced path 2 takes no account of the size.
+    // (6 rows, 8000 x 512: 7.1 us, 7.7 with the vocabulary on the lanes).  So a lower limit on the head's size for either band,
+    // from launches one after the other with the other form -> this one.  Up to 64 rows, 64 MB (d = 2048, 6 / 11 / 30 / 64 rows):
+    // 32 MB 11.8 / 12.0 / 12.9 / 13.4 -> 12.5 / 13.0 / 15.3 / 13.5 us; 64 MB 16.5 / 16.5 / 16.6 / 17.4 -> 16.6 / 16.8 / 18.4 / 17.2
+    // (17 to 32 rows catch up at 131 MB: 29.4 -> 28.6); 131 MB 29.3 / 29.3 / 29.4 / 29.9 -> 27.0 / 27.3 / 28.6 / 28.1.
+    // 129 to 160 rows, 45 MB, where the other form multiplies by 256 (130 / 160 rows): d = 1024, 32 MB 16.2 / 16.2 -> 15.0 / 15.0,
+    // 45 MB 18.3 / 18.4 -> 18.6 / 18.8, 96 MB 32.8 / 32.8 -> 32.3 / 33.3; d = 2048, 45 MB 20.4 / 20.3 -> 17.9 / 18.6, 131 MB
+    // 39.9 / 39.2 -> 34.3 / 36.1; d = 5120, 45 MB 29.6 / 29.6 -> 27.4 / 29.6, 320 MB 83.2 / 80.8 -> 67.1 / 71.3.  (It pays below
+    // 45 MB as well where the contraction is long.)  Forced path 2 takes no account of the size.
     const size_t head_bytes = (size_t)c->V * d * 2;
     const bool few = R <= 64 && (head_bytes >= (size_t)64 << 20 || c->path == 2);
     const bool beyond = R > 128 && R <= 160 && (head_bytes >= (size_t)45 << 20 || c->path == 2);
@@ -667,8 +674,8 @@ int draft_step_common(disco_ctx* c, const void* W_D, const void* h_D, int d, int
     p.feats = feats;
     p.probs = probs;
     p.nll_sum = nll_sum;
-    // The tensor-core kernel serves every batch (measured on the Vicuna head, us per step in a stream for 1 / 4 / 7 / 64
-    // sequences: 13.4 / 14.6 / 15.9 / 19.9); the CUDA-core streaming kernel is the path without tensor maps.
+    // The tensor-core kernel serves every batch (us per step in a stream, cold L2: one sequence of 32000 x 768 14.6, 7 of
+    // 40011 x 768 17.6, 64 of 32000 x 768 18.2); the CUDA-core streaming kernel is the path without tensor maps.
     const bool use_umma = draft_batch_possible(c, B) && c->path != 1;
     if (use_umma) {
         DraftFinalParams f{};
@@ -762,7 +769,11 @@ int verify_common(disco_ctx* c, const void* W_T, const void* H_T, const int32_t*
         p.padded.row_off_out = nullptr;
         dev_R = c->pack_off + B;
     }
-    if (B <= 16) {  // few sequences: the last CTA of the main kernel finishes the job, no second launch
+    // Few sequences: the last CTA of the main kernel finishes the job, no second launch.  Its eight warps take the sequences in
+    // turn behind a fence and a ticket, while the second kernel's launch hides under the first (us in one / two launches,
+    // 32000 x 2048, 5 rows each: 4 sequences 26.9 / 27.3, 8 26.5 / 26.8, 16 29.0 / 28.6, 20 30.2 / 29.7, 32 35.3 / 33.4; 32000 x
+    // 5120: 54.6 / 55.1, 55.8 / 56.0, 60.0 / 59.2, 63.2 / 59.6).
+    if (B <= 16) {
         UmmaParams fp{};
         fp.fuse_final = 1;
         fp.ticket = c->ticket + 32;

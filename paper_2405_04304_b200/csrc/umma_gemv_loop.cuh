@@ -10,8 +10,8 @@
 //     memory, so every CTA must be running);
 //   * the producer never stops: as soon as the MMAs of step i have released a ring stage it is refilled
 //     with the LM head's tiles for step i + 1, while the CTA folds, publishes its record, and the step is
-//     decided.  Only the hidden rows of step i + 1 are requested after step i has been decided -- in a
-//     decoder they would not exist before;
+//     decided.  The hidden rows of step i + 1, an input of the call like all others, follow as soon as the MMAs of step i
+//     are done with theirs;
 //   * the B operand is the one 8-row box of hidden rows read twice over (zero stride between the 8-row groups of the
 //     descriptor), so nothing outside it is read;
 //   * every warp folds its 32 logits of a hidden row (statistics, arg-max, a descending list of ten); one barrier later a
