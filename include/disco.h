@@ -260,9 +260,11 @@ int disco_verify_ragged(disco_ctx* ctx, const void* W_T, const void* H_T, const 
  * footnote on SL_max: fixed tensor shapes).  One enqueue runs up to sl_max draft steps; step i (1-based) is
  * disco_draft_step on the hidden states h_D[i-1] with pos = pos0 + i and n_drafted = i, for the sequences
  * that have not stopped yet, and the halt flag it produces is consumed on the device: no host round trip
- * between the steps.  A step that finds no sequence drafting any more returns at once.  (In this isolated
+ * between the steps.  A launch that finds no sequence drafting any more returns at once.  (In this isolated
  * tail the hidden state of every step is an input, complete before the call like any other: a decoder would
- * produce h_D[i] from token i-1, but the kernels may read it while step i-1 is still being decided.)
+ * produce h_D[i] from token i-1, but the kernels may read it before step i-1 has been decided.  With one head for
+ * all steps they project the rows of several steps in one pass over it; what a sequence's steps past its stop
+ * would have given, whatever their hidden states hold, is dropped.)
  *   W_D            bf16 [V, d_draft]            draft LM head
  *   w_step_stride  bytes between the LM heads used by consecutive steps; 0 = the same head for every step
  *                  (the normal case).  Non-zero lets a benchmark rotate through copies of the head so that

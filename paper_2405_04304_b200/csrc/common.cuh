@@ -44,11 +44,39 @@ struct ChainLink {
     const int32_t* pos0;       // [B] tokens generated before this iteration
     const int32_t* sl_forced;  // [B] or null
     int step;
+    // A launch may be `group` consecutive steps at once, `step` the first of them: row s * B + b is step `step + s` of
+    // sequence b.  Its verdicts meet in a word per sequence (group_step_taken).
+    int group = 1;
+    int B = 0;                 // sequences (group > 1)
 };
+// Sequence of a row of the launch, and its step.
+__device__ __forceinline__ int chain_seq(const ChainLink& c, int row) { return c.group > 1 ? row % c.B : row; }
+__device__ __forceinline__ int chain_step(const ChainLink& c, int row) { return c.step + (c.group > 1 ? row / c.B : 0); }
 
 __device__ __forceinline__ bool chain_seq_live(const ChainLink& c, const uint8_t* active, int b) {
     if (c.alive) return c.step == 1 || __ldcg(c.alive + b) != 0;
     return !active || active[b] != 0;
+}
+// Several steps in one launch: step s of a sequence takes place iff none of the launch's steps before it stopped.  The steps
+// of a sequence are finished by different warps; each leaves two bits in the sequence's word (finished, stops) and looks at
+// those below its own.  Nothing else passes between the warps, so relaxed accesses do.  Rows are handed out in ascending
+// order, so whatever is awaited here belongs to a warp that is at work (bounded all the same).
+constexpr int kMaxGroup = 16;
+__device__ __forceinline__ bool group_step_taken(unsigned int* word, int s, bool last, bool stops, int* status) {
+    const unsigned int below = (1u << (2 * s)) - 1u, fin = 0x55555555u & below, stop = 0xaaaaaaaau & below;
+    unsigned int v = 0u;
+    if (!last) v = atomicOr(word, (1u | (stops ? 2u : 0u)) << (2 * s));
+    const long long t0 = clock64();
+    for (int polls = 0;; ++polls) {
+        if (v & stop) return false;
+        if ((v & fin) == fin) return true;
+        asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(word) : "memory");
+        if ((polls & 63) == 63 &&
+            (*reinterpret_cast<volatile int*>(status) == DISCO_ERR_TIMEOUT || clock64() - t0 > kWaitBudgetClocks)) {
+            record_status(status, DISCO_ERR_TIMEOUT);
+            return false;
+        }
+    }
 }
 // Warp-collective: does any of the B sequences still draft?  (Always true outside a chain and at step 1.)
 __device__ __forceinline__ bool chain_any_live(const ChainLink& c, int B, int lane) {

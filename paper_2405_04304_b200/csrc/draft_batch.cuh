@@ -225,8 +225,8 @@ __device__ __forceinline__ void db_finish_row(const DraftBatchParams& p, const D
     float fpos = 0.f;
     int nd = 1;
     if (real) {
-        fpos = chain ? static_cast<float>(f.chain.pos0[b] + f.chain.step) : (f.pos ? static_cast<float>(f.pos[b]) : 0.f);
-        nd = chain ? f.chain.step : (f.n_drafted ? f.n_drafted[b] : 1);
+        nd = chain ? chain_step(f.chain, b) : (f.n_drafted ? f.n_drafted[b] : 1);
+        fpos = chain ? static_cast<float>(f.chain.pos0[chain_seq(f.chain, b)] + nd) : (f.pos ? static_cast<float>(f.pos[b]) : 0.f);
     }
     float4 q[PER][3];
     {
@@ -376,7 +376,9 @@ __device__ __forceinline__ void db_finish_row(const DraftBatchParams& p, const D
     SoftmaxState st;
     st.m = M, st.Z = Z, st.S = S;
     const unsigned long long key = idx != kDbNoIndex ? argmax_key(M, static_cast<int>(idx)) : 0ull;   // (0: token -1)
-    const DraftOutputs o{f.token, f.conf, f.halt, f.feats, f.final_stats, f.nll_sum, f.stats_only, f.chain, real};
+    // (a launch of several steps: the sequence's verdicts in a spare word of its first row's bounds, cleared with them)
+    unsigned int* verdicts = f.chain.group > 1 ? p.bound + (stamp & 1u) * p.set_words + (size_t)chain_seq(f.chain, b) * kDbBoundStride + kDbBoundSlots : nullptr;
+    const DraftOutputs o{f.token, f.conf, f.halt, f.feats, f.final_stats, f.nll_sum, f.stats_only, f.chain, real, verdicts, p.status};
     const int Hc = f.clf_H;
     warp_draft_epilogue(st, key, sel, fpos, nd, f.tau, f.sl_max, sm, clf_s, clf_s + Hc * kNFeat, clf_s + Hc * (kNFeat + 1),
                         clf_s + Hc * (kNFeat + 2), Hc, b, o, lane);
@@ -446,7 +448,7 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
     // A step of a draft phase that has ended already needs neither loads nor rehearsals.  The flags are looked at ahead of
     // the dependency wait for that, once for the whole CTA: they may be old and decide nothing else.
     if (warp == 2) {
-        const bool any = !chained || chain_any_live(f.chain, f.B, lane);
+        const bool any = !chained || chain_any_live(f.chain, f.chain.B, lane);
         if (lane == 0) *s_look = any ? 1u : 0u;
     }
     tc_fence_before();
@@ -525,7 +527,7 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
         bool live = true;
         if (chained) {
             asm volatile("griddepcontrol.wait;" ::: "memory");
-            live = chain_any_live(f.chain, f.B, lane);
+            live = chain_any_live(f.chain, f.chain.B, lane);
             if (lane == 0) *reinterpret_cast<volatile uint32_t*>(s_live) = live ? 1u : 2u;
         }
         if (live && elect_one()) {
@@ -607,7 +609,7 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
                     for (int i = ew * 32 + lane; i < f.clear_n; i += kDbEpiWarps * 32) f.clear_words[i] = 0u;
                 // Rows of sequences that are masked or have stopped drafting: nobody wants their candidates, and no record of
                 // them is written.
-                valid = valid && chain_seq_live(f.chain, f.active, row);
+                valid = valid && chain_seq_live(f.chain, f.active, chain_seq(f.chain, row));
                 keep_mask = __ballot_sync(kFullMask, p.probs && valid);
                 many_kept = __popc(keep_mask) > 8 && (reinterpret_cast<uintptr_t>(p.probs) & 15) == 0;
                 slots = p.bound + par * p.set_words + (size_t)(valid ? row : 0) * kDbBoundStride;
@@ -910,7 +912,7 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
         int b = 0;
         bool run = !epi && looks_live;
         for (bool real = false;; real = true) {
-            if (run && !(real && !chain_seq_live(f.chain, f.active, b))) db_finish_row(p, f, b, real, stamp + (real ? f.test_stamp_skew : 0u), sm, clf_s, STATS, lane);
+            if (run && !(real && !chain_seq_live(f.chain, f.active, chain_seq(f.chain, b)))) db_finish_row(p, f, b, real, stamp + (real ? f.test_stamp_skew : 0u), sm, clf_s, STATS, lane);
             run = true;
             if (!real) {
                 if (!epi) {

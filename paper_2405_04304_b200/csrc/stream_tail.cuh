@@ -557,6 +557,8 @@ struct DraftOutputs {
                      // 2: token and features, no classifier (bulk feature extraction)
     ChainLink chain; // draft phase chained on the device: the look-ahead bookkeeping goes with the halt flag
     bool write = true;   // false: compute, write nothing (a warp that only wants the code in its instruction cache)
+    unsigned int* verdicts = nullptr;   // chain.group > 1: the word of row b's sequence
+    int* status = nullptr;
 };
 __device__ __forceinline__ bool warp_draft_epilogue(const SoftmaxState& st, unsigned long long key, float sel, float fpos,
                                                     int n_drafted, float tau, int sl_max, float* feat_s, const float* W1,
@@ -601,8 +603,30 @@ __device__ __forceinline__ bool warp_draft_epilogue(const SoftmaxState& st, unsi
     }
     const float C = warp_halt_classifier(x, feat_s, W1, b1, w2, b2, Hc, lane);
     bool goes_on = false;
+    const bool halt = (C < tau) || (n_drafted >= sl_max);
+    if (o.verdicts) {   // one of several steps of this launch
+        if (!o.write) return false;
+        const int s = n_drafted - o.chain.step, seq = b - s * o.chain.B;
+        const bool last = s + 1 == o.chain.group;
+        const bool stop = o.chain.sl_forced ? n_drafted >= o.chain.sl_forced[seq] : halt;
+        bool taken = false;
+        if (lane == 0) {
+            taken = s == 0 && last ? true : group_step_taken(o.verdicts, s, last, stop, o.status);
+            if (taken) {
+                o.token[b] = key_index(key);
+                o.conf[b] = C;
+                o.halt[b] = halt ? 1 : 0;
+                if (stop || last) {
+                    __stcg(o.chain.sl + seq, n_drafted);
+                    __stcg(o.chain.alive + seq, static_cast<uint8_t>(stop ? 0 : 1));
+                }
+            }
+        }
+        taken = __shfl_sync(kFullMask, taken, 0);
+        if (taken && o.feats && lane < kNFeat) o.feats[(size_t)b * kNFeat + lane] = x;
+        return taken && !stop;
+    }
     if (lane == 0 && o.write) {
-        const bool halt = (C < tau) || (n_drafted >= sl_max);
         o.token[b] = key_index(key);
         o.conf[b] = C;
         o.halt[b] = halt ? 1 : 0;

@@ -350,3 +350,73 @@ def test_iteration_full_size_ragged_batch(oracle):
                if k != "row_off"}
         one["row_off"] = np.array([0, forced[b] + 1])
         check_iteration(oracle, one, ref, W_T, H_T[b:b + 1], wl.tau, S, ids[b:b + 1])
+
+
+def _draft_loop(ctx, W, h, pos0, clf, tau, S, forced=None, copies=1):
+    B = h.shape[1]
+    new = lambda *s, v, t: torch.full(s, v, dtype=t, device="cuda")
+    out = dict(token=new(S, B, v=-7, t=torch.int32), conf=new(S, B, v=-7.0, t=torch.float32),
+               halt=new(S, B, v=77, t=torch.uint8), feats=new(S, B, binding.NFEAT, v=-7.0, t=torch.float32),
+               sl=new(B, v=-7, t=torch.int32))
+    Wd = W.cuda() if copies == 1 else torch.stack([W] * copies).cuda()
+    ctx.draft_loop(Wd, h.cuda(), torch.as_tensor(pos0).cuda(), clf, tau, S, out["token"], out["conf"], out["halt"],
+                   out["sl"], feats=out["feats"], w_step_stride=0 if copies == 1 else W.numel() * 2,
+                   sl_forced=None if forced is None else torch.as_tensor(forced, dtype=torch.int32).cuda())
+    torch.cuda.synchronize()
+    return {k: v.cpu().numpy() for k, v in out.items()}
+
+
+def _check_draft_phase(got, ref, S):
+    for b in range(ref.sl.shape[0]):
+        n = int(ref.sl[b])
+        assert got["sl"][b] == n, f"seq {b}"
+        for i in range(n):
+            if ref.gap_D[i, b] >= GAP_EXEMPT:
+                assert got["token"][i, b] == ref.token[i, b], f"seq {b} step {i}"
+            assert abs(float(got["conf"][i, b]) - ref.conf[i, b]) <= PROB_TOL
+            assert got["halt"][i, b] == ref.halt[i, b], f"seq {b} step {i}"
+            np.testing.assert_allclose(got["feats"][i, b], ref.feats[i, b], rtol=0, atol=PROB_TOL)
+        assert np.all(got["token"][n:, b] == -7) and np.all(got["halt"][n:, b] == 77)
+        assert np.all(got["conf"][n:, b] == -7.0) and np.all(got["feats"][n:, b] == -7.0)
+
+
+# Steps share a launch: all of them, uneven shares, as many rows as a tile has, one more than a launch takes, and scratch for
+# one or three steps only.  A sequence's hidden states past its look-ahead are not numbers: nothing of them may be seen.
+@pytest.mark.parametrize("V,B,S,scratch", [(2000, 1, 16, 16), (700, 8, 16, 16), (1200, 9, 15, 15), (2000, 20, 9, 9),
+                                           (1500, 64, 5, 5), (300, 128, 3, 3), (300, 129, 3, 3), (30, 3, 40, 40),
+                                           (2000, 12, 10, 1), (2000, 12, 10, 3), (2000, 2, 10, 1), (2000, 2, 10, 3),
+                                           (900, 40, 16, 16), (5000, 256, 4, 4)])
+def test_steps_that_share_a_launch(oracle, V, B, S, scratch):
+    d = 72
+    W, h = inputs.lm_head(V, d, seed=V + B, std=0.3), inputs.hidden(S * B, d, seed=B + S).view(S, B, d)
+    pos0 = (np.arange(B, dtype=np.int32) * 7) % (S + 2)
+    params = position_clf(cut=float(S))                     # look-aheads S - pos0 + 1, at least one
+    ctx = binding.Context(V, d, 8, max_batch=B, max_rows=B * scratch, clf_hidden=8)
+    forced = (np.arange(B, dtype=np.int32) * 5) % (S + 3) + 1
+    for f in (None, forced, None):
+        sl = np.minimum(forced, S) if f is not None else np.minimum(np.maximum(S - pos0 + 1, 1), S)
+        poisoned = h.clone()
+        for b in range(B):
+            poisoned[sl[b]:, b] = float("nan")
+        got = _draft_loop(ctx, W, poisoned, pos0, to_gpu_clf(params), 0.5, S, forced=f)
+        ref = oracle.draft_loop(_bits(W), _bits(h), pos0, to_oracle_clf(oracle, params), 0.5, S, sl_forced=f, nthreads=8)
+        np.testing.assert_array_equal(ref.sl, sl)
+        _check_draft_phase(got, ref, S)
+    assert ctx.device_status() == 0
+    ctx.close()
+
+
+@pytest.mark.parametrize("B", [1, 2, 4])
+@pytest.mark.parametrize("V", [1, 9, 48, 1000])
+def test_steps_with_a_head_each(oracle, V, B):
+    """The persistent draft-phase kernel, which serves the calls whose steps read different copies of the head."""
+    d, S = 16, 4
+    W, h = inputs.lm_head(V, d, seed=500 + V, std=0.3), inputs.hidden(S * B, d, seed=B).view(S, B, d)
+    pos0 = (np.arange(B, dtype=np.int32) * 2 + 3) % 8
+    params = position_clf(cut=6.0)
+    ctx = binding.Context(V, d, 8, max_batch=B, max_rows=B * (S + 1), clf_hidden=8)
+    got = _draft_loop(ctx, W, h, pos0, to_gpu_clf(params), 0.5, S, copies=S)
+    ref = oracle.draft_loop(_bits(W), _bits(h), pos0, to_oracle_clf(oracle, params), 0.5, S, nthreads=4)
+    _check_draft_phase(got, ref, S)
+    assert ctx.device_status() == 0
+    ctx.close()
