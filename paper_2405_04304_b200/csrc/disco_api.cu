@@ -222,17 +222,41 @@ bool encode_bf16_2d(const disco_ctx* c, CUtensorMap* map, const void* base, int 
 }
 
 
+// Clusters of two CTAs, and programmatic stream serialization where that is on.
+int launch_attributes(const disco_ctx* c, bool pair, cudaLaunchAttribute (&attr)[2]) {
+    int n = 0;
+    if (pair) {
+        attr[n].id = cudaLaunchAttributeClusterDimension;
+        attr[n].val.clusterDim.x = 2;
+        attr[n].val.clusterDim.y = attr[n].val.clusterDim.z = 1;
+        ++n;
+    }
+    if (c->pdl) {
+        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[n].val.programmaticStreamSerializationAllowed = 1;
+        ++n;
+    }
+    return n;
+}
+
+// Verification by pairs of CTAs: half of the LM-head traffic from L2, but the rows are cut into tiles of 256.  Launches one after
+// the other, 32000 x 1024 / 2048 / 5120 (us, two tiles of hidden rows per CTA or one -> pairs): 250 rows 22.2 / 35.4 / 80.0 -> 20.3 /
+// 32.0 / 79.3, 300 rows 25.3 / 46.7 / 124 -> 32.0 / 55.2 / 130, 450 rows 33.9 / 60.4 / 122 -> 32.4 / 53.3 / 114, 600 rows 39.9 / 77.1 /
+// 165 -> 38.7 / 80.1 / 175; 2432 rows of 49152 x 6144: 3 % of the iteration.  So: no odd number of 128 rows unless it is large.
+bool umma_in_pairs(int R, int d) {
+    const int tiles = (R + 127) / 128;
+    return d >= 1024 && (tiles % 2 == 0 || tiles >= 9);
+}
+
 // Launch the tcgen05 verification kernel for R hidden rows of width d against the LM head W [V, d].
 int launch_umma(disco_ctx* c, const void* W, const void* H, int d, int R, const UmmaParams* fused, cudaStream_t st,
-                const int32_t* dev_R = nullptr) {
+                const int32_t* dev_R = nullptr, int likely_R = 0) {
     UmmaParams p{};
     if (fused) p = *fused;  // verification finished by the main kernel's last CTA
     p.V = c->V;
     p.d = d;
     p.R = R;
-    p.t = VerifyTiling::make(R, c->V, d, c->sm_count);
     p.dev_R = dev_R;
-    p.box_rows = dev_R ? 256 : p.t.TRN;   // (the kernel derives the tiling from the device-side row count)
     // Vocabulary on the TMEM lanes (umma_tail.cuh): few rows, and the first rows beyond one tile of 128, where the other form
     // multiplies by 256.  In between and beyond it has no fewer multiplications and the dearer epilogue.  (Launches one after
     // the other at the power limit, 32000 x 5120, 34 / 64 / 96 / 130 / 160 / 192 rows: 61.4 -> 56.2, 61.6 -> 58.2, 63.1 -> 62.5,
@@ -251,32 +275,36 @@ int launch_umma(disco_ctx* c, const void* W, const void* H, int d, int R, const 
     const bool beyond = R > 128 && R <= 160 && (head_bytes >= (size_t)45 << 20 || c->path == 2);
     const bool lanes = !dev_R && (few || beyond);
     const bool wide = lanes && R > kUmmaLaneRows;
-    p.a_rows = lanes ? (R + 15) / 16 * 16 : p.t.MT > 1 ? 128 : (R + 7) / 8 * 8;
-    p.pairs = !lanes && (dev_R || p.t.GS == 2);
+    // (a count in device memory: only where it is likely to be large, whatever its parity)
+    const bool pair = !lanes && R > 128 && VerifyTiling::pairs_possible(R, c->sm_count) &&
+                      (dev_R ? d >= 1024 && likely_R > 1024 : umma_in_pairs(R, d));
+    p.t = pair ? VerifyTiling::make_pairs(R, c->V, d, c->sm_count) : VerifyTiling::make(R, c->V, d, c->sm_count);
+    // (with the row count in device memory the kernel derives the tiling)
+    p.box_rows = (dev_R ? 256 : p.t.TRN) / (pair ? 2 : 1);
+    p.a_rows = lanes ? (R + 15) / 16 * 16 : pair || p.t.MT > 1 ? 128 : (R + 7) / 8 * 8;
+    p.a_tiles = !lanes && (dev_R || p.t.GS == 2) ? 2 : 1;
     // The A tile holds a_rows rows.  The MMA still reads 128 rows from its start: what lies behind the tile (other
     // stages of the ring, always inside it) only feeds accumulator lanes nobody reads.
     p.a_bytes = (p.a_rows * 128 + 1023) / 1024 * 1024;
     p.b_bytes = (p.box_rows * 128 + 1023) / 1024 * 1024;
-    p.stages = std::max(2, std::min(kUmmaMaxStages, kUmmaRingBytes / (p.a_bytes * (1 + p.pairs) + p.b_bytes)));
+    p.stages = std::max(2, std::min(kUmmaMaxStages, kUmmaRingBytes / (p.a_bytes * p.a_tiles + p.b_bytes)));
     p.status = c->status;
     p.keys = c->keys;
     CUtensorMap tmap_W, tmap_H;
     if (!encode_bf16_2d(c, &tmap_W, W, c->V, d, p.box_rows) || !encode_bf16_2d(c, &tmap_H, H, R, d, p.a_rows))
         return DISCO_ERR_CUDA;
-    static KernelSetup setup[3];
-    auto kern = wide ? umma_tail_kernel<true, true> : lanes ? umma_tail_kernel<true, false> : umma_tail_kernel<false, false>;
+    static KernelSetup setup[4];
+    auto kern = pair ? umma_tail_kernel<false, false, true> : wide ? umma_tail_kernel<true, true, false> : lanes ? umma_tail_kernel<true, false, false> : umma_tail_kernel<false, false, false>;
     const int smem_bytes = lanes ? kUmmaLaneSmemBytes : kUmmaSmemBytes;
-    if (!raise_smem_limit(c, setup[lanes + wide], kern, (size_t)smem_bytes, nullptr)) return DISCO_ERR_CUDA;
+    if (!raise_smem_limit(c, setup[pair ? 3 : lanes + wide], kern, (size_t)smem_bytes, nullptr)) return DISCO_ERR_CUDA;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)(dev_R ? c->sm_count : p.t.groups * p.t.CN));
+    cfg.gridDim = dim3((unsigned)(dev_R ? (pair ? c->sm_count & ~1 : c->sm_count) : p.t.groups * p.t.CN * (pair ? 2 : 1)));
     cfg.blockDim = dim3(kUmmaThreads);
     cfg.dynamicSmemBytes = (size_t)smem_bytes;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attr[2];
     cfg.attrs = attr;
-    cfg.numAttrs = c->pdl ? 1 : 0;
+    cfg.numAttrs = launch_attributes(c, pair, attr);
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tmap_W, tmap_H, p);
     c->launches += 1;
     return cuda_ok(e, "umma_tail_kernel launch") ? DISCO_OK : DISCO_ERR_CUDA;
@@ -288,6 +316,14 @@ bool draft_batch_possible(const disco_ctx* c, int R) {
     return c->encode_tiled != nullptr && MT <= c->sm_count && c->sm_count / MT <= kDbMaxRecords && c->V < (int)kDbNoIndex;
 }
 
+// Pairs of CTAs that share their vocabulary tiles, where the operands' way from L2 is the bound.  Launches one after the other,
+// 256 / 384 / 512 / 640 / 1000 rows (us, single CTAs -> pairs): 32000 x 768 23.1 / 28.5 / 36.5 / 41 / 58 -> 23.9 / 35.9 / 37.0 / 47 / 60;
+// 32000 x 2048 46.0 / 58.6 / 74.1 / 88.3 / 116 -> 41.8 / 64.5 / 65.7 / 91.1 / 114; 32000 x 5120 99.6 / 133 / 168 / 206 / 263 -> 90.5 / 144 /
+// 130 / 190 / 231.
+bool draft_batch_in_pairs(const disco_ctx* c, int MT, int d) {
+    return d >= 2048 && MT >= 2 && MT != 3 && ((MT + 1) & ~1) <= c->sm_count;
+}
+
 // Launch the batched draft step (STATS: arg-max and statistics only) for R hidden rows of width d against W [V, d].
 template <bool STATS>
 int launch_draft_batch(disco_ctx* c, const void* W, const void* H, int d, int R, float* probs, const DraftFinalParams& f,
@@ -297,6 +333,8 @@ int launch_draft_batch(disco_ctx* c, const void* W, const void* H, int d, int R,
     p.d = d;
     p.R = R;
     p.MT = (R + 127) / 128;
+    const bool pair = draft_batch_in_pairs(c, p.MT, d);
+    if (pair) p.MT = (p.MT + 1) & ~1;
     p.CN = c->sm_count / p.MT;
     // One tile of hidden rows: the LM head arrives slower than the tensor pipe works, so the tiles are small and the
     // epilogue of one runs under the loads of the next.  More tiles of rows: the rows' tile is loaded again for every
@@ -308,12 +346,12 @@ int launch_draft_batch(disco_ctx* c, const void* W, const void* H, int d, int R,
     p.TRN = std::max(16, (p.TR + 15) / 16 * 16);
     p.a_rows = p.MT > 1 ? 128 : std::max(8, (R + 7) / 8 * 8);
     p.a_bytes = (p.a_rows * 128 + 1023) / 1024 * 1024;
-    p.b_bytes = (p.TRN * 128 + 1023) / 1024 * 1024;
+    p.b_bytes = ((pair ? p.TRN / 2 : p.TRN) * 128 + 1023) / 1024 * 1024;
     if ((size_t)R * p.CN > (size_t)128 * c->sm_count || R > c->part_rows) return DISCO_ERR_WORKSPACE;
-    auto kern = umma_draft_batch_kernel<STATS>;
-    static KernelSetup setup;
+    auto kern = pair ? umma_draft_batch_kernel<STATS, true> : umma_draft_batch_kernel<STATS, false>;
+    static KernelSetup setup[2];
     size_t dyn_limit = 0;
-    if (!raise_smem_limit(c, setup, kern, 0, &dyn_limit)) return DISCO_ERR_CUDA;
+    if (!raise_smem_limit(c, setup[pair], kern, 0, &dyn_limit)) return DISCO_ERR_CUDA;
     p.all_finish = R > kDbFinWarps * p.MT * p.CN;
     const int fin_warps = kDbFinWarps + (p.all_finish ? kDbEpiWarps : 0);
     const size_t fixed = 1024 + 512 + kDbXchBytes + (size_t)(fin_warps * kDbFinWords + 128) * 4 +
@@ -328,18 +366,16 @@ int launch_draft_batch(disco_ctx* c, const void* W, const void* H, int d, int R,
     p.set_words = (size_t)c->part_rows * kDbBoundStride;
     p.sync = c->ticket + 48;
     CUtensorMap tmap_W, tmap_H;
-    if (!encode_bf16_2d(c, &tmap_W, W, c->V, d, p.TRN) || !encode_bf16_2d(c, &tmap_H, H, R, d, p.a_rows))
+    if (!encode_bf16_2d(c, &tmap_W, W, c->V, d, pair ? p.TRN / 2 : p.TRN) || !encode_bf16_2d(c, &tmap_H, H, R, d, p.a_rows))
         return DISCO_ERR_CUDA;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(p.MT * p.CN));
     cfg.blockDim = dim3(kDbThreads);
     cfg.dynamicSmemBytes = fixed + p.ring_bytes;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attr[2];
     cfg.attrs = attr;
-    cfg.numAttrs = c->pdl ? 1 : 0;
+    cfg.numAttrs = launch_attributes(c, pair, attr);
     if (layout) *layout = RecordLayout{p.part_rec, kStampedPieces, p.CN, p.TPC * p.TR};
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tmap_W, tmap_H, p, f);
     c->launches += 1;
@@ -783,6 +819,7 @@ int verify_common(disco_ctx* c, const void* W_T, const void* H_T, const int32_t*
     // Fixed-shape rows beyond one tile of 128: the projection is no longer free of charge for the rows that do not
     // count, so they are packed first and the tensor-core kernel tiles for the row count it finds on the device.
     const int32_t* dev_R = nullptr;
+    const int likely_R = pad ? (int)((long long)B * (SL + 3) / 2) : R;   // look-aheads anything from 1 to SL
     if (pad && R > 128) {
         PackParams pk{};
         pk.H = static_cast<const uint16_t*>(H_T);
@@ -817,9 +854,9 @@ int verify_common(disco_ctx* c, const void* W_T, const void* H_T, const int32_t*
         fp.bonus = bonus;
         fp.target_ids = target_ids;
         fp.padded = p.padded;
-        return launch_umma(c, W_T, H_T, c->d_target, R, &fp, st, dev_R);
+        return launch_umma(c, W_T, H_T, c->d_target, R, &fp, st, dev_R, likely_R);
     }
-    int rc = launch_umma(c, W_T, H_T, c->d_target, R, nullptr, st, dev_R);
+    int rc = launch_umma(c, W_T, H_T, c->d_target, R, nullptr, st, dev_R, likely_R);
     if (rc) return rc;
     VerifyFinalParams f{};
     f.keys = c->keys;

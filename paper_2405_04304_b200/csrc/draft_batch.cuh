@@ -388,7 +388,8 @@ __device__ __forceinline__ void db_finish_row(const DraftBatchParams& p, const D
 // main kernel
 // ---------------------------------------------------------------------------------------------
 // STATS: arg-max and soft-max statistics only (f.stats_only == 1), no list of the ten largest.
-template <bool STATS>
+// PAIR: clusters of two CTAs share every vocabulary tile: each loads its own 128 hidden rows and half of the LM-head box.
+template <bool STATS, bool PAIR>
 __global__ void __launch_bounds__(kDbThreads, 1)
 umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_constant__ CUtensorMap tmap_H,
                         const DraftBatchParams p, const DraftFinalParams f) {
@@ -431,7 +432,7 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
         }
         for (int b = 0; b < nbuf; ++b) {
             mbar_init(&tmem_full[b], 1);
-            mbar_init(&tmem_empty[b], kDbEpiWarps);
+            mbar_init(&tmem_empty[b], PAIR ? 2 * kDbEpiWarps : kDbEpiWarps);
         }
         *s_done = 0;
         *s_stamp = 0u;
@@ -442,8 +443,12 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
         prefetch_tensormap(&tmap_H);
     }
     if (warp == 1) {
-        tmem_alloc(tmem_base_s, 512);
-        tmem_relinquish();
+        if constexpr (PAIR) {
+            tmem_alloc_pair(tmem_base_s, 512);
+        } else {
+            tmem_alloc(tmem_base_s, 512);
+            tmem_relinquish();
+        }
     }
     // A step of a draft phase that has ended already needs neither loads nor rehearsals.  The flags are looked at ahead of
     // the dependency wait for that, once for the whole CTA: they may be old and decide nothing else.
@@ -452,10 +457,13 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
         if (lane == 0) *s_look = any ? 1u : 0u;
     }
     tc_fence_before();
-    __syncthreads();
+    if constexpr (PAIR) cluster_sync();    // (both CTAs' barriers are ready)
+    else __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_base_s;
-    const bool looks_live = *s_look != 0u;
+    const bool leader = !PAIR || cluster_rank() == 0;
+    // (the CTAs of a pair request the same stages ahead, so they go by the leader's look)
+    const bool looks_live = (leader ? *s_look : ld_cluster_u32(leader_addr(smem_addr(s_look)))) != 0u;
     // Does the step take place?  Read once per CTA, by the MMA issuer right after the dependency wait (a finishing warp of
     // this launch may clear flags once this CTA's records are out), and told to the others here.
     auto step_live = [&]() { return !chained || cold_smem_word(s_live, p.status) == 1u; };
@@ -463,7 +471,8 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
     if (warp == 0) {
         // ------------------------------ producer ------------------------------
         const int total = tiles * KB;
-        const uint32_t w_bytes = (uint32_t)p.TRN * 128u, h_bytes = (uint32_t)p.a_rows * 128u;
+        // (what a stage's barrier, the leader's, counts: the boxes of both CTAs)
+        const uint32_t w_bytes = (uint32_t)p.TRN * 128u, h_bytes = (uint32_t)p.a_rows * (PAIR ? 256u : 128u);
         // The LM head is never written by this library: its first stages are requested before the dependency wait.
         const int pre = looks_live ? min(p.stages, total) : 0;
         // Every CTA reads the same hidden rows.  Each starts at another k-block, so that they do not all ask the same few
@@ -472,7 +481,13 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
         // A single thread issues everything: running addresses and counters, as few instructions per stage as possible.
         const uint32_t full0 = smem_addr(full), empty0 = smem_addr(empty), a0 = smem_addr(a_tiles), b0 = smem_addr(b_tiles);
         const int k_end = KB * kUmmaBK, k_first = rot * kUmmaBK, h_row = m_tile * 128;
-        int k = k_first, v0 = v_first, left = KB;      // the next stage to request: k, vocabulary row, k-blocks left of the tile
+        const int v_own = v_first + (leader ? 0 : p.TRN / 2);
+        const uint32_t count0 = PAIR ? leader_addr(full0) : full0;
+        auto load = [&](uint32_t dst, const CUtensorMap* map, int c0, int c1, int slot) {
+            if constexpr (PAIR) tma_load_2d_pair(dst, map, c0, c1, count0 + slot * 8);
+            else tma_load_2d(dst, map, c0, c1, count0 + slot * 8);
+        };
+        int k = k_first, v0 = v_own, left = KB;        // the next stage to request: k, vocabulary row, k-blocks left of the tile
         auto advance = [&]() {
             k += kUmmaBK;
             if (k == k_end) k = 0;
@@ -483,35 +498,34 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
         };
         if (elect_one()) {
             for (int n = 0; n < pre; ++n, advance()) {
-                mbar_expect_tx(full0 + n * 8, w_bytes);
-                tma_load_2d(b0 + n * p.b_bytes, &tmap_W, k, v0, full0 + n * 8);
+                if (leader) mbar_expect_tx(full0 + n * 8, w_bytes);
+                load(b0 + n * p.b_bytes, &tmap_W, k, v0, n);
             }
         }
         asm volatile("griddepcontrol.wait;" ::: "memory");
         const bool live = step_live();
         if (!live) {
-            if (elect_one()) {
+            if (leader && elect_one()) {
                 for (int n = 0; n < pre; ++n) mbar_arrive(&full[n]);
                 for (int n = 0; n < pre; ++n) mbar_wait(&full[n], 0, p.status);   // nothing may still be landing at exit
             }
         } else if (elect_one()) {
             int kh = k_first;
             for (int n = 0; n < pre; ++n) {
-                mbar_arrive_expect_tx(full0 + n * 8, h_bytes);
-                tma_load_2d(a0 + n * p.a_bytes, &tmap_H, kh, h_row, full0 + n * 8);
+                if (leader) mbar_arrive_expect_tx(full0 + n * 8, h_bytes);
+                load(a0 + n * p.a_bytes, &tmap_H, kh, h_row, n);
                 kh += kUmmaBK;
                 if (kh == k_end) kh = 0;
             }
             int stage = pre == p.stages ? 0 : pre, phase = pre == p.stages ? 1 : 0;
-            k = k_first, v0 = v_first, left = KB;      // (the elected thread need not be the one of before)
+            k = k_first, v0 = v_own, left = KB;        // (the elected thread need not be the one of before)
             for (int n = 0; n < pre; ++n) advance();
             uint32_t at_a = a0 + stage * p.a_bytes, at_b = b0 + stage * p.b_bytes;
             for (int n = pre; n < total; ++n, advance()) {
-                const uint32_t bar = full0 + stage * 8;
                 mbar_wait(empty0 + stage * 8, phase ^ 1, p.status);
-                mbar_arrive_expect_tx(bar, w_bytes + h_bytes);
-                tma_load_2d(at_b, &tmap_W, k, v0, bar);
-                tma_load_2d(at_a, &tmap_H, k, h_row, bar);
+                if (leader) mbar_arrive_expect_tx(full0 + stage * 8, w_bytes + h_bytes);
+                load(at_b, &tmap_W, k, v0, stage);
+                load(at_a, &tmap_H, k, h_row, stage);
                 at_a += p.a_bytes;
                 at_b += p.b_bytes;
                 if (++stage == p.stages) {
@@ -519,6 +533,12 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
                     phase ^= 1;
                     at_a = a0;
                     at_b = b0;
+                }
+            }
+            if constexpr (PAIR) {   // the leader's arrivals at this CTA's barriers are all in before it leaves
+                for (int n = 0; n < p.stages; ++n) {
+                    mbar_wait(empty0 + stage * 8, phase ^ 1, p.status);
+                    if (++stage == p.stages) stage = 0, phase ^= 1;
                 }
             }
         }
@@ -530,8 +550,8 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
             live = chain_any_live(f.chain, f.chain.B, lane);
             if (lane == 0) *reinterpret_cast<volatile uint32_t*>(s_live) = live ? 1u : 2u;
         }
-        if (live && elect_one()) {
-            const uint32_t idesc = umma_idesc(p.TRN);
+        if (live && leader && elect_one()) {
+            const uint32_t idesc = umma_idesc(p.TRN, PAIR ? 256 : 128);
             const uint32_t full0 = smem_addr(full), empty0 = smem_addr(empty);
             // Up to eight rows: the A operand is the one 8-row box read 16 times over (zero stride between the 8-row groups
             // of the descriptor).  More: the MMA reads 128 rows from the start of the stage; what lies behind the box
@@ -543,16 +563,20 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
             int stage = 0, phase = 0;
             for (int t = 0; t < tiles; ++t) {
                 const int buf = t % nbuf;
-                mbar_wait(&tmem_empty[buf], ((t / nbuf) & 1) ^ 1, p.status);
+                if constexpr (PAIR) mbar_wait_cluster(smem_addr(&tmem_empty[buf]), ((t / nbuf) & 1) ^ 1, p.status);
+                else mbar_wait(&tmem_empty[buf], ((t / nbuf) & 1) ^ 1, p.status);
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + buf * buf_cols;
                 for (int kb = 0; kb < KB; ++kb) {
                     mbar_wait(full0 + stage * 8, phase, p.status);
                     tc_fence_after();
 #pragma unroll
-                    for (int k = 0; k < kUmmaBK / 16; ++k)  // 16 k-elements = 32 bytes = 2 descriptor units
-                        tc_mma_bf16(d_tmem, a_desc + 2 * k, b_desc + 2 * k, idesc, (kb | k) != 0);
-                    tc_commit(empty0 + stage * 8);
+                    for (int k = 0; k < kUmmaBK / 16; ++k) {  // 16 k-elements = 32 bytes = 2 descriptor units
+                        if constexpr (PAIR) tc_mma_bf16_pair(d_tmem, a_desc + 2 * k, b_desc + 2 * k, idesc, (kb | k) != 0);
+                        else tc_mma_bf16(d_tmem, a_desc + 2 * k, b_desc + 2 * k, idesc, (kb | k) != 0);
+                    }
+                    if constexpr (PAIR) tc_commit_pair(empty0 + stage * 8);
+                    else tc_commit(empty0 + stage * 8);
                     a_desc += a_step;
                     b_desc += b_step;
                     if (++stage == p.stages) {
@@ -562,7 +586,8 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
                         b_desc = b0;
                     }
                 }
-                tc_commit(&tmem_full[buf]);
+                if constexpr (PAIR) tc_commit_pair(smem_addr(&tmem_full[buf]));
+                else tc_commit(&tmem_full[buf]);
             }
         }
     }
@@ -830,7 +855,10 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
                     // this tile's accumulator columns are free again
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(&tmem_empty[tc % nbuf]);
+                    if (lane == 0) {
+                        if constexpr (PAIR) mbar_arrive_cluster(leader_addr(smem_addr(&tmem_empty[tc % nbuf])));
+                        else mbar_arrive(&tmem_empty[tc % nbuf]);
+                    }
                 }
             }
 
@@ -964,10 +992,13 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
     }
 
     tc_fence_before();
-    __syncthreads();
+    // (the CTAs of a pair arrive at each other's barriers: neither leaves before the other)
+    if constexpr (PAIR) cluster_sync();
+    else __syncthreads();
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem_base, 512);
+        if constexpr (PAIR) tmem_dealloc_pair(tmem_base, 512);
+        else tmem_dealloc(tmem_base, 512);
     }
 }
 

@@ -70,6 +70,31 @@ struct VerifyTiling {
         t.TRN = (t.TR + 15) / 16 * 16;
         return t;
     }
+    // Pairs of CTAs (cta_group::2): MT counts tiles of 256 hidden rows, GS of them (1 or 2) to a pair, CN pairs per group.  Of
+    // the two the cheaper one by the longer of tensor time and operand traffic (cycles per 64 k; an SM takes in about 61 bytes
+    // a cycle), and by the epilogue that GS = 2 does not hide.
+    __host__ __device__ static bool pairs_possible(int R, int grid) { return (R + 511) / 512 <= grid / 2; }
+    __host__ __device__ static VerifyTiling make_pairs(int R, int V, int d, int grid) {
+        VerifyTiling best{};
+        long long least = 0;
+        const int KB = (d + 63) / 64;
+        for (int gs = 1; gs <= 2; ++gs) {
+            VerifyTiling t;
+            t.MT = (R + 255) / 256;
+            t.GS = gs;
+            t.groups = (t.MT + gs - 1) / gs;
+            t.CN = grid / 2 / t.groups;
+            if (t.CN == 0) continue;
+            t.TPC = (V + 256 * t.CN - 1) / (256 * t.CN);
+            t.TR = (V + t.CN * t.TPC - 1) / (t.CN * t.TPC);
+            t.TRN = (t.TR + 15) / 16 * 16;
+            const int size = gs < t.MT ? gs : t.MT;
+            const int mma = 2 * t.TRN * size, feed = (size * 128 + t.TRN / 2) * 21 / 10;
+            const long long cost = (long long)t.TPC * ((long long)KB * (mma > feed ? mma : feed) + (size == 2 ? 1500 : 0));
+            if (best.CN == 0 || cost < least) best = t, least = cost;
+        }
+        return best;
+    }
 };
 
 struct UmmaParams {
@@ -79,7 +104,7 @@ struct UmmaParams {
     int a_rows;    // rows of the H box (multiple of 8, <= 128)
     int stages;    // ring depth (<= kUmmaMaxStages); stage s holds one or two A tiles of a_bytes and a B tile of b_bytes
     int a_bytes, b_bytes;  // multiples of 1024
-    int pairs;     // 1: stages have room for two A tiles
+    int a_tiles;   // A tiles a stage has room for
     int* status;
     unsigned long long* keys;  // [R]
     // verification finished inside this kernel by the last CTA (few sequences only)
@@ -143,6 +168,62 @@ __device__ __forceinline__ void tc_mma_bf16(uint32_t d_tmem, uint64_t a_desc, ui
         "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
+// ---- two CTAs of a cluster as one (cta_group::2): 256 rows of the A operand, 128 in each CTA, and a B operand of which each
+// CTA holds half; the even CTA (the leader) issues the MMAs for both ----
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm("mov.u32 %0, %cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+// The leader's word at the place of this CTA's one.
+__device__ __forceinline__ uint32_t leader_addr(uint32_t smem) {
+    uint32_t a;
+    asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(a) : "r"(smem));
+    return a;
+}
+__device__ __forceinline__ uint32_t ld_cluster_u32(uint32_t addr) {
+    uint32_t v;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+// A load into this CTA's shared memory that is counted on the leader's barrier.
+__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst_smem, const CUtensorMap* tmap, int c0, int c1, uint32_t leader_bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
+            dst_smem),
+        "l"(tmap), "r"(c0), "r"(c1), "r"(leader_bar)
+        : "memory");
+}
+__device__ __forceinline__ void tmem_alloc_pair(uint32_t* dst_smem, uint32_t ncols) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(dst_smem)), "r"(ncols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+}
+// Arrives at the barrier of this address in both CTAs once the MMAs issued so far are done.
+__device__ __forceinline__ void tc_commit_pair(uint32_t bar) {
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+                 "h"(static_cast<uint16_t>(3))
+                 : "memory");
+}
+__device__ __forceinline__ void tc_mma_bf16_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                                 uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
 // 32 lanes x 32 consecutive fp32 columns -> 32 registers per thread (the wait names the registers, so that the compiler
 // moves nothing that looks at them ahead of it)
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
@@ -183,9 +264,9 @@ __device__ __forceinline__ uint64_t umma_smem_desc(const void* tile) {
     desc |= static_cast<uint64_t>(2) << 61;                            // 128-byte swizzle
     return desc;
 }
-// Instruction descriptor: bf16 x bf16 -> fp32, both operands K-major, M = 128, N = n.
-__device__ __forceinline__ uint32_t umma_idesc(int n) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(n >> 3) << 17) | ((128u >> 4) << 24);
+// Instruction descriptor: bf16 x bf16 -> fp32, both operands K-major, M = m (256 for a pair of CTAs), N = n.
+__device__ __forceinline__ uint32_t umma_idesc(int n, uint32_t m = 128) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(n >> 3) << 17) | ((m >> 4) << 24);
 }
 
 // Draft step, second phase: one warp per sequence merges the per-CTA partial records, forms the
@@ -225,14 +306,16 @@ struct DraftFinalParams {
 // CTAs read as one B operand of 16 or 32 rows.
 // WIDE: the same with up to kUmmaWideRows hidden rows; the warp finds the largest logit of a column at once, and the running
 // keys live in shared memory.  130 rows, 32000 x 2048: 36.2 -> 32.3 us; 20.5 us at the measured copy bandwidth.
-template <bool VL, bool WIDE>
+// PAIR: clusters of two CTAs with 256 hidden rows to a tile (VerifyTiling::make_pairs): each loads its own 128 hidden rows and half
+// of the LM-head box, the even one issues the MMAs of both.
+template <bool VL, bool WIDE, bool PAIR>
 __global__ void __launch_bounds__(kUmmaThreads, 1)
 umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_constant__ CUtensorMap tmap_H,
                  const UmmaParams p) {
     extern __shared__ uint8_t smem_dyn[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023));
     uint8_t* a_tiles = smem;
-    uint8_t* b_tiles = smem + p.stages * p.a_bytes * (1 + p.pairs);
+    uint8_t* b_tiles = smem + p.stages * p.a_bytes * p.a_tiles;
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + kUmmaRingBytes);
     uint64_t* empty = full + kUmmaMaxStages;
     uint64_t* tmem_full = empty + kUmmaMaxStages;
@@ -252,12 +335,17 @@ umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_consta
     if (p.dev_R) {
         asm volatile("griddepcontrol.wait;" ::: "memory");   // the count is the predecessor's output
         R = min(max(__ldcg(p.dev_R), 1), p.R);
-        tl = VerifyTiling::make(R, p.V, p.d, (int)gridDim.x);
+        tl = PAIR ? VerifyTiling::make_pairs(R, p.V, p.d, (int)gridDim.x) : VerifyTiling::make(R, p.V, p.d, (int)gridDim.x);
     }
+    const int rank = PAIR ? (int)cluster_rank() : 0;
+    const bool leader = rank == 0;
+    const int cta = PAIR ? (int)blockIdx.x >> 1 : (int)blockIdx.x;      // (or pair of CTAs)
     // this CTA: `size` tiles of hidden rows from m_tile on, vocabulary rows v_begin .. v_end - 1 in tiles of TR
-    const int m_tile = (int)blockIdx.x % tl.groups * tl.GS;
+    const int m_tile = cta % tl.groups * tl.GS;
     const int size = VL ? 1 : min(tl.GS, tl.MT - m_tile);
-    const int slot = (int)blockIdx.x / tl.groups;
+    const int slot = cta / tl.groups;
+    constexpr int kTileStep = PAIR ? 256 : 128;
+    const int h_row = m_tile * kTileStep + rank * 128;                  // the first hidden row of this CTA; its second tile: kTileStep on
     const int v_begin = slot * tl.TPC * tl.TR;
     const int v_end = min(p.V, v_begin + tl.TPC * tl.TR);
 
@@ -268,18 +356,23 @@ umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_consta
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&tmem_full[b], 1);
-            mbar_init(&tmem_empty[b], kUmmaEpiWarps);
+            mbar_init(&tmem_empty[b], PAIR ? 2 * kUmmaEpiWarps : kUmmaEpiWarps);
         }
         fence_mbar_init();
         prefetch_tensormap(&tmap_W);
         prefetch_tensormap(&tmap_H);
     }
     if (warp == 1) {
-        tmem_alloc(tmem_base_s, 512);
-        tmem_relinquish();
+        if constexpr (PAIR) {
+            tmem_alloc_pair(tmem_base_s, 512);
+        } else {
+            tmem_alloc(tmem_base_s, 512);
+            tmem_relinquish();
+        }
     }
     tc_fence_before();
-    __syncthreads();
+    if constexpr (PAIR) cluster_sync();
+    else __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_base_s;
 
@@ -294,33 +387,38 @@ umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_consta
             // A single thread: running addresses and counters, as few instructions per stage as possible.
             const uint32_t full0 = smem_addr(full), empty0 = smem_addr(empty), a0 = smem_addr(a_tiles), b0 = smem_addr(b_tiles);
             const uint32_t a_box = (uint32_t)p.a_rows * 128u, w_box = (uint32_t)p.box_rows * 128u;   // bytes of the two boxes
-            const uint32_t a_step = (uint32_t)p.a_bytes * (1 + p.pairs);
+            const uint32_t a_step = (uint32_t)p.a_bytes * p.a_tiles;
             const int k_end = KB * kUmmaBK;
+            // (a pair's loads are counted on the leader's barriers)
+            const uint32_t count0 = PAIR ? leader_addr(full0) : full0, expected = (PAIR ? 2 : 1) * (w_box + size * a_box);
+            const int v_half = PAIR ? rank * (tl.TRN / 2) : 0;
+            auto load = [&](uint32_t dst, const CUtensorMap* map, int c0, int c1, int slot) {
+                if constexpr (PAIR) tma_load_2d_pair(dst, map, c0, c1, count0 + slot * 8);
+                else tma_load_2d(dst, map, c0, c1, count0 + slot * 8);
+            };
             // The LM head is never written by this library: its first tiles are requested before the
             // dependency wait, the hidden-state tiles of the same stages right after it.
-            const int h_row = m_tile * 128;
             int v0 = v_begin;
             const int pre = v0 < v_end ? min(p.stages, KB) : 0;
             for (int n = 0; n < pre; ++n) {
-                mbar_arrive_expect_tx(full0 + n * 8, w_box + size * a_box);
-                tma_load_2d(b0 + n * p.b_bytes, &tmap_W, n * kUmmaBK, v0, full0 + n * 8);
+                if (leader) mbar_arrive_expect_tx(full0 + n * 8, expected);
+                load(b0 + n * p.b_bytes, &tmap_W, n * kUmmaBK, v0 + v_half, n);
             }
             asm volatile("griddepcontrol.wait;" ::: "memory");
             for (int n = 0; n < pre; ++n) {
-                tma_load_2d(a0 + n * a_step, &tmap_H, n * kUmmaBK, h_row, full0 + n * 8);
-                if (size == 2) tma_load_2d(a0 + n * a_step + p.a_bytes, &tmap_H, n * kUmmaBK, h_row + 128, full0 + n * 8);
+                load(a0 + n * a_step, &tmap_H, n * kUmmaBK, h_row, n);
+                if (size == 2) load(a0 + n * a_step + p.a_bytes, &tmap_H, n * kUmmaBK, h_row + kTileStep, n);
             }
             int stage = pre == p.stages ? 0 : pre, phase = pre == p.stages ? 1 : 0;
             int k = pre * kUmmaBK;
             uint32_t at_a = a0 + stage * a_step, at_b = b0 + stage * p.b_bytes;
             for (; v0 < v_end; v0 += tl.TR, k = 0) {
                 for (; k < k_end; k += kUmmaBK) {
-                    const uint32_t bar = full0 + stage * 8;
                     mbar_wait(empty0 + stage * 8, phase ^ 1, p.status);
-                    mbar_arrive_expect_tx(bar, w_box + size * a_box);
-                    tma_load_2d(at_b, &tmap_W, k, v0, bar);
-                    tma_load_2d(at_a, &tmap_H, k, h_row, bar);
-                    if (size == 2) tma_load_2d(at_a + p.a_bytes, &tmap_H, k, h_row + 128, bar);
+                    if (leader) mbar_arrive_expect_tx(full0 + stage * 8, expected);
+                    load(at_b, &tmap_W, k, v0 + v_half, stage);
+                    load(at_a, &tmap_H, k, h_row, stage);
+                    if (size == 2) load(at_a + p.a_bytes, &tmap_H, k, h_row + kTileStep, stage);
                     at_a += a_step;
                     at_b += p.b_bytes;
                     if (++stage == p.stages) {
@@ -331,15 +429,29 @@ umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_consta
                     }
                 }
             }
+            if constexpr (PAIR) {   // the leader's arrivals at this CTA's barriers are all in before it leaves
+                for (int n = 0; n < p.stages; ++n) {
+                    mbar_wait(empty0 + stage * 8, phase ^ 1, p.status);
+                    if (++stage == p.stages) stage = 0, phase ^= 1;
+                }
+            }
         }
     } else if (warp == 1) {
         // ------------------------------ MMA issuer ------------------------------
-        if (live && elect_one()) {
-            const uint32_t idesc = umma_idesc(VL ? p.a_rows : tl.TRN);
+        if (live && leader && elect_one()) {
+            const uint32_t idesc = umma_idesc(VL ? p.a_rows : tl.TRN, PAIR ? 256 : 128);
+            auto mma = [&](uint32_t d, uint64_t a, uint64_t b, uint32_t accumulate) {
+                if constexpr (PAIR) tc_mma_bf16_pair(d, a, b, idesc, accumulate);
+                else tc_mma_bf16(d, a, b, idesc, accumulate);
+            };
+            auto commit = [&](uint32_t bar) {
+                if constexpr (PAIR) tc_commit_pair(bar);
+                else tc_commit(bar);
+            };
             const bool upper = tl.TRN > 128;   // (VL)
             const uint32_t full0 = smem_addr(full), empty0 = smem_addr(empty);
             const uint64_t a0 = umma_smem_desc(a_tiles), b0 = umma_smem_desc(b_tiles);
-            const uint32_t a_half = (uint32_t)p.a_bytes >> 4, a_step = a_half * (1 + p.pairs), b_step = (uint32_t)p.b_bytes >> 4;   // descriptor units
+            const uint32_t a_half = (uint32_t)p.a_bytes >> 4, a_step = a_half * p.a_tiles, b_step = (uint32_t)p.b_bytes >> 4;   // descriptor units
             uint64_t a_desc = a0, b_desc = b0;
             int stage = 0, phase = 0;
             // Two tiles of hidden rows use an accumulator each, one alternates between the two.
@@ -348,7 +460,10 @@ umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_consta
                 const bool alternate = VL ? lane_bufs == 2 : size == 1;
                 const int first = alternate ? it & 1 : 0;
                 const uint32_t parity = (alternate ? it >> 1 : it) & 1;
-                for (int j = 0; j < size; ++j) mbar_wait(&tmem_empty[first + j], parity ^ 1u, p.status);
+                for (int j = 0; j < size; ++j) {
+                    if constexpr (PAIR) mbar_wait_cluster(smem_addr(&tmem_empty[first + j]), parity ^ 1u, p.status);
+                    else mbar_wait(&tmem_empty[first + j], parity ^ 1u, p.status);
+                }
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + first * (VL ? 2 * lane_cols : 256);
                 for (int kb = 0; kb < KB; ++kb) {
@@ -366,14 +481,14 @@ umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_consta
                     } else {
 #pragma unroll
                         for (int k = 0; k < kUmmaBK / 16; ++k)  // 16 k-elements = 32 bytes = 2 descriptor units
-                            tc_mma_bf16(d_tmem, a_desc + 2 * k, b_desc + 2 * k, idesc, (kb | k) != 0);
+                            mma(d_tmem, a_desc + 2 * k, b_desc + 2 * k, (kb | k) != 0);
                     }
                     if (!VL && size == 2) {
 #pragma unroll
                         for (int k = 0; k < kUmmaBK / 16; ++k)
-                            tc_mma_bf16(d_tmem + 256, a_desc + a_half + 2 * k, b_desc + 2 * k, idesc, (kb | k) != 0);
+                            mma(d_tmem + 256, a_desc + a_half + 2 * k, b_desc + 2 * k, (kb | k) != 0);
                     }
-                    tc_commit(empty0 + stage * 8);
+                    commit(empty0 + stage * 8);
                     a_desc += a_step;
                     b_desc += b_step;
                     if (++stage == p.stages) {
@@ -383,7 +498,7 @@ umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_consta
                         b_desc = b0;
                     }
                 }
-                for (int j = 0; j < size; ++j) tc_commit(&tmem_full[first + j]);
+                for (int j = 0; j < size; ++j) commit(smem_addr(&tmem_full[first + j]));
             }
         }
     } else if (live) {
@@ -498,7 +613,7 @@ umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_consta
                     const int b = size == 2 ? j : it & 1;
                     mbar_wait(&tmem_full[b], (size == 2 ? it : it >> 1) & 1, p.status);
                     tc_fence_after();
-                    if ((m_tile + j) * 128 + quad * 32 < R) {
+                    if (h_row + j * kTileStep + quad * 32 < R) {
                         for (int c = c_lo; c < c_hi; ++c) {
                             float z[32];
                             tmem_ld32(tmem_base + b * 256 + c * 32 + (static_cast<uint32_t>(quad * 32) << 16), z);
@@ -526,13 +641,16 @@ umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_consta
                     }
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(&tmem_empty[b]);
+                    if (lane == 0) {
+                        if constexpr (PAIR) mbar_arrive_cluster(leader_addr(smem_addr(&tmem_empty[b])));
+                        else mbar_arrive(&tmem_empty[b]);
+                    }
                 }
             }
             // one result per hidden row and CTA
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
-                const int row = (m_tile + j) * 128 + quad * 32 + lane;
+                const int row = h_row + j * kTileStep + quad * 32 + lane;
                 if (j < size && row < R && best_i[j] != kNoIndex)
                     atomicMax(p.keys + row, argmax_key(__fadd_rn(best_v[j], 0.f), best_i[j]));
             }
@@ -542,7 +660,7 @@ umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_consta
             __shared__ int s_last;
             __threadfence();
             named_barrier_sync(2, kUmmaEpiWarps * 32);
-            if (ew == 0 && lane == 0) s_last = atomicAdd(p.ticket, 1u) == (unsigned)(tl.groups * tl.CN) - 1u;   // CTAs beyond the tiling take none
+            if (ew == 0 && lane == 0) s_last = atomicAdd(p.ticket, 1u) == (unsigned)(tl.groups * tl.CN * (PAIR ? 2 : 1)) - 1u;   // CTAs beyond the tiling take none
             named_barrier_sync(2, kUmmaEpiWarps * 32);
             if (s_last) {
                 __threadfence();
@@ -558,10 +676,12 @@ umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_consta
     }
 
     tc_fence_before();
-    __syncthreads();
+    if constexpr (PAIR) cluster_sync();    // (neither CTA of a pair leaves before the other)
+    else __syncthreads();
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem_base, 512);
+        if constexpr (PAIR) tmem_dealloc_pair(tmem_base, 512);
+        else tmem_dealloc(tmem_base, 512);
     }
 }
 

@@ -420,3 +420,20 @@ def test_steps_with_a_head_each(oracle, V, B):
     _check_draft_phase(got, ref, S)
     assert ctx.device_status() == 0
     ctx.close()
+
+
+def test_iteration_of_many_rows_counted_on_the_device(oracle):
+    """More rows than the pairs of CTAs are meant for, their number known to the device alone."""
+    V, dD, dT, B, S = 300, 16, 1032, 300, 6
+    W_D, W_T, h_D, H_T = make_inputs(V, dD, dT, B, S, seed=5)
+    pos0 = (np.arange(B, dtype=np.int32) * 3) % 7
+    params = position_clf(cut=6.0)
+    ctx = binding.Context(V, dD, dT, max_batch=B, max_rows=B * (S + 1), clf_hidden=8)
+    ids = np.random.default_rng(3).integers(0, V, size=(B, S)).astype(np.int32)
+    for f in (None, np.full(B, 1, np.int32)):               # about 1400 rows, then 600
+        got = gpu_iteration(ctx, W_D, W_T, h_D, H_T, pos0, to_gpu_clf(params), 0.5, S, sl_forced=f, draft_ids=ids)
+        ref = oracle.iteration(_bits(W_D), _bits(h_D), _bits(W_T), _bits(H_T), pos0, to_oracle_clf(oracle, params), 0.5, S,
+                               sl_forced=f, draft_ids=ids, nthreads=16)
+        check_iteration(oracle, got, ref, W_T, H_T, 0.5, S, ids)
+    assert ctx.device_status() == 0
+    ctx.close()

@@ -353,3 +353,35 @@ def test_features_with_rows_that_are_and_are_not_aligned(oracle, V, N):
     assert torch.equal(lab.cpu().bool(), tD.cpu() == tT.cpu())
     assert ctx.device_status() == 0
     ctx.close()
+
+
+# Tiles of hidden rows in pairs of CTAs: full and part-filled pairs, a last pair with one tile, kept logits
+@pytest.mark.parametrize("N,V,d", [(129, 700, 2048), (256, 3000, 2048), (257, 401, 2056), (520, 5003, 2048), (1000, 300, 2048)])
+def test_feature_extraction_by_pairs_of_ctas(N, V, d):
+    """The ten probabilities, the distribution and the token of every row against float64.  A logit is a sum of 2048 products of
+    fp32 accumulation: good to 2048 * 2^-24 of the sum of the products' sizes (2048 * 0.8 * 0.016 = 26), 3.2e-3 at most."""
+    ctx = binding.Context(V, 64, d, max_batch=1, max_rows=N)
+    W_D, H_D = inputs.lm_head(V, 64, seed=1).cuda(), inputs.hidden(N, 64, seed=2).cuda()
+    W_T, H_T = inputs.lm_head(V, d, seed=3).cuda(), inputs.hidden(N, d, seed=4).cuda()
+    z = lambda *s, t=torch.float32: torch.zeros(*s, dtype=t, device="cuda")
+    pos, tv, label = torch.arange(N, dtype=torch.int32, device="cuda"), z(N), z(N, t=torch.uint8)
+    fD, fT, tD, tT, yD, yT = z(N, 12), z(N, 12), z(N, t=torch.int32), z(N, t=torch.int32), z(N, V), z(N, V)
+    for _ in range(2):
+        ctx.extract_features(W_D, H_D, W_T, H_T, pos, fD, fT, tv, label, tD, tT, yD, yT)
+    assert ctx.device_status() == 0
+    ctx.close()
+    for W, H, feats, token, y in ((W_D, H_D, fD, tD, yD), (W_T, H_T, fT, tT, yT)):
+        logits = H.double() @ W.double().T
+        want = torch.softmax(logits, -1)
+        assert float((y.double() / want - 1).abs().max()) < 3.2e-3
+        assert float((feats[:, :10].double() / want.topk(10, -1).values - 1).abs().max()) < 3.2e-3
+        picked = logits.gather(1, token.long()[:, None])[:, 0]
+        assert float((logits.max(-1).values - picked).max()) < 3.2e-3
+    assert float((tv.double() - 0.5 * (yD.double() - yT.double()).abs().sum(-1)).abs().max()) < 1e-5
+
+
+# Pairs of CTAs: two tiles of 128 rows (the second nearly empty, full), four, ten and an odd number of them; one and several
+# vocabulary tiles per pair
+@pytest.mark.parametrize("V,rows", [(300, 129), (300, 256), (2500, 500), (20000, 180), (400, 1160), (700, 1409)])
+def test_verification_by_pairs_of_ctas(oracle, V, rows):
+    _verification_agrees(oracle, V, rows // 8, rows, 1032)
