@@ -13,6 +13,7 @@
 #include "stream_tail.cuh"
 #include "umma_tail.cuh"
 #include "draft_batch.cuh"
+#include "draft_few.cuh"
 #include "sample.cuh"
 #include "umma_gemv_loop.cuh"
 
@@ -38,7 +39,7 @@ struct KernelSetup {
 // Where an LM-head pass leaves its records (m, Z first) of consecutive vocabulary slabs: what a draw is located with.
 struct RecordLayout {
     const float4* recs;
-    int pieces, NP, slab;
+    int step, row, NP, slab;   // record and row strides in float4; records per row, vocabulary rows per record
 };
 
 struct StreamPlan {
@@ -239,13 +240,37 @@ int launch_attributes(const disco_ctx* c, bool pair, cudaLaunchAttribute (&attr)
     return n;
 }
 
+// Vocabulary on the TMEM lanes (umma_tail.cuh): few rows, and the first rows beyond one tile of 128, where the other form
+// multiplies by 256.  In between and beyond it has no fewer multiplications and the dearer epilogue.  (Launches one after
+// the other at the power limit, 32000 x 5120, 34 / 64 / 96 / 130 / 160 / 192 rows: 61.4 -> 56.2, 61.6 -> 58.2, 63.1 -> 62.5,
+// 79.7 -> 68.9, 81.2 -> 72.6, 82.8 -> 81.1 us; 49152 x 6144, 64 / 96 / 160 / 192 rows: 113 -> 109, 115 -> 121, 158 -> 153,
+// 160 -> 171 us.)  A head that takes less than some 10 us does not reach the power limit, and its epilogue is a larger part
+// (6 rows, 8000 x 512: 7.1 us, 7.7 with the vocabulary on the lanes).  So a lower limit on the head's size for either band,
+// from launches one after the other with the other form -> this one.  Up to 64 rows, 64 MB (d = 2048, 6 / 11 / 30 / 64 rows):
+// 32 MB 11.8 / 12.0 / 12.9 / 13.4 -> 12.5 / 13.0 / 15.3 / 13.5 us; 64 MB 16.5 / 16.5 / 16.6 / 17.4 -> 16.6 / 16.8 / 18.4 / 17.2
+// (17 to 32 rows catch up at 131 MB: 29.4 -> 28.6); 131 MB 29.3 / 29.3 / 29.4 / 29.9 -> 27.0 / 27.3 / 28.6 / 28.1.
+// 129 to 160 rows, 45 MB, where the other form multiplies by 256 (130 / 160 rows): d = 1024, 32 MB 16.2 / 16.2 -> 15.0 / 15.0,
+// 45 MB 18.3 / 18.4 -> 18.6 / 18.8, 96 MB 32.8 / 32.8 -> 32.3 / 33.3; d = 2048, 45 MB 20.4 / 20.3 -> 17.9 / 18.6, 131 MB
+// 39.9 / 39.2 -> 34.3 / 36.1; d = 5120, 45 MB 29.6 / 29.6 -> 27.4 / 29.6, 320 MB 83.2 / 80.8 -> 67.1 / 71.3.  (It pays below
+// 45 MB as well where the contraction is long.)  Forced path 2 takes no account of the size.
+bool verify_on_lanes(const disco_ctx* c, int R, int d) {
+    const size_t head_bytes = (size_t)c->V * d * 2;
+    const bool few = R <= 64 && (head_bytes >= (size_t)64 << 20 || c->path == 2);
+    const bool beyond = R > 128 && R <= 160 && (head_bytes >= (size_t)45 << 20 || c->path == 2);
+    return few || beyond;
+}
+
 // Verification by pairs of CTAs: half of the LM-head traffic from L2, but the rows are cut into tiles of 256.  Launches one after
 // the other, 32000 x 1024 / 2048 / 5120 (us, two tiles of hidden rows per CTA or one -> pairs): 250 rows 22.2 / 35.4 / 80.0 -> 20.3 /
 // 32.0 / 79.3, 300 rows 25.3 / 46.7 / 124 -> 32.0 / 55.2 / 130, 450 rows 33.9 / 60.4 / 122 -> 32.4 / 53.3 / 114, 600 rows 39.9 / 77.1 /
-// 165 -> 38.7 / 80.1 / 175; 2432 rows of 49152 x 6144: 3 % of the iteration.  So: no odd number of 128 rows unless it is large.
-bool umma_in_pairs(int R, int d) {
-    const int tiles = (R + 127) / 128;
-    return d >= 1024 && (tiles % 2 == 0 || tiles >= 9);
+// 165 -> 38.7 / 80.1 / 175; 2432 rows of 49152 x 6144: 3 % of the iteration; 1186 rows of 17960 x 3064, an even number of tiles that
+// leaves pairs idle, 118 -> 120.  So: where a CTA's share of the tensor work does not grow by more than a few hundredths.
+// (A count in device memory: only where it is likely to be large.)
+bool verify_in_pairs(const disco_ctx* c, int R, int d, bool dev_R, int likely_R) {
+    if (d < 1024 || R <= 128 || !VerifyTiling::pairs_possible(R, c->sm_count)) return false;
+    if (dev_R) return likely_R > 1024;
+    const VerifyTiling one = VerifyTiling::make(R, c->V, d, c->sm_count), two = VerifyTiling::make_pairs(R, c->V, d, c->sm_count);
+    return 32ll * two.TPC * two.TRN * std::min(two.GS, two.MT) <= 33ll * one.TPC * one.TRN * std::min(one.GS, one.MT);
 }
 
 // Launch the tcgen05 verification kernel for R hidden rows of width d against the LM head W [V, d].
@@ -257,27 +282,9 @@ int launch_umma(disco_ctx* c, const void* W, const void* H, int d, int R, const 
     p.d = d;
     p.R = R;
     p.dev_R = dev_R;
-    // Vocabulary on the TMEM lanes (umma_tail.cuh): few rows, and the first rows beyond one tile of 128, where the other form
-    // multiplies by 256.  In between and beyond it has no fewer multiplications and the dearer epilogue.  (Launches one after
-    // the other at the power limit, 32000 x 5120, 34 / 64 / 96 / 130 / 160 / 192 rows: 61.4 -> 56.2, 61.6 -> 58.2, 63.1 -> 62.5,
-    // 79.7 -> 68.9, 81.2 -> 72.6, 82.8 -> 81.1 us; 49152 x 6144, 64 / 96 / 160 / 192 rows: 113 -> 109, 115 -> 121, 158 -> 153,
-    // 160 -> 171 us.)  A head that takes less than some 10 us does not reach the power limit, and its epilogue is a larger part
-    // (6 rows, 8000 x 512: 7.1 us, 7.7 with the vocabulary on the lanes).  So a lower limit on the head's size for either band,
-    // from launches one after the other with the other form -> this one.  Up to 64 rows, 64 MB (d = 2048, 6 / 11 / 30 / 64 rows):
-    // 32 MB 11.8 / 12.0 / 12.9 / 13.4 -> 12.5 / 13.0 / 15.3 / 13.5 us; 64 MB 16.5 / 16.5 / 16.6 / 17.4 -> 16.6 / 16.8 / 18.4 / 17.2
-    // (17 to 32 rows catch up at 131 MB: 29.4 -> 28.6); 131 MB 29.3 / 29.3 / 29.4 / 29.9 -> 27.0 / 27.3 / 28.6 / 28.1.
-    // 129 to 160 rows, 45 MB, where the other form multiplies by 256 (130 / 160 rows): d = 1024, 32 MB 16.2 / 16.2 -> 15.0 / 15.0,
-    // 45 MB 18.3 / 18.4 -> 18.6 / 18.8, 96 MB 32.8 / 32.8 -> 32.3 / 33.3; d = 2048, 45 MB 20.4 / 20.3 -> 17.9 / 18.6, 131 MB
-    // 39.9 / 39.2 -> 34.3 / 36.1; d = 5120, 45 MB 29.6 / 29.6 -> 27.4 / 29.6, 320 MB 83.2 / 80.8 -> 67.1 / 71.3.  (It pays below
-    // 45 MB as well where the contraction is long.)  Forced path 2 takes no account of the size.
-    const size_t head_bytes = (size_t)c->V * d * 2;
-    const bool few = R <= 64 && (head_bytes >= (size_t)64 << 20 || c->path == 2);
-    const bool beyond = R > 128 && R <= 160 && (head_bytes >= (size_t)45 << 20 || c->path == 2);
-    const bool lanes = !dev_R && (few || beyond);
+    const bool lanes = !dev_R && verify_on_lanes(c, R, d);
     const bool wide = lanes && R > kUmmaLaneRows;
-    // (a count in device memory: only where it is likely to be large, whatever its parity)
-    const bool pair = !lanes && R > 128 && VerifyTiling::pairs_possible(R, c->sm_count) &&
-                      (dev_R ? d >= 1024 && likely_R > 1024 : umma_in_pairs(R, d));
+    const bool pair = !lanes && verify_in_pairs(c, R, d, dev_R != nullptr, likely_R);
     p.t = pair ? VerifyTiling::make_pairs(R, c->V, d, c->sm_count) : VerifyTiling::make(R, c->V, d, c->sm_count);
     // (with the row count in device memory the kernel derives the tiling)
     p.box_rows = (dev_R ? 256 : p.t.TRN) / (pair ? 2 : 1);
@@ -319,27 +326,109 @@ bool draft_batch_possible(const disco_ctx* c, int R) {
 // Pairs of CTAs that share their vocabulary tiles, where the operands' way from L2 is the bound.  Launches one after the other,
 // 256 / 384 / 512 / 640 / 1000 rows (us, single CTAs -> pairs): 32000 x 768 23.1 / 28.5 / 36.5 / 41 / 58 -> 23.9 / 35.9 / 37.0 / 47 / 60;
 // 32000 x 2048 46.0 / 58.6 / 74.1 / 88.3 / 116 -> 41.8 / 64.5 / 65.7 / 91.1 / 114; 32000 x 5120 99.6 / 133 / 168 / 206 / 263 -> 90.5 / 144 /
-// 130 / 190 / 231.
-bool draft_batch_in_pairs(const disco_ctx* c, int MT, int d) {
-    return d >= 2048 && MT >= 2 && MT != 3 && ((MT + 1) & ~1) <= c->sm_count;
+// 130 / 190 / 231.  With the logits kept the narrow heads gain as well where no tile is left over (feature extraction, heads of 768 and
+// 1024, 300 / 512 / 640 / 760 / 1000 positions: 111 / 157 / 178 / 209 / 251 -> 124 / 156 / 190 / 202 / 244).
+bool draft_batch_in_pairs(const disco_ctx* c, int MT, int d, bool kept) {
+    return ((MT + 1) & ~1) <= c->sm_count && (d >= 2048 ? MT >= 2 && MT != 3 : kept && MT >= 6 && MT % 2 == 0);
+}
+
+// CTAs that finish rows and do nothing else (draft_batch.cuh): a warp for each row.  (us per step, any CTA may finish -> CTAs of
+// their own: one row of 32000 x 768 14.7 -> 11.4, 7 rows of 40011 x 768 17.5 -> 14.3, 64 rows of 32000 x 768 17.8 -> 16.4, 128 rows
+// 16.0 -> 15.1, of 49152 x 768 25.0 -> 23.5.)
+int draft_finishers(const disco_ctx* c, int R) {
+    constexpr int per_cta = kDbEpiWarps + kDbFinWarps;
+    return std::max(1, std::min((R + per_cta - 1) / per_cta, c->sm_count / 4));
+}
+
+// Few hidden rows: the vocabulary on the TMEM lanes.  Up to 32, and beyond 16 only where a CTA has more than 32 vocabulary rows: with
+// fewer there is no shared bound, and then the lists of four rows are one warp's work after another (us, 512-wide heads of
+// 4000 / 8000 / 16000, vocabulary on the columns -> on the lanes: 32 rows 9.9 / 11.7 / 12.4 -> 13.5 / 11.7 / 11.6, 16 rows 9.7 / 11.5 /
+// 12.2 -> 9.9 / 10.3 / 10.4, 4 rows 9.7 / 9.8 / 10.5 -> 9.4 / 9.2 / 9.3).
+bool draft_few_possible(const disco_ctx* c, int R) {
+    return R <= 32 && c->sm_count >= 8 && (R <= 16 || c->V > 32 * (c->sm_count - draft_finishers(c, R)));
+}
+
+template <bool STATS, int NR>
+int launch_draft_few(disco_ctx* c, const void* W, const void* H, int d, int R, float* probs, const DraftFinalParams& f,
+                     cudaStream_t st, RecordLayout* layout) {
+    DraftBatchParams p{};
+    p.V = c->V;
+    p.d = d;
+    p.R = R;
+    p.MT = 1;
+    p.finishers = draft_finishers(c, R);
+    p.CN = c->sm_count - p.finishers;
+    p.TPC = std::max(1, (c->V + 128 * p.CN - 1) / (128 * p.CN));
+    p.TR = (c->V + p.CN * p.TPC - 1) / (p.CN * p.TPC);
+    p.TRN = std::max(16, (p.TR + 15) / 16 * 16);
+    p.a_rows = 8 * NR;
+    p.a_bytes = p.a_rows * 128;
+    p.b_bytes = (p.TRN * 128 + 1023) / 1024 * 1024;
+    if ((size_t)R * p.CN > (size_t)128 * c->sm_count || R > c->part_rows) return DISCO_ERR_WORKSPACE;
+    auto kern = umma_draft_few_kernel<STATS, NR>;
+    static KernelSetup setup;
+    size_t dyn_limit = 0;
+    if (!raise_smem_limit(c, setup, kern, 0, &dyn_limit)) return DISCO_ERR_CUDA;
+    const size_t fixed = draft_few_fixed_smem(NR, f.clf_H);
+    // (an MMA reads 128 rows from the start of the last stage of W)
+    const int stage_bytes = p.a_bytes + p.b_bytes;
+    const size_t least = std::max((size_t)2 * stage_bytes, (size_t)p.b_bytes + 16384);
+    if (dyn_limit < fixed + least) return DISCO_ERR_UNSUPPORTED_SHAPE;
+    p.stages = (int)std::min<size_t>(kDbMaxStages, (dyn_limit - fixed) / stage_bytes);
+    while (p.stages > 2 && fixed + (size_t)(p.stages - 1) * p.b_bytes + 16384 > dyn_limit) --p.stages;
+    p.ring_bytes = std::max(p.stages * stage_bytes, (p.stages - 1) * p.b_bytes + 16384);
+    p.status = c->status;
+    p.part_rec = reinterpret_cast<float4*>(c->stamped_rec);
+    p.probs = probs;
+    p.bound = c->row_bound;
+    p.set_words = (size_t)c->part_rows * kDbBoundStride;
+    p.sync = c->ticket + 48;
+    CUtensorMap tmap_W, tmap_H;
+    if (!encode_bf16_2d(c, &tmap_W, W, c->V, d, p.TRN) || !encode_bf16_2d(c, &tmap_H, H, R, d, p.a_rows))
+        return DISCO_ERR_CUDA;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(p.CN + p.finishers));
+    cfg.blockDim = dim3(kDbThreads);
+    cfg.dynamicSmemBytes = fixed + p.ring_bytes;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = c->pdl ? 1 : 0;
+    if (layout) *layout = RecordLayout{p.part_rec, 1, kStampedPieces * p.CN, p.CN, p.TPC * p.TR};
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tmap_W, tmap_H, p, f);
+    c->launches += 1;
+    return cuda_ok(e, "umma_draft_few_kernel launch") ? DISCO_OK : DISCO_ERR_CUDA;
 }
 
 // Launch the batched draft step (STATS: arg-max and statistics only) for R hidden rows of width d against W [V, d].
 template <bool STATS>
 int launch_draft_batch(disco_ctx* c, const void* W, const void* H, int d, int R, float* probs, const DraftFinalParams& f,
                        cudaStream_t st, RecordLayout* layout) {
+    if (draft_few_possible(c, R)) {
+        if (R <= 8) return launch_draft_few<STATS, 1>(c, W, H, d, R, probs, f, st, layout);
+        if (R <= 16) return launch_draft_few<STATS, 2>(c, W, H, d, R, probs, f, st, layout);
+        return launch_draft_few<STATS, 4>(c, W, H, d, R, probs, f, st, layout);
+    }
     DraftBatchParams p{};
     p.V = c->V;
     p.d = d;
     p.R = R;
     p.MT = (R + 127) / 128;
-    const bool pair = draft_batch_in_pairs(c, p.MT, d);
+    const bool pair = draft_batch_in_pairs(c, p.MT, d, probs != nullptr);
     if (pair) p.MT = (p.MT + 1) & ~1;
-    p.CN = c->sm_count / p.MT;
     // One tile of hidden rows: the LM head arrives slower than the tensor pipe works, so the tiles are small and the
     // epilogue of one runs under the loads of the next.  More tiles of rows: the rows' tile is loaded again for every
     // vocabulary tile, and that traffic (L2 to shared memory) is the bound, so the vocabulary tiles are the widest.
     const int tile_target = R <= 128 ? 128 : 256;
+    // (one tile of rows: CTAs of their own finish the rows, unless the others would need a vocabulary tile more for it, or one
+    // that is too large to do without the shared bound)
+    auto tiles_each = [&](int CN) { return (c->V + tile_target * CN - 1) / (tile_target * CN); };
+    p.finishers = p.MT == 1 ? draft_finishers(c, R) : 0;
+    const int without = c->sm_count / p.MT, with = without - p.finishers;
+    if (tiles_each(with) > tiles_each(without) || (c->V > 32 * with && c->V <= 32 * without)) p.finishers = 0;
+    p.CN = c->sm_count / p.MT - p.finishers;
     p.TPC = std::max(1, (c->V + tile_target * p.CN - 1) / (tile_target * p.CN));
     p.TR = (c->V + p.CN * p.TPC - 1) / (p.CN * p.TPC);
     if (probs) p.TR = (p.TR + 3) & ~3;   // rows of logits are stored 16 bytes at a time
@@ -352,8 +441,8 @@ int launch_draft_batch(disco_ctx* c, const void* W, const void* H, int d, int R,
     static KernelSetup setup[2];
     size_t dyn_limit = 0;
     if (!raise_smem_limit(c, setup[pair], kern, 0, &dyn_limit)) return DISCO_ERR_CUDA;
-    p.all_finish = R > kDbFinWarps * p.MT * p.CN;
-    const int fin_warps = kDbFinWarps + (p.all_finish ? kDbEpiWarps : 0);
+    p.all_finish = p.finishers == 0 && R > kDbFinWarps * p.MT * p.CN;
+    const int fin_warps = kDbFinWarps + (p.all_finish || p.finishers ? kDbEpiWarps : 0);
     const size_t fixed = 1024 + 512 + kDbXchBytes + (size_t)(fin_warps * kDbFinWords + 128) * 4 +
                          (probs ? kDbEpiWarps * 32 * kDbTurnStride * 4 : 0) + umma_clf_bytes(f.clf_H) + 128;
     if (dyn_limit < fixed + 2 * (size_t)(p.a_bytes + p.b_bytes)) return DISCO_ERR_UNSUPPORTED_SHAPE;
@@ -369,14 +458,14 @@ int launch_draft_batch(disco_ctx* c, const void* W, const void* H, int d, int R,
     if (!encode_bf16_2d(c, &tmap_W, W, c->V, d, pair ? p.TRN / 2 : p.TRN) || !encode_bf16_2d(c, &tmap_H, H, R, d, p.a_rows))
         return DISCO_ERR_CUDA;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)(p.MT * p.CN));
+    cfg.gridDim = dim3((unsigned)(p.MT * p.CN + p.finishers));
     cfg.blockDim = dim3(kDbThreads);
     cfg.dynamicSmemBytes = fixed + p.ring_bytes;
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
     cfg.attrs = attr;
     cfg.numAttrs = launch_attributes(c, pair, attr);
-    if (layout) *layout = RecordLayout{p.part_rec, kStampedPieces, p.CN, p.TPC * p.TR};
+    if (layout) *layout = RecordLayout{p.part_rec, 1, kStampedPieces * p.CN, p.CN, p.TPC * p.TR};
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tmap_W, tmap_H, p, f);
     c->launches += 1;
     return cuda_ok(e, "umma_draft_batch_kernel launch") ? DISCO_OK : DISCO_ERR_CUDA;
@@ -742,8 +831,8 @@ int draft_step_common(disco_ctx* c, const void* W_D, const void* h_D, int d, int
     p.feats = feats;
     p.probs = probs;
     p.nll_sum = nll_sum;
-    // The tensor-core kernel serves every batch (us per step in a stream, cold L2: one sequence of 32000 x 768 14.6, 7 of
-    // 40011 x 768 17.6, 64 of 32000 x 768 18.2); the CUDA-core streaming kernel is the path without tensor maps.
+    // The tensor-core kernels serve every batch (us per step in a stream, cold L2: one sequence of 32000 x 768 11.4, 7 of
+    // 40011 x 768 14.4, 64 of 32000 x 768 16.5); the CUDA-core streaming kernel is the path without tensor maps.
     const bool use_umma = draft_batch_possible(c, B) && c->path != 1;
     if (use_umma) {
         DraftFinalParams f{};
@@ -775,7 +864,8 @@ int draft_step_common(disco_ctx* c, const void* W_D, const void* h_D, int d, int
     } else {
         rc = run_stream<true>(c, p, clf->H, st);
         if (rc) return rc;
-        if (layout) *layout = RecordLayout{p.part_rec, 4, (p.V + p.rows_per_cta - 1) / p.rows_per_cta, p.rows_per_cta};
+        const int slabs = (p.V + p.rows_per_cta - 1) / p.rows_per_cta;
+        if (layout) *layout = RecordLayout{p.part_rec, 4, 4 * slabs, slabs, p.rows_per_cta};
     }
     if (probs && normalize) {
         dim3 grid((unsigned)std::min(64, (c->V + 255) / 256), (unsigned)B);
@@ -910,7 +1000,8 @@ int disco_draft_step_sample(disco_ctx* c, const void* W_D, const void* h_D, int 
     if (rc) return rc;
     // probs holds the logits: the kernel turns them into y^D and replaces the greedy token by the draw
     DrawRowsParams dp{};
-    dp.rec_pieces = rl.pieces;
+    dp.rec_step = rl.step;
+    dp.rec_row = rl.row;
     dp.NP = rl.NP;
     dp.slab = rl.slab;
     // about two CTAs per SM, at least one slab each
@@ -921,7 +1012,7 @@ int disco_draft_step_sample(disco_ctx* c, const void* W_D, const void* h_D, int 
     for (size_t b0 = 0; b0 < (size_t)B; b0 += kMaxRows) {
         dp.probs = probs + b0 * c->V;
         dp.stats = c->final_stats + 2 * b0;
-        dp.recs = rl.recs + b0 * rl.NP * rl.pieces;
+        dp.recs = rl.recs + b0 * rl.row;
         dp.u = u + b0;
         dp.active = active ? active + b0 : nullptr;
         dp.token = token + b0;

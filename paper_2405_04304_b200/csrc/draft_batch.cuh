@@ -10,7 +10,8 @@
 //   * warps 2-9   epilogue: every thread owns one hidden row and walks over its share of a tile's columns: soft-max
 //                 statistics in registers, and the few logits that can still be among the row's ten largest;
 //   * warps 10-11 finish rows: one warp merges the per-CTA records of a hidden row, forms the features of Eq. 2, runs
-//                 the halt classifier and the stopping rule.
+//                 the halt classifier and the stopping rule.  With one tile of rows (up to 128) the grid's last CTAs do that,
+//                 with ten warps each, and have no vocabulary of their own (db_finish_dedicated).
 //
 // What the design is built around:
 //   * The ten largest.  A CTA sees a few hundred columns of each row, so "above this CTA's tenth largest" is no
@@ -20,12 +21,14 @@
 //     of the row's tenth largest logit, at any time and whatever the timing; the final list is exact.  About twenty of a
 //     row's logits pass it, over all CTAs.
 //   * No waiting on CTAs that may not run.  The finishing warps wait for other CTAs' records, but only once every CTA of
-//     the grid has started (a counter); a CTA that is done before that leaves.  The CTA that starts last always finds
-//     the counter full, so every row is finished by somebody, with any number of other kernels on the device.  So the
-//     launch need not be cooperative, and its prologue and first loads run under the tail of the kernel before it (a
-//     cooperative launch was measured to cost 4 - 5 us in a stream).
+//     the grid has started (a counter); with more than one tile of rows a CTA that is done before that leaves, and the CTA
+//     that starts last always finds the counter full, so every row is finished by somebody, with any number of other
+//     kernels on the device.  So the launch need not be cooperative, and its prologue and first loads run under the tail of
+//     the kernel before it (a cooperative launch was measured to cost 4 - 5 us in a stream).
 //   * Code that runs once per launch is fetched from L2 instruction by instruction.  Both the finishing code and what
-//     follows the column loop run once for nothing while the first tile is awaited.
+//     follows the column loop run once for nothing while the first tile is awaited, and the finishing code is short: the
+//     wait for the records and what follows it took 12.5 thousand cycles of a launch of 28 (one row of 32000 x 768), now 6
+//     of 21.
 #pragma once
 
 #include "umma_tail.cuh"
@@ -37,9 +40,8 @@ constexpr int kDbFinWarps = 2;
 constexpr int kDbThreads = (2 + kDbEpiWarps + kDbFinWarps) * 32;
 constexpr int kDbMaxStages = 16;
 constexpr int kDbMaxRecords = 160;     // records per row a finishing warp takes in: five per lane
-constexpr int kDbCandidates = 128;
 constexpr int kDbXchBytes = 128 * 64;  // states handed between the two warps that share a hidden row
-constexpr int kDbFinWords = 16 + kDbCandidates + 16;   // features, candidates, result; per finishing warp
+constexpr int kDbFinWords = 16;        // features; per finishing warp
 constexpr int kDbBoundSlots = 12;      // words of the shared bound per row
 constexpr int kDbBoundStride = 16;     // (rows 64 bytes apart)
 constexpr int kDbTurnStride = 36;      // floats per row of the area that turns a chunk of logits round (no bank conflicts)
@@ -57,7 +59,7 @@ struct DraftBatchParams {
     int a_rows;  // rows of the H box (multiple of 8, <= 128)
     int stages, a_bytes, b_bytes, ring_bytes;
     int* status;
-    float4* part_rec;      // [R][CN] stamped records of 80 bytes
+    float4* part_rec;      // [R][kStampedPieces][CN]: stamped records, piece by piece
     float* probs;          // optional [R][V]: raw logits are written here
     // Two sets of [set_words / kDbBoundStride] rows: ordered bits of the groups' maxima.  A launch uses the set of its
     // stamp's parity, which starts zeroed, and zeroes the other one (whose launch is over, so nothing of it is in flight).
@@ -67,6 +69,7 @@ struct DraftBatchParams {
     // [4] on two sets of (CTAs started, rows claimed), four words apart, used by parity: a launch clears the other
     unsigned int* sync;
     int all_finish;        // more rows than finishing warps in the grid: the epilogue warps help
+    int finishers;         // CTAs behind the CN others that finish the rows and have no vocabulary (0: every CTA may finish rows)
 };
 
 __device__ __forceinline__ float ex2_approx(float x) {
@@ -168,7 +171,9 @@ static_assert(kDbBoundSlots - kTopK == 2, "the third smallest of the words bound
 // ---------------------------------------------------------------------------------------------
 // second phase: one warp finishes one hidden row
 // ---------------------------------------------------------------------------------------------
-// A record (five stamped 16-byte pieces, see kStampedPieces): m Z S | word l0 bound | l1 l2 l3 | l4 l5 l6 | l7 l8 l9.
+// A record (five stamped 16-byte pieces, see kStampedPieces): m Z S | word l0 bound | l1 l2 l3 | l4 l5 l6 | l7 l8 l9.  The
+// same piece of all CTAs lies side by side: a load of a warp reads four lines (records of 80 bytes one after the other were
+// 32 requests each: 2000 cycles for the pieces of a row, against 900).
 // word: the arg-max index if the CTA's largest logit passed the bound (kDbNoIndex otherwise), and the number of list
 // entries.  l: the CTA's logits above the bound (at most its ten largest), descending.  bound: the largest bound used.
 // The last two pieces are written only if there are more than four entries.
@@ -176,48 +181,34 @@ static_assert(kDbBoundSlots - kTopK == 2, "the third smallest of the words bound
 // What the lists leave out is at most B = the largest of the records' bounds, and at least ten logits of the row are at
 // or above B: so the row's k-th largest logit is max(B, the k-th largest list entry), for k <= 10.
 
-// Many list entries that cannot be told apart by a threshold (ties, or one CTA holding them all): ten rounds of
-// "largest entry after the last one" over the lists in memory, entries ordered by value, then position.
-static __device__ __noinline__ void db_select_slow(const float4* recs, int NP, uint32_t stamp, float* res, int lane) {
-    float last_v = __int_as_float(0x7f800000);
-    int last_pos = -1;
-    for (int k = 0; k < kTopK; ++k) {
-        float bv = DISCO_NEG_INF;
-        int bp = kNoIndex;
-        for (int c = lane; c < NP; c += 32) {
-            const float4* src = recs + (size_t)c * kStampedPieces;
-            const float4 h = load_relaxed_v4(src + 1);
-            const int cnt = min(kTopK, static_cast<int>(__float_as_uint(h.x) >> 28));
-            for (int i = 0; i < cnt; ++i) {
-                const float4 x = load_relaxed_v4(src + 2 + (i - 1) / 3);
-                // (a late piece of a list is not stamped yet only if nothing of it is wanted: the caller has seen the others)
-                if (i > 0 && __float_as_uint(x.w) != stamp) continue;
-                const int w = (i - 1) % 3;
-                const float v = i == 0 ? h.y : (w == 0 ? x.x : (w == 1 ? x.y : x.z));
-                const int pos = c * 16 + i;
-                const bool after = v < last_v || (v == last_v && pos > last_pos);
-                if (after && v > bv) {   // (positions ascend: the first of equal values stays)
-                    bv = v;
-                    bp = pos;
-                }
-            }
-        }
-        const uint32_t top = __reduce_max_sync(kFullMask, ordered_bits(bv));
-        const int pos = __reduce_min_sync(kFullMask, ordered_bits(bv) == top ? bp : kNoIndex);
-        last_v = from_ordered_bits(top);
-        last_pos = pos;
-        if (lane == 0) res[k] = last_v;
-        if (pos == kNoIndex) break;
+// The fifth and further entries of record c's list go into the row's ten largest (lane k < 10 holds the k-th) where they are
+// above `least`.  They are in the record's last two pieces, which may still be on their way.
+static __device__ __noinline__ float db_long_list(const float4* recs, int NP, int c, int cnt, uint32_t stamp, int* status, float sel,
+                                                  float least, int lane) {
+    float x = DISCO_NEG_INF;
+    if (lane < cnt - 4) {
+        const float4* piece = recs + (3 + lane / 3) * NP + c;
+        float4 v = load_relaxed_v4(piece);
+        const long long t0 = clock64();
+        while (__float_as_uint(v.w) != stamp && clock64() - t0 < kWaitBudgetClocks) v = load_relaxed_v4(piece);
+        if (__float_as_uint(v.w) != stamp) record_status(status, DISCO_ERR_TIMEOUT);
+        const int w = lane % 3;
+        x = w == 0 ? v.x : (w == 1 ? v.y : v.z);
     }
     __syncwarp();
+    for (unsigned mask = __ballot_sync(kFullMask, x > least); mask; mask &= mask - 1u) {
+        const float v = __shfl_sync(kFullMask, x, __ffs(mask) - 1);
+        const int at = __popc(__ballot_sync(kFullMask, lane < kTopK && sel >= v));
+        const float up = __shfl_up_sync(kFullMask, sel, 1);
+        if (lane < kTopK && lane >= at) sel = lane == at ? v : up;
+    }
+    return sel;
 }
 
 // real = false: the same instructions on made-up records, nothing read from or written to global memory.
 __device__ __forceinline__ void db_finish_row(const DraftBatchParams& p, const DraftFinalParams& f, int b, bool real,
                                               uint32_t stamp, float* sm, const float* clf_s, bool stats, int lane) {
     constexpr int PER = kDbMaxRecords / 32;
-    float* cand = sm + 16;
-    float* res = cand + kDbCandidates;
     const int NP = real ? p.CN : 0;
     const float4* recs = p.part_rec + (size_t)b * p.CN * kStampedPieces;
     // issued with the first poll: what the epilogue needs besides the records
@@ -232,9 +223,11 @@ __device__ __forceinline__ void db_finish_row(const DraftBatchParams& p, const D
     {
         const long long t0 = clock64();
 #pragma unroll
-        for (int j = 0; j < PER; ++j)
-#pragma unroll
-            for (int i = 0; i < 3; ++i) q[j][i] = make_float4(0.f, 0.f, 0.f, __uint_as_float(stamp));
+        for (int j = 0; j < PER; ++j) {   // (no record: Z = 0 and an empty list)
+            q[j][0] = make_float4(0.f, 0.f, 0.f, __uint_as_float(stamp));
+            q[j][1] = make_float4(0.f, DISCO_NEG_INF, DISCO_NEG_INF, q[j][0].w);
+            q[j][2] = make_float4(DISCO_NEG_INF, DISCO_NEG_INF, DISCO_NEG_INF, q[j][0].w);
+        }
         if (!real) {   // made-up records, so that the loops below run
             q[0][0] = make_float4(lane * 0.125f, 1.f, 0.f, q[0][0].w);
             q[0][1] = make_float4(__uint_as_float(1u << 28 | lane), lane * 0.125f, 0.f, q[0][1].w);
@@ -245,10 +238,10 @@ __device__ __forceinline__ void db_finish_row(const DraftBatchParams& p, const D
         for (int polls = 0;;) {
 #pragma unroll
             for (int j = 0; j < PER; ++j) {
-                const float4* src = recs + (size_t)(j * 32 + lane) * kStampedPieces;
+                const float4* src = recs + (j * 32 + lane);
                 if ((pend >> j) & 1u)
 #pragma unroll
-                    for (int i = 0; i < 3; ++i) q[j][i] = load_relaxed_v4(src + i);
+                    for (int i = 0; i < 3; ++i) q[j][i] = load_relaxed_v4(src + i * NP);
             }
 #pragma unroll
             for (int j = 0; j < PER; ++j)
@@ -296,82 +289,71 @@ __device__ __forceinline__ void db_finish_row(const DraftBatchParams& p, const D
     idx = __reduce_min_sync(kFullMask, idx);
     float sel = DISCO_NEG_INF;
     if (!stats) {
-        // Entries above the bound move to shared memory (about twenty, over all records).  More than 64 of them (a grid that
-        // had no bound in time): only those not below theta, the tenth largest of the lanes' largest entries.
-        float theta = DISCO_NEG_INF;
-        int n = 0;
-        bool more = false;    // some list goes on past its fourth entry
-        const unsigned lt = (1u << lane) - 1u;
-        for (int round = 0; round < 2; ++round) {
-            n = 0;
-            more = false;
+        // One warp is at work here, on code that it runs once, so what counts is the number of instructions: the four largest
+        // entries of each lane's lists (places without an entry hold -inf), then ten times the largest of all, taken from the
+        // lane that has it; a lane that has given four looks for its next four.  (Collecting the 30 - 50 entries above the bound
+        // and ranking them: 4400 cycles; only those not below the tenth largest of the lanes' heads: 3300; this: 1300.)
+        float fourth[PER], more = DISCO_NEG_INF;      // the fourth entry of a list that goes on past it
 #pragma unroll
-            for (int j = 0; j < PER; ++j) {
-                const int cnt = static_cast<int>(__float_as_uint(q[j][1].x) >> 28);
-                const float l[4] = {q[j][1].y, q[j][2].x, q[j][2].y, q[j][2].z};
+        for (int j = 0; j < PER; ++j) {
+            fourth[j] = (__float_as_uint(q[j][1].x) >> 28) > 4u ? q[j][2].z : DISCO_NEG_INF;
+            more = fmaxf(more, fourth[j]);
+        }
+        float t = DISCO_NEG_INF;
+        bool ended = false;
+#pragma unroll 1
+        for (int k = 0; k < kTopK && !ended;) {
+            float a[4] = {q[0][1].y, q[0][2].x, q[0][2].y, q[0][2].z};
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const bool take = k < cnt && l[k] > bound && l[k] >= theta;
-                    const unsigned mask = __ballot_sync(kFullMask, take);
-                    if (mask == 0u) break;
-                    const int at = n + __popc(mask & lt);
-                    if (take && at < kDbCandidates) cand[at] = l[k];
-                    n += __popc(mask);
-                    if (k == 3) more = more || (take && cnt > 4);
-                }
+            for (int j = 1; j < PER; ++j) {
+                // two descending lists, one reversed: the larger of each pair are the four largest, two steps sort them
+                const float c0 = fmaxf(a[0], q[j][2].z), c1 = fmaxf(a[1], q[j][2].y), c2 = fmaxf(a[2], q[j][2].x), c3 = fmaxf(a[3], q[j][1].y);
+                const float d0 = fmaxf(c0, c2), d2 = fminf(c0, c2), d1 = fmaxf(c1, c3), d3 = fminf(c1, c3);
+                a[0] = fmaxf(d0, d1), a[1] = fminf(d0, d1), a[2] = fmaxf(d2, d3), a[3] = fminf(d2, d3);
             }
-            if (n <= 64) break;
-            float head = DISCO_NEG_INF;
+            int taken = 0;
+#pragma unroll 1
+            for (;;) {
+                t = warp_max_f32(a[0]);
+                ended = !(t > bound);
+                if (ended) break;
+                if (lane == k) sel = t;
+                if (lane == __ffs(__ballot_sync(kFullMask, a[0] == t)) - 1) {
+                    a[0] = a[1], a[1] = a[2], a[2] = a[3], a[3] = DISCO_NEG_INF;
+                    ++taken;
+                }
+                if (++k == kTopK || __any_sync(kFullMask, taken == 4)) break;
+            }
+            if (k < kTopK && !ended) {   // (seldom) what the lanes gave leaves their lists
+#pragma unroll 1
+                for (; taken > 0; --taken) {
+                    float h = q[0][1].y;
+#pragma unroll
+                    for (int j = 1; j < PER; ++j) h = fmaxf(h, q[j][1].y);
+                    bool out = false;
+#pragma unroll
+                    for (int j = 0; j < PER; ++j)
+                        if (!out && q[j][1].y == h) {
+                            q[j][1].y = q[j][2].x, q[j][2].x = q[j][2].y, q[j][2].y = q[j][2].z, q[j][2].z = DISCO_NEG_INF;
+                            out = true;
+                        }
+                }
+                __syncwarp();
+            }
+        }
+        // A list that goes on may hold more of the ten largest if its fourth entry is above the tenth of those found.
+        float least = ended ? bound : t;
+        if (__any_sync(kFullMask, more > least)) {
 #pragma unroll
             for (int j = 0; j < PER; ++j)
-                if (__float_as_uint(q[j][1].x) >> 28) head = fmaxf(head, q[j][1].y);
-            __syncwarp();
-            const int rank = rank_in_warp(head, lane, cand);
-            theta = __shfl_sync(kFullMask, head, __ffs(__ballot_sync(kFullMask, rank == kTopK - 1)) - 1);
-            if (round == 1) n = kDbCandidates + 1;   // (the candidates were overwritten)
-        }
-        if (__any_sync(kFullMask, more)) {   // (rare) the rest of the long lists
-#pragma unroll 1
-            for (int j = 0; j < PER; ++j) {
-                const int c = j * 32 + lane;
-                int cnt = 0;
-                if (c < NP) cnt = static_cast<int>(__float_as_uint(__ldcg(&recs[(size_t)c * kStampedPieces + 1].x)) >> 28);
-#pragma unroll 1
-                for (int i = 4; i < kTopK; ++i) {
-                    float v = DISCO_NEG_INF;
-                    if (i < cnt) {
-                        const float4* piece = recs + (size_t)c * kStampedPieces + 3 + (i - 4) / 3;
-                        float4 x = load_relaxed_v4(piece);
-                        const long long t0 = clock64();
-                        while (__float_as_uint(x.w) != stamp && clock64() - t0 < kWaitBudgetClocks) x = load_relaxed_v4(piece);
-                        if (__float_as_uint(x.w) != stamp) record_status(p.status, DISCO_ERR_TIMEOUT);
-                        const int w = (i - 4) % 3;
-                        v = w == 0 ? x.x : (w == 1 ? x.y : x.z);
-                    }
-                    const bool take = v > bound && v >= theta && v > DISCO_NEG_INF;
-                    const unsigned mask = __ballot_sync(kFullMask, take);
-                    const int slot = n + __popc(mask & ((1u << lane) - 1u));
-                    if (take && slot < kDbCandidates) cand[slot] = v;
-                    n += __popc(mask);
+                for (unsigned mask = __ballot_sync(kFullMask, fourth[j] > least); mask; mask &= mask - 1u) {
+                    const int src = __ffs(mask) - 1;
+                    const int cnt = static_cast<int>(__shfl_sync(kFullMask, __float_as_uint(q[j][1].x), src) >> 28);
+                    sel = db_long_list(recs, NP, j * 32 + src, cnt, stamp, p.status, sel, least, lane);
+                    least = fmaxf(least, __shfl_sync(kFullMask, sel, kTopK - 1));
                 }
-            }
         }
-        if (lane < kTopK) res[lane] = DISCO_NEG_INF;
-        __syncwarp();
-        if (n <= kDbCandidates) {
-            for (int i = n + lane; i < ((n + 31) & ~31); i += 32) cand[i] = DISCO_NEG_INF;
-            __syncwarp();
-            for (int i = lane; i < n; i += 32) {
-                const float x = cand[i];
-                const int r = rank_in_list(cand, n, x, i);
-                if (r < kTopK) res[r] = x;
-            }
-            __syncwarp();
-        } else {
-            db_select_slow(recs, NP, stamp, res, lane);
-        }
-        if (lane < kTopK) sel = fmaxf(res[lane], bound);
-        __syncwarp();
+        if (lane < kTopK) sel = fmaxf(sel, bound);
     }
     SoftmaxState st;
     st.m = M, st.Z = Z, st.S = S;
@@ -382,6 +364,167 @@ __device__ __forceinline__ void db_finish_row(const DraftBatchParams& p, const D
     const int Hc = f.clf_H;
     warp_draft_epilogue(st, key, sel, fpos, nd, f.tau, f.sl_max, sm, clf_s, clf_s + Hc * kNFeat, clf_s + Hc * (kNFeat + 1),
                         clf_s + Hc * (kNFeat + 2), Hc, b, o, lane);
+}
+
+// A number the compiler cannot know: a loop that rehearses and then runs the same code must stay one copy of it.
+__device__ __forceinline__ int opaque(int x) {
+    asm volatile("" : "+r"(x));
+    return x;
+}
+
+// This launch's stamp, by the epilogue warps (eight of the CTA, ew their number) once what went before is over: the set of
+// bounds of the launch before is cleared and the CTA counts as started.
+__device__ __forceinline__ uint32_t db_begin(const DraftBatchParams& p, const DraftFinalParams& f, int ew, uint32_t* s_stamp, int lane) {
+    const uint32_t stamp = *reinterpret_cast<volatile unsigned int*>(p.sync) + 1u;
+    const uint32_t par = stamp & 1u;
+    // (that word is the other parity's: only a launch after this one writes it)
+    const int old_rows = *reinterpret_cast<volatile unsigned int*>(p.sync + 2 + (par ^ 1u));
+    if (blockIdx.x == 0)
+        for (int i = ew * 32 + lane; i < f.clear_n; i += kDbEpiWarps * 32) f.clear_words[i] = 0u;
+    uint4* old = reinterpret_cast<uint4*>(p.bound + (par ^ 1u) * p.set_words);
+    for (int i = blockIdx.x * (kDbEpiWarps * 32) + ew * 32 + lane; i < old_rows * (kDbBoundStride / 4);
+         i += gridDim.x * (kDbEpiWarps * 32))
+        old[i] = make_uint4(0, 0, 0, 0);
+    __syncwarp();
+    // This CTA has started once all of its eight reads of the stamp are done: the stamp may be moved on as soon as every
+    // CTA counts as started, and a warp that read the moved word would work on the next launch's set of bounds.  (One
+    // warp that reads and hands the stamp to the others through shared memory: their polling costs the step up to 3 %,
+    // eight rows of 49152 x 768 kept and drawn 30.9 us against 30.1.)
+    named_barrier_sync_after(8, kDbEpiWarps * 32, stamp);
+    if (ew == 0 && lane == 0) {
+        *reinterpret_cast<volatile uint32_t*>(s_stamp) = stamp;
+        atomicAdd(p.sync + 4 + 4 * par, 1u);
+    }
+    return stamp;
+}
+// All CTAs have started: the stamp can move on, and the counters of the next launch (this one's may still be looked at) start
+// at zero.
+__device__ __forceinline__ void db_move_on(const DraftBatchParams& p, uint32_t stamp) {
+    unsigned int* other = p.sync + 4 + 4 * ((stamp + 1u) & 1u);
+    other[0] = 0u;
+    other[1] = 0u;
+    p.sync[2 + (stamp & 1u)] = (unsigned int)p.R;
+    p.sync[0] = stamp == 0xffffffffu ? 1u : stamp;   // never zero, and the two sets keep alternating
+}
+__device__ __forceinline__ void db_stage_classifier(const DraftFinalParams& f, float* clf_s, int first, int step) {
+    const int Hc = f.clf_H, n1 = Hc * kNFeat;
+    if (Hc > 0) {
+        for (int i = first; i < n1 + 2 * Hc + 1; i += step) {
+            const float* src = i < n1 ? f.clf_W1 + i
+                                      : (i < n1 + Hc ? f.clf_b1 + (i - n1)
+                                                     : (i < n1 + 2 * Hc ? f.clf_w2 + (i - n1 - Hc) : f.clf_b2));
+            cp_async4(clf_s + i, src);
+        }
+        cp_async_commit();
+    }
+}
+
+// Up to 128 rows: the last CTAs of the grid have no vocabulary, ten warps of theirs finish a row each.  The CTAs with vocabulary
+// leave when their records are out, so the next launch finds their SMs free and has its share of the LM head on the way while
+// this one ends; a CTA that finished a row as well was replaced when the launch ended, and its successor's records came 3 us
+// after the others'.  A CTA here that starts before the others (blocks start in order, so that is not expected) waits for
+// them, bounded; its own place is one that no other CTA of the launch needs.
+template <bool STATS, class Live>
+__device__ __forceinline__ void db_finish_dedicated(const DraftBatchParams& p, const DraftFinalParams& f, int warp, bool looks_live,
+                                                    float* fin_s, float* clf_s, uint32_t* s_stamp, const Live& step_live, int lane) {
+    constexpr int kWarps = kDbEpiWarps + kDbFinWarps;
+    const int fw = warp - 2;
+    float* sm = fin_s + fw * kDbFinWords;
+    db_stage_classifier(f, clf_s, fw * 32 + lane, kWarps * 32);
+    cp_async_wait_all();
+    named_barrier_sync(3, kWarps * 32);
+    uint32_t stamp = 1u;
+    int b = 0;
+    bool run = looks_live;
+#pragma unroll 1
+    for (int real = opaque(0);; real = opaque(1)) {
+        if (run) db_finish_row(p, f, b, real != 0, stamp + (real ? f.test_stamp_skew : 0u), sm, clf_s, STATS, lane);
+        if (real) {
+            b += kWarps * p.finishers;
+        } else {
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            if (!step_live()) break;
+            b = (int)blockIdx.x - p.CN + fw * p.finishers;
+            if (fw < kDbEpiWarps) stamp = db_begin(p, f, fw, s_stamp, lane);
+            else stamp = smem_word(s_stamp, p.status);
+            if (lane == 0) {
+                const unsigned int* started = p.sync + 4 + 4 * (stamp & 1u);
+                const long long t0 = clock64();
+                for (int polls = 0; ld_relaxed_u32(started) != gridDim.x; ++polls) {
+                    __nanosleep(100);
+                    if ((polls & 63) == 63 && (*reinterpret_cast<volatile int*>(p.status) == DISCO_ERR_TIMEOUT ||
+                                               clock64() - t0 > 64 * kWaitBudgetClocks)) {
+                        record_status(p.status, DISCO_ERR_TIMEOUT);
+                        break;
+                    }
+                }
+                if (b == 0) db_move_on(p, stamp);
+            }
+            __syncwarp();
+        }
+        if (b >= f.B) break;
+        run = chain_seq_live(f.chain, f.active, chain_seq(f.chain, b));
+    }
+}
+
+// The finishing warps, from the start of the launch; with more rows than those of the whole grid, the epilogue warps as
+// well once their records are out.  warp: the warp's number in the CTA; step_live: whether the step takes place.
+template <bool STATS, class Live>
+__device__ __forceinline__ void db_finish_rows(const DraftBatchParams& p, const DraftFinalParams& f, int warp, bool looks_live,
+                                               float* fin_s, float* clf_s, int* s_done, uint32_t* s_clf, const uint32_t* s_stamp,
+                                               const Live& step_live, int lane) {
+    const bool epi = warp < 2 + kDbEpiWarps;
+    if (epi && !p.all_finish) return;
+    const int fw = epi ? kDbFinWarps + warp - 2 : warp - 2 - kDbEpiWarps;
+    float* sm = fin_s + fw * kDbFinWords;
+    if (!epi) db_stage_classifier(f, clf_s, fw * 32 + lane, kDbFinWarps * 32);
+    uint32_t stamp = 1u;
+    unsigned int* set = nullptr;
+    int b = 0;
+    bool run = !epi && looks_live;
+#pragma unroll 1
+    for (int real = opaque(0);; real = opaque(1)) {
+        if (run) db_finish_row(p, f, b, real != 0, stamp + (real ? f.test_stamp_skew : 0u), sm, clf_s, STATS, lane);
+        if (!real) {
+            if (!epi) {
+                cp_async_wait_all();
+                named_barrier_sync(3, kDbFinWarps * 32);
+                if (fw == 0 && lane == 0) {
+                    __threadfence_block();
+                    *reinterpret_cast<volatile uint32_t*>(s_clf) = 1u;
+                }
+                asm volatile("griddepcontrol.wait;" ::: "memory");
+            }
+            if (!step_live()) break;
+            if (epi) smem_word(s_clf, p.status);
+            stamp = smem_word(s_stamp, p.status);
+            __syncwarp();
+            set = p.sync + 4 + 4 * (stamp & 1u);
+            // Have all CTAs of the grid started?  Until then none of their records may be waited for.
+            int all = 0;
+            if (lane == 0) {
+                for (;;) {
+                    const bool done = *reinterpret_cast<volatile int*>(s_done) == kDbEpiWarps;
+                    __threadfence_block();
+                    all = ld_relaxed_u32(set) == gridDim.x;
+                    if (all || done) break;
+                    __nanosleep(300);   // (148 CTAs polling one word without a pause held everybody up by 5 us)
+                }
+            }
+            if (!__shfl_sync(kFullMask, all, 0)) break;
+        }
+        // the next row nobody has taken
+        int first = 0;
+        if (lane == 0) first = (int)atomicAdd(set + 1, 1u);
+        b = __shfl_sync(kFullMask, first, 0);
+        if (b == 0 && lane == 0) db_move_on(p, stamp);
+        if (b >= f.B) break;
+        run = chain_seq_live(f.chain, f.active, chain_seq(f.chain, b));
+        // The records of the other CTAs will not be there before this CTA's own: polling them earlier only loads L2.
+        if (lane == 0 && !epi)
+            for (int i = 0; i < (1 << 20) && *reinterpret_cast<volatile int*>(s_done) != kDbEpiWarps; ++i) __nanosleep(32);
+        __syncwarp();
+    }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -409,7 +552,7 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
     uint32_t* s_stamp = tmem_base_s + 2;                      // stamp of this launch (0: not read yet, or nothing to do)
     float4* xch = reinterpret_cast<float4*>(reinterpret_cast<uint8_t*>(full) + 512);
     float* fin_s = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(xch) + kDbXchBytes);
-    float* row_thr_s = fin_s + (p.all_finish ? kDbFinWarps + kDbEpiWarps : kDbFinWarps) * kDbFinWords;     // [128] the rows' bounds
+    float* row_thr_s = fin_s + (p.all_finish || p.finishers ? kDbFinWarps + kDbEpiWarps : kDbFinWarps) * kDbFinWords;     // [128] the rows' bounds
     float* turn_s = row_thr_s + 128;                          // with probs: 32 rows of one chunk per epilogue warp
     float* clf_s = turn_s + (p.probs ? kDbEpiWarps * 32 * kDbTurnStride : 0);
 
@@ -591,7 +734,8 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
             }
         }
     }
-    if (warp >= 2 && warp < 2 + kDbEpiWarps) {
+    const bool finisher = p.finishers > 0 && nslot >= p.CN;
+    if (warp >= 2 && warp < 2 + kDbEpiWarps && !finisher) {
         // ------------------------------ epilogue ------------------------------
         const int ew = warp - 2;
         const int quad = warp & 3;              // TMEM lane quadrant this warp may read
@@ -609,7 +753,8 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
         float* turn = turn_s + ew * 32 * kDbTurnStride;
         // Twice: a rehearsal without columns before the dependency wait (what follows the column loop is on the critical
         // path, and its instructions would come from L2 one after the other), then for good.
-        for (int phase = looks_live ? 0 : 1; phase < 2; ++phase) {
+#pragma unroll 1
+        for (int phase = opaque(looks_live ? 0 : 1); phase < 2; phase = opaque(phase + 1)) {
             bool many_kept = false;        // enough of them to store four rows per instruction
             unsigned keep_mask = 0u;       // rows of this warp whose raw logits go to probs (none of a masked sequence's)
             unsigned int *slots = nullptr, *my_slot = nullptr;
@@ -626,33 +771,14 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
             } else {
                 asm volatile("griddepcontrol.wait;" ::: "memory");  // scratch and outputs belong to the predecessor until now
                 if (!step_live()) break;
-                const uint32_t stamp = *reinterpret_cast<volatile unsigned int*>(p.sync) + 1u;
-                const uint32_t par = stamp & 1u;
-                // (that word is the other parity's: only a launch after this one writes it)
-                const int old_rows = *reinterpret_cast<volatile unsigned int*>(p.sync + 2 + (par ^ 1u));
-                if (blockIdx.x == 0)
-                    for (int i = ew * 32 + lane; i < f.clear_n; i += kDbEpiWarps * 32) f.clear_words[i] = 0u;
                 // Rows of sequences that are masked or have stopped drafting: nobody wants their candidates, and no record of
                 // them is written.
                 valid = valid && chain_seq_live(f.chain, f.active, chain_seq(f.chain, row));
                 keep_mask = __ballot_sync(kFullMask, p.probs && valid);
                 many_kept = __popc(keep_mask) > 8 && (reinterpret_cast<uintptr_t>(p.probs) & 15) == 0;
-                slots = p.bound + par * p.set_words + (size_t)(valid ? row : 0) * kDbBoundStride;
+                const uint32_t stamp = db_begin(p, f, ew, s_stamp, lane);
+                slots = p.bound + (stamp & 1u) * p.set_words + (size_t)(valid ? row : 0) * kDbBoundStride;
                 my_slot = slots + nslot % kDbBoundSlots;
-                uint4* old = reinterpret_cast<uint4*>(p.bound + (par ^ 1u) * p.set_words);
-                for (int i = blockIdx.x * (kDbEpiWarps * 32) + ew * 32 + lane; i < old_rows * (kDbBoundStride / 4);
-                     i += gridDim.x * (kDbEpiWarps * 32))
-                    old[i] = make_uint4(0, 0, 0, 0);
-                __syncwarp();
-                // This CTA has started once all of its eight reads of the stamp are done: the stamp may be moved on as soon as every
-                // CTA counts as started, and a warp that read the moved word would work on the next launch's set of bounds.  (One
-                // warp that reads and hands the stamp to the others through shared memory: their polling costs the step up to 3 %,
-                // eight rows of 49152 x 768 kept and drawn 30.9 us against 30.1.)
-                named_barrier_sync_after(8, kDbEpiWarps * 32, stamp);
-                if (ew == 0 && lane == 0) {
-                    *reinterpret_cast<volatile uint32_t*>(s_stamp) = stamp;
-                    atomicAdd(p.sync + 4 + 4 * par, 1u);
-                }
             }
             const int phase_tiles = phase == 0 ? 0 : tiles;
 
@@ -897,17 +1023,20 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
                     }
                 }
                 // Statistics that are no numbers (logits that are infinite or no numbers themselves): the record is as good as empty.
-                if (!(Z > 0.f)) cnt = 0u;
+                if (!(Z > 0.f)) {
+                    cnt = 0u;
+                    top.init();
+                }
                 if (valid && phase == 1) {
                     const uint32_t word = (cnt << 28) | (best_v == m && Z > 0.f ? (uint32_t)best_i : kDbNoIndex);
-                    float4* rec = p.part_rec + ((size_t)row * p.CN + nslot) * kStampedPieces;
+                    float4* rec = p.part_rec + (size_t)row * p.CN * kStampedPieces + nslot;
                     const float sf = __uint_as_float(smem_word(s_stamp, p.status));   // (written microseconds ago)
                     store_relaxed_v4(rec, m + 0.f, Z, S, sf);
-                    store_relaxed_v4(rec + 1, __uint_as_float(word), top.t[0], bound_used, sf);
-                    store_relaxed_v4(rec + 2, top.t[1], top.t[2], top.t[3], sf);
+                    store_relaxed_v4(rec + p.CN, __uint_as_float(word), top.t[0], bound_used, sf);
+                    store_relaxed_v4(rec + 2 * p.CN, top.t[1], top.t[2], top.t[3], sf);
                     if (cnt > 4) {
-                        store_relaxed_v4(rec + 3, top.t[4], top.t[5], top.t[6], sf);
-                        store_relaxed_v4(rec + 4, top.t[7], top.t[8], top.t[9], sf);
+                        store_relaxed_v4(rec + 3 * p.CN, top.t[4], top.t[5], top.t[6], sf);
+                        store_relaxed_v4(rec + 4 * p.CN, top.t[7], top.t[8], top.t[9], sf);
                     }
                 }
             }
@@ -918,77 +1047,10 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
             }
         }
     }
-    // ------------------------------ finishing rows ------------------------------
-    // The finishing warps, from the start of the launch; with more rows than those of the whole grid, the epilogue warps as
-    // well once their records are out.
-    const bool epi = warp < 2 + kDbEpiWarps;
-    if (warp >= 2 && (!epi || p.all_finish)) {
-        const int fw = epi ? kDbFinWarps + warp - 2 : warp - 2 - kDbEpiWarps;
-        float* sm = fin_s + fw * kDbFinWords;
-        if (!epi && f.clf_H > 0) {   // classifier parameters -> shared
-            const int Hc = f.clf_H, n1 = Hc * kNFeat;
-            for (int i = fw * 32 + lane; i < n1 + 2 * Hc + 1; i += kDbFinWarps * 32) {
-                const float* src = i < n1 ? f.clf_W1 + i
-                                          : (i < n1 + Hc ? f.clf_b1 + (i - n1)
-                                                         : (i < n1 + 2 * Hc ? f.clf_w2 + (i - n1 - Hc) : f.clf_b2));
-                cp_async4(clf_s + i, src);
-            }
-            cp_async_commit();
-        }
-        uint32_t stamp = 1u;
-        unsigned int* set = nullptr;
-        int b = 0;
-        bool run = !epi && looks_live;
-        for (bool real = false;; real = true) {
-            if (run && !(real && !chain_seq_live(f.chain, f.active, chain_seq(f.chain, b)))) db_finish_row(p, f, b, real, stamp + (real ? f.test_stamp_skew : 0u), sm, clf_s, STATS, lane);
-            run = true;
-            if (!real) {
-                if (!epi) {
-                    cp_async_wait_all();
-                    named_barrier_sync(3, kDbFinWarps * 32);
-                    if (fw == 0 && lane == 0) {
-                        __threadfence_block();
-                        *reinterpret_cast<volatile uint32_t*>(s_clf) = 1u;
-                    }
-                    asm volatile("griddepcontrol.wait;" ::: "memory");
-                }
-                if (!step_live()) break;
-                if (epi) smem_word(s_clf, p.status);
-                stamp = smem_word(s_stamp, p.status);
-                __syncwarp();
-                set = p.sync + 4 + 4 * (stamp & 1u);
-                // Have all CTAs of the grid started?  Until then none of their records may be waited for.
-                int all = 0;
-                if (lane == 0) {
-                    for (;;) {
-                        const bool done = *reinterpret_cast<volatile int*>(s_done) == kDbEpiWarps;
-                        __threadfence_block();
-                        all = ld_relaxed_u32(set) == gridDim.x;
-                        if (all || done) break;
-                        __nanosleep(300);   // (148 CTAs polling one word without a pause held everybody up by 5 us)
-                    }
-                }
-                if (!__shfl_sync(kFullMask, all, 0)) break;
-                // The records of the other CTAs will not be there before this CTA's own: polling them earlier only loads L2.
-                if (lane == 0 && !epi)
-                    for (int i = 0; i < (1 << 20) && *reinterpret_cast<volatile int*>(s_done) != kDbEpiWarps; ++i) __nanosleep(100);
-                __syncwarp();
-            }
-            // the next row nobody has taken
-            int first = 0;
-            if (lane == 0) first = (int)atomicAdd(set + 1, 1u);
-            b = __shfl_sync(kFullMask, first, 0);
-            if (b == 0 && lane == 0) {
-                // All CTAs have started: the stamp can move on, and the counters of the next launch (this one's may
-                // still be looked at) start at zero.
-                unsigned int* other = p.sync + 4 + 4 * ((stamp + 1u) & 1u);
-                other[0] = 0u;
-                other[1] = 0u;
-                p.sync[2 + (stamp & 1u)] = (unsigned int)p.R;
-                p.sync[0] = stamp == 0xffffffffu ? 1u : stamp;   // never zero, and the two sets keep alternating
-            }
-            if (b >= f.B) break;
-        }
+    if (finisher) {
+        if (warp >= 2) db_finish_dedicated<STATS>(p, f, warp, looks_live, fin_s, clf_s, s_stamp, step_live, lane);
+    } else if (warp >= 2 && p.finishers == 0) {
+        db_finish_rows<STATS>(p, f, warp, looks_live, fin_s, clf_s, s_done, s_clf, s_stamp, step_live, lane);
     }
 
     tc_fence_before();

@@ -91,8 +91,8 @@ __device__ __forceinline__ void block_cdf_walk(WeightFn w, int c0, int c1, doubl
 struct DrawRowsParams {
     float* probs;             // [B, V]
     const float* stats;       // [B][2]
-    const float4* recs;       // [B][NP] records of rec_pieces * 16 bytes that start with m, Z
-    int rec_pieces, NP;
+    const float4* recs;       // records that start with m, Z: NP per row, rec_step * 16 bytes apart, rows rec_row * 16 bytes
+    int rec_step, rec_row, NP;
     int slab;                 // vocabulary rows per record
     int seg_slabs;            // slabs per segment
     int V;
@@ -119,14 +119,14 @@ static __global__ void __launch_bounds__(kSampleThreads) draw_rows_kernel(const 
     if (t < 32) {
         // a few consecutive records per lane, running sums in record order
         const int q = (p.NP + 31) / 32, c0 = min(p.NP, lane * q), c1 = min(p.NP, c0 + q);
-        const float4* rec = p.recs + (size_t)b * p.NP * p.rec_pieces;
+        const float4* rec = p.recs + (size_t)b * p.rec_row;
         // (the first few are fetched side by side: a loop of dependent loads is a round trip each)
         constexpr int kAhead = 5;
         float2 mz[kAhead];
 #pragma unroll
         for (int i = 0; i < kAhead; ++i) {
             mz[i] = make_float2(0.f, 0.f);
-            if (c0 + i < c1) mz[i] = __ldcg(reinterpret_cast<const float2*>(rec + (size_t)(c0 + i) * p.rec_pieces));
+            if (c0 + i < c1) mz[i] = __ldcg(reinterpret_cast<const float2*>(rec + (size_t)(c0 + i) * p.rec_step));
         }
         auto mass_of = [&](const float2& r) {
             return r.y > 0.f ? static_cast<double>(r.y) * static_cast<double>(expf(r.x - m)) : 0.0;
@@ -140,7 +140,7 @@ static __global__ void __launch_bounds__(kSampleThreads) draw_rows_kernel(const 
             mine += w_first[i];
             if (w_first[i] > 0.0) last = c0 + i;
         }
-        auto mass = [&](int c) { return mass_of(__ldcg(reinterpret_cast<const float2*>(rec + (size_t)c * p.rec_pieces))); };
+        auto mass = [&](int c) { return mass_of(__ldcg(reinterpret_cast<const float2*>(rec + (size_t)c * p.rec_step))); };
         for (int c = c0 + kAhead; c < c1; ++c) {
             const double w = mass(c);
             mine += w;

@@ -385,3 +385,23 @@ def test_feature_extraction_by_pairs_of_ctas(N, V, d):
 @pytest.mark.parametrize("V,rows", [(300, 129), (300, 256), (2500, 500), (20000, 180), (400, 1160), (700, 1409)])
 def test_verification_by_pairs_of_ctas(oracle, V, rows):
     _verification_agrees(oracle, V, rows // 8, rows, 1032)
+
+
+# Few hidden rows, the vocabulary on the lanes: the rows a warp holds (8, 16, 32), tiles of exactly 32 and 128 vocabulary rows
+# and one more or less, more tiles than accumulators (2100 rows per SM: 17 tiles), CTAs without a vocabulary row
+@pytest.mark.parametrize("rows_per_sm,extra,B", [(31, 0, 1), (32, 1, 8), (33, 0, 9), (127, 3, 16), (128, 1, 17), (129, 0, 32),
+                                                 (257, -2, 33), (2100, 5, 3), (2100, 0, 20), (1, -100, 2)])
+def test_few_rows_at_the_edges_of_their_tiling(oracle, rows_per_sm, extra, B):
+    V, d = _sms() * rows_per_sm + extra, 40 if rows_per_sm < 1000 else 16
+    W, h = inputs.lm_head(V, d, seed=V + B, std=0.3), inputs.hidden(B, d, seed=B)
+    params = make_clf(16, seed=1)
+    pos, nd = np.arange(1, B + 1, dtype=np.int32), (np.arange(B, dtype=np.int32) % 4) + 1
+    active = (np.arange(B) % 5 != 2).astype(np.uint8)
+    ctx = binding.Context(V, d, 8, max_batch=B, max_rows=8, clf_hidden=16)
+    Wg, clf = W.cuda(), to_gpu_clf(params)
+    for act in (None, active, None):
+        got = gpu_draft_step(ctx, Wg, h, pos, nd, clf, 0.5, 3, active=act, want_probs=True)
+        ref = oracle.draft_step(_bits(W), _bits(h), pos, nd, to_oracle_clf(oracle, params), 0.5, 3, active=act, want_probs=True, nthreads=8)
+        _check_draft_and_each_probability(got, ref, 0.5, active=act)
+    assert ctx.device_status() == 0
+    ctx.close()
