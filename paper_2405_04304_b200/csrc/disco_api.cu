@@ -14,6 +14,7 @@
 #include "umma_tail.cuh"
 #include "draft_batch.cuh"
 #include "draft_few.cuh"
+#include "fetch.cuh"
 #include "sample.cuh"
 #include "umma_gemv_loop.cuh"
 
@@ -26,6 +27,11 @@ constexpr int kMaxHidden = 16384;    // widest hidden dimension the kernels acce
 constexpr int kSlotTargetBytes = 6144;
 
 constexpr int kMaxDevices = 64;
+// Hidden states that disco_iteration_host has a kernel bring over rather than the copy engine: by then the engine's second copy,
+// which runs beside the draft phase, has made up for what its first one and the events around it cost (us per call, 32000 x 768
+// and a target of the width given, engine -> kernel: 37 KB 69.0 -> 65.0, 150 KB 107.6 -> 104.4, 230 KB 108.1 -> 106.0, 256 KB 106.6 ->
+// 104.0, 420 KB 106.7 -> 109.5, 490 KB 84.4 -> 86.5).
+constexpr size_t kFetchBytes = 288 * 1024;
 
 // One-time, per-device configuration of one kernel (its dynamic shared-memory limit).  Every template
 // instance of a launcher owns one of these; the lock makes first calls from several host threads, and
@@ -83,9 +89,11 @@ struct disco_ctx {
     unsigned int* row_bound;       // batched draft step: two sets of [part_rows][kDbBoundStride] words, see DraftBatchParams
     int part_slots;                // partials per row the buffers can hold
     void* encode_tiled;            // cuTensorMapEncodeTiled, resolved through the runtime
+    void* pointer_attributes;      // cuPointerGetAttributes, the same way
     // device staging for the *_host entry points
     void* stage_hidden;
     void* stage_hidden_draft;      // disco_iteration_host: the draft hidden states of all steps
+    int32_t* stage_dev;            // disco_iteration_host: pos0 | sl_forced (max_batch each) | draft_ids (max_rows)
     cudaStream_t copy_stream;      // disco_iteration_host: the target hidden states travel beside the draft phase
     cudaEvent_t copy_done;
     // Small inputs and outputs of the *_host entry points live in pinned host memory that the GPU maps:
@@ -642,6 +650,9 @@ int disco_create(disco_ctx** out, int V, int d_draft, int d_target, int max_batc
         if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres) == cudaSuccess &&
             qres == cudaDriverEntryPointSuccess)
             c->encode_tiled = fn;
+        if (cudaGetDriverEntryPoint("cuPointerGetAttributes", &fn, cudaEnableDefault, &qres) == cudaSuccess &&
+            qres == cudaDriverEntryPointSuccess)
+            c->pointer_attributes = fn;
     }
     // the largest layout is disco_iteration_host's: 6 arrays of max_batch words and 2 of max_rows
     const size_t n_int = (size_t)8 * max_batch + (size_t)3 * max_rows + 64;
@@ -679,6 +690,7 @@ int disco_create(disco_ctx** out, int V, int d_draft, int d_target, int max_batc
     device(&c->pack_off, ((size_t)std::max(max_batch, max_rows) + 1) * sizeof(int32_t));
     device(&c->stage_hidden, hid);
     device(&c->stage_hidden_draft, (size_t)max_rows * d_draft * 2);
+    device(&c->stage_dev, (2 * (size_t)max_batch + (size_t)max_rows) * sizeof(int32_t));
     auto pinned = [&](size_t bytes) {
         const size_t at = host_bytes;
         host_bytes += (bytes + 255) & ~(size_t)255;
@@ -771,6 +783,22 @@ cudaError_t launch_after(const disco_ctx* c, void (*kern)(KArgs...), dim3 grid, 
     cfg.attrs = attr;
     cfg.numAttrs = c->pdl ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+}
+
+// Host memory as the device sees it, if all of [p, p + bytes) is pinned, 16-byte aligned memory of one allocation.
+const void* device_view(const disco_ctx* c, const void* p, size_t bytes) {
+    if (!c->pointer_attributes || !aligned16(p)) return nullptr;
+    unsigned int type = 0;
+    unsigned long long dev = 0, start = 0;
+    size_t size = 0;
+    CUpointer_attribute what[4] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                   CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void* where[4] = {&type, &dev, &start, &size};
+    using Fn = CUresult (*)(unsigned int, CUpointer_attribute*, void**, CUdeviceptr);
+    const unsigned long long at = reinterpret_cast<unsigned long long>(p);
+    if (reinterpret_cast<Fn>(c->pointer_attributes)(4, what, where, at) != CUDA_SUCCESS) return nullptr;
+    if (type != CU_MEMORYTYPE_HOST || dev == 0 || (dev & 15u) || at < start || at + bytes > start + size) return nullptr;
+    return reinterpret_cast<const void*>(dev);
 }
 
 // Shared body of the LM-head + soft-max passes: B rows of hidden size d against the head W.
@@ -1320,29 +1348,63 @@ int disco_iteration_host(disco_ctx* c, const void* W_D, size_t w_step_stride, co
     std::memcpy(h_tok, token_host, SB * 4);
     std::memcpy(h_conf, conf_host, SB * 4);
     std::memcpy(h_halt, halt_host, SB);
+    auto hand_back = [&]() {
+        std::memcpy(token_host, h_tok, SB * 4);
+        std::memcpy(conf_host, h_conf, SB * 4);
+        std::memcpy(halt_host, h_halt, SB);
+        std::memcpy(sl_host, h_sl, (size_t)B * 4);
+        std::memcpy(n_accept_host, h_nacc, (size_t)B * 4);
+        std::memcpy(bonus_host, h_bonus, (size_t)B * 4);
+        if (pos_next_host) std::memcpy(pos_next_host, h_next, (size_t)B * 4);
+        return (int)DISCO_OK;
+    };
+    const size_t bytes_D = SB * c->d_draft * 2, bytes_T = R * c->d_target * 2;
+    const void *src_D = nullptr, *src_T = nullptr;
+    const bool fetch = bytes_D + bytes_T <= kFetchBytes && (src_D = device_view(c, h_D_host, bytes_D)) != nullptr &&
+                       (src_T = device_view(c, H_T_host, bytes_T)) != nullptr;
+    if (fetch) {
+        // Little to move, all of it pinned: one kernel brings it over, and the draft phase's launch and its first loads of the
+        // LM head run meanwhile.
+        FetchParams fp{};
+        int32_t* dev = c->stage_dev;     // pos0 | forced | ids
+        auto part = [&fp](const void* src, void* dst, size_t bytes, unsigned unit) {
+            fp.part[fp.n++] = FetchPart{src, dst, (unsigned)(bytes / unit), unit == 16 ? 1u : 0u};
+        };
+        part(src_D, c->stage_hidden_draft, bytes_D, 16);
+        part(src_T, c->stage_hidden, bytes_T, 16);
+        part(dev_i(h_pos), dev, (size_t)B * 4, 4);
+        if (sl_forced_host) part(dev_i(h_forced), dev + mb, (size_t)B * 4, 4);
+        if (draft_ids_host) part(dev_i(h_ids), dev + 2 * mb, SB * 4, 4);
+        unsigned pieces = 0;
+        for (int i = 0; i < fp.n; ++i) pieces += fp.part[i].pieces;
+        cudaError_t e = launch_after(c, fetch_kernel, dim3((pieces + kFetchThreads - 1) / kFetchThreads), dim3(kFetchThreads), 0, st, fp);
+        c->launches += 1;
+        if (!cuda_ok(e, "fetch_kernel launch")) return DISCO_ERR_CUDA;
+        const int rc = iteration_impl(c, W_D, w_step_stride, c->stage_hidden_draft, W_T, c->stage_hidden, B, dev, clf, tau, sl_max,
+                                      sl_forced_host ? dev + mb : nullptr, draft_ids_host ? dev + 2 * mb : nullptr,
+                                      dev_i(h_tok), c->stage_float_d, c->stage_byte_d, nullptr, dev_i(h_sl), dev_i(h_nacc),
+                                      dev_i(h_bonus), nullptr, nullptr, pos_next_host ? dev_i(h_next) : nullptr, stream, nullptr, 0);
+        const bool done = cudaStreamSynchronize(st) == cudaSuccess;   // (the user's memory is read until here)
+        if (rc) return rc;
+        if (!done) return DISCO_ERR_CUDA;
+        return hand_back();
+    }
     // The draft phase needs the draft hidden states only: the (larger) target hidden states are sent once it is
     // enqueued, on a stream of their own, and the verification waits for them.  (Every host entry point returns with its
     // work done, so nothing earlier still reads the staging buffers.)
-    if (cudaMemcpyAsync(c->stage_hidden_draft, h_D_host, SB * c->d_draft * 2, cudaMemcpyHostToDevice, st) != cudaSuccess)
+    if (cudaMemcpyAsync(c->stage_hidden_draft, h_D_host, bytes_D, cudaMemcpyHostToDevice, st) != cudaSuccess)
         return DISCO_ERR_CUDA;
     int rc = iteration_impl(c, W_D, w_step_stride, c->stage_hidden_draft, W_T, c->stage_hidden, B, dev_i(h_pos), clf, tau,
                             sl_max, sl_forced_host ? dev_i(h_forced) : nullptr, draft_ids_host ? dev_i(h_ids) : nullptr,
                             dev_i(h_tok), c->stage_float_d, c->stage_byte_d, nullptr, dev_i(h_sl), dev_i(h_nacc),
                             dev_i(h_bonus), nullptr, nullptr, pos_next_host ? dev_i(h_next) : nullptr, stream, H_T_host,
-                            R * c->d_target * 2);
+                            bytes_T);
     if (rc) {
         cudaStreamSynchronize(c->copy_stream);   // the copy must not outlive the call
         return rc;
     }
     if (cudaStreamSynchronize(st) != cudaSuccess) return DISCO_ERR_CUDA;
-    std::memcpy(token_host, h_tok, SB * 4);
-    std::memcpy(conf_host, h_conf, SB * 4);
-    std::memcpy(halt_host, h_halt, SB);
-    std::memcpy(sl_host, h_sl, (size_t)B * 4);
-    std::memcpy(n_accept_host, h_nacc, (size_t)B * 4);
-    std::memcpy(bonus_host, h_bonus, (size_t)B * 4);
-    if (pos_next_host) std::memcpy(pos_next_host, h_next, (size_t)B * 4);
-    return DISCO_OK;
+    return hand_back();
 }
 
 }  // extern "C"

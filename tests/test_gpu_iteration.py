@@ -437,3 +437,38 @@ def test_iteration_of_many_rows_counted_on_the_device(oracle):
         check_iteration(oracle, got, ref, W_T, H_T, 0.5, S, ids)
     assert ctx.device_status() == 0
     ctx.close()
+
+
+@pytest.mark.parametrize("memory", ["pinned", "pageable", "pinned, 8 bytes in"])
+@pytest.mark.parametrize("B,forced", [(1, False), (3, True), (40, False)])
+def test_host_iteration_from_any_host_memory(memory, B, forced):
+    """Pinned hidden states of up to 288 KB are fetched by a kernel, others by the copy engine (40 sequences: 700 KB)."""
+    V, dD, dT, S = 1000, 72, 1032, 7
+    W_D, W_T, h_D, H_T = make_inputs(V, dD, dT, B, S, seed=17)
+    pos0 = (np.arange(B, dtype=np.int32) * 3) % 6
+    clf = to_gpu_clf(position_clf(cut=6.0))
+    ids = np.random.default_rng(B).integers(0, V, size=(B, S)).astype(np.int32)
+    fs = (np.arange(B, dtype=np.int32) % S) + 1 if forced else None
+    ctx = binding.Context(V, dD, dT, max_batch=B + 2, max_rows=(B + 2) * (S + 1), clf_hidden=8)
+    dev = gpu_iteration(ctx, W_D, W_T, h_D, H_T, pos0, clf, 0.5, S, sl_forced=fs, draft_ids=ids)
+
+    def host(t):
+        if memory == "pageable":
+            return t.contiguous().clone()
+        skip = 0 if memory == "pinned" else 8 // t.element_size()
+        buf = torch.empty(t.numel() + skip, dtype=t.dtype).pin_memory()
+        buf[skip:] = t.reshape(-1)
+        return buf[skip:].view(t.shape)
+
+    token, conf = host(torch.full((S, B), -7, dtype=torch.int32)), host(torch.full((S, B), -7.0))
+    halt = host(torch.full((S, B), 77, dtype=torch.uint8))
+    sl, n_acc, bonus, nxt = (host(torch.full((B,), -7, dtype=torch.int32)) for _ in range(4))
+    for _ in range(2):
+        ctx.iteration_host(W_D.cuda(), host(h_D), W_T.cuda(), host(H_T), host(torch.from_numpy(pos0)), clf, 0.5, S, token, conf,
+                           halt, sl, n_acc, bonus, draft_ids=host(torch.from_numpy(ids)), pos_next=nxt,
+                           sl_forced=None if fs is None else host(torch.from_numpy(fs)))
+    for k, t in (("token", token), ("conf", conf), ("halt", halt), ("sl", sl), ("n_accept", n_acc), ("bonus", bonus),
+                 ("pos_next", nxt)):
+        np.testing.assert_array_equal(t.numpy(), dev[k])
+    assert ctx.device_status() == 0
+    ctx.close()
