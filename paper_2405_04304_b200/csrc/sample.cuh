@@ -257,15 +257,26 @@ struct SampleRowsParams {
     int* status;
 };
 
-static __global__ void __launch_bounds__(kSampleThreads) sample_rows_fused_kernel(const SampleRowsParams p) {
+static __global__ void __launch_bounds__(kSampleThreads, 2) sample_rows_fused_kernel(const SampleRowsParams p) {
     __shared__ double sh[40];
     __shared__ double red[4][kSampleWarps];
-    __shared__ int s_b, s_n, s_skip, s_last, s_lastpos[2];
+    __shared__ int s_b, s_r0, s_r1, s_n, s_skip, s_last, s_lastpos[2];
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int r = blockIdx.x / p.SEG, s = blockIdx.x - r * p.SEG;
     const int V = p.V;
+    // A chain of round trips to L2 bounds this kernel, so whatever waits for nothing is on its way first: the row's statistics
+    // and this CTA's logits.
+    float* y = p.y_T + (size_t)r * V;
+    const float m = p.stats[2 * r], Z = p.stats[2 * r + 1];
+    const int v_lo = min(V, s * p.seg_len), v_hi = min(V, v_lo + p.seg_len);
+    float z_first[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const int v = v_lo + t + k * kSampleThreads;
+        z_first[k] = v < v_hi ? __ldcg(y + v) : 0.f;
+    }
     // malformed offsets are reported once per sequence, by the first CTA of row b
     if (p.row_off && r < p.B && s == 0 && t == 0) {
         const int b = r, r0 = p.row_off[b], r1 = p.row_off[b + 1];
@@ -277,37 +288,33 @@ static __global__ void __launch_bounds__(kSampleThreads) sample_rows_fused_kerne
     }
     if (t == 0) {
         s_b = p.row_off ? -1 : r / (p.SL + 1);
+        s_r0 = s_b * (p.SL + 1);
+        s_r1 = s_r0 + p.SL + 1;
         s_skip = -1;
         s_lastpos[0] = s_lastpos[1] = -1;
     }
     __syncthreads();
     if (p.row_off) {
-        for (int b = t; b < p.B; b += kSampleThreads)
-            if (p.row_off[b] <= r && r < p.row_off[b + 1]) s_b = b;
+        for (int b = t; b < p.B; b += kSampleThreads) {
+            const int lo = p.row_off[b], hi = p.row_off[b + 1];
+            if (lo <= r && r < hi && atomicCAS(&s_b, -1, b) == -1) s_r0 = lo, s_r1 = hi;   // (one of them, if the offsets are malformed)
+        }
         __syncthreads();
     }
-    const int b = s_b;
+    const int b = s_b, r0 = s_r0, r1 = s_r1;
     if (b < 0) return;
-    int r0, r1;
-    if (p.row_off) {
-        r0 = p.row_off[b];
-        r1 = p.row_off[b + 1];
-        if (r0 < b || r1 <= r0 || r1 > p.R - (p.B - 1 - b) || (b == 0 && r0 != 0) || (b == p.B - 1 && r1 != p.R)) return;
-    } else {
-        r0 = b * (p.SL + 1);
-        r1 = r0 + p.SL + 1;
-    }
+    if (p.row_off && (r0 < b || r1 <= r0 || r1 > p.R - (p.B - 1 - b) || (b == 0 && r0 != 0) || (b == p.B - 1 && r1 != p.R))) return;
     const int sl = r1 - r0 - 1;
-    // (loads that wait for nothing are issued first: the uniform of the draw, this CTA's first logits)
     const float u_draw = p.u_sample[b];
-    float* y = p.y_T + (size_t)r * V;
-    const float m = p.stats[2 * r], inv_Z = 1.f / p.stats[2 * r + 1];
-    const int v_lo = min(V, s * p.seg_len), v_hi = min(V, v_lo + p.seg_len);
-    float z_first[8];
+    const float inv_Z = 1.f / Z;
+    // If this row is the one drawn from, it is so after r - r0 accepted tokens, and that is the draft distribution it takes:
+    // requested before the acceptance tests say whether (3 MB in all for 30 rows of 32000).
+    const float* yD_here = r - r0 < sl ? p.draft_probs + ((size_t)(r - r0) * p.B + b) * V : nullptr;
+    float d_first[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
         const int v = v_lo + t + k * kSampleThreads;
-        z_first[k] = v < v_hi ? __ldcg(y + v) : 0.f;
+        d_first[k] = (yD_here && v < v_hi) ? __ldg(yD_here + v) : 0.f;
     }
     // acceptance tests of all positions side by side, then the first that fails
     if (t == 0) s_n = sl;
@@ -335,7 +342,7 @@ static __global__ void __launch_bounds__(kSampleThreads) sample_rows_fused_kerne
     __syncthreads();
     const int n = s_n, skip = s_skip;
     const bool draw_row = r == r0 + n;
-    const float* yD = (draw_row && n < sl) ? p.draft_probs + ((size_t)n * p.B + b) * V : nullptr;
+    const float* yD = draw_row ? yD_here : nullptr;
     double acc_w = 0.0, acc_y = 0.0;
     int last_w = -1, last_y = -1;
     for (int v0 = v_lo + t; v0 < v_hi; v0 += 8 * kSampleThreads) {
@@ -344,7 +351,7 @@ static __global__ void __launch_bounds__(kSampleThreads) sample_rows_fused_kerne
         for (int k = 0; k < 8; ++k) {
             const int v = v0 + k * kSampleThreads;
             z[k] = v0 == v_lo + t ? z_first[k] : (v < v_hi ? __ldcg(y + v) : 0.f);
-            d[k] = (yD && v < v_hi) ? __ldg(yD + v) : 0.f;
+            d[k] = v0 == v_lo + t ? d_first[k] : (yD && v < v_hi) ? __ldg(yD + v) : 0.f;
         }
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
@@ -377,12 +384,17 @@ static __global__ void __launch_bounds__(kSampleThreads) sample_rows_fused_kerne
             atomicMax(&s_lastpos[1], last_y);
         }
         __syncthreads();
-        if (t == 0) {
-            double tw = 0.0, ty = 0.0;
-            for (int k = 0; k < kSampleWarps; ++k) {
-                tw += red[0][k];
-                ty += red[1][k];
+        if (warp == 0) {
+            double tw = lane < kSampleWarps ? red[0][lane] : 0.0, ty = lane < kSampleWarps ? red[1][lane] : 0.0;
+#pragma unroll
+            for (int off = kSampleWarps / 2; off > 0; off >>= 1) {
+                tw += __shfl_xor_sync(kFullMask, tw, off);
+                ty += __shfl_xor_sync(kFullMask, ty, off);
             }
+            acc_w = tw, acc_y = ty;
+        }
+        if (t == 0) {
+            const double tw = acc_w, ty = acc_y;
             const size_t at = ((size_t)b * kSampleMaxSegments + s) * 2;
             p.seg_tot[at] = tw;
             p.seg_tot[at + 1] = ty;
