@@ -281,6 +281,16 @@ bool verify_in_pairs(const disco_ctx* c, int R, int d, bool dev_R, int likely_R)
     return 32ll * two.TPC * two.TRN * std::min(two.GS, two.MT) <= 33ll * one.TPC * one.TRN * std::min(one.GS, one.MT);
 }
 
+// CTAs that do nothing but finish a verification in the kernel that projects it (umma_tail.cuh), a warp for each sequence; 0: the
+// rest must not get more to do for it, and there is a limit.  (us, 32000 x 5120 head, 11 rows of one sequence, launches one
+// after the other: the last CTA to take a ticket finishes 53.5, a CTA of its own 52.3.)
+int verify_finishers(const disco_ctx* c, int R, int d, int B) {
+    const int n = (B + kUmmaEpiWarps - 1) / kUmmaEpiWarps;
+    if (n > 8 || !VerifyTiling::possible(R, c->sm_count - n)) return 0;
+    const VerifyTiling all = VerifyTiling::make(R, c->V, d, c->sm_count), less = VerifyTiling::make(R, c->V, d, c->sm_count - n);
+    return less.TPC == all.TPC && less.GS == all.GS && less.TRN <= all.TRN + (R <= 128 ? 16 : 0) ? n : 0;   // (one tile: HBM is the bound)
+}
+
 // Launch the tcgen05 verification kernel for R hidden rows of width d against the LM head W [V, d].
 int launch_umma(disco_ctx* c, const void* W, const void* H, int d, int R, const UmmaParams* fused, cudaStream_t st,
                 const int32_t* dev_R = nullptr, int likely_R = 0) {
@@ -293,7 +303,7 @@ int launch_umma(disco_ctx* c, const void* W, const void* H, int d, int R, const 
     const bool lanes = !dev_R && verify_on_lanes(c, R, d);
     const bool wide = lanes && R > kUmmaLaneRows;
     const bool pair = !lanes && verify_in_pairs(c, R, d, dev_R != nullptr, likely_R);
-    p.t = pair ? VerifyTiling::make_pairs(R, c->V, d, c->sm_count) : VerifyTiling::make(R, c->V, d, c->sm_count);
+    p.t = pair ? VerifyTiling::make_pairs(R, c->V, d, c->sm_count) : VerifyTiling::make(R, c->V, d, c->sm_count - p.finishers);
     // (with the row count in device memory the kernel derives the tiling)
     p.box_rows = (dev_R ? 256 : p.t.TRN) / (pair ? 2 : 1);
     p.a_rows = lanes ? (R + 15) / 16 * 16 : pair || p.t.MT > 1 ? 128 : (R + 7) / 8 * 8;
@@ -313,7 +323,7 @@ int launch_umma(disco_ctx* c, const void* W, const void* H, int d, int R, const 
     const int smem_bytes = lanes ? kUmmaLaneSmemBytes : kUmmaSmemBytes;
     if (!raise_smem_limit(c, setup[pair ? 3 : lanes + wide], kern, (size_t)smem_bytes, nullptr)) return DISCO_ERR_CUDA;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)(dev_R ? (pair ? c->sm_count & ~1 : c->sm_count) : p.t.groups * p.t.CN * (pair ? 2 : 1)));
+    cfg.gridDim = dim3((unsigned)(dev_R ? (pair ? c->sm_count & ~1 : c->sm_count) : p.t.groups * p.t.CN * (pair ? 2 : 1) + p.finishers));
     cfg.blockDim = dim3(kUmmaThreads);
     cfg.dynamicSmemBytes = (size_t)smem_bytes;
     cfg.stream = st;
@@ -956,13 +966,18 @@ int verify_common(disco_ctx* c, const void* W_T, const void* H_T, const int32_t*
         p.padded.row_off_out = nullptr;
         dev_R = c->pack_off + B;
     }
-    // Few sequences: the last CTA of the main kernel finishes the job, no second launch.  Its eight warps take the sequences in
-    // turn behind a fence and a ticket, while the second kernel's launch hides under the first (us in one / two launches,
-    // 32000 x 2048, 5 rows each: 4 sequences 26.9 / 27.3, 8 26.5 / 26.8, 16 29.0 / 28.6, 20 30.2 / 29.7, 32 35.3 / 33.4; 32000 x
-    // 5120: 54.6 / 55.1, 55.8 / 56.0, 60.0 / 59.2, 63.2 / 59.6).
-    if (B <= 16) {
+    // CTAs of their own finish the job in the same launch where that costs the others nothing (us, a second launch -> finishing
+    // CTAs, rows of 2 and 4 a sequence: 17 sequences of 32000 x 2048 26.8 / 26.5 -> 24.7 / 25.1, 32 26.8 / 27.2 -> 24.9 / 26.0, 64 28.7 /
+    // 34.8 -> 28.1 / 31.0; 17 of 8000 x 2048 13.6 / 13.3 -> 12.9 / 12.4).  Where it does not: with few sequences the last CTA of the main
+    // kernel, whose eight warps take the sequences in turn behind a fence and a ticket; with more a second launch, which hides
+    // under the first (us in one / two launches, 32000 x 2048, 5 rows each: 4 sequences 26.9 / 27.3, 8 26.5 / 26.8, 16 29.0 / 28.6, 20
+    // 30.2 / 29.7, 32 35.3 / 33.4; 32000 x 5120: 54.6 / 55.1, 55.8 / 56.0, 60.0 / 59.2, 63.2 / 59.6).
+    const bool pairs = !verify_on_lanes(c, R, c->d_target) && verify_in_pairs(c, R, c->d_target, false, R);
+    const int finishers = dev_R || pairs ? 0 : verify_finishers(c, R, c->d_target, B);
+    if (B <= 16 || finishers) {
         UmmaParams fp{};
         fp.fuse_final = 1;
+        fp.finishers = finishers;
         fp.ticket = c->ticket + 32;
         fp.draft_ids = draft_ids;
         fp.row_off = row_off;

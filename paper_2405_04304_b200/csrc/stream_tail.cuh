@@ -660,36 +660,48 @@ __device__ __forceinline__ void finalize_draft_seq(const TailParams& p, int b, i
 // One warp per sequence; lane j looks at row j of the sequence.  Three row layouts: packed rows with
 // offsets (row_off), a uniform look-ahead SL, or the fixed-shape layout with the look-ahead read from
 // device memory (pad.sl).
-__device__ __forceinline__ void verify_one_sequence(const unsigned long long* keys, const int32_t* draft_ids,
-                                                    const int32_t* row_off, int B, int SL, int R, int b,
-                                                    int32_t* n_accept, int32_t* bonus, int32_t* target_ids,
-                                                    int* status, int lane, const VerifyPadded& pad) {
+// First half: where the sequence's rows and draft ids are; lane j's first id (independent of the arg-max keys).
+struct VerifySeq {
     int r0, r1;
-    int out0 = -1;            // first row of the sequence in target_ids when that differs from its first key row
-    long long id0, idj = 1;
+    int out0;                 // first row of the sequence in target_ids when that differs from its first key row (else -1)
+    long long id0, idj;
     bool bad;
+    int first_id;
+};
+__device__ __forceinline__ VerifySeq verify_locate(const int32_t* draft_ids, const int32_t* row_off, int B, int SL, int R, int b,
+                                                   int lane, const VerifyPadded& pad) {
+    VerifySeq q;
+    q.out0 = -1;
+    q.idj = 1;
     if (pad.sl) {
         const int s = __ldcg(pad.sl + b);
-        out0 = b * (SL + 1);
-        r0 = pad.packed_off ? __ldcg(pad.packed_off + b) : out0;
-        r1 = r0 + s + 1;
-        id0 = (long long)b * pad.stride_b;
-        idj = pad.stride_j;
-        bad = s < 0 || s > SL || r0 < 0 || r1 > R;
+        q.out0 = b * (SL + 1);
+        q.r0 = pad.packed_off ? __ldcg(pad.packed_off + b) : q.out0;
+        q.r1 = q.r0 + s + 1;
+        q.id0 = (long long)b * pad.stride_b;
+        q.idj = pad.stride_j;
+        q.bad = s < 0 || s > SL || q.r0 < 0 || q.r1 > R;
     } else {
         if (row_off) {
-            r0 = row_off[b];
-            r1 = row_off[b + 1];
+            q.r0 = row_off[b];
+            q.r1 = row_off[b + 1];
         } else {
-            r0 = b * (SL + 1);
-            r1 = r0 + SL + 1;
+            q.r0 = b * (SL + 1);
+            q.r1 = q.r0 + SL + 1;
         }
-        id0 = r0 - b;
+        q.id0 = q.r0 - b;
         // every sequence owns at least one row, so row_off[b] >= b and R - row_off[b+1] >= B - 1 - b: offsets that
         // break this would put the sequence's draft ids (which start at r0 - b) outside the [R - B] array
-        bad = r0 < b || r1 <= r0 || r1 > R - (B - 1 - b) || (b == 0 && r0 != 0) || (b == B - 1 && r1 != R);
+        q.bad = q.r0 < b || q.r1 <= q.r0 || q.r1 > R - (B - 1 - b) || (b == 0 && q.r0 != 0) || (b == B - 1 && q.r1 != R);
     }
-    if (bad) {
+    q.first_id = !q.bad && lane < q.r1 - q.r0 - 1 ? __ldcg(draft_ids + q.id0 + lane * q.idj) : -1;
+    return q;
+}
+// Second half, once the keys are complete.
+__device__ __forceinline__ void verify_match(const VerifySeq& q, const unsigned long long* keys, const int32_t* draft_ids, int b,
+                                             int32_t* n_accept, int32_t* bonus, int32_t* target_ids, int* status, int lane,
+                                             const VerifyPadded& pad) {
+    if (q.bad) {
         if (lane == 0) {
             record_status(status, DISCO_ERR_INVALID_ARG);
             n_accept[b] = -1;
@@ -697,16 +709,16 @@ __device__ __forceinline__ void verify_one_sequence(const unsigned long long* ke
         }
         return;
     }
-    const int sl = r1 - r0 - 1;
+    const int sl = q.r1 - q.r0 - 1;
     int n_acc = -1, bonus_tok = -1;
     for (int j0 = 0; j0 <= sl; j0 += 32) {
         const int j = j0 + lane;
         int a = -1;
         bool match = false;
         if (j <= sl) {
-            a = key_index(__ldcg(keys + r0 + j));
-            if (target_ids) target_ids[(out0 >= 0 ? out0 : r0) + j] = a;
-            match = (j < sl) && (__ldcg(draft_ids + id0 + j * idj) == a);
+            a = key_index(__ldcg(keys + q.r0 + j));
+            if (target_ids) target_ids[(q.out0 >= 0 ? q.out0 : q.r0) + j] = a;
+            match = (j < sl) && ((j0 == 0 ? q.first_id : __ldcg(draft_ids + q.id0 + j * q.idj)) == a);
         }
         if (n_acc < 0) {  // warp-uniform
             const unsigned miss = ~__ballot_sync(kFullMask, match);  // bit set: that row ends the prefix
@@ -722,6 +734,13 @@ __device__ __forceinline__ void verify_one_sequence(const unsigned long long* ke
         bonus[b] = bonus_tok;
         if (pad.sl && pad.pos_next) pad.pos_next[b] = pad.pos0[b] + n_acc + 1;   // n_acc accepted tokens and the bonus token
     }
+}
+__device__ __forceinline__ void verify_one_sequence(const unsigned long long* keys, const int32_t* draft_ids,
+                                                    const int32_t* row_off, int B, int SL, int R, int b,
+                                                    int32_t* n_accept, int32_t* bonus, int32_t* target_ids,
+                                                    int* status, int lane, const VerifyPadded& pad) {
+    const VerifySeq q = verify_locate(draft_ids, row_off, B, SL, R, b, lane, pad);
+    verify_match(q, keys, draft_ids, b, n_accept, bonus, target_ids, status, lane, pad);
 }
 
 // Fixed-shape verification: offsets of the packed rows, row_off[b] = sum over b' < b of (sl[b'] + 1), for the

@@ -21,7 +21,9 @@
 //
 // A CTA keeps one or two tiles of hidden rows and walks over a contiguous range of vocabulary tiles (VerifyTiling).  CTAs
 // that share a vocabulary tile run side by side, so the LM head crosses HBM once and is shared through L2.
-// Results leave the CTA as one atomicMax per row; the last CTA (few sequences) or a small separate kernel finishes the job.
+// With many rows two CTAs may work as one (cta_group::2, VerifyTiling::make_pairs): the operands' way from L2 is the bound there.
+// Results leave the CTA as one atomicMax per row; CTAs of their own finish the job, a warp per sequence, or the last CTA to take
+// a ticket, or a small separate kernel (verify_finishers and what follows it in disco_api.cu say which).
 #pragma once
 
 #include <cuda.h>
@@ -110,6 +112,7 @@ struct UmmaParams {
     // verification finished inside this kernel by the last CTA (few sequences only)
     int fuse_final;
     unsigned int* ticket;
+    int finishers;         // with fuse_final: the grid's last CTAs finish eight sequences each and have no vocabulary of their own
     const int32_t* draft_ids;
     const int32_t* row_off;
     int B, SL;
@@ -655,7 +658,11 @@ umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_consta
                     atomicMax(p.keys + row, argmax_key(__fadd_rn(best_v[j], 0.f), best_i[j]));
             }
         }
-        if (p.fuse_final) {
+        if (p.finishers) {
+            __threadfence();
+            named_barrier_sync(2, kUmmaEpiWarps * 32);
+            if (ew == 0 && lane == 0) atomicAdd(p.ticket, 1u);
+        } else if (p.fuse_final) {
             // ticket: the last CTA to get here matches the prefixes and clears the keys
             __shared__ int s_last;
             __threadfence();
@@ -672,6 +679,43 @@ umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_consta
                 for (int r = ew * 32 + lane; r < p.R; r += kUmmaEpiWarps * 32) p.keys[r] = 0ull;
                 if (ew == 0 && lane == 0) *p.ticket = 0u;
             }
+        }
+    } else if (p.finishers && warp < 2 + kUmmaEpiWarps) {
+        // ------------------------------ finishers ------------------------------
+        // What does not depend on the keys is read while the others work; then the CTAs that are done are counted.  The others
+        // leave at once, so the next launch sets itself up on their SMs meanwhile.  (Blocks start in order, so these CTAs are
+        // the last ones; should one start after them, it has an SM of its own to wait for.)
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        const int ew = warp - 2, first = (int)gridDim.x - p.finishers, step = kUmmaEpiWarps * p.finishers;
+        const int b0 = ((int)blockIdx.x - first) * kUmmaEpiWarps + ew;
+        VerifySeq q{};
+        if (b0 < p.B) q = verify_locate(p.draft_ids, p.row_off, p.B, p.SL, R, b0, lane, p.padded);
+        if (lane == 0) {
+            const long long t0 = clock64();
+            for (int polls = 0; ld_relaxed_u32(p.ticket) != (unsigned)first; ++polls) {
+                __nanosleep(40);
+                if ((polls & 255) == 255 && (*reinterpret_cast<volatile int*>(p.status) == DISCO_ERR_TIMEOUT ||
+                                             clock64() - t0 > 64 * kWaitBudgetClocks)) {
+                    record_status(p.status, DISCO_ERR_TIMEOUT);
+                    break;
+                }
+            }
+            __threadfence();
+        }
+        __syncwarp();
+        for (int b = b0; b < p.B; b += step) {
+            if (b != b0) q = verify_locate(p.draft_ids, p.row_off, p.B, p.SL, R, b, lane, p.padded);
+            verify_match(q, p.keys, p.draft_ids, b, p.n_accept, p.bonus, p.target_ids, p.status, lane, p.padded);
+        }
+        if (b0 == 0) warp_write_row_offsets(p.padded, p.B, p.SL, lane);
+        // the last of them leaves the keys and the counters at zero
+        __shared__ int s_clear;
+        named_barrier_sync(2, kUmmaEpiWarps * 32);
+        if (ew == 0 && lane == 0) s_clear = p.finishers == 1 || atomicAdd(p.ticket + 1, 1u) == (unsigned)p.finishers - 1u;
+        named_barrier_sync(2, kUmmaEpiWarps * 32);
+        if (s_clear) {
+            for (int r = ew * 32 + lane; r < p.R; r += kUmmaEpiWarps * 32) p.keys[r] = 0ull;
+            if (ew == 0 && lane == 0) p.ticket[0] = p.ticket[1] = 0u;
         }
     }
 

@@ -355,6 +355,26 @@ def test_features_with_rows_that_are_and_are_not_aligned(oracle, V, N):
     ctx.close()
 
 
+# Few hidden rows, the vocabulary on the lanes: the rows a warp holds (8, 16, 32), tiles of exactly 32 and 128 vocabulary rows
+# and one more or less, more tiles than accumulators (2100 rows per SM: 17 tiles), CTAs without a vocabulary row
+@pytest.mark.parametrize("rows_per_sm,extra,B", [(31, 0, 1), (32, 1, 8), (33, 0, 9), (127, 3, 16), (128, 1, 17), (129, 0, 32),
+                                                 (257, -2, 33), (2100, 5, 3), (2100, 0, 20), (1, -100, 2)])
+def test_few_rows_at_the_edges_of_their_tiling(oracle, rows_per_sm, extra, B):
+    V, d = _sms() * rows_per_sm + extra, 40 if rows_per_sm < 1000 else 16
+    W, h = inputs.lm_head(V, d, seed=V + B, std=0.3), inputs.hidden(B, d, seed=B)
+    params = make_clf(16, seed=1)
+    pos, nd = np.arange(1, B + 1, dtype=np.int32), (np.arange(B, dtype=np.int32) % 4) + 1
+    active = (np.arange(B) % 5 != 2).astype(np.uint8)
+    ctx = binding.Context(V, d, 8, max_batch=B, max_rows=8, clf_hidden=16)
+    Wg, clf = W.cuda(), to_gpu_clf(params)
+    for act in (None, active, None):
+        got = gpu_draft_step(ctx, Wg, h, pos, nd, clf, 0.5, 3, active=act, want_probs=True)
+        ref = oracle.draft_step(_bits(W), _bits(h), pos, nd, to_oracle_clf(oracle, params), 0.5, 3, active=act, want_probs=True, nthreads=8)
+        _check_draft_and_each_probability(got, ref, 0.5, active=act)
+    assert ctx.device_status() == 0
+    ctx.close()
+
+
 # Tiles of hidden rows in pairs of CTAs: full and part-filled pairs, a last pair with one tile, kept logits
 @pytest.mark.parametrize("N,V,d", [(129, 700, 2048), (256, 3000, 2048), (257, 401, 2056), (520, 5003, 2048), (1000, 300, 2048)])
 def test_feature_extraction_by_pairs_of_ctas(N, V, d):
@@ -380,28 +400,33 @@ def test_feature_extraction_by_pairs_of_ctas(N, V, d):
     assert float((tv.double() - 0.5 * (yD.double() - yT.double()).abs().sum(-1)).abs().max()) < 1e-5
 
 
+def _ragged_verification(oracle, V, d, sls, seed, ctx):
+    """One verification with look-aheads `sls`, most offered ids the target's own, against the oracle."""
+    off = np.concatenate([[0], np.cumsum(np.asarray(sls) + 1)]).astype(np.int32)
+    R, B = int(off[-1]), len(sls)
+    W, H = inputs.lm_head(V, d, seed=seed, std=0.3), inputs.hidden(R, d, seed=seed + 1)
+    free = oracle.verify_ragged(_bits(W), _bits(H), np.zeros(R - B, np.int32), off, nthreads=16)
+    keep = np.ones(R, bool)
+    keep[off[1:] - 1] = False
+    draft = inputs.corrupt_ids(torch.from_numpy(free.target_ids[keep].astype(np.int32)), 0.2, V, seed=seed).numpy()
+    ref = oracle.verify_ragged(_bits(W), _bits(H), draft, off, nthreads=16)
+    got = gpu_verify(ctx, W.cuda(), H, draft, row_off=off)
+    check_verify(got, ref, off, draft, near_tie_ids(oracle, _bits(W), _bits(H), ref.gap))
+
+
+# CTAs that finish eight sequences each: one of them, full, one sequence more, the most there are and more than that; the
+# second call of a context finds keys and counters as the first has left them
+@pytest.mark.parametrize("B", [1, 8, 9, 33, 64, 65])
+def test_verification_finished_by_ctas_of_their_own(oracle, B):
+    ctx = binding.Context(3001, 8, 72, max_batch=B, max_rows=4 * B)
+    for k in range(2):
+        _ragged_verification(oracle, 3001, 72, [(b + k) % 4 for b in range(B)], 50 + B + k, ctx)
+    assert ctx.device_status() == 0
+    ctx.close()
+
+
 # Pairs of CTAs: two tiles of 128 rows (the second nearly empty, full), four, ten and an odd number of them; one and several
 # vocabulary tiles per pair
 @pytest.mark.parametrize("V,rows", [(300, 129), (300, 256), (2500, 500), (20000, 180), (400, 1160), (700, 1409)])
 def test_verification_by_pairs_of_ctas(oracle, V, rows):
     _verification_agrees(oracle, V, rows // 8, rows, 1032)
-
-
-# Few hidden rows, the vocabulary on the lanes: the rows a warp holds (8, 16, 32), tiles of exactly 32 and 128 vocabulary rows
-# and one more or less, more tiles than accumulators (2100 rows per SM: 17 tiles), CTAs without a vocabulary row
-@pytest.mark.parametrize("rows_per_sm,extra,B", [(31, 0, 1), (32, 1, 8), (33, 0, 9), (127, 3, 16), (128, 1, 17), (129, 0, 32),
-                                                 (257, -2, 33), (2100, 5, 3), (2100, 0, 20), (1, -100, 2)])
-def test_few_rows_at_the_edges_of_their_tiling(oracle, rows_per_sm, extra, B):
-    V, d = _sms() * rows_per_sm + extra, 40 if rows_per_sm < 1000 else 16
-    W, h = inputs.lm_head(V, d, seed=V + B, std=0.3), inputs.hidden(B, d, seed=B)
-    params = make_clf(16, seed=1)
-    pos, nd = np.arange(1, B + 1, dtype=np.int32), (np.arange(B, dtype=np.int32) % 4) + 1
-    active = (np.arange(B) % 5 != 2).astype(np.uint8)
-    ctx = binding.Context(V, d, 8, max_batch=B, max_rows=8, clf_hidden=16)
-    Wg, clf = W.cuda(), to_gpu_clf(params)
-    for act in (None, active, None):
-        got = gpu_draft_step(ctx, Wg, h, pos, nd, clf, 0.5, 3, active=act, want_probs=True)
-        ref = oracle.draft_step(_bits(W), _bits(h), pos, nd, to_oracle_clf(oracle, params), 0.5, 3, active=act, want_probs=True, nthreads=8)
-        _check_draft_and_each_probability(got, ref, 0.5, active=act)
-    assert ctx.device_status() == 0
-    ctx.close()
