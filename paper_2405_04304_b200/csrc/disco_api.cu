@@ -1375,7 +1375,9 @@ int disco_iteration_host(disco_ctx* c, const void* W_D, size_t w_step_stride, co
     };
     const size_t bytes_D = SB * c->d_draft * 2, bytes_T = R * c->d_target * 2;
     const void *src_D = nullptr, *src_T = nullptr;
-    const bool fetch = bytes_D + bytes_T <= kFetchBytes && (src_D = device_view(c, h_D_host, bytes_D)) != nullptr &&
+    // (not ahead of the persistent draft phase: a cooperative launch starts when all before it has ended, and the engine's second
+    // copy runs beside it: 11 rows of 5120 and ten steps of 768 with a head each 141 us, fetched 150)
+    const bool fetch = w_step_stride == 0 && bytes_D + bytes_T <= kFetchBytes && (src_D = device_view(c, h_D_host, bytes_D)) != nullptr &&
                        (src_T = device_view(c, H_T_host, bytes_T)) != nullptr;
     if (fetch) {
         // Little to move, all of it pinned: one kernel brings it over, and the draft phase's launch and its first loads of the
