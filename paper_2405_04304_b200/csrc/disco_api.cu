@@ -439,7 +439,10 @@ int launch_draft_batch(disco_ctx* c, const void* W, const void* H, int d, int R,
     // One tile of hidden rows: the LM head arrives slower than the tensor pipe works, so the tiles are small and the
     // epilogue of one runs under the loads of the next.  More tiles of rows: the rows' tile is loaded again for every
     // vocabulary tile, and that traffic (L2 to shared memory) is the bound, so the vocabulary tiles are the widest.
-    const int tile_target = R <= 128 ? 128 : 256;
+    // (Heads of more than two such tiles per CTA: three narrow tiles take longer than two wide ones; 40 / 64 / 100 / 128 rows of 40000 x
+    // 768 20.6 / 20.1 / 21.3 / 22.0 -> 19.1 / 19.2 / 20.2 / 21.7 us, of 32000 x 768, two tiles or one, 15.8 / 16.9 / 17.5 / 18.4 -> 17.6 / 18.7 /
+    // 20.2 / 20.0.)
+    const int tile_target = R <= 128 && (probs || c->V <= 256 * (c->sm_count - draft_finishers(c, R))) ? 128 : 256;
     // (one tile of rows: CTAs of their own finish the rows, unless the others would need a vocabulary tile more for it, or one
     // that is too large to do without the shared bound)
     auto tiles_each = [&](int CN) { return (c->V + tile_target * CN - 1) / (tile_target * CN); };
