@@ -283,7 +283,7 @@ bool verify_in_pairs(const disco_ctx* c, int R, int d, bool dev_R, int likely_R)
 
 // CTAs that do nothing but finish a verification in the kernel that projects it (umma_tail.cuh), a warp for each sequence; 0: the
 // rest must not get more to do for it, and there is a limit.  (us, 32000 x 5120 head, 11 rows of one sequence, launches one
-// after the other: the last CTA to take a ticket finishes 53.5, a CTA of its own 52.3.)
+// after the other: the last CTA to take a ticket finishes 53.5, a CTA of its own 52.3; in a graph 53.3 and 51.9.)
 int verify_finishers(const disco_ctx* c, int R, int d, int B) {
     const int n = (B + kUmmaEpiWarps - 1) / kUmmaEpiWarps;
     if (n > 8 || !VerifyTiling::possible(R, c->sm_count - n)) return 0;
@@ -318,10 +318,13 @@ int launch_umma(disco_ctx* c, const void* W, const void* H, int d, int R, const 
     CUtensorMap tmap_W, tmap_H;
     if (!encode_bf16_2d(c, &tmap_W, W, c->V, d, p.box_rows) || !encode_bf16_2d(c, &tmap_H, H, R, d, p.a_rows))
         return DISCO_ERR_CUDA;
-    static KernelSetup setup[4];
-    auto kern = pair ? umma_tail_kernel<false, false, true> : wide ? umma_tail_kernel<true, true, false> : lanes ? umma_tail_kernel<true, false, false> : umma_tail_kernel<false, false, false>;
+    static KernelSetup setup[7];
+    auto kern = pair    ? umma_tail_kernel<false, false, true, false>
+                : wide  ? (p.finishers ? umma_tail_kernel<true, true, false, true> : umma_tail_kernel<true, true, false, false>)
+                : lanes ? (p.finishers ? umma_tail_kernel<true, false, false, true> : umma_tail_kernel<true, false, false, false>)
+                        : (p.finishers ? umma_tail_kernel<false, false, false, true> : umma_tail_kernel<false, false, false, false>);
     const int smem_bytes = lanes ? kUmmaLaneSmemBytes : kUmmaSmemBytes;
-    if (!raise_smem_limit(c, setup[pair ? 3 : lanes + wide], kern, (size_t)smem_bytes, nullptr)) return DISCO_ERR_CUDA;
+    if (!raise_smem_limit(c, setup[pair ? 6 : lanes + wide + (p.finishers ? 3 : 0)], kern, (size_t)smem_bytes, nullptr)) return DISCO_ERR_CUDA;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(dev_R ? (pair ? c->sm_count & ~1 : c->sm_count) : p.t.groups * p.t.CN * (pair ? 2 : 1) + p.finishers));
     cfg.blockDim = dim3(kUmmaThreads);
@@ -976,7 +979,8 @@ int verify_common(disco_ctx* c, const void* W_T, const void* H_T, const int32_t*
     // under the first (us in one / two launches, 32000 x 2048, 5 rows each: 4 sequences 26.9 / 27.3, 8 26.5 / 26.8, 16 29.0 / 28.6, 20
     // 30.2 / 29.7, 32 35.3 / 33.4; 32000 x 5120: 54.6 / 55.1, 55.8 / 56.0, 60.0 / 59.2, 63.2 / 59.6).
     const bool pairs = !verify_on_lanes(c, R, c->d_target) && verify_in_pairs(c, R, c->d_target, false, R);
-    const int finishers = dev_R || pairs ? 0 : verify_finishers(c, R, c->d_target, B);
+    // (behind a draft phase, pad: 89.0 us in the other form against 92.4, 11 rows of 32000 x 5120 and steps with a head each)
+    const int finishers = dev_R || pairs || pad ? 0 : verify_finishers(c, R, c->d_target, B);
     if (B <= 16 || finishers) {
         UmmaParams fp{};
         fp.fuse_final = 1;

@@ -311,7 +311,9 @@ struct DraftFinalParams {
 // keys live in shared memory.  130 rows, 32000 x 2048: 36.2 -> 32.3 us; 20.5 us at the measured copy bandwidth.
 // PAIR: clusters of two CTAs with 256 hidden rows to a tile (VerifyTiling::make_pairs): each loads its own 128 hidden rows and half
 // of the LM-head box, the even one issues the MMAs of both.
-template <bool VL, bool WIDE, bool PAIR>
+// FIN: the grid's last p.finishers CTAs finish the sequences (an instance of its own: the code behind the last load comes from memory
+// line by line when another kernel ran before, and a verification behind its draft phase lost 3 us to code that it did not use).
+template <bool VL, bool WIDE, bool PAIR, bool FIN>
 __global__ void __launch_bounds__(kUmmaThreads, 1)
 umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_constant__ CUtensorMap tmap_H,
                  const UmmaParams p) {
@@ -658,7 +660,7 @@ umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_consta
                     atomicMax(p.keys + row, argmax_key(__fadd_rn(best_v[j], 0.f), best_i[j]));
             }
         }
-        if (p.finishers) {
+        if constexpr (FIN) {
             __threadfence();
             named_barrier_sync(2, kUmmaEpiWarps * 32);
             if (ew == 0 && lane == 0) atomicAdd(p.ticket, 1u);
@@ -680,13 +682,13 @@ umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_consta
                 if (ew == 0 && lane == 0) *p.ticket = 0u;
             }
         }
-    } else if (p.finishers && warp < 2 + kUmmaEpiWarps) {
+    } else if constexpr (FIN) {
         // ------------------------------ finishers ------------------------------
         // What does not depend on the keys is read while the others work; then the CTAs that are done are counted.  The others
         // leave at once, so the next launch sets itself up on their SMs meanwhile.  (Blocks start in order, so these CTAs are
         // the last ones; should one start after them, it has an SM of its own to wait for.)
         asm volatile("griddepcontrol.wait;" ::: "memory");
-        const int ew = warp - 2, first = (int)gridDim.x - p.finishers, step = kUmmaEpiWarps * p.finishers;
+        const int ew = warp - 2, first = (int)gridDim.x - p.finishers;
         const int b0 = ((int)blockIdx.x - first) * kUmmaEpiWarps + ew;
         VerifySeq q{};
         if (b0 < p.B) q = verify_locate(p.draft_ids, p.row_off, p.B, p.SL, R, b0, lane, p.padded);
@@ -703,12 +705,8 @@ umma_tail_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_consta
             __threadfence();
         }
         __syncwarp();
-        for (int b = b0; b < p.B; b += step) {
-            if (b != b0) q = verify_locate(p.draft_ids, p.row_off, p.B, p.SL, R, b, lane, p.padded);
-            verify_match(q, p.keys, p.draft_ids, b, p.n_accept, p.bonus, p.target_ids, p.status, lane, p.padded);
-        }
-        if (b0 == 0) warp_write_row_offsets(p.padded, p.B, p.SL, lane);
-        // the last of them leaves the keys and the counters at zero
+        if (b0 < p.B) verify_match(q, p.keys, p.draft_ids, b0, p.n_accept, p.bonus, p.target_ids, p.status, lane, p.padded);
+        // the last of these CTAs leaves the keys and the counters at zero
         __shared__ int s_clear;
         named_barrier_sync(2, kUmmaEpiWarps * 32);
         if (ew == 0 && lane == 0) s_clear = p.finishers == 1 || atomicAdd(p.ticket + 1, 1u) == (unsigned)p.finishers - 1u;
