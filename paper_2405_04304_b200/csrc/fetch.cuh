@@ -2,7 +2,8 @@
 //
 // Bound: the latency of one round trip over PCIe, then its bandwidth; every thread has its one load in flight at once.  A copy
 // by the copy engine in the stream keeps the kernel behind it from being launched early; this one lets the draft phase set
-// itself up and request the LM head while the hidden states arrive.
+// itself up and request the LM head while the hidden states arrive.  It looks at the caller's memory only once the work before
+// it in the stream is done, as a copy there would: that work may be what writes the hidden states.
 #pragma once
 
 #include "common.cuh"
@@ -23,7 +24,7 @@ struct FetchParams {
 
 static __global__ void __launch_bounds__(kFetchThreads) fetch_kernel(const FetchParams p) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    // (the buffers belong to the host entry points, which return with their work done: nothing earlier still reads them)
+    asm volatile("griddepcontrol.wait;" ::: "memory");   // (every thread: no part of this kernel ends before what went before it)
     unsigned i = blockIdx.x * kFetchThreads + threadIdx.x;
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
@@ -36,8 +37,6 @@ static __global__ void __launch_bounds__(kFetchThreads) fetch_kernel(const Fetch
         }
         i -= pieces;
     }
-    // (the kernel behind this one takes its end for the end of all that went before)
-    asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 }  // namespace disco

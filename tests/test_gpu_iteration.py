@@ -472,3 +472,41 @@ def test_host_iteration_from_any_host_memory(memory, B, forced):
         np.testing.assert_array_equal(t.numpy(), dev[k])
     assert ctx.device_status() == 0
     ctx.close()
+
+
+def test_host_iteration_behind_a_kernel_that_writes_its_hidden_states():
+    """The draft hidden states are the tokens of a draft step in front of the call in the same stream: int32 words below 16640 in
+    pinned memory, each two finite bf16 numbers.  That step lets its successor start early and writes them when it ends."""
+    V, B, S, dD, dT = 16500, 256, 2, 256, 64                # 256 words are the 2 x 256 bf16 numbers of one sequence's two steps
+    W, h = inputs.lm_head(V, 768, seed=1).cuda(), inputs.hidden(2 * B, 768, seed=2).view(2, B, 768).cuda()
+    first = binding.Context(V, 768, 8, max_batch=B, max_rows=8, clf_hidden=8)
+    clf = to_gpu_clf(position_clf(cut=100.0))
+    one, token, conf = torch.ones(B, dtype=torch.int32, device="cuda"), torch.zeros(B, dtype=torch.int32).pin_memory(), torch.zeros(B, device="cuda")
+    halt, ids = torch.zeros(B, dtype=torch.uint8, device="cuda"), torch.zeros(B, dtype=torch.int32, device="cuda")
+    W_D, W_T, _, H_T = make_inputs(V, dD, dT, 1, S, seed=3)
+    W_D, W_T, pos0 = W_D.cuda(), W_T.cuda(), torch.zeros(1, dtype=torch.int32).pin_memory()
+    ctx = binding.Context(V, dD, dT, max_batch=1, max_rows=S + 1, clf_hidden=8)
+    pin = lambda *s, t=torch.int32: torch.zeros(*s, dtype=t).pin_memory()
+    out = dict(token=pin(S, 1), conf=pin(S, 1, t=torch.float32), halt=pin(S, 1, t=torch.uint8), sl=pin(1), n_accept=pin(1), bonus=pin(1))
+    H_T = H_T.pin_memory()
+    seen = []
+    for k in range(4):
+        first.draft_step(W, h[k % 2], one, one, clf, 0.5, 2, ids, conf, halt)
+        torch.cuda.synchronize()
+        want = ids.cpu()
+        got_dev = {n: torch.zeros_like(t, device="cuda") for n, t in out.items()}
+        ctx.iteration(W_D, want.view(torch.bfloat16).view(S, 1, dD).cuda(), W_T, H_T.cuda(), pos0.cuda(), clf, 0.0, S, **got_dev)
+        token.zero_()
+        torch.cuda.synchronize()
+        rc = first._lib.disco_draft_step(first._h, W.data_ptr(), h[k % 2].data_ptr(), B, one.data_ptr(), one.data_ptr(), None, clf._c, 0.5, 2,
+                                         token.data_ptr(), conf.data_ptr(), halt.data_ptr(), None, None, torch.cuda.current_stream().cuda_stream)
+        assert rc == 0
+        ctx.iteration_host(W_D, token.view(torch.bfloat16).view(S, 1, dD), W_T, H_T, pos0, clf, 0.0, S, **out)
+        assert torch.equal(token, want)
+        for n, t in out.items():
+            assert torch.equal(t, got_dev[n].cpu()), n
+        seen.append(tuple(out["token"].flatten().tolist()))
+    assert seen[0] != seen[1]                               # the hidden states do decide the tokens
+    assert ctx.device_status() == 0 and first.device_status() == 0
+    ctx.close()
+    first.close()
