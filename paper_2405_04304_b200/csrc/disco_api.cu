@@ -817,6 +817,14 @@ const void* device_view(const disco_ctx* c, const void* p, size_t bytes) {
     return reinterpret_cast<const void*>(dev);
 }
 
+// The end of a *_host entry point, failed or not: its copies read the caller's memory and its kernels the staging buffers, so
+// nothing of the call may still be on its way when it returns.
+int host_call_done(const disco_ctx* c, int rc, cudaStream_t st, bool used_copy_stream = false) {
+    if (rc && used_copy_stream) cudaStreamSynchronize(c->copy_stream);   // (a call that did not fail made st wait for it)
+    const bool ok = cudaStreamSynchronize(st) == cudaSuccess;
+    return rc ? rc : (ok ? (int)DISCO_OK : (int)DISCO_ERR_CUDA);
+}
+
 // Shared body of the LM-head + soft-max passes: B rows of hidden size d against the head W.
 //   * nll_sum != null selects the perplexity rule (no classifier; tau is the perplexity bound);
 //   * stats_only = 1: arg-max (token, optional) and soft-max statistics only, no classifier: the target
@@ -1291,8 +1299,8 @@ int disco_draft_step_host(disco_ctx* c, const void* W_D, const void* h_D_host, i
     int rc = disco_draft_step(c, W_D, c->stage_hidden, B, dev_i(h_pos), dev_i(h_nd), active_host ? dev_b(h_act) : nullptr,
                               clf, tau, sl_max, dev_i(h_tok), dev_f(h_conf), dev_b(h_halt),
                               feats_host ? dev_f(h_feats) : nullptr, nullptr, stream);
+    rc = host_call_done(c, rc, st);
     if (rc) return rc;
-    if (cudaStreamSynchronize(st) != cudaSuccess) return DISCO_ERR_CUDA;
     // inactive sequences keep the caller's values: hand back only what the kernel wrote
     for (int b = 0; b < B; ++b) {
         if (active_host && !active_host[b]) continue;
@@ -1329,8 +1337,8 @@ int disco_verify_ragged_host(disco_ctx* c, const void* W_T, const void* H_T_host
         return DISCO_ERR_CUDA;
     int rc = disco_verify_ragged(c, W_T, c->stage_hidden, dev_i(h_ids), dev_i(h_off), B, R, dev_i(h_nacc), dev_i(h_bonus),
                                  target_ids_host ? dev_i(h_tids) : nullptr, stream);
+    rc = host_call_done(c, rc, st);
     if (rc) return rc;
-    if (cudaStreamSynchronize(st) != cudaSuccess) return DISCO_ERR_CUDA;
     std::memcpy(n_accept_host, h_nacc, (size_t)B * 4);
     std::memcpy(bonus_host, h_bonus, (size_t)B * 4);
     if (target_ids_host) std::memcpy(target_ids_host, h_tids, (size_t)R * 4);
@@ -1408,27 +1416,21 @@ int disco_iteration_host(disco_ctx* c, const void* W_D, size_t w_step_stride, co
                                       sl_forced_host ? dev + mb : nullptr, draft_ids_host ? dev + 2 * mb : nullptr,
                                       dev_i(h_tok), c->stage_float_d, c->stage_byte_d, nullptr, dev_i(h_sl), dev_i(h_nacc),
                                       dev_i(h_bonus), nullptr, nullptr, pos_next_host ? dev_i(h_next) : nullptr, stream, nullptr, 0);
-        const bool done = cudaStreamSynchronize(st) == cudaSuccess;   // (the user's memory is read until here)
-        if (rc) return rc;
-        if (!done) return DISCO_ERR_CUDA;
-        return hand_back();
+        const int end = host_call_done(c, rc, st);
+        return end ? end : hand_back();
     }
     // The draft phase needs the draft hidden states only: the (larger) target hidden states are sent once it is
     // enqueued, on a stream of their own, and the verification waits for them.  (Every host entry point returns with its
     // work done, so nothing earlier still reads the staging buffers.)
     if (cudaMemcpyAsync(c->stage_hidden_draft, h_D_host, bytes_D, cudaMemcpyHostToDevice, st) != cudaSuccess)
         return DISCO_ERR_CUDA;
-    int rc = iteration_impl(c, W_D, w_step_stride, c->stage_hidden_draft, W_T, c->stage_hidden, B, dev_i(h_pos), clf, tau,
+    const int rc = iteration_impl(c, W_D, w_step_stride, c->stage_hidden_draft, W_T, c->stage_hidden, B, dev_i(h_pos), clf, tau,
                             sl_max, sl_forced_host ? dev_i(h_forced) : nullptr, draft_ids_host ? dev_i(h_ids) : nullptr,
                             dev_i(h_tok), c->stage_float_d, c->stage_byte_d, nullptr, dev_i(h_sl), dev_i(h_nacc),
                             dev_i(h_bonus), nullptr, nullptr, pos_next_host ? dev_i(h_next) : nullptr, stream, H_T_host,
                             bytes_T);
-    if (rc) {
-        cudaStreamSynchronize(c->copy_stream);   // the copy must not outlive the call
-        return rc;
-    }
-    if (cudaStreamSynchronize(st) != cudaSuccess) return DISCO_ERR_CUDA;
-    return hand_back();
+    const int end = host_call_done(c, rc, st, true);
+    return end ? end : hand_back();
 }
 
 }  // extern "C"

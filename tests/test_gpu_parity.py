@@ -336,6 +336,38 @@ def test_errors_are_codes_not_faults():
     ctx.close()
 
 
+def test_failing_host_calls_leave_nothing_in_flight():
+    """A *_host call that fails behind its first copy: the copy reads the caller's memory and fills the staging buffer of the next
+    call, so the call returns when the stream is through.  20 ms of other work are in front of it."""
+    V, d, B, S = 300, 16, 3, 4
+    ctx = binding.Context(V, d, d, max_batch=B, max_rows=B * (S + 1), clf_hidden=8)
+    W, odd = inputs.lm_head(V, d, seed=1).cuda(), inputs.lm_head(V + 1, d, seed=1).cuda().view(-1)[4:4 + V * d].view(V, d)
+    good, wide = to_gpu_clf(make_clf(8, seed=2)), to_gpu_clf(make_clf(16, seed=2))
+    z = lambda *s, t=torch.int32: torch.zeros(*s, dtype=t).pin_memory()
+    bf16, f32, u8 = torch.bfloat16, torch.float32, torch.uint8
+    off = torch.tensor([0, 5, 10, 15], dtype=torch.int32).pin_memory()
+
+    def iteration(W_T, clf, pin):
+        hidden = (lambda *s: z(*s, t=bf16)) if pin else (lambda *s: torch.zeros(*s, dtype=bf16))   # fetched, or copied by the engine
+        ctx.iteration_host(W, hidden(S, B, d), W_T, hidden(B, S + 1, d), z(B), clf, 0.5, S, z(S, B), z(S, B, t=f32), z(S, B, t=u8), z(B), z(B), z(B))
+
+    calls = [(binding.ERR_WORKSPACE, lambda: ctx.draft_step_host(W, z(B, d, t=bf16), z(B), z(B), wide, 0.5, S, z(B), z(B, t=f32), z(B, t=u8))),
+             (binding.ERR_INVALID_ARG, lambda: ctx.verify_ragged_host(odd, z(15, d, t=bf16), z(12), off, B, 15, z(B), z(B))),
+             (binding.ERR_WORKSPACE, lambda: iteration(W, wide, True)), (binding.ERR_WORKSPACE, lambda: iteration(W, wide, False)),
+             (binding.ERR_INVALID_ARG, lambda: iteration(odd, good, True)), (binding.ERR_INVALID_ARG, lambda: iteration(odd, good, False))]
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        for want, call in calls:
+            torch.cuda._sleep(int(4e7))
+            with pytest.raises(binding.DiscoError) as e:
+                call()
+            assert e.value.code == want
+            assert stream.query(), "work of the failed call is still on its way"
+    iteration(W, good, True)
+    assert ctx.device_status() == 0
+    ctx.close()
+
+
 # ---------------------------------------------------------------------------------- both kernel families
 @pytest.mark.parametrize("path", [1, 2, 3])
 @pytest.mark.parametrize("V,d,B", [(50, 16, 1), (1000, 72, 3), (4099, 264, 7), (32000, 768, 1), (20011, 320, 16),
