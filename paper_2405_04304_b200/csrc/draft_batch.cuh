@@ -122,7 +122,7 @@ __device__ __forceinline__ void tmem_ld_columns(uint32_t a, uint32_t b, float& x
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
     asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
-// A barrier that a warp reaches only once it has the (non-zero) word it read: the barrier takes a predicate made from it.
+// A barrier that a warp reaches only once it has the words it read: the barrier takes a predicate made from them.
 __device__ __forceinline__ void named_barrier_sync_after(int id, int nthreads, uint32_t word) {
     asm volatile(
         "{\n\t.reg .pred p, q;\n\t"
@@ -374,7 +374,12 @@ __device__ __forceinline__ int opaque(int x) {
 
 // This launch's stamp, by the epilogue warps (eight of the CTA, ew their number) once what went before is over: the set of
 // bounds of the launch before is cleared and the CTA counts as started.
-__device__ __forceinline__ uint32_t db_begin(const DraftBatchParams& p, const DraftFinalParams& f, int ew, uint32_t* s_stamp, int lane) {
+// seen: anything made from what the thread has read of the rows' liveness.  Where several steps share a launch, a row that is
+// finished may end its sequence and clear the byte that the sequence's other rows, in other CTAs and other warps, went by; that
+// happens once all CTAs count as started, so no CTA counts before its threads have their bytes.  (A row that is dead here and
+// live to the warp that finishes it would be waited for in vain.)
+__device__ __forceinline__ uint32_t db_begin(const DraftBatchParams& p, const DraftFinalParams& f, int ew, uint32_t* s_stamp, uint32_t seen,
+                                             int lane) {
     const uint32_t stamp = *reinterpret_cast<volatile unsigned int*>(p.sync) + 1u;
     const uint32_t par = stamp & 1u;
     // (that word is the other parity's: only a launch after this one writes it)
@@ -390,7 +395,7 @@ __device__ __forceinline__ uint32_t db_begin(const DraftBatchParams& p, const Dr
     // CTA counts as started, and a warp that read the moved word would work on the next launch's set of bounds.  (One
     // warp that reads and hands the stamp to the others through shared memory: their polling costs the step up to 3 %,
     // eight rows of 49152 x 768 kept and drawn 30.9 us against 30.1.)
-    named_barrier_sync_after(8, kDbEpiWarps * 32, stamp);
+    named_barrier_sync_after(8, kDbEpiWarps * 32, stamp | seen);
     if (ew == 0 && lane == 0) {
         *reinterpret_cast<volatile uint32_t*>(s_stamp) = stamp;
         atomicAdd(p.sync + 4 + 4 * par, 1u);
@@ -445,7 +450,7 @@ __device__ __forceinline__ void db_finish_dedicated(const DraftBatchParams& p, c
             asm volatile("griddepcontrol.wait;" ::: "memory");
             if (!step_live()) break;
             b = (int)blockIdx.x - p.CN + fw * p.finishers;
-            if (fw < kDbEpiWarps) stamp = db_begin(p, f, fw, s_stamp, lane);
+            if (fw < kDbEpiWarps) stamp = db_begin(p, f, fw, s_stamp, 0u, lane);   // (reads its rows' bytes when all have started)
             else stamp = smem_word(s_stamp, p.status);
             if (lane == 0) {
                 const unsigned int* started = p.sync + 4 + 4 * (stamp & 1u);
@@ -607,8 +612,9 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
     const bool leader = !PAIR || cluster_rank() == 0;
     // (the CTAs of a pair request the same stages ahead, so they go by the leader's look)
     const bool looks_live = (leader ? *s_look : ld_cluster_u32(leader_addr(smem_addr(s_look)))) != 0u;
-    // Does the step take place?  Read once per CTA, by the MMA issuer right after the dependency wait (a finishing warp of
-    // this launch may clear flags once this CTA's records are out), and told to the others here.
+    // Does the step take place?  Read once per CTA, by the MMA issuer right after the dependency wait, and told to the others
+    // here.  (A finishing warp of this launch may clear flags once every CTA counts as started: db_begin, which the epilogue warps
+    // reach only when they have been told.)
     auto step_live = [&]() { return !chained || cold_smem_word(s_live, p.status) == 1u; };
 
     if (warp == 0) {
@@ -776,7 +782,7 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
                 valid = valid && chain_seq_live(f.chain, f.active, chain_seq(f.chain, row));
                 keep_mask = __ballot_sync(kFullMask, p.probs && valid);
                 many_kept = __popc(keep_mask) > 8 && (reinterpret_cast<uintptr_t>(p.probs) & 15) == 0;
-                const uint32_t stamp = db_begin(p, f, ew, s_stamp, lane);
+                const uint32_t stamp = db_begin(p, f, ew, s_stamp, valid ? 1u : 0u, lane);
                 slots = p.bound + (stamp & 1u) * p.set_words + (size_t)(valid ? row : 0) * kDbBoundStride;
                 my_slot = slots + nslot % kDbBoundSlots;
             }

@@ -283,10 +283,13 @@ umma_draft_few_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_c
             } else {
                 asm volatile("griddepcontrol.wait;" ::: "memory");  // scratch and outputs belong to the predecessor until now
                 if (!step_live()) break;
+                uint32_t seen = 0u;
 #pragma unroll
-                for (int q = 0; q < NR; ++q)
+                for (int q = 0; q < NR; ++q) {
                     valid[q] = valid[q] && chain_seq_live(f.chain, f.active, chain_seq(f.chain, ew + 8 * q));
-                stamp = db_begin(p, f, ew, s_stamp, lane);
+                    seen |= valid[q] ? 1u << q : 0u;
+                }
+                stamp = db_begin(p, f, ew, s_stamp, seen, lane);
                 slots = p.bound + (stamp & 1u) * p.set_words + (size_t)ew * kDbBoundStride;    // row q: 8 q rows on
             }
             const int phase_tiles = phase == 0 ? 0 : tiles;

@@ -387,6 +387,18 @@ def _check_draft_phase(got, ref, S):
                                            (2000, 12, 10, 1), (2000, 12, 10, 3), (2000, 2, 10, 1), (2000, 2, 10, 3),
                                            (900, 40, 16, 16), (5000, 256, 4, 4)])
 def test_steps_that_share_a_launch(oracle, V, B, S, scratch):
+    _steps_that_share_launches(oracle, V, B, S, scratch)
+
+
+# ... and several of them, each with the rows of two or three steps, in two to six tiles of hidden rows or one of few: what one row's
+# verdict does to the sequence's others meets rows of every tile
+@pytest.mark.parametrize("V,B,S,scratch,launches", [(2000, 160, 6, 2, 3), (3000, 250, 8, 3, 3), (900, 130, 7, 2, 4), (20000, 65, 9, 3, 3),
+                                                    (2000, 2, 9, 3, 3), (8000, 8, 12, 4, 3)])
+def test_several_launches_of_several_steps(oracle, V, B, S, scratch, launches):
+    _steps_that_share_launches(oracle, V, B, S, scratch, launches)
+
+
+def _steps_that_share_launches(oracle, V, B, S, scratch, launches=None):
     d = 72
     W, h = inputs.lm_head(V, d, seed=V + B, std=0.3), inputs.hidden(S * B, d, seed=B + S).view(S, B, d)
     pos0 = (np.arange(B, dtype=np.int32) * 7) % (S + 2)
@@ -398,8 +410,10 @@ def test_steps_that_share_a_launch(oracle, V, B, S, scratch):
         poisoned = h.clone()
         for b in range(B):
             poisoned[sl[b]:, b] = float("nan")
+        before = ctx.launch_count()
         got = _draft_loop(ctx, W, poisoned, pos0, to_gpu_clf(params), 0.5, S, forced=f)
         ref = oracle.draft_loop(_bits(W), _bits(h), pos0, to_oracle_clf(oracle, params), 0.5, S, sl_forced=f, nthreads=8)
+        assert launches in (None, ctx.launch_count() - before)
         np.testing.assert_array_equal(ref.sl, sl)
         _check_draft_phase(got, ref, S)
     assert ctx.device_status() == 0
