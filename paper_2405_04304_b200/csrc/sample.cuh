@@ -267,7 +267,10 @@ static __global__ void __launch_bounds__(kSampleThreads, 2) sample_rows_fused_ke
     const int r = blockIdx.x / p.SEG, s = blockIdx.x - r * p.SEG;
     const int V = p.V;
     // A chain of round trips to L2 bounds this kernel, so whatever waits for nothing is on its way first: the row's statistics
-    // and this CTA's logits.
+    // and this CTA's logits.  (Not the draft distribution that the row would be compared with were it the one drawn from: a load from
+    // memory that nearly every CTA waits for in vain.  us per call with it -> without, 17000 x 2048, 8 / 26 / 65 / 126 / 323 / 505 rows:
+    // 24.4 / 29.5 / 37.7 / 46.3 / 122 / 131 -> 24.2 / 29.1 / 37.4 / 45.3 / 118 / 129; 32000 x 5120: 65.5 / 70.6 / 88.6 / 115 / 269 / 294 ->
+    // 64.9 / 70.0 / 87.6 / 113 / 259 / 291.)
     float* y = p.y_T + (size_t)r * V;
     const float m = p.stats[2 * r], Z = p.stats[2 * r + 1];
     const int v_lo = min(V, s * p.seg_len), v_hi = min(V, v_lo + p.seg_len);
@@ -307,15 +310,6 @@ static __global__ void __launch_bounds__(kSampleThreads, 2) sample_rows_fused_ke
     const int sl = r1 - r0 - 1;
     const float u_draw = p.u_sample[b];
     const float inv_Z = 1.f / Z;
-    // If this row is the one drawn from, it is so after r - r0 accepted tokens, and that is the draft distribution it takes:
-    // requested before the acceptance tests say whether (3 MB in all for 30 rows of 32000).
-    const float* yD_here = r - r0 < sl ? p.draft_probs + ((size_t)(r - r0) * p.B + b) * V : nullptr;
-    float d_first[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        const int v = v_lo + t + k * kSampleThreads;
-        d_first[k] = (yD_here && v < v_hi) ? __ldg(yD_here + v) : 0.f;
-    }
     // acceptance tests of all positions side by side, then the first that fails
     if (t == 0) s_n = sl;
     __syncthreads();
@@ -342,7 +336,7 @@ static __global__ void __launch_bounds__(kSampleThreads, 2) sample_rows_fused_ke
     __syncthreads();
     const int n = s_n, skip = s_skip;
     const bool draw_row = r == r0 + n;
-    const float* yD = draw_row ? yD_here : nullptr;
+    const float* yD = (draw_row && n < sl) ? p.draft_probs + ((size_t)n * p.B + b) * V : nullptr;
     double acc_w = 0.0, acc_y = 0.0;
     int last_w = -1, last_y = -1;
     for (int v0 = v_lo + t; v0 < v_hi; v0 += 8 * kSampleThreads) {
@@ -351,7 +345,7 @@ static __global__ void __launch_bounds__(kSampleThreads, 2) sample_rows_fused_ke
         for (int k = 0; k < 8; ++k) {
             const int v = v0 + k * kSampleThreads;
             z[k] = v0 == v_lo + t ? z_first[k] : (v < v_hi ? __ldcg(y + v) : 0.f);
-            d[k] = v0 == v_lo + t ? d_first[k] : (yD && v < v_hi) ? __ldg(yD + v) : 0.f;
+            d[k] = (yD && v < v_hi) ? __ldg(yD + v) : 0.f;
         }
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
