@@ -1121,7 +1121,8 @@ int disco_verify_sample_ragged(disco_ctx* c, const void* W_T, const void* H_T, c
     sp.seg_last = c->sample_seg_last;
     sp.tickets = c->sample_tickets;
     sp.status = c->status;
-    const cudaError_t e = launch_after(c, sample_rows_fused_kernel, dim3((unsigned)R * sp.SEG), dim3(kSampleThreads), 0, st, sp);
+    const auto kern = sp.seg_len > kSampleShortWalk ? sample_rows_fused_kernel<true> : sample_rows_fused_kernel<false>;
+    const cudaError_t e = launch_after(c, kern, dim3((unsigned)R * sp.SEG), dim3(kSampleThreads), 0, st, sp);
     c->launches += 1;
     return cuda_ok(e, "sample_rows_fused_kernel launch") ? DISCO_OK : DISCO_ERR_CUDA;
 }

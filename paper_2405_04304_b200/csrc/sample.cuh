@@ -14,10 +14,89 @@ namespace disco {
 constexpr int kSampleThreads = 512;
 constexpr int kSampleWarps = kSampleThreads / 32;
 
-// The last step of a draw: entries [c0, c1) hold the crossing of `target` (the running
-// sum before c0 is `before`).  They are dealt out, a few consecutive entries per thread of the whole CTA: sums in
-// vocabulary order, a scan over the CTA, and the thread that holds the crossing walks its entries and writes
-// the token to found[0].  piece_tot: kSampleWarps doubles of shared memory.  Ends without a barrier.
+// The last step of a draw: entries [c0, c1) hold the crossing of `target` (the running sum before c0 is `before`); the token is
+// written to found[0].  piece_tot: kSampleWarps doubles of shared memory.  Ends without a barrier.
+//
+// Long ranges (a segment of a row that few CTAs share): consecutive entries per warp, read in whole lines, 256 at a time; the warp
+// that holds the crossing goes through its part again.  Bound: the round trips of the 256-entry batches to L2.  (Entries dealt out
+// to threads, as below, are 32 lines per load, which only a large L1 survives: the walk of 32000 entries took 31 or 61 us, as the
+// SM happened to be configured behind the LM-head kernel.)
+template <typename WeightFn>
+__device__ __forceinline__ void block_cdf_walk_long(WeightFn w, int c0, int c1, double before, double target, double* piece_tot,
+                                                    int* found) {
+    constexpr int kRows = 8, kBatch = 32 * kRows;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int q = ((c1 - c0 + kSampleWarps - 1) / kSampleWarps + 31) & ~31;
+    const int p0 = min(c1, c0 + warp * q), p1 = min(c1, p0 + q);
+    auto batch = [&](int v0, float (&x)[kRows]) {
+#pragma unroll
+        for (int k = 0; k < kRows; ++k) x[k] = v0 + 32 * k + lane < p1 ? w(v0 + 32 * k + lane) : 0.f;
+    };
+    auto warp_sum = [](double x) {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(kFullMask, x, off);
+        return x;
+    };
+    double mine = 0.0;
+    int last = -1;      // the warp's last entry with weight
+    for (int v0 = p0; v0 < p1; v0 += kBatch) {
+        float x[kRows];
+        batch(v0, x);
+#pragma unroll
+        for (int k = 0; k < kRows; ++k) {
+            mine += static_cast<double>(x[k]);
+            if (x[k] > 0.f) last = v0 + 32 * k + lane;
+        }
+    }
+    mine = warp_sum(mine);
+    last = __reduce_max_sync(kFullMask, last);
+    if (lane == 0) piece_tot[warp] = mine;
+    __syncthreads();
+    double run = before;
+    for (int k = 0; k < warp; ++k) run += piece_tot[k];
+    const double end = run + mine;
+    if (run <= target && end > target) {   // at most one warp
+        int tok = -1;
+        for (int v0 = p0; v0 < p1 && tok < 0; v0 += kBatch) {
+            float x[kRows];
+            batch(v0, x);
+            double sum = 0.0;
+#pragma unroll
+            for (int k = 0; k < kRows; ++k) sum += static_cast<double>(x[k]);
+            sum = warp_sum(sum);
+            if (!(run + sum > target)) {
+                run += sum;
+                continue;
+            }
+#pragma unroll
+            for (int k = 0; k < kRows; ++k) {
+                double incl = static_cast<double>(x[k]);
+#pragma unroll
+                for (int off = 1; off < 32; off <<= 1) {
+                    const double o = __shfl_up_sync(kFullMask, incl, off);
+                    if (lane >= off) incl += o;
+                }
+                const unsigned hit = __ballot_sync(kFullMask, x[k] > 0.f && run + incl > target);
+                if (tok < 0 && hit) tok = v0 + 32 * k + __ffs(hit) - 1;
+                run += __shfl_sync(kFullMask, incl, 31);
+            }
+        }
+        if (lane == 0) found[0] = tok >= 0 ? tok : last;   // (sums in another order: the last bit may fall short of the target)
+    }
+    // ... or that of the whole range may: its last entry with weight
+    if (warp == kSampleWarps - 1 && !(end > target)) {
+        int sl = -1;
+        for (int v0 = c1 - 32; v0 > c0 - 32 && sl < 0; v0 -= 32) {
+            const unsigned some = __ballot_sync(kFullMask, v0 + lane >= c0 && w(v0 + lane) > 0.f);
+            if (some) sl = v0 + 31 - __clz(some);
+        }
+        if (lane == 0) found[0] = sl;
+    }
+}
+// Short ranges: a few consecutive entries per thread, a scan over the CTA, and the thread that holds the crossing has its first eight
+// entries in registers still.  Up to 5632 entries (sampled verifications of 32000 x 2048, one form -> the other: 43 rows, segments of
+// 4572 entries, 46.6 -> 47.9 us; 65 rows, 6400, 52.8 -> 51.8; 126 rows, 10668, 78.3 -> 62.5; 288 rows, 16000, 142 -> 92).
+constexpr int kSampleShortWalk = 11 * kSampleThreads;
 template <typename WeightFn>
 __device__ __forceinline__ void block_cdf_walk(WeightFn w, int c0, int c1, double before, double target,
                                                double* piece_tot, int* found) {
@@ -257,6 +336,9 @@ struct SampleRowsParams {
     int* status;
 };
 
+// LONG: segments of more than kSampleShortWalk entries (an instance of its own: with both walks in one kernel the calls with short
+// segments were 1 - 3 % slower).
+template <bool LONG>
 static __global__ void __launch_bounds__(kSampleThreads, 2) sample_rows_fused_kernel(const SampleRowsParams p) {
     __shared__ double sh[40];
     __shared__ double red[4][kSampleWarps];
@@ -454,11 +536,12 @@ static __global__ void __launch_bounds__(kSampleThreads, 2) sample_rows_fused_ke
     __syncthreads();
     if (win >= 0) {
         const int c0 = min(V, win * p.seg_len), c1 = min(V, c0 + p.seg_len);
-        if (yDn && which == 0)
-            block_cdf_walk([&](int v) { return fmaxf(0.f, __ldcg(yn + v) - __ldg(yDn + v)); }, c0, c1, before, target,
-                           sh + kSampleWarps, found);
-        else
-            block_cdf_walk([&](int v) { return __ldcg(yn + v); }, c0, c1, before, target, sh + kSampleWarps, found);
+        auto walk = [&](auto w) {
+            if constexpr (LONG) block_cdf_walk_long(w, c0, c1, before, target, sh + kSampleWarps, found);
+            else block_cdf_walk(w, c0, c1, before, target, sh + kSampleWarps, found);
+        };
+        if (yDn && which == 0) walk([&](int v) { return fmaxf(0.f, __ldcg(yn + v) - __ldg(yDn + v)); });
+        else walk([&](int v) { return __ldcg(yn + v); });
     }
     __syncthreads();
     if (t == 0) {

@@ -707,6 +707,37 @@ def test_verify_sample_small_shapes(oracle, path, V, d, sls):
     _verify_sample_case(oracle, V, d, sls, seed=V + len(sls), path=path)
 
 
+# Rows that one or two CTAs share: segments around the limit beyond which a draw walks a segment by warps (5632 entries), and a
+# segment of several batches per warp that ends in the middle of one
+@pytest.mark.parametrize("V,sls", [(5629, [1] * 150), (5633, [1] * 150), (11268, [0, 1, 2, 3] * 20), (20011, [2] * 100)])
+def test_verify_sample_by_long_segments(oracle, V, sls):
+    _verify_sample_case(oracle, V, 16, sls, seed=V)
+
+
+@pytest.mark.parametrize("scale", [1.0, 40.0])
+@pytest.mark.parametrize("V,B", [(5633, 300), (9001, 300), (17000, 160), (40, 300)])
+def test_draws_are_where_the_running_sum_says(V, B, scale):
+    """Draws without draft tokens against the running sums of the distributions the call itself returns (scale 40: most entries are
+    zero), at uniforms from 0 to the largest below 1.  The sums are of doubles, so anything but rounding at 2^-52 of V terms is a
+    wrong token: the draw's interval has to hold the target within V * 2^-52."""
+    d = 16
+    W, H = inputs.lm_head(V, d, seed=V, std=0.25).cuda(), (inputs.hidden(B, d, seed=B).float() * scale).to(torch.bfloat16).cuda()
+    u = torch.rand(B, generator=torch.Generator().manual_seed(1))
+    u[:3] = torch.tensor([0.0, 1.0 - 2.0 ** -24, 0.5])
+    ctx = _ctx(V, 8, d, max_batch=B, max_rows=B)
+    z = lambda *s, t=torch.int32: torch.zeros(*s, dtype=t, device="cuda")
+    n, tok, y = z(B), z(B), z(B, V, t=torch.float32)
+    for _ in range(2):
+        ctx.verify_sample_ragged(W, H, None, None, None, B, B, None, u.cuda(), n, tok, y)
+    assert ctx.device_status() == 0
+    ctx.close()
+    upto = torch.cumsum(y.double(), -1)
+    target, at = u.cuda().double() * upto[:, -1], tok.long()[:, None]
+    mass, end = y.gather(1, at)[:, 0], upto.gather(1, at)[:, 0]
+    slack = V * 2.0 ** -52
+    assert bool((mass > 0).all()) and bool((end > target - slack).all()) and bool((end - mass.double() <= target + slack).all())
+
+
 def test_verify_sample_uniform_look_ahead_and_acceptance_range(oracle):
     acc, tot = _verify_sample_case(oracle, 2000, 64, [4] * 12, seed=77, uniform=True, noise=0.3)
     assert 0.3 * tot < acc <= tot                # close distributions: most tokens pass
