@@ -384,7 +384,8 @@ int launch_draft_few(disco_ctx* c, const void* W, const void* H, int d, int R, f
     p.TRN = std::max(16, (p.TR + 15) / 16 * 16);
     p.a_rows = 8 * NR;
     p.a_bytes = p.a_rows * 128;
-    p.b_bytes = (p.TRN * 128 + 1023) / 1024 * 1024;
+    p.w_rows = p.TR;
+    p.b_bytes = (p.w_rows * 128 + 1023) / 1024 * 1024;
     if ((size_t)R * p.CN > (size_t)128 * c->sm_count || R > c->part_rows) return DISCO_ERR_WORKSPACE;
     auto kern = umma_draft_few_kernel<STATS, NR>;
     static KernelSetup setup;
@@ -405,7 +406,7 @@ int launch_draft_few(disco_ctx* c, const void* W, const void* H, int d, int R, f
     p.set_words = (size_t)c->part_rows * kDbBoundStride;
     p.sync = c->ticket + 48;
     CUtensorMap tmap_W, tmap_H;
-    if (!encode_bf16_2d(c, &tmap_W, W, c->V, d, p.TRN) || !encode_bf16_2d(c, &tmap_H, H, R, d, p.a_rows))
+    if (!encode_bf16_2d(c, &tmap_W, W, c->V, d, p.w_rows) || !encode_bf16_2d(c, &tmap_H, H, R, d, p.a_rows))
         return DISCO_ERR_CUDA;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(p.CN + p.finishers));
@@ -459,7 +460,7 @@ int launch_draft_batch(disco_ctx* c, const void* W, const void* H, int d, int R,
     p.TRN = std::max(16, (p.TR + 15) / 16 * 16);
     p.a_rows = p.MT > 1 ? 128 : std::max(8, (R + 7) / 8 * 8);
     p.a_bytes = (p.a_rows * 128 + 1023) / 1024 * 1024;
-    p.b_bytes = ((pair ? p.TRN / 2 : p.TRN) * 128 + 1023) / 1024 * 1024;
+    p.w_rows = pair ? p.TRN / 2 : p.TR;
     if ((size_t)R * p.CN > (size_t)128 * c->sm_count || R > c->part_rows) return DISCO_ERR_WORKSPACE;
     auto kern = pair ? umma_draft_batch_kernel<STATS, true> : umma_draft_batch_kernel<STATS, false>;
     static KernelSetup setup[2];
@@ -469,8 +470,15 @@ int launch_draft_batch(disco_ctx* c, const void* W, const void* H, int d, int R,
     const int fin_warps = kDbFinWarps + (p.all_finish || p.finishers ? kDbEpiWarps : 0);
     const size_t fixed = 1024 + 512 + kDbXchBytes + (size_t)(fin_warps * kDbFinWords + 128) * 4 +
                          (probs ? kDbEpiWarps * 32 * kDbTurnStride * 4 : 0) + umma_clf_bytes(f.clf_H) + 128;
-    if (dyn_limit < fixed + 2 * (size_t)(p.a_bytes + p.b_bytes)) return DISCO_ERR_UNSUPPORTED_SHAPE;
-    p.stages = (int)std::min<size_t>(kDbMaxStages, (dyn_limit - fixed) / (p.a_bytes + p.b_bytes));
+    // Room for what the MMA takes, or for the box alone where that makes one more stage (us, the former -> the latter: 90 rows of
+    // 49152 x 768, five stages -> six, 22.9 -> 22.2; 100 rows of 49152 x 1024, five either way, 25.8 -> 26.2).
+    const int roomy = ((pair ? p.TRN / 2 : p.TRN) * 128 + 1023) / 1024 * 1024, close = (p.w_rows * 128 + 1023) / 1024 * 1024;
+    auto fit = [&](int b_bytes) {
+        return dyn_limit < fixed ? 0 : (int)std::min<size_t>(kDbMaxStages, (dyn_limit - fixed) / (p.a_bytes + b_bytes));
+    };
+    p.b_bytes = fit(close) > fit(roomy) ? close : roomy;
+    p.stages = fit(p.b_bytes);
+    if (p.stages < 2) return DISCO_ERR_UNSUPPORTED_SHAPE;
     p.ring_bytes = p.stages * (p.a_bytes + p.b_bytes);
     p.status = c->status;
     p.part_rec = reinterpret_cast<float4*>(c->stamped_rec);
@@ -479,7 +487,7 @@ int launch_draft_batch(disco_ctx* c, const void* W, const void* H, int d, int R,
     p.set_words = (size_t)c->part_rows * kDbBoundStride;
     p.sync = c->ticket + 48;
     CUtensorMap tmap_W, tmap_H;
-    if (!encode_bf16_2d(c, &tmap_W, W, c->V, d, pair ? p.TRN / 2 : p.TRN) || !encode_bf16_2d(c, &tmap_H, H, R, d, p.a_rows))
+    if (!encode_bf16_2d(c, &tmap_W, W, c->V, d, p.w_rows) || !encode_bf16_2d(c, &tmap_H, H, R, d, p.a_rows))
         return DISCO_ERR_CUDA;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(p.MT * p.CN + p.finishers));

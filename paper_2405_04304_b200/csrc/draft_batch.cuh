@@ -54,8 +54,13 @@ struct DraftBatchParams {
     int MT;      // tiles of 128 hidden rows
     int CN;      // CTAs per tile of hidden rows (grid = MT * CN)
     int TPC;     // vocabulary tiles per CTA
-    int TR;      // vocabulary rows per tile; the MMA and the TMA box use TRN = TR rounded up to 16
+    int TR;      // vocabulary rows per tile; the MMA takes TRN = TR rounded up to 16
     int TRN;
+    // Rows of the LM-head box: TR.  What the MMA reads behind them (shared memory of this CTA) only feeds columns, or lanes, that
+    // nobody looks at.  (Half of TRN for each CTA of a pair.)  With boxes of TRN rows the CTAs that are set aside for finishing could
+    // cost a long head more than they gain: 113 rows in a tile instead of 111 were a box of 128 instead of 112, and the rows loaded
+    // for nothing come from memory (12 / 32 rows of 49152 x 5120 101.9 / 111.1 -> 93.2 / 102.4 us, 12 rows of 49152 x 3072 68.5 -> 63.0).
+    int w_rows;
     int a_rows;  // rows of the H box (multiple of 8, <= 128)
     int stages, a_bytes, b_bytes, ring_bytes;
     int* status;
@@ -621,7 +626,7 @@ umma_draft_batch_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid
         // ------------------------------ producer ------------------------------
         const int total = tiles * KB;
         // (what a stage's barrier, the leader's, counts: the boxes of both CTAs)
-        const uint32_t w_bytes = (uint32_t)p.TRN * 128u, h_bytes = (uint32_t)p.a_rows * (PAIR ? 256u : 128u);
+        const uint32_t w_bytes = (uint32_t)p.w_rows * (PAIR ? 256u : 128u), h_bytes = (uint32_t)p.a_rows * (PAIR ? 256u : 128u);
         // The LM head is never written by this library: its first stages are requested before the dependency wait.
         const int pre = looks_live ? min(p.stages, total) : 0;
         // Every CTA reads the same hidden rows.  Each starts at another k-block, so that they do not all ask the same few

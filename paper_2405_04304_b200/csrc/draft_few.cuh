@@ -151,7 +151,7 @@ umma_draft_few_kernel(const __grid_constant__ CUtensorMap tmap_W, const __grid_c
     if (warp == 0) {
         // ------------------------------ producer ------------------------------
         const int total = tiles * KB;
-        const uint32_t w_bytes = (uint32_t)p.TRN * 128u, h_bytes = (uint32_t)kRows * 128u;
+        const uint32_t w_bytes = (uint32_t)p.w_rows * 128u, h_bytes = (uint32_t)kRows * 128u;
         const int pre = looks_live ? min(p.stages, total) : 0;
         const int rot = nslot % KB;       // (every CTA reads the same hidden rows: each starts at another k-block)
         const uint32_t full0 = smem_addr(full), empty0 = smem_addr(empty), w0 = smem_addr(w_tiles), h0 = smem_addr(h_tiles);
