@@ -353,20 +353,12 @@ bool draft_batch_in_pairs(const disco_ctx* c, int MT, int d, bool kept) {
     return ((MT + 1) & ~1) <= c->sm_count && (d >= 2048 ? MT >= 2 && MT != 3 : kept && MT >= 6 && MT % 2 == 0);
 }
 
-// CTAs that finish rows and do nothing else (draft_batch.cuh): a warp for each row.  (us per step, any CTA may finish -> CTAs of
-// their own: one row of 32000 x 768 14.7 -> 11.4, 7 rows of 40011 x 768 17.5 -> 14.3, 64 rows of 32000 x 768 17.8 -> 16.4, 128 rows
-// 16.0 -> 15.1, of 49152 x 768 25.0 -> 23.5.)
-int draft_finishers(const disco_ctx* c, int R) {
-    constexpr int per_cta = kDbEpiWarps + kDbFinWarps;
-    return std::max(1, std::min((R + per_cta - 1) / per_cta, c->sm_count / 4));
-}
-
 // Few hidden rows: the vocabulary on the TMEM lanes.  Up to 32, and beyond 16 only where a CTA has more than 32 vocabulary rows: with
 // fewer there is no shared bound, and then the lists of four rows are one warp's work after another (us, 512-wide heads of
 // 4000 / 8000 / 16000, vocabulary on the columns -> on the lanes: 32 rows 9.9 / 11.7 / 12.4 -> 13.5 / 11.7 / 11.6, 16 rows 9.7 / 11.5 /
 // 12.2 -> 9.9 / 10.3 / 10.4, 4 rows 9.7 / 9.8 / 10.5 -> 9.4 / 9.2 / 9.3).
 bool draft_few_possible(const disco_ctx* c, int R) {
-    return R <= 32 && c->sm_count >= 8 && (R <= 16 || c->V > 32 * (c->sm_count - draft_finishers(c, R)));
+    return R <= 32 && c->sm_count >= 8 && (R <= 16 || c->V > 32 * (c->sm_count - draft_finishers(c->sm_count, R)));
 }
 
 template <bool STATS, int NR>
@@ -377,7 +369,7 @@ int launch_draft_few(disco_ctx* c, const void* W, const void* H, int d, int R, f
     p.d = d;
     p.R = R;
     p.MT = 1;
-    p.finishers = draft_finishers(c, R);
+    p.finishers = draft_finishers(c->sm_count, R);
     p.CN = c->sm_count - p.finishers;
     p.TPC = std::max(1, (c->V + 128 * p.CN - 1) / (128 * p.CN));
     p.TR = (c->V + p.CN * p.TPC - 1) / (p.CN * p.TPC);
@@ -437,27 +429,14 @@ int launch_draft_batch(disco_ctx* c, const void* W, const void* H, int d, int R,
     p.V = c->V;
     p.d = d;
     p.R = R;
-    p.MT = (R + 127) / 128;
-    const bool pair = draft_batch_in_pairs(c, p.MT, d, probs != nullptr);
-    if (pair) p.MT = (p.MT + 1) & ~1;
-    // One tile of hidden rows: the LM head arrives slower than the tensor pipe works, so the tiles are small and the
-    // epilogue of one runs under the loads of the next.  More tiles of rows: the rows' tile is loaded again for every
-    // vocabulary tile, and that traffic (L2 to shared memory) is the bound, so the vocabulary tiles are the widest.
-    // (Heads of more than two such tiles per CTA: three narrow tiles take longer than two wide ones; 40 / 64 / 100 / 128 rows of 40000 x
-    // 768 20.6 / 20.1 / 21.3 / 22.0 -> 19.1 / 19.2 / 20.2 / 21.7 us, of 32000 x 768, two tiles or one, 15.8 / 16.9 / 17.5 / 18.4 -> 17.6 / 18.7 /
-    // 20.2 / 20.0.)
-    const int tile_target = R <= 128 && (probs || c->V <= 256 * (c->sm_count - draft_finishers(c, R))) ? 128 : 256;
-    // (one tile of rows: CTAs of their own finish the rows, unless the others would need a vocabulary tile more for it, or one
-    // that is too large to do without the shared bound)
-    auto tiles_each = [&](int CN) { return (c->V + tile_target * CN - 1) / (tile_target * CN); };
-    p.finishers = p.MT == 1 ? draft_finishers(c, R) : 0;
-    const int without = c->sm_count / p.MT, with = without - p.finishers;
-    if (tiles_each(with) > tiles_each(without) || (c->V > 32 * with && c->V <= 32 * without)) p.finishers = 0;
-    p.CN = c->sm_count / p.MT - p.finishers;
-    p.TPC = std::max(1, (c->V + tile_target * p.CN - 1) / (tile_target * p.CN));
-    p.TR = (c->V + p.CN * p.TPC - 1) / (p.CN * p.TPC);
-    if (probs) p.TR = (p.TR + 3) & ~3;   // rows of logits are stored 16 bytes at a time
-    p.TRN = std::max(16, (p.TR + 15) / 16 * 16);
+    const bool pair = draft_batch_in_pairs(c, (R + 127) / 128, d, probs != nullptr);
+    const DraftTiling t = DraftTiling::make(c->V, d, R, probs != nullptr, pair, c->sm_count);
+    p.MT = t.MT;
+    p.finishers = t.finishers;
+    p.CN = t.CN;
+    p.TPC = t.TPC;
+    p.TR = t.TR;
+    p.TRN = t.TRN;
     p.a_rows = p.MT > 1 ? 128 : std::max(8, (R + 7) / 8 * 8);
     p.a_bytes = (p.a_rows * 128 + 1023) / 1024 * 1024;
     p.w_rows = pair ? p.TRN / 2 : p.TR;

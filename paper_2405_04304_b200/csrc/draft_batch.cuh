@@ -31,12 +31,11 @@
 //     of 21.
 #pragma once
 
+#include "draft_rules.cuh"
 #include "umma_tail.cuh"
 
 namespace disco {
 
-constexpr int kDbEpiWarps = 8;
-constexpr int kDbFinWarps = 2;
 constexpr int kDbThreads = (2 + kDbEpiWarps + kDbFinWarps) * 32;
 constexpr int kDbMaxStages = 16;
 constexpr int kDbMaxRecords = 160;     // records per row a finishing warp takes in: five per lane

@@ -1,0 +1,56 @@
+// How the LM-head passes with soft-max statistics (draft_batch.cuh, draft_few.cuh) are cut.  Host code on plain sizes, so that a
+// test without a GPU can go through them.
+#pragma once
+
+#include <algorithm>
+
+namespace disco {
+
+constexpr int kDbEpiWarps = 8;
+constexpr int kDbFinWarps = 2;
+
+// CTAs that finish rows and do nothing else: a warp for each row.  (us per step, any CTA may finish -> CTAs of their own: one row of
+// 32000 x 768 14.7 -> 11.4, 7 rows of 40011 x 768 17.5 -> 14.3, 64 rows of 32000 x 768 17.1 -> 16.7, 126 rows 18.4 -> 18.1, of 49152 x
+// 768 24.1 -> 23.2.)
+inline int draft_finishers(int sms, int R) {
+    constexpr int per_cta = kDbEpiWarps + kDbFinWarps;
+    return std::max(1, std::min((R + per_cta - 1) / per_cta, sms / 4));
+}
+
+// MT tiles of 128 hidden rows (an even number by pairs of CTAs), CN CTAs (or pairs' halves) for each, TPC tiles of TR vocabulary rows
+// for each of those, TRN what the MMA takes.
+struct DraftTiling {
+    int MT, finishers, CN, TPC, TR, TRN;
+    // One tile of hidden rows: CTAs of their own finish the rows, unless the others would need a vocabulary tile more for it, or one
+    // that is too large to do without the shared bound.
+    static DraftTiling cut(int V, int R, bool kept, bool pair, int sms, int target) {
+        DraftTiling t;
+        t.MT = (R + 127) / 128;
+        if (pair) t.MT = (t.MT + 1) & ~1;
+        auto tiles_each = [&](int CN) { return (V + target * CN - 1) / (target * CN); };
+        const int without = sms / t.MT, with = t.MT == 1 ? without - draft_finishers(sms, R) : without;
+        t.CN = with < 1 || tiles_each(with) > tiles_each(without) || (V > 32 * with && V <= 32 * without) ? without : with;
+        t.finishers = without - t.CN;
+        t.TPC = std::max(1, tiles_each(t.CN));
+        t.TR = (V + t.CN * t.TPC - 1) / (t.CN * t.TPC);
+        if (kept) t.TR = (t.TR + 3) & ~3;   // rows of logits are stored 16 bytes at a time
+        t.TRN = std::max(16, (t.TR + 15) / 16 * 16);
+        return t;
+    }
+    // One tile of hidden rows: the LM head arrives slower than the tensor pipe works, so the vocabulary tiles are small and the
+    // epilogue of one runs under the loads of the next.  More tiles of rows: the rows' tile is loaded again for every
+    // vocabulary tile, and that traffic (L2 to shared memory) is the bound, so the vocabulary tiles are the widest.
+    // Heads of more than two small tiles for each CTA that there is in the end: three narrow tiles take longer than two wide ones
+    // (40 / 64 / 100 / 128 rows of 40000 x 768 20.6 / 20.9 / 21.6 / 22.0 -> 19.1 / 20.0 / 20.8 / 21.9 us; of 32000 x 768, two or one, 15.8 /
+    // 16.9 / 17.5 / 18.4 -> 17.6 / 18.7 / 20.2 / 20.0).  Two narrow ones without CTAs for the finishing, for which they are too full, still
+    // beat a wide one (37000 x 768 20.7 / 20.9 / 21.6 / 21.9 -> 18.7 / 19.0 / 19.4 / 19.8; 36000 x 512 18.5 -> 17.3 at 100 rows, x 384 16.1 ->
+    // 15.5), but for short contractions, whose tile is done before the epilogue (x 256 14.7 -> 16.0).
+    static DraftTiling make(int V, int d, int R, bool kept, bool pair, int sms) {
+        const DraftTiling narrow = cut(V, R, kept, pair, sms, 128);
+        if (R > 128) return cut(V, R, kept, pair, sms, 256);
+        if (kept || narrow.TPC < 2 || (narrow.TPC == 2 && (narrow.finishers > 0 || d > 320))) return narrow;
+        return cut(V, R, kept, pair, sms, 256);
+    }
+};
+
+}  // namespace disco

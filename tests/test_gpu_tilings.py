@@ -18,14 +18,14 @@ def _sms():
     return torch.cuda.get_device_properties(0).multi_processor_count
 
 
-def _check_draft_and_each_probability(got, ref, tau, active=None):
+def _check_draft_and_each_probability(got, ref, tau, active=None, rel=5e-5):
     """check_draft compares probabilities absolutely, which says nothing about those of a flat distribution: here each of the ten
     largest relatively.  A logit of these tests is a sum of at most 40 products of some 10 in all, in fp32, so that it is good to
     40 * 10 * 2^-24 = 2.4e-5 and e^z to as much; the exponentials and their sum add 1e-6."""
     check_draft(got, ref, tau, active=active)
     on = np.ones(len(ref.token), bool) if active is None else np.asarray(active) != 0
     want = ref.feats[on, :10]
-    assert float(np.abs(got["feats"][on, :10] / want - 1.0).max()) < 5e-5
+    assert float(np.abs(got["feats"][on, :10] / want - 1.0).max()) < rel
 
 
 # vocabulary rows per SM: one and two tiles of up to 128, a tile of exactly 32 / 33 rows (with and without the shared bound)
@@ -43,6 +43,25 @@ def test_batched_draft_step_at_the_edges_of_its_tiling(oracle, rows_per_sm, extr
         got = gpu_draft_step(ctx, Wg, h, pos, nd, clf, 0.5, 3, active=act)
         ref = oracle.draft_step(_bits(W), _bits(h), pos, nd, to_oracle_clf(oracle, params), 0.5, 3, active=act, nthreads=8)
         _check_draft_and_each_probability(got, ref, 0.5, active=act)
+    assert ctx.device_status() == 0
+    ctx.close()
+
+
+# Two narrow vocabulary tiles per CTA with CTAs of their own for the finishing, without them, and two wide ones; contractions around
+# the limit of the rule
+@pytest.mark.parametrize("d", [320, 328])
+@pytest.mark.parametrize("B", [33, 128])
+@pytest.mark.parametrize("finishers,extra", [(True, 0), (True, 1), (False, 0), (False, 1)])
+def test_batched_draft_step_where_its_tiles_grow(oracle, finishers, extra, B, d):
+    """A logit is a sum of 328 products of some 328 * 0.1 * 0.64 = 21 in all, in fp32: good to 328 * 21 * 2^-24 = 4.1e-4."""
+    V = 256 * (_sms() - ((B + 9) // 10 if finishers else 0)) + extra
+    W, h = inputs.lm_head(V, d, seed=V, std=0.1), inputs.hidden(B, d, seed=B)
+    params = make_clf(16, seed=1)
+    pos, nd = np.arange(1, B + 1, dtype=np.int32), (np.arange(B, dtype=np.int32) % 4) + 1
+    ctx = binding.Context(V, d, 8, max_batch=B, max_rows=8, clf_hidden=16)
+    got = gpu_draft_step(ctx, W.cuda(), h, pos, nd, to_gpu_clf(params), 0.5, 3)
+    ref = oracle.draft_step(_bits(W), _bits(h), pos, nd, to_oracle_clf(oracle, params), 0.5, 3, nthreads=16)
+    _check_draft_and_each_probability(got, ref, 0.5, rel=4.1e-4)
     assert ctx.device_status() == 0
     ctx.close()
 

@@ -28,12 +28,48 @@ int main() {
 """
 
 
-def test_verification_tiling_covers_everything_with_the_ctas_there_are(tmp_path):
-    src, exe = tmp_path / "tiling.cu", tmp_path / "tiling"
-    src.write_text(_TILING)
+def _run(tmp_path, source):
+    src, exe = tmp_path / "rules.cu", tmp_path / "rules"
+    src.write_text(source)
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
     include = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "include")
     subprocess.run([nvcc, "-gencode", "arch=compute_100a,code=sm_100a", "-std=c++17", "-I", build.CSRC, "-I", include, "-o", str(exe),
                     str(src)], check=True)
     run = subprocess.run([str(exe)], capture_output=True, text=True)
     assert run.returncode == 0, (run.returncode, run.stdout)
+
+
+def test_verification_tiling_covers_everything_with_the_ctas_there_are(tmp_path):
+    _run(tmp_path, _TILING)
+
+
+_DRAFT = r"""
+#include "draft_rules.cuh"
+#include <cstdio>
+using disco::DraftTiling;
+int main() {
+    const int grids[] = {1, 2, 16, 148}, ds[] = {8, 320, 328, 768, 5120}, rows[] = {1, 33, 40, 64, 100, 128, 129, 256, 257, 640, 1000};
+    for (int sms : grids)
+        for (int V = 1; V < 80000; V += V < 300 || (V > 34000 && V < 38200) ? 1 : 97)
+            for (int R : rows) {
+                if ((R + 127) / 128 > sms) continue;
+                for (int d : ds)
+                    for (int kind = 0; kind < 4; ++kind) {
+                        const bool kept = kind & 1, pair = (kind & 2) && R > 128 && (((R + 127) / 128 + 1) & ~1) <= sms;
+                        const DraftTiling t = DraftTiling::make(V, d, R, kept, pair, sms);
+                        const bool covered = t.MT * 128 >= R && t.CN >= 1 && t.TPC >= 1 && t.TR >= 1 && (long long)t.CN * t.TPC * t.TR >= V;
+                        const bool fits = t.MT * t.CN + t.finishers <= sms && t.TRN >= t.TR && t.TRN % 16 == 0 && t.TRN <= 256 &&
+                                          (!pair || t.MT % 2 == 0) && (!kept || t.TR % 4 == 0) && (t.finishers == 0 || R <= 128);
+                        // one tile of rows: one wide vocabulary tile and nobody to finish the rows is the worst of both
+                        const bool lame = R <= 128 && t.TRN > 128 && t.TPC == 1 && t.finishers == 0 && d > 320;
+                        if (!covered || !fits || (lame && sms > 16))
+                            return std::printf("V %d d %d R %d kept %d pair %d sms %d\n", V, d, R, kept, pair, sms), 1;
+                    }
+            }
+    return 0;
+}
+"""
+
+
+def test_draft_tiling_covers_everything_with_the_ctas_there_are(tmp_path):
+    _run(tmp_path, _DRAFT)
