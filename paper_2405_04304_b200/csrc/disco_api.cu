@@ -344,15 +344,6 @@ bool draft_batch_possible(const disco_ctx* c, int R) {
     return c->encode_tiled != nullptr && MT <= c->sm_count && c->sm_count / MT <= kDbMaxRecords && c->V < (int)kDbNoIndex;
 }
 
-// Pairs of CTAs that share their vocabulary tiles, where the operands' way from L2 is the bound.  Launches one after the other,
-// 256 / 384 / 512 / 640 / 1000 rows (us, single CTAs -> pairs): 32000 x 768 23.1 / 28.5 / 36.5 / 41 / 58 -> 23.9 / 35.9 / 37.0 / 47 / 60;
-// 32000 x 2048 46.0 / 58.6 / 74.1 / 88.3 / 116 -> 41.8 / 64.5 / 65.7 / 91.1 / 114; 32000 x 5120 99.6 / 133 / 168 / 206 / 263 -> 90.5 / 144 /
-// 130 / 190 / 231.  With the logits kept the narrow heads gain as well where no tile is left over (feature extraction, heads of 768 and
-// 1024, 300 / 512 / 640 / 760 / 1000 positions: 111 / 157 / 178 / 209 / 251 -> 124 / 156 / 190 / 202 / 244).
-bool draft_batch_in_pairs(const disco_ctx* c, int MT, int d, bool kept) {
-    return ((MT + 1) & ~1) <= c->sm_count && (d >= 2048 ? MT >= 2 && MT != 3 : kept && MT >= 6 && MT % 2 == 0);
-}
-
 // Few hidden rows: the vocabulary on the TMEM lanes.  Up to 32, and beyond 16 only where a CTA has more than 32 vocabulary rows: with
 // fewer there is no shared bound, and then the lists of four rows are one warp's work after another (us, 512-wide heads of
 // 4000 / 8000 / 16000, vocabulary on the columns -> on the lanes: 32 rows 9.9 / 11.7 / 12.4 -> 13.5 / 11.7 / 11.6, 16 rows 9.7 / 11.5 /
@@ -429,7 +420,7 @@ int launch_draft_batch(disco_ctx* c, const void* W, const void* H, int d, int R,
     p.V = c->V;
     p.d = d;
     p.R = R;
-    const bool pair = draft_batch_in_pairs(c, (R + 127) / 128, d, probs != nullptr);
+    const bool pair = draft_in_pairs(c->V, d, (R + 127) / 128, probs != nullptr, STATS, c->sm_count);
     const DraftTiling t = DraftTiling::make(c->V, d, R, probs != nullptr, pair, c->sm_count);
     p.MT = t.MT;
     p.finishers = t.finishers;

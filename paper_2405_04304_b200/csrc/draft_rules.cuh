@@ -17,6 +17,26 @@ inline int draft_finishers(int sms, int R) {
     return std::max(1, std::min((R + per_cta - 1) / per_cta, sms / 4));
 }
 
+// Pairs of CTAs that share their vocabulary tiles, for passes over MT tiles of 128 hidden rows: where the operands' way from L2 is the
+// bound, which takes a long contraction.  kept: the logits are written; stats: no lists of the ten largest.  us, single CTAs ->
+// pairs, under continuous load (a few launches in a row differ by as much):
+//   an even number of tiles, d = 2048, kept (both heads of a feature extraction), 200 / 450 / 700 / 1000 rows: V = 5000 42 / 54 / 69 /
+//   83 -> 43 / 55 / 68 / 83, 17000 77 / 123 / 170 / 220 -> 74 / 116 / 159 / 210, 32000 119 / 208 / 285 / 376 -> 111 / 194 / 260 / 340; not
+//   kept: 5000 16.5 / 19.7 / 23.8 / 27.3 -> 17.8 / 20.6 / 25.3 / 28.1, 17000 26.7 / 40.6 / 54.5 / 69.9 -> 26.4 / 40.3 / 53.2 / 67.0, 32000
+//   43.5 / 69.8 / 101 / 120 -> 40.7 / 65.7 / 93 / 115;
+//   an odd one, where a pair works on a tile of nothing, kept, 600 / 850 rows: 5000 x 2048 63 / 76 -> 66 / 77, 17000 x 2048 153 / 198 -> 149 /
+//   197, 32000 x 5120 475 / 645 -> 458 / 600; not kept: 32000 x 2048 88 / 106 -> 92 / 113, x 5120 165 / 228 -> 174 / 236; three tiles lose
+//   wherever they are narrower than 49152;
+//   narrow heads, 700 / 1000 rows kept: 32000 x 768 182 / 229 -> 187 / 245, x 1024 199 / 252 -> 200 / 260, x 1536 240 / 314 -> 229 / 298, 17000 x
+//   1536 142 / 184 -> 145 / 190; statistics only, 1006 rows of 32000 x 1024 169 -> 164, of 17000 x 1024 108 -> 112.
+inline bool draft_in_pairs(int V, int d, int MT, bool kept, bool stats, int sms) {
+    if (MT < 2 || ((MT + 1) & ~1) > sms) return false;
+    const long long head = (long long)V * d;
+    if (d < 2048) return kept && MT >= 6 && MT % 2 == 0 && V >= 24000 && d >= (stats ? 1024 : 1536);
+    if (MT % 2) return kept && MT >= 5 && head >= 25000000;
+    return kept ? MT >= 6 || head >= 16000000 : head >= 32000000;
+}
+
 // MT tiles of 128 hidden rows (an even number by pairs of CTAs), CN CTAs (or pairs' halves) for each, TPC tiles of TR vocabulary rows
 // for each of those, TRN what the MMA takes.
 struct DraftTiling {

@@ -48,6 +48,15 @@ _DRAFT = r"""
 #include <cstdio>
 using disco::DraftTiling;
 int main() {
+    // head, tiles of rows, logits kept, statistics only: whether pairs of CTAs were measured to be the faster form
+    struct { int V, d, MT; bool kept, stats, pairs; } measured[] = {
+        {32000, 2048, 5, false, false, false}, {49152, 4096, 7, false, false, false}, {32000, 5120, 5, true, false, true},
+        {32000, 5120, 3, true, true, false}, {32000, 768, 8, true, false, false}, {17000, 1024, 8, true, true, false},
+        {32000, 1536, 8, true, false, true}, {5000, 2048, 2, true, false, false}, {5000, 2048, 8, false, false, false},
+        {32000, 2048, 2, false, false, true}, {32000, 2048, 4, false, false, true}, {17000, 2048, 4, true, true, true}};
+    for (auto& m : measured)
+        if (disco::draft_in_pairs(m.V, m.d, m.MT, m.kept, m.stats, 148) != m.pairs) return std::printf("pairs: %d x %d, %d\\n", m.V, m.d, m.MT), 1;
+    if (disco::draft_in_pairs(32000, 5120, 148, true, false, 147) || disco::draft_in_pairs(32000, 5120, 1, true, false, 148)) return 1;
     const int grids[] = {1, 2, 16, 148}, ds[] = {8, 320, 328, 768, 5120}, rows[] = {1, 33, 40, 64, 100, 128, 129, 256, 257, 640, 1000};
     for (int sms : grids)
         for (int V = 1; V < 80000; V += V < 300 || (V > 34000 && V < 38200) ? 1 : 97)
