@@ -268,17 +268,14 @@ bool verify_on_lanes(const disco_ctx* c, int R, int d) {
     return few || beyond;
 }
 
-// Verification by pairs of CTAs: half of the LM-head traffic from L2, but the rows are cut into tiles of 256.  Launches one after
-// the other, 32000 x 1024 / 2048 / 5120 (us, two tiles of hidden rows per CTA or one -> pairs): 250 rows 22.2 / 35.4 / 80.0 -> 20.3 /
-// 32.0 / 79.3, 300 rows 25.3 / 46.7 / 124 -> 32.0 / 55.2 / 130, 450 rows 33.9 / 60.4 / 122 -> 32.4 / 53.3 / 114, 600 rows 39.9 / 77.1 /
-// 165 -> 38.7 / 80.1 / 175; 2432 rows of 49152 x 6144: 3 % of the iteration; 1186 rows of 17960 x 3064, an even number of tiles that
-// leaves pairs idle, 118 -> 120.  So: where a CTA's share of the tensor work does not grow by more than a few hundredths.
-// (A count in device memory: only where it is likely to be large.)
+// Verification by pairs of CTAs (VerifyTiling::in_pairs).  A count in device memory: only where it is likely to be large, since the
+// tiling that the kernel derives then may be one that pays or one that does not (whole iterations of 256 / 180 sequences with
+// look-aheads up to 16 / 12, single CTAs -> pairs, us under continuous load: 32000 x 5120, 769 / 1350 / 1408 / 1676 / 2432 rows 384 / 547 /
+// 547 / 542 / 832 -> 372 / 506 / 498 / 571 / 828; 49152 x 6144, 662 / 906 / 899 / 930 / 1421 -> 601 / 819 / 807 / 973 / 1438; 17000 x 2048, 1408 /
+// 2432 rows 236 / 277 -> 227 / 281).
 bool verify_in_pairs(const disco_ctx* c, int R, int d, bool dev_R, int likely_R) {
-    if (d < 1024 || R <= 128 || !VerifyTiling::pairs_possible(R, c->sm_count)) return false;
-    if (dev_R) return likely_R > 1024;
-    const VerifyTiling one = VerifyTiling::make(R, c->V, d, c->sm_count), two = VerifyTiling::make_pairs(R, c->V, d, c->sm_count);
-    return 32ll * two.TPC * two.TRN * std::min(two.GS, two.MT) <= 33ll * one.TPC * one.TRN * std::min(one.GS, one.MT);
+    if (dev_R) return d >= 1024 && likely_R > 1024 && VerifyTiling::pairs_possible(R, c->sm_count);
+    return VerifyTiling::in_pairs(R, c->V, d, c->sm_count);
 }
 
 // CTAs that do nothing but finish a verification in the kernel that projects it (umma_tail.cuh), a warp for each sequence; 0: the

@@ -97,6 +97,23 @@ struct VerifyTiling {
         }
         return best;
     }
+    // Whether pairs are the faster form (us under continuous load, single CTAs -> pairs; few launches in a row differ by as much).
+    // They halve the LM head's traffic from L2, but cut the rows into tiles of 256: a CTA's share of the tensor work may not grow by
+    // more than a few hundredths.  Then
+    //   * a pair with one tile of rows, whose epilogue runs under the next vocabulary tile, beats CTAs with two (32000 x 1024 / 2048 /
+    //     5120, 251 rows 23.2 / 39.3 / 95 -> 20.4 / 34.1 / 88; x 2048 / 5120, 650 rows 87 / 202 -> 79 / 193; 4000 x 5120, 512 rows 35.2 ->
+    //     24.8), and CTAs with one where it has three vocabulary tiles to gain on (32000 x 1024, 650 / 974 / 2432 rows 47.1 / 59.2 / 133
+    //     -> 43.4 / 56.5 / 127, but 8000 x 1024, 512 rows 10.9 -> 12.0);
+    //   * a pair with two has its epilogue exposed like a CTA with two, and waits for more (32000 x 2048 / 5120, 1520 rows 156 / 364 -> 162 /
+    //     371; against CTAs with one: 49152 x 1024, 428 rows 45.4 -> 49.6, 8000 x 1024, 2432 rows 33.4 -> 39.9).  It pays on a short head
+    //     of a long contraction only (4000 / 8000 x 5120, 1520 rows 57 / 109 -> 54 / 105, 4000 x 6144, 2432 rows 113 -> 102).
+    __host__ __device__ static bool in_pairs(int R, int V, int d, int grid) {
+        if (d < 1024 || R <= 128 || !pairs_possible(R, grid)) return false;
+        const VerifyTiling one = make(R, V, d, grid), two = make_pairs(R, V, d, grid);
+        auto share = [](const VerifyTiling& t) { return (long long)t.TPC * t.TRN * (t.GS < t.MT ? t.GS : t.MT); };
+        if (32 * share(two) > 33 * share(one)) return false;
+        return two.GS == 1 ? one.GS == 2 || two.TPC >= 3 : d >= 4096 && V <= 8192 && two.TPC <= 2;
+    }
 };
 
 struct UmmaParams {

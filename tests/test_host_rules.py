@@ -9,6 +9,13 @@ _TILING = r"""
 #include <cstdio>
 using disco::VerifyTiling;
 int main() {
+    // head, rows: whether pairs of CTAs were measured to be the faster form
+    struct { int V, d, R; bool pairs; } measured[] = {
+        {32000, 2048, 251, true}, {32000, 5120, 650, true}, {32000, 1024, 2432, true}, {32000, 2048, 1520, false}, {49152, 1024, 428, false},
+        {8000, 1024, 512, false}, {8000, 1024, 2432, false}, {32000, 5120, 300, false}, {4000, 5120, 1520, true}, {32000, 5120, 1520, false},
+        {4000, 1024, 650, false}, {32000, 768, 650, false}, {32000, 5120, 128, false}};
+    for (auto& m : measured)
+        if (VerifyTiling::in_pairs(m.R, m.V, m.d, 148) != m.pairs) return std::printf("pairs: %d x %d, %d\\n", m.V, m.d, m.R), 1;
     const int grids[] = {1, 2, 148}, vs[] = {1, 300, 32000, 151936}, ds[] = {8, 768, 2040, 2048, 6144};
     for (int grid : grids)
         for (int R = 1; R <= 128 * 2 * grid + 129; R += R < 1000 ? 1 : 127) {
@@ -21,6 +28,14 @@ int main() {
                     const bool rows = t.groups * t.GS * 128 >= R && t.groups * t.CN <= grid && t.CN >= 1 && (t.GS == 1 || t.GS == 2);
                     const bool cols = (long long)t.CN * t.TPC * t.TR >= V && t.TR >= 1 && t.TRN >= t.TR && t.TRN <= 256 && t.TRN % 16 == 0;
                     if (!rows || !cols) return std::printf("R %d V %d d %d grid %d\n", R, V, d, grid), 1;
+                    // pairs of CTAs: what the kernel derives from a count in device memory
+                    const bool pairs = (R + 511) / 512 <= grid / 2;
+                    if (VerifyTiling::pairs_possible(R, grid) != pairs) return std::printf("pairs_possible(%d, %d)\n", R, grid), 1;
+                    if (!pairs) continue;
+                    const VerifyTiling u = VerifyTiling::make_pairs(R, V, d, grid);
+                    const bool u_rows = u.groups * u.GS * 256 >= R && 2 * u.groups * u.CN <= grid && u.CN >= 1 && (u.GS == 1 || u.GS == 2);
+                    const bool u_cols = (long long)u.CN * u.TPC * u.TR >= V && u.TR >= 1 && u.TRN >= u.TR && u.TRN <= 256 && u.TRN % 16 == 0;
+                    if (!u_rows || !u_cols) return std::printf("pairs: R %d V %d d %d grid %d\n", R, V, d, grid), 1;
                 }
         }
     return 0;
