@@ -509,36 +509,11 @@ bool gemv_loop_possible(const disco_ctx* c, int B, int sl_max, size_t w_step_str
     return (size_t)((c->d_draft + kUmmaBK - 1) / kUmmaBK) * 8 * 128 <= 48 * 1024;
 }
 
-// Steps of a draft phase that one launch of the batched draft step takes on (1: none but its own).  A launch costs the head's
-// way through HBM and the chain behind it once, and a tensor-bound part per tile of 128 rows; a step after the last sequence
-// has stopped costs a launch that returns (3 us, 5 with more than 128 rows), and rows of such steps that shared a launch were
-// projected for nothing.  So: the number that is the cheapest on average, the longest look-ahead being anything from 1 to
-// sl_max, of those that are no dearer than single steps even if every sequence stops at once.  us per call of the whole
-// iteration with 1 / 2 / 4 / 8 / 16 steps to a launch, all stop after the first of 16, 32000 x 768: 64 sequences 91 / 69 / 63 / 65 / 87, 256
-// sequences 139 / 114 / 116 / - / -; after the third, 64 sequences 123 / 89 / 67 / 69 / 91.  1 sequence, 4 steps of 10: 104 -> 78 us.  64
-// sequences, look-aheads up to 10 of 10: 303 -> 200 us; 256 sequences of 49152 x 768, up to 16 of 16: 1710 -> 1555 us.
 int steps_per_launch(const disco_ctx* c, int B, int sl_max, size_t w_step_stride) {
     if (w_step_stride != 0 || c->path != 0) return 1;
     const int most = std::min(std::min(kMaxGroup, sl_max), c->part_rows / B);
     if (most < 2 || !draft_batch_possible(c, most * B)) return 1;
-    const double per_tile = 256.0 * c->V * c->d_draft / 1.1e9;                                  // us
-    const double once = 6.0 + std::max(7.0, 2.0 * c->V * c->d_draft / 6.5e6);
-    const double idle = B <= 128 ? 3.0 : 5.0;
-    auto cost = [&](int k) { return once + per_tile * ((k * B + 127) / 128); };
-    int best = 1;
-    double least = 0.0;
-    for (int k = 1; k <= most; ++k) {
-        const int launches = (sl_max + k - 1) / k;
-        if ((k * B + 127) / 128 > c->sm_count || cost(k) - cost(1) > (sl_max - launches) * idle) continue;
-        double mean = 0.0;
-        for (int l = 0; l < launches; ++l) {
-            const double lives = 1.0 - (double)l * k / sl_max;
-            mean += lives * cost(k) + (1.0 - lives) * idle;
-        }
-        if (k == 1 || mean < least) best = k, least = mean;
-    }
-    const int launches = (sl_max + best - 1) / best;
-    return (sl_max + launches - 1) / launches;
+    return draft_steps_per_launch(c->V, c->d_draft, B, sl_max, most, c->sm_count);
 }
 
 int launch_gemv_loop(disco_ctx* c, const TailParams& t, int steps, size_t w_step_stride, cudaStream_t st) {

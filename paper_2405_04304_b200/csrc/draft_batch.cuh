@@ -41,7 +41,6 @@ constexpr int kDbMaxStages = 16;
 constexpr int kDbMaxRecords = 160;     // records per row a finishing warp takes in: five per lane
 constexpr int kDbXchBytes = 128 * 64;  // states handed between the two warps that share a hidden row
 constexpr int kDbFinWords = 16;        // features; per finishing warp
-constexpr int kDbBoundSlots = 12;      // words of the shared bound per row
 constexpr int kDbBoundStride = 16;     // (rows 64 bytes apart)
 constexpr int kDbTurnStride = 36;      // floats per row of the area that turns a chunk of logits round (no bank conflicts)
 constexpr int kDbChunks = 4;           // chunks of 32 columns per warp and tile, at most

@@ -8,6 +8,7 @@ namespace disco {
 
 constexpr int kDbEpiWarps = 8;
 constexpr int kDbFinWarps = 2;
+constexpr int kDbBoundSlots = 12;      // words of the shared bound per row
 
 // CTAs that finish rows and do nothing else: a warp for each row.  (us per step, any CTA may finish -> CTAs of their own: one row of
 // 32000 x 768 14.7 -> 11.4, 7 rows of 40011 x 768 17.5 -> 14.3, 64 rows of 32000 x 768 17.1 -> 16.7, 126 rows 18.4 -> 18.1, of 49152 x
@@ -72,5 +73,41 @@ struct DraftTiling {
         return cut(V, R, kept, pair, sms, 256);
     }
 };
+
+// Steps of a draft phase that one launch takes on, at most `most` (1: none but its own).  A launch costs the head's way through HBM
+// and the chain behind it once, and a part per tile of 128 rows: the MMAs, or the epilogue where the contraction is short (us per
+// tile, 4000 / 12000 / 32000 / 49152 x 256 1.0 / 1.8 / 4.0 / 5.3, x 768 1.1 / 2.1 / 5.8 / 8.8); a step after the last sequence has stopped
+// costs a launch that returns (3 us, 5 with more than 128 rows), and rows of such steps that shared a launch were projected for
+// nothing.  So: the number that is the cheapest on average, the longest look-ahead being anything from 1 to sl_max, of those that are
+// no dearer than single steps even if every sequence stops at once (a seventh dearer at most on narrow heads: 200 sequences of 32000 x
+// 256, all stop after the first / third step of 3, 27 / 54 us step by step, 31 / 31 in one launch).  us per call of the whole iteration with 1 / 2 / 4 / 8 / 16 steps to
+// a launch, all stop after the first of 16, 32000 x 768: 64 sequences 91 / 69 / 63 / 65 / 87, 256 sequences 139 / 114 / 116 / - / -; after the
+// third, 64 sequences 123 / 89 / 67 / 69 / 91.  1 sequence, 4 steps of 10: 104 -> 78 us.  64 sequences, look-aheads up to 10 of 10: 303 ->
+// 200 us; 256 sequences of 49152 x 768, up to 16 of 16: 1710 -> 1555 us.
+// Not so many rows that a row has fewer than ten CTAs: with three of its twelve words empty the shared bound bounds nothing (32000 x
+// 256, 1536 / 2048 rows, 12 / 9 CTAs to a row: 59 / 119 us).
+inline int draft_steps_per_launch(int V, int d, int B, int sl_max, int most, int sms) {
+    const double epilogue = 0.6 + 1.05e-4 * V, mma = 256.0 * V * d / 1.1e9, per_tile = std::max(epilogue, mma);   // us
+    const double allowed = epilogue > mma ? 1.15 : 1.0;
+    const double once = 6.0 + std::max(7.0, 2.0 * V * d / 6.5e6);
+    const double idle = B <= 64 ? 3.0 : B <= 128 ? 4.0 : 5.0;
+    auto tiles = [&](int k) { return (k * B + 127) / 128; };
+    auto cost = [&](int k) { return once + per_tile * tiles(k); };
+    int best = 1;
+    double least = 0.0;
+    for (int k = 1; k <= most; ++k) {
+        const int launches = (sl_max + k - 1) / k;
+        if (k > 1 && (sms / tiles(k) < kDbBoundSlots - 2 || cost(k) + (launches - 1) * idle > allowed * (cost(1) + (sl_max - 1) * idle)))
+            continue;
+        double mean = 0.0;
+        for (int l = 0; l < launches; ++l) {
+            const double lives = 1.0 - (double)l * k / sl_max;
+            mean += lives * cost(k) + (1.0 - lives) * idle;
+        }
+        if (k == 1 || mean < least) best = k, least = mean;
+    }
+    const int launches = (sl_max + best - 1) / best;
+    return (sl_max + launches - 1) / launches;
+}
 
 }  // namespace disco

@@ -72,6 +72,20 @@ int main() {
     for (auto& m : measured)
         if (disco::draft_in_pairs(m.V, m.d, m.MT, m.kept, m.stats, 148) != m.pairs) return std::printf("pairs: %d x %d, %d\\n", m.V, m.d, m.MT), 1;
     if (disco::draft_in_pairs(32000, 5120, 148, true, false, 147) || disco::draft_in_pairs(32000, 5120, 1, true, false, 148)) return 1;
+    // steps to a launch: as many as there is scratch for, in even shares, and never more rows than have a shared bound
+    for (int B : {1, 2, 3, 8, 12, 64, 100, 128, 130, 200, 256})
+        for (int d : {64, 256, 768, 1024})
+            for (int V : {1, 4000, 32000, 49152})
+                for (int S = 1; S <= 40; ++S)
+                    for (int most = 1; most <= 16; ++most) {
+                        const int k = disco::draft_steps_per_launch(V, d, B, S, most, 148);
+                        const int launches = (S + k - 1) / k;
+                        if (k < 1 || k > most || k > S || (launches > 1 && (S + launches - 1) / launches != k) ||
+                            (k > 1 && 148 / ((k * B + 127) / 128) < 10))
+                            return std::printf("steps: %d x %d, B %d, %d, most %d: %d\\n", V, d, B, S, most, k), 1;
+                    }
+    // one sequence's ten steps fit a launch; narrow heads of many sequences, whose rows cost an epilogue each, do not gain by sixteen
+    if (disco::draft_steps_per_launch(32000, 768, 1, 10, 10, 148) != 10 || disco::draft_steps_per_launch(32000, 256, 130, 16, 16, 148) > 8) return 1;
     const int grids[] = {1, 2, 16, 148}, ds[] = {8, 320, 328, 768, 5120}, rows[] = {1, 33, 40, 64, 100, 128, 129, 256, 257, 640, 1000};
     for (int sms : grids)
         for (int V = 1; V < 80000; V += V < 300 || (V > 34000 && V < 38200) ? 1 : 97)
