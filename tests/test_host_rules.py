@@ -13,7 +13,10 @@ int main() {
     struct { int V, d, R; bool pairs; } measured[] = {
         {32000, 2048, 251, true}, {32000, 5120, 650, true}, {32000, 1024, 2432, true}, {32000, 2048, 1520, false}, {49152, 1024, 428, false},
         {8000, 1024, 512, false}, {8000, 1024, 2432, false}, {32000, 5120, 300, false}, {4000, 5120, 1520, true}, {32000, 5120, 1520, false},
-        {4000, 1024, 650, false}, {32000, 768, 650, false}, {32000, 5120, 128, false}};
+        {4000, 1024, 650, false}, {32000, 768, 650, false}, {32000, 5120, 128, false},
+        // (sizes at which the GPU tests check pairs)
+        {300, 1032, 129, true}, {300, 1032, 256, true}, {2500, 2056, 500, true}, {20000, 1032, 180, true}, {400, 2056, 1160, true},
+        {700, 2056, 1409, true}, {9000, 1032, 1409, true}, {4000, 4104, 1409, true}};
     for (auto& m : measured)
         if (VerifyTiling::in_pairs(m.R, m.V, m.d, 148) != m.pairs) return std::printf("pairs: %d x %d, %d\\n", m.V, m.d, m.R), 1;
     const int grids[] = {1, 2, 148}, vs[] = {1, 300, 32000, 151936}, ds[] = {8, 768, 2040, 2048, 6144};
@@ -68,7 +71,10 @@ int main() {
         {32000, 2048, 5, false, false, false}, {49152, 4096, 7, false, false, false}, {32000, 5120, 5, true, false, true},
         {32000, 5120, 3, true, true, false}, {32000, 768, 8, true, false, false}, {17000, 1024, 8, true, true, false},
         {32000, 1536, 8, true, false, true}, {5000, 2048, 2, true, false, false}, {5000, 2048, 8, false, false, false},
-        {32000, 2048, 2, false, false, true}, {32000, 2048, 4, false, false, true}, {17000, 2048, 4, true, true, true}};
+        {32000, 2048, 2, false, false, true}, {32000, 2048, 4, false, false, true}, {17000, 2048, 4, true, true, true},
+        // (sizes at which the GPU tests check pairs)
+        {8000, 2048, 2, true, false, true}, {8003, 2048, 4, true, false, true}, {12300, 2048, 5, true, false, true},
+        {300, 2048, 8, true, false, true}};
     for (auto& m : measured)
         if (disco::draft_in_pairs(m.V, m.d, m.MT, m.kept, m.stats, 148) != m.pairs) return std::printf("pairs: %d x %d, %d\\n", m.V, m.d, m.MT), 1;
     if (disco::draft_in_pairs(32000, 5120, 148, true, false, 147) || disco::draft_in_pairs(32000, 5120, 1, true, false, 148)) return 1;
