@@ -342,9 +342,9 @@ bool draft_batch_possible(const disco_ctx* c, int R) {
 }
 
 // Few hidden rows: the vocabulary on the TMEM lanes.  Up to 32, and beyond 16 only where a CTA has more than 32 vocabulary rows: with
-// fewer there is no shared bound, and then the lists of four rows are one warp's work after another (us, 512-wide heads of
-// 4000 / 8000 / 16000, vocabulary on the columns -> on the lanes: 32 rows 9.9 / 11.7 / 12.4 -> 13.5 / 11.7 / 11.6, 16 rows 9.7 / 11.5 /
-// 12.2 -> 9.9 / 10.3 / 10.4, 4 rows 9.7 / 9.8 / 10.5 -> 9.4 / 9.2 / 9.3).
+// fewer there is no shared bound, and then the lists of four rows are one warp's work after another (us, 512-wide heads of 4000 /
+// 8000, vocabulary on the columns -> on the lanes: 32 rows 9.9 / 11.7 -> 13.5 / 11.7, 16 rows 9.6 / 11.0 -> 9.6 / 9.5, 12 rows 9.5 / 9.8 -> 9.4 /
+// 9.2, 4 rows 9.8 / 9.9 -> 9.2 / 9.3; of 1024 x 2000, 4 / 9 / 16 rows 9.8 / 10.0 / 9.7 -> 9.3 / 10.1 / 10.5).
 bool draft_few_possible(const disco_ctx* c, int R) {
     return R <= 32 && c->sm_count >= 8 && (R <= 16 || c->V > 32 * (c->sm_count - draft_finishers(c->sm_count, R)));
 }

@@ -295,7 +295,7 @@ __device__ __forceinline__ void db_finish_row(const DraftBatchParams& p, const D
         // One warp is at work here, on code that it runs once, so what counts is the number of instructions: the four largest
         // entries of each lane's lists (places without an entry hold -inf), then ten times the largest of all, taken from the
         // lane that has it; a lane that has given four looks for its next four.  (Collecting the 30 - 50 entries above the bound
-        // and ranking them: 4400 cycles; only those not below the tenth largest of the lanes' heads: 3300; this: 1300.)
+        // and ranking them: 4400 cycles; only those not below the tenth largest of the lanes' heads: 3300; this: 1800.)
         float fourth[PER], more = DISCO_NEG_INF;      // the fourth entry of a list that goes on past it
 #pragma unroll
         for (int j = 0; j < PER; ++j) {

@@ -1,6 +1,6 @@
 // Merging the per-CTA partial records of one sequence with SEVERAL warps (the single-warp merge is
 // warp_merge_partials in stream_tail.cuh), and the small ranking helpers it is built from.  Used by the
-// persistent draft-phase kernel (its finishing CTA); the batched draft step uses the ranking helpers.  These
+// persistent draft-phase kernel (its finishing CTA); draft_few.cuh uses the ranking helpers.  These
 // phases are chains of dependent instructions on a few warps, so the code is written for short chains (values
 // through shared memory and independent comparisons instead of shuffle chains, the loads of a batch in flight
 // before the first use), not for few instructions.

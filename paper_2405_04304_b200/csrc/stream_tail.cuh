@@ -218,7 +218,8 @@ struct MergedPartials {
 };
 
 // Stamped records (80 bytes): five 16-byte pieces, each three payload words and the stamp of the launch
-// that wrote it: (m, Z, S | l0 l1 l2 | l3 l4 l5 | l6 l7 l8 | l9, key lo, key hi).  A 16-byte piece is
+// that wrote it: (m, Z, S | l0 l1 l2 | l3 l4 l5 | l6 l7 l8 | l9, key lo, key hi) in the persistent draft-phase
+// kernel (umma_gemv_loop.cuh); draft_batch.cuh has its own words and order.  A 16-byte piece is
 // written and read as one access, so a reader that finds the current stamp in a piece holds that
 // piece's payload of this launch, whatever the order in which the pieces travel: no fence, barrier or
 // counter lies between writer and reader (a fence at GPU scope costs about 1.5 us here).  The buffer is
@@ -234,16 +235,6 @@ __device__ __forceinline__ float4 load_relaxed_v4(const float4* p) {
                  : "l"(p)
                  : "memory");
     return v;
-}
-__device__ __forceinline__ void store_stamped_record(float4* rec, float m, float Z, float S, const float (&l)[kTopK],
-                                                     unsigned long long key, uint32_t stamp) {
-    const float sf = __uint_as_float(stamp);
-    store_relaxed_v4(rec, m, Z, S, sf);
-    store_relaxed_v4(rec + 1, l[0], l[1], l[2], sf);
-    store_relaxed_v4(rec + 2, l[3], l[4], l[5], sf);
-    store_relaxed_v4(rec + 3, l[6], l[7], l[8], sf);
-    store_relaxed_v4(rec + 4, l[9], __uint_as_float(static_cast<uint32_t>(key & 0xffffffffull)),
-                     __uint_as_float(static_cast<uint32_t>(key >> 32)), sf);
 }
 
 // Merge the NP partial records of one sequence (consecutive) by one warp.
