@@ -327,7 +327,8 @@ int disco_iteration(disco_ctx* ctx, const void* W_D, size_t w_step_stride, const
  * the hidden states, integer inputs and every output are host pointers.  Each call copies the
  * hidden states to device staging owned by the context, passes the small inputs and outputs through
  * pinned host memory that the GPU maps (the kernels read and write it in place), runs the kernels
- * and synchronises the stream before returning.  feats / target_ids may be NULL.
+ * and synchronises the stream before returning, also when it fails behind its first copy: nothing of it
+ * is in flight any more.  feats / target_ids may be NULL.
  */
 int disco_draft_step_host(disco_ctx* ctx, const void* W_D /*device*/, const void* h_D_host, int B,
                           const int32_t* pos_host, const int32_t* n_drafted_host,
@@ -346,7 +347,8 @@ int disco_verify_ragged_host(disco_ctx* ctx, const void* W_T /*device*/, const v
  * outputs token, conf, halt [sl_max, B], sl, n_accept, bonus [B] and pos_next [B] (or NULL; may be pos0_host
  * itself).  One copy of each hidden-state block to device staging (the target rows travel on a stream the
  * context owns while the draft phase runs on the caller's; the verification waits for them; small blocks of
- * pinned, 16-byte aligned memory are read by a kernel instead), the small arrays
+ * pinned, 16-byte aligned memory are read by a kernel instead, once the work before the call in the stream is
+ * done), the small arrays
  * through pinned memory that the GPU maps, the whole iteration on the device, one synchronisation.  The LM
  * heads and the classifier stay on the device.  Entries of steps a sequence did not take keep the caller's
  * values.  Like every *_host entry point it returns with its work done, and it cannot be captured in a graph.
